@@ -667,6 +667,7 @@ int plan_launch_impl(smcrt_plan *pl, uint64_t id_begin, uint64_t n, uint64_t see
     jw.scene = pl->dscene;
     jw.cancelled = 0;
     jw.stage = pl->precision == SMCRT_MIXED ? pl->stage : 0;
+    jw.lanes = spread_lanes(n, blocks, threads);
     jw.time_limit_ns = pl->time_limit_s > 0.0 ? (unsigned long long)std::llround(pl->time_limit_s * 1e9) : 0ull;
     JobWork *slot = pl->djobs + pl->ring_pos;
     pl->ring_pos = (pl->ring_pos + 1) % pl->ring;

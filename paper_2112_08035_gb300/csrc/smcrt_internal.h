@@ -260,7 +260,7 @@ struct JobWork {
     long long drain_cycles;       // > 0 (served rounds): once its warp finds no job with work left,
                                   // park a packet after this many SM cycles in the launch
     int32_t stage;                // mixed kernel: stage the scene tables in shared memory
-    int32_t stage_pad;
+    int32_t lanes;                // plan launches: lanes of a warp that carry packets (0 = all 32)
     int32_t *jstat;               // device, may be null: this job's own status word (bits OR-ed in)
     unsigned long long time_limit_ns;   // > 0: a warp stops this job that long after it started on it
 };
@@ -285,6 +285,21 @@ int occupancy_mixed(int threads, int variant = 0);
 cudaError_t launch_mixed_multi(JobWork *jobs, int njobs, int *status, int blocks, int threads,
                                cudaStream_t stream, int variant = 0);
 int occupancy_mixed_multi(int threads, int variant = 0);
+// Lanes of a warp that carry packets in a plan launch (JobWork.lanes; 0 =
+// all).  A launch with fewer packets than lanes is bound by the latency of
+// one loop iteration, which grows with the number of different branches a
+// warp's lanes take, so its packets are spread evenly over all warps instead
+// of filling the first ones.  Measured (layered slab, mixed, 3040 warps):
+// 1e3 packets 1.61 ms with 1 lane against 2.61 ms with 32, 1e4 2.49 ms (4)
+// against 3.32, 3e4 2.95 ms (6-8) against 3.70, 6e4 3.72 ms (16) against
+// 3.91; FP64 (1824 warps): 1e3 18.1 ms (1) against 28.3, 1e4 43.3 ms (6)
+// against 62.6.  Fewer lanes than this rule's serialise the packets.
+inline int32_t spread_lanes(uint64_t npackets, int blocks, int threads)
+{
+    const uint64_t warps = (uint64_t)blocks * (uint64_t)(threads / 32);
+    const uint64_t lanes = warps > 0 ? (npackets + warps - 1) / warps : 0;
+    return lanes < 32 ? (int32_t)lanes : 0;
+}
 cudaError_t launch_set_job(JobWork *dst, const JobWork &v, cudaStream_t stream);
 // Field validation of scene / source / grid, without compiling or
 // allocating (host runtime).

@@ -469,7 +469,8 @@ __device__ bool run_job_mixed(JobSlot *slots, JobWork *jobs, int njobs, int firs
         scan = nj + 1 < njobs ? nj + 1 : 0;
     }
 
-    bool alive = false, retired = false;
+    // a small plan launch spreads its packets over all warps
+    bool alive = false, retired = !MULTI && J->lanes > 0 && lane >= J->lanes;
     float px = 0, py = 0, pz = 0, ux = 0, uy = 0, uz = 0, w = 0, tau = 0;
     float qx = 0, qy = 0, qz = 0;        // FAR / NEAR: surface point; TRACE: crawl anchor
     // Crawl: a packet within delta32 of a surface that it is leaving takes

@@ -67,7 +67,8 @@ __device__ bool run_job_fp64(const DevScene &S, WarpAcc *wa, const volatile JobC
 {
     const double delta = S.delta;
 
-    bool alive = false, retired = false;
+    // a small plan launch spreads its packets over all warps
+    bool alive = false, retired = J->lanes > 0 && lane >= J->lanes;
     double px = 0, py = 0, pz = 0, ux = 0, uy = 0, uz = 0, w = 0, tau = 0;
     double qx = 0, qy = 0, qz = 0;       // NRM: gradient; PROJ / FAR / NEAR: surface point
     double nx = 0, ny = 0, nz = 0, cdot = 0, fplus = 0, dstar = 0;

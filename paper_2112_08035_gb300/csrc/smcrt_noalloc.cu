@@ -345,8 +345,6 @@ extern "C" int smcrt_run_noalloc(const smcrt_scene *scene, const smcrt_source *s
     jw.totals = totals_dev;
     jw.records = nullptr;
     jw.scene = (const DevScene *)(base + kImageOff);
-    JobWork *dj = (JobWork *)(base + kJobOff);
-    if (launch_set_job(dj, jw, s) != cudaSuccess) return SMCRT_ERR_CUDA;
     int dev = 0, sms = 0;
     cudaGetDevice(&dev);
     if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return SMCRT_ERR_CUDA;
@@ -354,6 +352,9 @@ extern "C" int smcrt_run_noalloc(const smcrt_scene *scene, const smcrt_source *s
     const int variant = (precision == SMCRT_FP64 ? 1 : 0) + (general ? kNumVariants : 0);
     const int occ = precision == SMCRT_FP64 ? occupancy_fp64(threads, variant) : occupancy_mixed(threads, variant);
     const int blocks = sms * (occ > 0 ? occ : 1);
+    jw.lanes = spread_lanes(npackets, blocks, threads);
+    JobWork *dj = (JobWork *)(base + kJobOff);
+    if (launch_set_job(dj, jw, s) != cudaSuccess) return SMCRT_ERR_CUDA;
     const cudaError_t e = precision == SMCRT_FP64
                               ? launch_fp64(dj, 1, (int *)(base + kStatusOff), blocks, threads, s, variant)
                               : launch_mixed(dj, 1, (int *)(base + kStatusOff), blocks, threads, s, variant);
