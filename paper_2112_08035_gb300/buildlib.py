@@ -40,7 +40,7 @@ UNITS = {
     "smcrt_noalloc.cu": [],
     "smcrt_microbench.cu": [],
 }
-HEADERS = ["smcrt_internal.h", "smcrt_kernel.cuh"]
+HEADERS = ["smcrt_internal.h", "smcrt_kernel.cuh", "smcrt_screen.cuh"]
 
 
 def _newer(src_list, target):

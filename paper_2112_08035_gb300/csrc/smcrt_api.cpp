@@ -580,6 +580,7 @@ int build_plan(smcrt_ctx *ctx, const smcrt_scene *sc, const smcrt_source *src, c
     }
     H.src_radius = src->radius;
     H.src_radius32 = (float)src->radius;
+    if (precision == SMCRT_FP64) fill_screen(H, sc, src, g, ins.data(), rr.data());
 
     std::vector<char> hb(total, 0);
     std::memcpy(hb.data() + o_scene, &H, sizeof H);

@@ -221,7 +221,54 @@ struct DevScene {
     double g_lo[3], g_hi[3], g_dl[3];
     float g_lo32[3], g_hi32[3], g_dl32[3], g_idl32[3];
     int32_t g_n[3], pad1;
+    // FP64 kernel: FP32 screening (smcrt_screen.cuh).  feps = 0: none.
+    uint64_t screen_mask;     // regions whose FP32 value has an error below feps
+    uint64_t fold_mask;       // regions that are left folds of unions and smooth unions
+    uint64_t soft_mask;       // soft regions (segment stepping)
+    float feps;               // error bound of an FP32 distance
+    float gm32[3];            // error bound of an FP32 position in voxels, per axis
 };
+
+// The screening fields of a compiled scene without general shapes: the error
+// bounds and region classes that smcrt_screen.cuh states.
+inline void fill_screen(DevScene &H, const smcrt_scene *sc, const smcrt_source *src, const smcrt_grid *g,
+                        const Instr *ins, const int2 *rr)
+{
+    double R = 0.0;
+    for (int a = 0; a < 3; ++a) {
+        R = std::fmax(R, std::fmax(std::fabs(sc->bbox_lo[a]), std::fabs(sc->bbox_hi[a])));
+        R = std::fmax(R, std::fabs(src->pos[a]) + std::fabs(src->radius));
+    }
+    for (int i = 0; i < sc->nprims; ++i) {
+        const smcrt_prim &P = sc->prims[i];
+        for (int a = 0; a < 3; ++a) {
+            if (P.kind == SMCRT_SPHERE) R = std::fmax(R, std::fabs(P.p[a]) + P.p[3]);
+            else if (P.kind == SMCRT_BOX) R = std::fmax(R, std::fabs(P.p[a]) + P.p[3 + a]);
+            else if (P.kind == SMCRT_CAPSULE)
+                R = std::fmax(R, std::fmax(std::fabs(P.p[a]), std::fabs(P.p[3 + a])) + P.p[6]);
+        }
+    }
+    R = R + 4.0 * sc->delta;
+    H.screen_mask = H.fold_mask = H.soft_mask = 0;
+    H.feps = 0.f;
+    for (int a = 0; a < 3; ++a) H.gm32[a] = INFINITY;
+    if (H.general || !(R > 1e-6 && R < 1e12)) return;   // FP32 squares stay in range
+    H.feps = (float)(R / 65536.0);
+    for (int r = 0; r < sc->nregions; ++r) {
+        const uint64_t bit = 1ull << r;
+        bool fold = rr[r].y - rr[r].x <= 60000;   // list entries are 16 bits
+        int smooth = 0;
+        for (int i = rr[r].x; i < rr[r].y; ++i) {
+            const int op = ins[i].op & 0xff;
+            if (op == SMCRT_OP_SMOOTH_UNION) ++smooth;
+            if (i > rr[r].x && (ins[i].prim < 0 || (op != SMCRT_OP_UNION && op != SMCRT_OP_SMOOTH_UNION))) fold = false;
+        }
+        if (fold) H.fold_mask |= bit;
+        if (fold || smooth <= 8) H.screen_mask |= bit;
+        if (region_is_soft(sc, r)) H.soft_mask |= bit;
+    }
+    for (int a = 0; a < 3; ++a) H.gm32[a] = (float)(g->n[a] * (16.0 / 16777216.0));
+}
 
 // A packet parked between serving rounds: its complete state at a trace
 // boundary (FP32 values are stored widened, which round-trips exactly), so

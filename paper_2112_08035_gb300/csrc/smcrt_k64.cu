@@ -4,7 +4,7 @@
 // reference algorithm (Sec. 2.3 sphere tracing and interface handling,
 // Eq. 1 free path, Sec. 3.1 HG scattering), so the int64 tallies equal the
 // FP64 CPU reference bit for bit for any packet count.
-#include "smcrt_kernel.cuh"
+#include "smcrt_screen.cuh"
 
 namespace smcrt {
 
@@ -16,23 +16,23 @@ __device__ __forceinline__ double hg_cos64(double g, double xi)
     if (fabs(g) < 1e-6) {
         c = 2.0 * xi - 1.0;
     } else {
-        const double t = (1.0 - g * g) / (1.0 - g + 2.0 * g * xi);
-        c = (1.0 + g * g - t * t) / (2.0 * g);
+        const double t = div64(1.0 - g * g, 1.0 - g + 2.0 * g * xi);
+        c = div64(1.0 + g * g - t * t, 2.0 * g);
     }
     return fmin(fmax(c, -1.0), 1.0);
 }
 
 __device__ __forceinline__ void normalise64(double &x, double &y, double &z)
 {
-    const double l = sqrt(x * x + y * y + z * z);
-    x = x / l;
-    y = y / l;
-    z = z / l;
+    const double l = sqrt64(x * x + y * y + z * z);
+    x = div64(x, l);
+    y = div64(y, l);
+    z = div64(z, l);
 }
 
 __device__ __forceinline__ void scatter64(double &ux, double &uy, double &uz, double ct, double xi_phi)
 {
-    const double st = sqrt((1.0 - ct) * (1.0 + ct));
+    const double st = sqrt64((1.0 - ct) * (1.0 + ct));
     double sp, cp;
     sincos2pi64(xi_phi, &sp, &cp);
     double b1[3], b2[3];
@@ -45,9 +45,72 @@ __device__ __forceinline__ void scatter64(double &ux, double &uy, double &uz, do
     ux = vx; uy = vy; uz = vz;
 }
 
-__device__ __forceinline__ double region_n64(const DevScene &S, int r)
+// Photon release (Sec. 2.1), out of line: position and direction from the
+// source and the first optical depth (Eq. 1), from one Philox call's words.
+struct Launched64 {
+    double px, py, pz, ux, uy, uz, tau;
+};
+
+static __device__ __noinline__ Launched64 launch64(const DevScene &S, uint4 r)
 {
-    return r < 0 ? S.ambient_n : __ldg(S.reg64 + 8 * r + 3);
+    Launched64 o;
+    const double x0 = u01_64(r.x), x1 = u01_64(r.y), x3 = u01_64(r.w);
+    o.px = S.src_pos[0]; o.py = S.src_pos[1]; o.pz = S.src_pos[2];
+    o.ux = S.src_dir[0]; o.uy = S.src_dir[1]; o.uz = S.src_dir[2];
+    if (S.src_kind == 1 || S.src_kind == 2) {
+        double c1, c2;
+        if (S.src_kind == 1) {
+            const double rho = S.src_radius * sqrt64(x0);
+            double sn, cs;
+            sincos2pi64(x1, &sn, &cs);
+            c1 = rho * cs;
+            c2 = rho * sn;
+        } else {
+            c1 = S.src_radius * (2.0 * x0 - 1.0);
+            c2 = S.src_radius * (2.0 * x1 - 1.0);
+        }
+        o.px = S.src_pos[0] + c1 * S.src_b1[0] + c2 * S.src_b2[0];
+        o.py = S.src_pos[1] + c1 * S.src_b1[1] + c2 * S.src_b2[1];
+        o.pz = S.src_pos[2] + c1 * S.src_b1[2] + c2 * S.src_b2[2];
+    } else if (S.src_kind == 3) {
+        const double ctt = 2.0 * x0 - 1.0;
+        const double st = sqrt64((1.0 - ctt) * (1.0 + ctt));
+        double sn, cs;
+        sincos2pi64(x1, &sn, &cs);
+        o.ux = st * cs; o.uy = st * sn; o.uz = ctt;
+    }
+    o.tau = -ln64(x3);
+    return o;
+}
+
+// After a Fresnel decision at the surface point q (Sec. 2.3), out of line:
+// the reflected or refracted direction and the point 2 delta beyond q on the
+// packet's side (ee = 2 delta, signed like u.n).
+struct Crossed64 {
+    double px, py, pz, ux, uy, uz;
+};
+
+static __device__ __noinline__ Crossed64 cross64(double ux, double uy, double uz, double qx, double qy, double qz,
+                                                 double nx, double ny, double nz, double cdot, double ee, double n1,
+                                                 double n2, double ct, bool reflect)
+{
+    Crossed64 o;
+    double sx;
+    if (reflect) {
+        const double c2 = 2.0 * cdot;
+        ux = ux - c2 * nx; uy = uy - c2 * ny; uz = uz - c2 * nz;
+        sx = -ee;
+    } else {
+        const double eta = div64(n1, n2);
+        const double ci = fabs(cdot);
+        const double k = (cdot > 0.0 ? 1.0 : -1.0) * (eta * ci - ct);
+        ux = eta * ux - k * nx; uy = eta * uy - k * ny; uz = eta * uz - k * nz;
+        sx = ee;
+    }
+    normalise64(ux, uy, uz);
+    o.ux = ux; o.uy = uy; o.uz = uz;
+    o.px = qx + sx * nx; o.py = qy + sx * ny; o.pz = qz + sx * nz;
+    return o;
 }
 
 struct WarpShared {
@@ -70,11 +133,11 @@ __device__ bool run_job_fp64(const DevScene &S, WarpAcc *wa, const volatile JobC
     // a small plan launch spreads its packets over all warps
     bool alive = false, retired = J->lanes > 0 && lane >= J->lanes;
     double px = 0, py = 0, pz = 0, ux = 0, uy = 0, uz = 0, w = 0, tau = 0;
-    double qx = 0, qy = 0, qz = 0;       // NRM: gradient; PROJ / FAR / NEAR: surface point
-    double nx = 0, ny = 0, nz = 0, cdot = 0, fplus = 0, dstar = 0;
-    int phase = kTrace, sub = 0, istar = -1, reg = -1, rfar = -1;
+    double dstar = 0;
+    int phase = kTrace, istar = -1, reg = -1;
     int nsteps = 0;
-    unsigned pscat = 0, npieces = 0;
+    unsigned pscat = 0, npieces = 0, nev = 0;
+    int waited = 0;                      // lane iterations that arrived packets have waited (warp-uniform)
     long long pA = 0, pG = 0;
     uint32_t id_lo = 0, id_hi = 0, event = 0;
     uint32_t t_acq = 0;
@@ -143,123 +206,77 @@ __device__ bool run_job_fp64(const DevScene &S, WarpAcc *wa, const volatile JobC
         }
 
         // ---- 2. the scene evaluation of this iteration
-        const double ee = 2.0 * delta * (cdot > 0.0 ? 1.0 : -1.0);
-        double ex = px, ey = py, ez = pz;
-        int sel = -2;
-        if (phase == kNrm) {
-            const double hh = (sub & 1) ? -delta : delta;
-            const int a = sub >> 1;
-            if (a == 0) ex = px + hh; else if (a == 1) ey = py + hh; else ez = pz + hh;
-            sel = istar;
-        } else if (phase == kProj) {
-            ex = qx; ey = qy; ez = qz;
-            sel = istar;
-        } else if (phase == kFar) {
-            ex = qx + ee * nx; ey = qy + ee * ny; ez = qz + ee * nz;
-        } else if (phase == kNear) {
-            ex = qx - ee * nx; ey = qy - ee * ny; ez = qz - ee * nz;
-        }
-        const Eval64 E = scene_eval64<G>(S, ex, ey, ez, sel);
-        {
-            const unsigned ev = __ballot_sync(SMCRT_FULL, alive && phase != kLaunch);
-            if (lane == 0) wadd(wa, kEvals, __popc(ev));
-        }
+        Eval64 E{};
+        const bool evals = alive && phase == kTrace;
+        if (G)
+            E = scene_eval64<G>(S, px, py, pz, -2);
+        else if (evals)
+            E = scene_eval64_screened(S, px, py, pz, -2, kForTrace);
+        nev += evals;
 
         // ---- 3. classify
         bool move = false, fresnel = false, iter_done = false;
         bool seg_step = false;                 // a tracing move that segment stepping may lengthen
         bool fin = false;                      // the packet ends this iteration
+        bool out = false;                      // ... leaving the volume: R or T
         long long fin_R = 0, fin_T = 0, fin_K = 0;
-        double L = 0.0, R = 1.0, ct = 0.0, n1 = 0.0, n2 = 0.0;
-        if (alive) {
-            if (phase == kTrace) {
-                if (E.dbox > 0.0) {                      // outside the volume of interest
-                    {                                          // leaves the volume: R or T
-                        const long long v = fx64(w);
-                        if (ux * S.src_dir[0] + uy * S.src_dir[1] + uz * S.src_dir[2] < 0.0) fin_R = v; else fin_T = v;
-                        fin = true;
-                        alive = false;
-                    }
+        double L = 0.0;
+        if (evals) {
+            if (E.dbox > 0.0) {                          // outside the volume of interest
+                out = true;
+            } else {
+                reg = E.region;
+                if (E.dmin < delta) {                    // on a boundary
+                    istar = E.istar;
+                    dstar = E.dstar;
+                    phase = kArrive;
                 } else {
-                    reg = E.region;
-                    if (E.dmin < delta) {                // on a boundary: find its normal
-                        istar = E.istar;
-                        dstar = E.dstar;
-                        phase = kNrm;
-                        sub = 0;
-                    } else {
-                        L = E.dmin - 0.5 * delta;        // stop short of the surface
-                        move = true;
-                        seg_step = S.stepping == SMCRT_STEP_SEGMENT;
-                    }
+                    L = E.dmin - 0.5 * delta;            // stop short of the surface
+                    move = true;
+                    seg_step = S.stepping == SMCRT_STEP_SEGMENT;
                 }
-            } else if (phase == kNrm) {
-                const double f = E.dsel;
-                if ((sub & 1) == 0) {
-                    fplus = f;
-                } else {
-                    const double gg = fplus - f;
-                    const int a = sub >> 1;
-                    if (a == 0) qx = gg; else if (a == 1) qy = gg; else qz = gg;
-                }
-                if (++sub == 6) {
-                    const double l2 = qx * qx + qy * qy + qz * qz;
-                    bool approaching = false;
-                    if (l2 > 0.0) {
-                        const double l = sqrt(l2);
-                        nx = qx / l; ny = qy / l; nz = qz / l;
-                        cdot = ux * nx + uy * ny + uz * nz;
-                        approaching = (cdot > 0.0 && dstar < 0.0) || (cdot < 0.0 && dstar >= 0.0);
-                    }
-                    if (!approaching) {
+            }
+        }
+
+        // ---- 3b. the packets at a surface, once enough of them wait: the
+        // routine costs as much for one lane as for all, about ten times
+        // what a waiting lane loses per iteration
+        Interface64 I;
+        I.R = 1.0;
+        const unsigned arrived = __ballot_sync(SMCRT_FULL, alive && phase == kArrive);
+        if (arrived != 0u) {
+            waited += __popc(arrived);
+            const unsigned here = __ballot_sync(SMCRT_FULL, alive);
+            if (3 * waited >= __popc(here) || here == arrived) {
+                waited = 0;
+                if (alive && phase == kArrive) {
+                    I = interface64<G>(S, px, py, pz, ux, uy, uz, istar, dstar);
+                    nev += I.evals;
+                    phase = kTrace;
+                    if (I.what == kIntfForced) {
                         L = delta;                       // forced step along u
                         move = true;
-                    } else if (istar < 0) {
-                        {                                          // leaves the volume: R or T
-                        const long long v = fx64(w);
-                        if (ux * S.src_dir[0] + uy * S.src_dir[1] + uz * S.src_dir[2] < 0.0) fin_R = v; else fin_T = v;
-                        fin = true;
-                        alive = false;
-                    }                        // outward through the bounding box
+                    } else if (I.what == kIntfEscape) {
+                        out = true;                      // outward through the bounding box
                     } else {
                         wadd(wa, kIntf, 1);
-                        qx = px; qy = py; qz = pz;
-                        phase = kProj;
-                        sub = 0;
-                    }
-                }
-            } else if (phase == kProj) {
-                const double dq = E.dsel;
-                if (fabs(dq) <= delta * 1e-3) {
-                    phase = kFar;
-                } else {
-                    qx = qx - dq * nx; qy = qy - dq * ny; qz = qz - dq * nz;
-                    if (++sub == 3) phase = kFar;
-                }
-            } else if (phase == kFar) {
-                rfar = E.region;
-                phase = kNear;
-            } else if (phase == kNear) {
-                n1 = region_n64(S, E.region);
-                n2 = region_n64(S, rfar);
-                if (n1 == n2) {
-                    px = qx + ee * nx; py = qy + ee * ny; pz = qz + ee * nz;
-                    phase = kTrace;
-                    iter_done = true;
-                } else {
-                    wadd(wa, kFres, 1);
-                    fresnel = true;
-                    const double ci = fabs(cdot);
-                    const double eta = n1 / n2;
-                    const double st2 = eta * eta * ((1.0 - ci) * (1.0 + ci));
-                    if (st2 < 1.0) {
-                        ct = sqrt(1.0 - st2);
-                        const double rs = (n1 * ci - n2 * ct) / (n1 * ci + n2 * ct);
-                        const double rp = (n1 * ct - n2 * ci) / (n1 * ct + n2 * ci);
-                        R = 0.5 * (rs * rs + rp * rp);
+                        if (I.what == kIntfMatched) {
+                            const double ee = 2.0 * delta * (I.cdot > 0.0 ? 1.0 : -1.0);
+                            px = I.qx + ee * I.nx; py = I.qy + ee * I.ny; pz = I.qz + ee * I.nz;
+                            iter_done = true;
+                        } else {
+                            wadd(wa, kFres, 1);
+                            fresnel = true;
+                        }
                     }
                 }
             }
+        }
+        if (SMCRT_RARE(out)) {
+            const long long v = fx64(w);
+            if (ux * S.src_dir[0] + uy * S.src_dir[1] + uz * S.src_dir[2] < 0.0) fin_R = v; else fin_T = v;
+            fin = true;
+            alive = false;
         }
 
         // ---- 4. move: interaction point or sphere-trace step, one tally site
@@ -269,12 +286,27 @@ __device__ bool run_job_fp64(const DevScene &S, WarpAcc *wa, const volatile JobC
             if (reg >= 0) mu_t = __ldg(S.reg64 + 8 * reg + 4);
             interact = mu_t > 0.0 && tau < mu_t * L;
             if (seg_step && !interact) {           // segment stepping: a longer move along u
-                L = fmax(L, segment_bound64<G>(S, E.dsoft, E.dbox, px, py, pz, ux, uy, uz));
-                interact = mu_t > 0.0 && tau < mu_t * L;
+                if (G) {
+                    L = fmax(L, segment_bound64<G>(S, E.dsoft, E.dbox, px, py, pz, ux, uy, uz));
+                    interact = mu_t > 0.0 && tau < mu_t * L;
+                } else {
+                    // FP32 first: most of these packets interact before the
+                    // bound, whose value then does not matter
+                    const float p[3] = {(float)px, (float)py, (float)pz}, u[3] = {(float)ux, (float)uy, (float)uz};
+                    const float lo = segment_screen(S, (float)E.dsoft, p, u);
+                    interact = mu_t > 0.0 && (float)tau * kScrUp < (float)mu_t * lo * kScrDown;
+                    if (!interact) {
+                        L = fmax(L, segment_bound64_screened(S, E.dsoft, E.dbox, px, py, pz, ux, uy, uz));
+                        interact = mu_t > 0.0 && tau < mu_t * L;
+                    }
+                }
             }
-            const double seg = interact ? tau / mu_t : L;
+            const double seg = interact ? div64(tau, mu_t) : L;
             long long *const flu = (long long *)jc->flu;
-            if (flu) tally64(S, flu, px, py, pz, ux, uy, uz, seg, w, &npieces);
+            if (flu) {
+                if (G) npieces += tally64(S, flu, px, py, pz, ux, uy, uz, seg, w);
+                else npieces += tally64_screened(S, flu, px, py, pz, ux, uy, uz, seg, w);
+            }
             px = px + seg * ux; py = py + seg * uy; pz = pz + seg * uz;
             if (!interact) tau = tau - mu_t * L;
             phase = kTrace;
@@ -282,7 +314,7 @@ __device__ bool run_job_fp64(const DevScene &S, WarpAcc *wa, const volatile JobC
         }
 
         // ---- 5. one Philox call for every lane that draws this iteration
-        const bool draws = alive && (phase == kLaunch || interact || (fresnel && R < 1.0));
+        const bool draws = alive && (phase == kLaunch || interact || (fresnel && I.R < 1.0));
         uint4 r = make_uint4(0u, 0u, 0u, 0u);
         if (__any_sync(SMCRT_FULL, draws)) {
             r = philox4x32_10(make_uint4(event, 0u, id_lo, id_hi), jc->k0, jc->k1);
@@ -290,33 +322,11 @@ __device__ bool run_job_fp64(const DevScene &S, WarpAcc *wa, const volatile JobC
         }
 
         // ---- 6. consumers
-        if (alive && phase == kLaunch) {                 // photon release
-            const double x0 = u01_64(r.x), x1 = u01_64(r.y), x3 = u01_64(r.w);
-            px = S.src_pos[0]; py = S.src_pos[1]; pz = S.src_pos[2];
-            ux = S.src_dir[0]; uy = S.src_dir[1]; uz = S.src_dir[2];
-            if (S.src_kind == 1 || S.src_kind == 2) {
-                double c1, c2;
-                if (S.src_kind == 1) {
-                    const double rho = S.src_radius * sqrt(x0);
-                    double sn, cs;
-                    sincos2pi64(x1, &sn, &cs);
-                    c1 = rho * cs;
-                    c2 = rho * sn;
-                } else {
-                    c1 = S.src_radius * (2.0 * x0 - 1.0);
-                    c2 = S.src_radius * (2.0 * x1 - 1.0);
-                }
-                px = S.src_pos[0] + c1 * S.src_b1[0] + c2 * S.src_b2[0];
-                py = S.src_pos[1] + c1 * S.src_b1[1] + c2 * S.src_b2[1];
-                pz = S.src_pos[2] + c1 * S.src_b1[2] + c2 * S.src_b2[2];
-            } else if (S.src_kind == 3) {
-                const double ctt = 2.0 * x0 - 1.0;
-                const double st = sqrt((1.0 - ctt) * (1.0 + ctt));
-                double sn, cs;
-                sincos2pi64(x1, &sn, &cs);
-                ux = st * cs; uy = st * sn; uz = ctt;
-            }
-            tau = -ln64(x3);
+        if (SMCRT_RARE(alive && phase == kLaunch)) {                 // photon release
+            const Launched64 o = launch64(S, r);
+            px = o.px; py = o.py; pz = o.pz;
+            ux = o.ux; uy = o.uy; uz = o.uz;
+            tau = o.tau;
             w = 1.0;
             nsteps = 0; pA = 0; pG = 0; pscat = 0;
             phase = kTrace;
@@ -340,21 +350,13 @@ __device__ bool run_job_fp64(const DevScene &S, WarpAcc *wa, const volatile JobC
             }
             tau = -ln64(u01_64(r.w));
         }
-        if (fresnel) {                                   // Fresnel reflection / Snell refraction
-            const bool reflect = R < 1.0 ? (u01_64(r.x) <= R) : true;
-            if (reflect) {
-                const double c2 = 2.0 * cdot;
-                ux = ux - c2 * nx; uy = uy - c2 * ny; uz = uz - c2 * nz;
-                normalise64(ux, uy, uz);
-                px = qx - ee * nx; py = qy - ee * ny; pz = qz - ee * nz;
-            } else {
-                const double eta = n1 / n2;
-                const double ci = fabs(cdot);
-                const double k = (cdot > 0.0 ? 1.0 : -1.0) * (eta * ci - ct);
-                ux = eta * ux - k * nx; uy = eta * uy - k * ny; uz = eta * uz - k * nz;
-                normalise64(ux, uy, uz);
-                px = qx + ee * nx; py = qy + ee * ny; pz = qz + ee * nz;
-            }
+        if (SMCRT_RARE(fresnel)) {                                 // Fresnel reflection / Snell refraction
+            const bool reflect = I.R < 1.0 ? (u01_64(r.x) <= I.R) : true;
+            const double ee = 2.0 * delta * (I.cdot > 0.0 ? 1.0 : -1.0);
+            const Crossed64 o = cross64(ux, uy, uz, I.qx, I.qy, I.qz, I.nx, I.ny, I.nz, I.cdot, ee, I.n1, I.n2, I.ct,
+                                        reflect);
+            px = o.px; py = o.py; pz = o.pz;
+            ux = o.ux; uy = o.uy; uz = o.uz;
             phase = kTrace;
             iter_done = true;
         }
@@ -368,10 +370,11 @@ __device__ bool run_job_fp64(const DevScene &S, WarpAcc *wa, const volatile JobC
             }
         }
         // ---- a terminated packet: one bookkeeping site per iteration
-        if (fin) {
+        if (SMCRT_RARE(fin)) {
             wadd(wa, kR, fin_R); wadd(wa, kT, fin_T); wadd(wa, kKilled, fin_K);
             wadd(wa, kA, pA); wadd(wa, kGain, pG); wadd(wa, kScat, pscat); wadd(wa, kSteps, nsteps);
-            wadd(wa, kPackets, 1);
+            wadd(wa, kPackets, 1); wadd(wa, kEvals, nev);
+            nev = 0;
             smcrt_packet_record *const recs = (smcrt_packet_record *)jc->recs;
             if (recs) {
                 smcrt_packet_record r;
@@ -382,7 +385,7 @@ __device__ bool run_job_fp64(const DevScene &S, WarpAcc *wa, const volatile JobC
             }
         }
         // ---- park a straggler at a trace boundary (serving rounds only)
-        if (alive && phase == kTrace && jc->budget > 0u && (uint32_t)clock() - t_acq > jc->budget) {
+        if (SMCRT_RARE(alive && phase == kTrace && jc->budget > 0u && (uint32_t)clock() - t_acq > jc->budget)) {
             JobDefer *const dfr = (JobDefer *)jc->dfr;
             const int din = jc->din;
             const unsigned k = atomicAdd(&dfr->count[1 - din], 1u);
@@ -394,7 +397,8 @@ __device__ bool run_job_fp64(const DevScene &S, WarpAcc *wa, const volatile JobC
                 d.pA = pA; d.pG = pG;
                 d.id_lo = id_lo; d.id_hi = id_hi; d.event = event;
                 d.nsteps = (uint32_t)nsteps; d.pscat = pscat;
-                wadd(wa, kParked, 1);
+                wadd(wa, kParked, 1); wadd(wa, kEvals, nev);
+                nev = 0;
                 alive = false;
             } else {
                 atomicAdd(&dfr->overflow, 1u);

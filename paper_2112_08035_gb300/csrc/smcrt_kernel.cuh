@@ -88,6 +88,13 @@ __device__ __forceinline__ float u01_32(uint32_t w) { return ((float)(w >> 9) + 
 // series to s^21; sin/cos by reduction to the nearest quarter turn and the
 // Taylor series of sin to a^17, cos to a^16 on |a| <= pi/4.
 // ---------------------------------------------------------------------------
+// FP64 quotient and square root, one copy each: a call costs far less than
+// the ten or so FP64 instructions (16 cycles each) it leads to, while inline
+// copies made the FP64 kernel 194 KB of code, more than the instruction cache
+// holds (15 cycles of fetch stall per instruction).
+static __device__ __noinline__ double div64(double a, double b) { return a / b; }
+static __device__ __noinline__ double sqrt64(double a) { return sqrt(a); }
+
 __device__ __forceinline__ double ln64(double x)
 {
     const long long b = __double_as_longlong(x);
@@ -97,7 +104,7 @@ __device__ __forceinline__ double ln64(double x)
         m = m * 0.5;
         e = e + 1;
     }
-    const double s = (m - 1.0) / (m + 1.0);
+    const double s = div64(m - 1.0, m + 1.0);
     const double z = s * s;
     double t = 1.0 / 21.0;
     t = t * z + 1.0 / 19.0;
@@ -163,12 +170,34 @@ __device__ __forceinline__ long long fx32(float x) { return __float2ll_rn(x * 42
 struct Eval64 { double dmin, dstar, dsel, dbox, dsoft; int istar, region; };
 struct Eval32 { float dmin, dstar, dsel, dbox, dsoft; int istar, region; };
 
+// The larger of two numbers (not NaN), compared as integers.
+__device__ __forceinline__ double max64(double a, double b)
+{
+    long long x = __double_as_longlong(a), y = __double_as_longlong(b);
+    x ^= (long long)((unsigned long long)(x >> 63) >> 1);
+    y ^= (long long)((unsigned long long)(y >> 63) >> 1);
+    return x > y ? a : b;
+}
+
+// a < b for numbers that are not negative (nor NaN).
+__device__ __forceinline__ bool less64(double a, double b)
+{
+    return __double_as_longlong(a) < __double_as_longlong(b);
+}
+
 __device__ __forceinline__ double box64(double x, double y, double z, double cx, double cy, double cz,
                                         double hx, double hy, double hz)
 {
     const double qx = fabs(x - cx) - hx, qy = fabs(y - cy) - hy, qz = fabs(z - cz) - hz;
+    // At most one axis outside: the root of a square is the value itself
+    // (binary, round to nearest, no underflow), and the sum adds zeros.  The
+    // largest q is found with integer compares, off the FP64 pipe.
+    const double q = max64(qx, max64(qy, qz));
+    const int one = (__double2hiint(qx) >= 0) + (__double2hiint(qy) >= 0) + (__double2hiint(qz) >= 0);
+    const int hq = __double2hiint(q);
+    if (one == 0 || (one == 1 && hq > 0x20000000 && hq < 0x5f000000)) return q;
     const double mx = fmax(qx, 0.0), my = fmax(qy, 0.0), mz = fmax(qz, 0.0);
-    const double outside = sqrt(mx * mx + my * my + mz * mz);
+    const double outside = sqrt64(mx * mx + my * my + mz * mz);
     const double inside = fmin(fmax(qx, fmax(qy, qz)), 0.0);
     return outside + inside;
 }
@@ -189,13 +218,13 @@ static __device__ __noinline__ double round64(int kind, const double *P, double 
 {
     const double dx = x - __ldg(P), dy = y - __ldg(P + 1), dz = z - __ldg(P + 2);
     if (kind == 3) {                     // torus about z: core circle distance - tube radius
-        const double ring = sqrt(dx * dx + dy * dy) - __ldg(P + 3);
-        return sqrt(ring * ring + dz * dz) - __ldg(P + 4);
+        const double ring = sqrt64(dx * dx + dy * dy) - __ldg(P + 3);
+        return sqrt64(ring * ring + dz * dz) - __ldg(P + 4);
     }
-    const double a = sqrt(dx * dx + dy * dy) - __ldg(P + 3);   // capped cylinder along z
+    const double a = sqrt64(dx * dx + dy * dy) - __ldg(P + 3);   // capped cylinder along z
     const double b = fabs(dz) - __ldg(P + 4);
     const double ma = fmax(a, 0.0), mb = fmax(b, 0.0);
-    return fmin(fmax(a, b), 0.0) + sqrt(ma * ma + mb * mb);
+    return fmin(fmax(a, b), 0.0) + sqrt64(ma * ma + mb * mb);
 }
 
 // Primitive distances in local coordinates (kind 0..4, Sec. 2.2 and the
@@ -208,17 +237,17 @@ __device__ __forceinline__ double base64(int kind, const double *P, double x, do
 {
     if (kind == 0) {
         const double dx = x - __ldg(P), dy = y - __ldg(P + 1), dz = z - __ldg(P + 2);
-        return sqrt(dx * dx + dy * dy + dz * dz) - __ldg(P + 3);
+        return sqrt64(dx * dx + dy * dy + dz * dz) - __ldg(P + 3);
     }
     if (kind == 1)
         return box64(x, y, z, __ldg(P), __ldg(P + 1), __ldg(P + 2), __ldg(P + 3), __ldg(P + 4), __ldg(P + 5));
     if (!G || kind == 2) {
         const double pax = x - __ldg(P), pay = y - __ldg(P + 1), paz = z - __ldg(P + 2);
         const double bax = __ldg(P + 3), bay = __ldg(P + 4), baz = __ldg(P + 5);
-        double t = (pax * bax + pay * bay + paz * baz) / __ldg(P + 7);
+        double t = div64(pax * bax + pay * bay + paz * baz, __ldg(P + 7));
         t = fmin(fmax(t, 0.0), 1.0);
         const double dx = pax - bax * t, dy = pay - bay * t, dz = paz - baz * t;
-        return sqrt(dx * dx + dy * dy + dz * dz) - __ldg(P + 6);
+        return sqrt64(dx * dx + dy * dy + dz * dz) - __ldg(P + 6);
     }
     return round64(kind, P, x, y, z);
 }
@@ -231,9 +260,9 @@ static __device__ __noinline__ double xprim64(const DevScene &S, int kind, int i
     const double *X = S.xf64 + kXf64 * i;
     const double vx = x - __ldg(X + 9), vy = y - __ldg(X + 10), vz = z - __ldg(X + 11);
     const double s = __ldg(X + 12);
-    double q0 = (__ldg(X) * vx + __ldg(X + 3) * vy + __ldg(X + 6) * vz) / s;
-    double q1 = (__ldg(X + 1) * vx + __ldg(X + 4) * vy + __ldg(X + 7) * vz) / s;
-    double q2 = (__ldg(X + 2) * vx + __ldg(X + 5) * vy + __ldg(X + 8) * vz) / s;
+    double q0 = div64(__ldg(X) * vx + __ldg(X + 3) * vy + __ldg(X + 6) * vz, s);
+    double q1 = div64(__ldg(X + 1) * vx + __ldg(X + 4) * vy + __ldg(X + 7) * vz, s);
+    double q2 = div64(__ldg(X + 2) * vx + __ldg(X + 5) * vy + __ldg(X + 8) * vz, s);
     const int op = (int)__ldg(X + 13);
     const double a0 = __ldg(X + 14), a1 = __ldg(X + 15), a2 = __ldg(X + 16), a3 = __ldg(X + 17);
     double L = 1.0;
@@ -242,20 +271,20 @@ static __device__ __noinline__ double xprim64(const DevScene &S, int kind, int i
         q1 = q1 - fmin(fmax(q1, -a1), a1);
         q2 = q2 - fmin(fmax(q2, -a2), a2);
     } else if (op == 2 || op == 3) {     // twist about z / bend in x-y
-        const double rho = sqrt(q0 * q0 + q1 * q1);
+        const double rho = sqrt64(q0 * q0 + q1 * q1);
         double sn, cs;
         sincos2pi64(a0 * (op == 2 ? q2 : q0), &sn, &cs);
         const double rx = cs * q0 - sn * q1;
         const double ry = sn * q0 + cs * q1;
         q0 = rx; q1 = ry;
         const double m = 6.283185307179586 * a0 * fmax(rho, a1);   // stretch bound of the map
-        L = op == 2 ? 0.5 * (m + sqrt(m * m + 4.0)) : 1.0 + m;
+        L = op == 2 ? 0.5 * (m + sqrt64(m * m + 4.0)) : 1.0 + m;
     } else if (op == 4) {                // repetition: nearest copy
         if (a0 > 0.0) { double k = floor(q0 / a0 + 0.5); k = fmin(fmax(k, -a3), a3); q0 = q0 - a0 * k; }
         if (a1 > 0.0) { double k = floor(q1 / a1 + 0.5); k = fmin(fmax(k, -a3), a3); q1 = q1 - a1 * k; }
         if (a2 > 0.0) { double k = floor(q2 / a2 + 0.5); k = fmin(fmax(k, -a3), a3); q2 = q2 - a2 * k; }
     }
-    return s * base64<true>(kind, S.p64 + 8 * i, q0, q1, q2) / L;
+    return div64(s * base64<true>(kind, S.p64 + 8 * i, q0, q1, q2), L);
 }
 
 template <bool G>
@@ -344,7 +373,7 @@ __device__ __forceinline__ double csg64(int op, double a, double b, double k)
     if (op == 1) return fmin(a, b);
     if (op == 3) return fmax(a, b);
     if (op == 4) return fmax(a, -b);
-    double h = 0.5 + 0.5 * (b - a) / k;
+    double h = 0.5 + div64(0.5 * (b - a), k);
     h = fmin(fmax(h, 0.0), 1.0);
     const double m = b * (1.0 - h) + a * h;
     return m - k * h * (1.0 - h);
@@ -695,16 +724,16 @@ __device__ __forceinline__ double seg_sphere64(const double *P, double d, double
     double t;
     if (d > 0.0) {                       // outside: entry of the grown sphere (near root)
         if (b >= 0.0 || disc < 0.0) return __longlong_as_double(0x7ff0000000000000LL);
-        t = cc / (sqrt(disc) - b);
+        t = div64(cc, sqrt64(disc) - b);
     } else {                             // inside: exit of the shrunk sphere
         if (disc < 0.0) return 0.0;
-        if (b > 0.0) t = -cc / (b + sqrt(disc));
-        else t = sqrt(disc) - b;
+        if (b > 0.0) t = div64(-cc, b + sqrt64(disc));
+        else t = sqrt64(disc) - b;
     }
     return t > 0.0 ? t : 0.0;
 }
 
-__device__ __forceinline__ double seg_box64(double cx, double cy, double cz, double hx, double hy, double hz,
+static __device__ __noinline__ double seg_box64(double cx, double cy, double cz, double hx, double hy, double hz,
                                             double d, double px, double py, double pz, double ux, double uy,
                                             double uz, double dh)
 {
@@ -716,7 +745,7 @@ __device__ __forceinline__ double seg_box64(double cx, double cy, double cz, dou
     for (int a = 0; a < 3; ++a) {
         const double lo = c[a] - (h[a] + e), hi = c[a] + (h[a] + e);
         if (u[a] != 0.0) {
-            const double t0 = (lo - p[a]) / u[a], t1 = (hi - p[a]) / u[a];
+            const double t0 = div64(lo - p[a], u[a]), t1 = div64(hi - p[a], u[a]);
             tn = fmax(tn, fmin(t0, t1));
             tf = fmin(tf, fmax(t0, t1));
         } else if (p[a] < lo || p[a] > hi) {
@@ -742,13 +771,13 @@ __device__ __forceinline__ void ray_ball64(double ox, double oy, double oz, doub
     t0 = __longlong_as_double(0x7ff0000000000000LL);
     t1 = -t0;
     if (disc < 0.0) return;
-    const double sq = sqrt(disc);
+    const double sq = sqrt64(disc);
     if (b > 0.0) {
         const double q = -(b + sq);
-        t0 = q; t1 = cc / q;
+        t0 = q; t1 = div64(cc, q);
     } else {
         const double q = sq - b;
-        if (q > 0.0) { t1 = q; t0 = cc / q; }
+        if (q > 0.0) { t1 = q; t0 = div64(cc, q); }
         else { t0 = 0.0; t1 = 0.0; }
     }
 }
@@ -766,12 +795,12 @@ __device__ __forceinline__ void ray_cylinder64(double ox, double oy, double oz, 
     double lo = -inf, hi = inf;
     t0 = inf; t1 = -inf;
     if (uw != 0.0) {                     // between the end planes
-        const double s0 = -ow / uw, s1 = (L2 - ow) / uw;
+        const double s0 = div64(-ow, uw), s1 = div64(L2 - ow, uw);
         lo = fmin(s0, s1); hi = fmax(s0, s1);
     } else if (ow < 0.0 || ow > L2) {
         return;
     }
-    const double k = uw / L2, m = ow / L2;
+    const double k = div64(uw, L2), m = div64(ow, L2);
     const double vx = ux - k * bax, vy = uy - k * bay, vz = uz - k * baz;
     const double wx = ox - m * bax, wy = oy - m * bay, wz = oz - m * baz;
     const double A = vx * vx + vy * vy + vz * vz;
@@ -780,14 +809,14 @@ __device__ __forceinline__ void ray_cylinder64(double ox, double oy, double oz, 
     if (A > 0.0) {                       // A t^2 + 2 B t + C <= 0
         const double disc = B * B - A * C;
         if (disc < 0.0) return;
-        const double sq = sqrt(disc);
+        const double sq = sqrt64(disc);
         double c0, c1;
         if (B > 0.0) {
             const double q = -(B + sq);
-            c0 = q / A; c1 = C / q;
+            c0 = div64(q, A); c1 = div64(C, q);
         } else {
             const double q = sq - B;
-            if (q > 0.0) { c1 = q / A; c0 = C / q; }
+            if (q > 0.0) { c1 = div64(q, A); c0 = div64(C, q); }
             else { c0 = 0.0; c1 = 0.0; }
         }
         lo = fmax(lo, c0); hi = fmin(hi, c1);
@@ -856,9 +885,9 @@ static __device__ __noinline__ double seg_torus64(const double *P, double d, dou
     const double inf = __longlong_as_double(0x7ff0000000000000LL);
     if (d < 0.0) {
         const double dx = px - __ldg(P), dy = py - __ldg(P + 1);
-        const double rho = sqrt(dx * dx + dy * dy);
+        const double rho = sqrt64(dx * dx + dy * dy);
         if (!(rho > 0.0)) return -d - e;
-        const double cx = __ldg(P) + __ldg(P + 3) * dx / rho, cy = __ldg(P + 1) + __ldg(P + 3) * dy / rho;
+        const double cx = __ldg(P) + div64(__ldg(P + 3) * dx, rho), cy = __ldg(P + 1) + div64(__ldg(P + 3) * dy, rho);
         const double rr = __ldg(P + 4) - e;
         const double ox = px - cx, oy = py - cy, oz = pz - __ldg(P + 2);
         const double b = ox * ux + oy * uy + oz * uz;
@@ -866,8 +895,8 @@ static __device__ __noinline__ double seg_torus64(const double *P, double d, dou
         const double disc = b * b - cc;
         if (disc < 0.0) return 0.0;
         double t;
-        if (b > 0.0) t = -cc / (b + sqrt(disc));
-        else t = sqrt(disc) - b;
+        if (b > 0.0) t = div64(-cc, b + sqrt64(disc));
+        else t = sqrt64(disc) - b;
         return t > 0.0 ? t : 0.0;
     }
     const double R = __ldg(P + 3), rt = __ldg(P + 4) + e;
@@ -897,13 +926,13 @@ static __device__ __noinline__ double seg_xprim64(const DevScene &S, int kind, i
     if ((int)__ldg(X + 13) != 0) return fabs(d) - e;
     const double vx = px - __ldg(X + 9), vy = py - __ldg(X + 10), vz = pz - __ldg(X + 11);
     const double s = __ldg(X + 12);
-    const double q0 = (__ldg(X) * vx + __ldg(X + 3) * vy + __ldg(X + 6) * vz) / s;
-    const double q1 = (__ldg(X + 1) * vx + __ldg(X + 4) * vy + __ldg(X + 7) * vz) / s;
-    const double q2 = (__ldg(X + 2) * vx + __ldg(X + 5) * vy + __ldg(X + 8) * vz) / s;
+    const double q0 = div64(__ldg(X) * vx + __ldg(X + 3) * vy + __ldg(X + 6) * vz, s);
+    const double q1 = div64(__ldg(X + 1) * vx + __ldg(X + 4) * vy + __ldg(X + 7) * vz, s);
+    const double q2 = div64(__ldg(X + 2) * vx + __ldg(X + 5) * vy + __ldg(X + 8) * vz, s);
     const double w0 = __ldg(X) * ux + __ldg(X + 3) * uy + __ldg(X + 6) * uz;
     const double w1 = __ldg(X + 1) * ux + __ldg(X + 4) * uy + __ldg(X + 7) * uz;
     const double w2 = __ldg(X + 2) * ux + __ldg(X + 5) * uy + __ldg(X + 8) * uz;
-    const double dl = d / s, el = e / s;
+    const double dl = div64(d, s), el = div64(e, s);
     const double *P = S.p64 + 8 * i;
     double t;
     if (kind == 0) t = seg_sphere64(P, dl, q0, q1, q2, w0, w1, w2, el);
@@ -1224,8 +1253,8 @@ __device__ __forceinline__ void red_add(long long *a, long long v)
 __device__ __forceinline__ bool clip64(double lo, double hi, double p, double u, double &tin, double &tout)
 {
     if (u != 0.0) {
-        const double t0 = (lo - p) / u;
-        const double t1 = (hi - p) / u;
+        const double t0 = div64(lo - p, u);
+        const double t1 = div64(hi - p, u);
         tin = fmax(tin, fmin(t0, t1));
         tout = fmin(tout, fmax(t0, t1));
         return true;
@@ -1233,37 +1262,32 @@ __device__ __forceinline__ bool clip64(double lo, double hi, double p, double u,
     return !(p < lo || p > hi);
 }
 
-__device__ __forceinline__ void dda_axis64(double lo, double dl, int n, double p, double u, double tin, int &i,
-                                           double &tn)
+// The plane ahead of voxel i on one axis, along the segment.
+__device__ __forceinline__ double plane64(double lo, double dl, double p, double u, int i)
 {
-    const double xa = p + tin * u;
-    const double f = floor((xa - lo) / dl);
-    i = (int)fmin(fmax(f, 0.0), (double)(n - 1));
-    if (u > 0.0)
-        tn = ((lo + (double)(i + 1) * dl) - p) / u;
-    else if (u < 0.0)
-        tn = ((lo + (double)i * dl) - p) / u;
-    else
-        tn = __longlong_as_double(0x7ff0000000000000LL);
+    if (u > 0.0) return div64((lo + (double)(i + 1) * dl) - p, u);
+    if (u < 0.0) return div64((lo + (double)i * dl) - p, u);
+    return __longlong_as_double(0x7ff0000000000000LL);
 }
 
-static __device__ __noinline__ void tally64(const DevScene &S, long long *flu, double px, double py, double pz,
-                                            double ux, double uy, double uz, double len, double w,
-                                            unsigned *npieces)
+__device__ __forceinline__ void dda_axis64(double lo, double dl, int n, double p, double u, double tin, int &i)
 {
-    if (!(len > 0.0) || !(w > 0.0)) return;
-    double tin = 0.0, tout = len;
-    if (!clip64(S.g_lo[0], S.g_hi[0], px, ux, tin, tout)) return;
-    if (!clip64(S.g_lo[1], S.g_hi[1], py, uy, tin, tout)) return;
-    if (!clip64(S.g_lo[2], S.g_hi[2], pz, uz, tin, tout)) return;
-    if (!(tin < tout)) return;
+    const double xa = p + tin * u;
+    const double f = floor(div64(xa - lo, dl));
+    i = (int)fmin(fmax(f, 0.0), (double)(n - 1));
+}
+
+// The walk from voxel (ix, iy, iz), reached at t, along the segment to tout;
+// returns the number of pieces.
+static __device__ __noinline__ unsigned walk64(const DevScene &S, long long *flu, double px, double py, double pz,
+                                               double ux, double uy, double uz, int ix, int iy, int iz, double t,
+                                               double tout, double w)
+{
+    unsigned npieces = 0u;
+    double tx = plane64(S.g_lo[0], S.g_dl[0], px, ux, ix);
+    double ty = plane64(S.g_lo[1], S.g_dl[1], py, uy, iy);
+    double tz = plane64(S.g_lo[2], S.g_dl[2], pz, uz, iz);
     const int nx = S.g_n[0], ny = S.g_n[1], nz = S.g_n[2];
-    int ix, iy, iz;
-    double tx, ty, tz;
-    dda_axis64(S.g_lo[0], S.g_dl[0], nx, px, ux, tin, ix, tx);
-    dda_axis64(S.g_lo[1], S.g_dl[1], ny, py, uy, tin, iy, ty);
-    dda_axis64(S.g_lo[2], S.g_dl[2], nz, pz, uz, tin, iz, tz);
-    double t = tin;
     int guard = nx + ny + nz + 3;
     while (guard-- > 0) {
         const int ax = (tx <= ty && tx <= tz) ? 0 : ((ty <= tz) ? 1 : 2);
@@ -1273,28 +1297,43 @@ static __device__ __noinline__ void tally64(const DevScene &S, long long *flu, d
         if (piece > 0.0) {
             const long long off = ((long long)iz * ny + iy) * nx + ix;
             red_add(flu + off, fx64(w * piece));
-            *npieces += 1u;
+            npieces += 1u;
             t = tend;
         }
         if (ta >= tout) break;
         if (ax == 0) {
             ix += ux > 0.0 ? 1 : -1;
             if (ix < 0 || ix >= nx) break;
-            tx = ux > 0.0 ? ((S.g_lo[0] + (double)(ix + 1) * S.g_dl[0]) - px) / ux
-                          : ((S.g_lo[0] + (double)ix * S.g_dl[0]) - px) / ux;
+            tx = plane64(S.g_lo[0], S.g_dl[0], px, ux, ix);
         } else if (ax == 1) {
             iy += uy > 0.0 ? 1 : -1;
             if (iy < 0 || iy >= ny) break;
-            ty = uy > 0.0 ? ((S.g_lo[1] + (double)(iy + 1) * S.g_dl[1]) - py) / uy
-                          : ((S.g_lo[1] + (double)iy * S.g_dl[1]) - py) / uy;
+            ty = plane64(S.g_lo[1], S.g_dl[1], py, uy, iy);
         } else {
             iz += uz > 0.0 ? 1 : -1;
             if (iz < 0 || iz >= nz) break;
-            tz = uz > 0.0 ? ((S.g_lo[2] + (double)(iz + 1) * S.g_dl[2]) - pz) / uz
-                          : ((S.g_lo[2] + (double)iz * S.g_dl[2]) - pz) / uz;
+            tz = plane64(S.g_lo[2], S.g_dl[2], pz, uz, iz);
         }
     }
+    return npieces;
 }
+
+static __device__ __noinline__ unsigned tally64(const DevScene &S, long long *flu, double px, double py, double pz,
+                                                double ux, double uy, double uz, double len, double w)
+{
+    if (!(len > 0.0) || !(w > 0.0)) return 0u;
+    double tin = 0.0, tout = len;
+    if (!clip64(S.g_lo[0], S.g_hi[0], px, ux, tin, tout)) return 0u;
+    if (!clip64(S.g_lo[1], S.g_hi[1], py, uy, tin, tout)) return 0u;
+    if (!clip64(S.g_lo[2], S.g_hi[2], pz, uz, tin, tout)) return 0u;
+    if (!(tin < tout)) return 0u;
+    int ix, iy, iz;
+    dda_axis64(S.g_lo[0], S.g_dl[0], S.g_n[0], px, ux, tin, ix);
+    dda_axis64(S.g_lo[1], S.g_dl[1], S.g_n[1], py, uy, tin, iy);
+    dda_axis64(S.g_lo[2], S.g_dl[2], S.g_n[2], pz, uz, tin, iz);
+    return walk64(S, flu, px, py, pz, ux, uy, uz, ix, iy, iz, tin, tout, w);
+}
+
 
 // FP32 (mixed): reciprocal directions, incremental voxel offset.
 __device__ __forceinline__ bool clip32(float lo, float hi, float p, float iu, bool nz_, float &tin, float &tout)
@@ -1374,7 +1413,7 @@ __device__ __forceinline__ void tally32(const DevScene &S, long long *flu, float
 __device__ __forceinline__ void onb64(double nx, double ny, double nz, double b1[3], double b2[3])
 {
     const double sg = copysign(1.0, nz);
-    const double a = -1.0 / (sg + nz);
+    const double a = div64(-1.0, sg + nz);
     const double b = nx * ny * a;
     b1[0] = 1.0 + sg * nx * nx * a; b1[1] = sg * b; b1[2] = -sg * nx;
     b2[0] = b; b2[1] = sg + ny * ny * a; b2[2] = -ny;
@@ -1403,9 +1442,18 @@ struct WarpAcc {
     unsigned long long v[kNumSlots];
 };
 
+// A 64-bit add as two 32-bit ones (the low word's old value tells the
+// carry): shared memory has no 64-bit add, and the compare-and-swap loop in
+// its place is 48 instructions at each of the packet loop's 17 call sites.
 __device__ __forceinline__ void wadd(WarpAcc *a, int slot, long long x)
 {
-    if (x != 0) atomicAdd(&a->v[slot], (unsigned long long)x);
+    if (x != 0) {
+        unsigned *const p = reinterpret_cast<unsigned *>(&a->v[slot]);
+        const unsigned lo = (unsigned)x;
+        const unsigned old = atomicAdd(p, lo);
+        const unsigned hi = (unsigned)((unsigned long long)x >> 32) + (old + lo < lo ? 1u : 0u);
+        if (hi != 0u) atomicAdd(p + 1, hi);
+    }
 }
 
 __device__ __forceinline__ long long warp_sum(long long v)
@@ -1479,7 +1527,7 @@ __device__ __forceinline__ void jobconst_fill(volatile JobConst *jc, const JobWo
     jc->deadline = J->time_limit_ns > 0ull ? globaltimer_ns() + J->time_limit_ns : 0ull;
 }
 
-enum Phase { kTrace = 0, kNrm = 1, kProj = 2, kFar = 3, kNear = 4, kLaunch = 5 };
+enum Phase { kTrace = 0, kNrm = 1, kFar = 3, kNear = 4, kLaunch = 5, kArrive = 6 };
 
 constexpr double kWRoulette = 1e-4;   // roulette threshold (MCML convention)
 constexpr double kRouletteM = 10.0;   // survival 1/m, weight x m

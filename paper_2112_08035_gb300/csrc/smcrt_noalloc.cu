@@ -276,6 +276,7 @@ int build_image(const smcrt_scene *sc, const smcrt_source *src, const smcrt_grid
     }
     H.src_radius = src->radius;
     H.src_radius32 = (float)src->radius;
+    if (precision == SMCRT_FP64) fill_screen(H, sc, src, g, ins, rr);
     std::memcpy(img + o_scene, &H, sizeof H);
     *used = off;
     return SMCRT_OK;
