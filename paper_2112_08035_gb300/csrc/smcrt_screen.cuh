@@ -55,15 +55,17 @@ __device__ __forceinline__ float scr_prim(const DevScene &S, int kind, int i, fl
 // primitive leaves the fold as it is, a nearer one makes everything before it
 // irrelevant.  What is left to fold in FP64 are the instructions since the
 // last such reset that do not leave the fold alone: `list`, 16 bits each, in
-// order; cnt > kFoldList: too many, all of them count.  On the 64-capsule
-// vessel tree 1 to 3 capsules are left of 64.
+// order; cnt > kFoldList: too many, all of them count.  Each blend of two
+// operands adds 14 u R to the value's error; beyond the 8 that feps covers
+// the bound grows with them (err).  On the 64-capsule vessel tree 1 to 3
+// capsules are left of 64.
 constexpr int kFoldList = 4;
 
 __device__ __noinline__ float fold_screen(const DevScene &S, int i0, int i1, float x, float y, float z,
-                                          unsigned long long &list, int &cnt)
+                                          unsigned long long &list, int &cnt, float &err)
 {
-    const float eps2 = 2.f * S.feps;
-    float acc = 0.f;
+    const float eps = S.feps;
+    float acc = 0.f, ea = eps;
     unsigned long long li = 0ull;
     int n = 0;
     for (int i = i0; i < i1; ++i) {
@@ -71,22 +73,25 @@ __device__ __noinline__ float fold_screen(const DevScene &S, int i0, int i1, flo
         const int op = ins.x & 0xff;
         const float d = scr_prim(S, (ins.x >> 8) & 0xff, ins.y, x, y, z);
         const float kinv = __int_as_float(ins.w);
-        const float gap = fabsf(acc - d) - eps2;
+        const float gap = fabsf(acc - d) - (ea + eps);
         const bool sure = op == 2 ? gap * kinv > kScrUp : gap > 0.f;
         if (op == 0 || sure) {
             if (op == 0 || d < acc) {
                 acc = d;
+                ea = eps;
                 li = (unsigned long long)(unsigned)(i - i0);
                 n = 1;
             }
         } else {
             if (n < kFoldList) li |= (unsigned long long)(unsigned)(i - i0) << (16 * n);
-            n = min(n + 1, kFoldList + 1);
+            ++n;
+            if (n > 9) ea = __fmaf_rn(eps, 1.f / 16.f, ea) * kScrUp;
             acc = op == 2 ? csg32(2, acc, d, kinv) : fminf(acc, d);
         }
     }
     list = li;
     cnt = n;
+    err = ea;
     return acc;
 }
 
@@ -144,9 +149,11 @@ __device__ __forceinline__ void fold_list(const DevScene &S, int r, double x, do
                                           unsigned long long &list, int &cnt)
 {
     cnt = -1;
+    list = 0ull;
     if (!((S.fold_mask >> r) & 1ull)) return;
     const int2 rr = __ldg(S.rrange + r);
-    if (rr.y - rr.x > kFoldList) fold_screen(S, rr.x, rr.y, (float)x, (float)y, (float)z, list, cnt);
+    float err;
+    if (rr.y - rr.x > kFoldList) fold_screen(S, rr.x, rr.y, (float)x, (float)y, (float)z, list, cnt, err);
 }
 
 // What an evaluation is for: a trace position (region, nearest surface), one
@@ -182,13 +189,13 @@ static __device__ __noinline__ Eval64 scene_eval64_screened(const DevScene &S, d
                 continue;
             }
             const int2 rr = __ldg(S.rrange + r);
-            float d;
+            float d, err = eps;
             unsigned long long li = 0ull;
             int n = 0;
-            if (S.fold_mask & bit) d = fold_screen(S, rr.x, rr.y, fx, fy, fz, li, n);
+            if (S.fold_mask & bit) d = fold_screen(S, rr.x, rr.y, fx, fy, fz, li, n, err);
             else d = prog_screen(S, rr.x, rr.y, fx, fy, fz);
             if (d < 0.f) neg |= bit;
-            const float lo = fabsf(d) - eps, hi = fabsf(d) + eps;
+            const float lo = fabsf(d) - err, hi = fabsf(d) + err;
             if (S.soft_mask & bit) soft = fminf(soft, lo);
             bool in;
             if (mode == kForRegion) {
@@ -213,8 +220,10 @@ static __device__ __noinline__ Eval64 scene_eval64_screened(const DevScene &S, d
         const int r = __ffsll((long long)mask) - 1;
         const unsigned long long bit = 1ull << r;
         mask ^= bit;
-        if (r != flr) fold_list(S, r, x, y, z, list, cnt);
-        const double d = region_exact(S, r, x, y, z, list, cnt);
+        unsigned long long li = list;
+        int n = cnt;
+        if (r != flr) fold_list(S, r, x, y, z, li, n);
+        const double d = region_exact(S, r, x, y, z, li, n);
         if (d < 0.0) neg |= bit; else neg &= ~bit;
         const double ad = fabs(d);
         if (less64(ad, E.dmin)) { E.dmin = ad; E.istar = r; E.dstar = d; }
