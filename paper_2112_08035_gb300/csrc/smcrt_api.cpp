@@ -259,6 +259,7 @@ struct smcrt_plan {
     int ring = 64, ring_pos = 0;
     int *dstatus = nullptr;
     int blocks = 0, threads = 0, variant = 0;
+    bool chosen = false;       // the caller or the autotuner chose the variant
     int stage = 0;             // mixed: stage the scene tables in shared memory
     double time_limit_s = 0.0; // device time limit of a launch (0 = none)
     size_t cells = 0;
@@ -270,7 +271,7 @@ namespace {
 
 // Kernel instantiation of a plan: its register variant, in the general-shape
 // family when the scene has tori, cylinders or primitive frames.
-int kvariant(const smcrt_plan *pl) { return pl->variant + (pl->host.general ? kNumVariants : 0); }
+int kvariant(const smcrt_plan *pl, int variant) { return variant + (pl->host.general ? kNumVariants : 0); }
 
 int occupancy(int precision, int threads, int variant)
 {
@@ -442,14 +443,13 @@ int build_plan(smcrt_ctx *ctx, const smcrt_scene *sc, const smcrt_source *src, c
         fill_prim(sc, i, &p64[(size_t)8 * i], &p32[(size_t)2 * i], has_xf ? &xf64[(size_t)kXf64 * i] : nullptr,
                   has_xf ? &xf32[(size_t)kXf32 * i] : nullptr);
     }
-    std::vector<double> reg64((size_t)nr * 8, 0.0);
+    std::vector<double> reg64((size_t)nr * kReg64, 0.0);
     std::vector<float4> reg32((size_t)nr * 2);
     for (int r = 0; r < nr; ++r) {
         const smcrt_region &R = sc->regions[r];
         const double mu_t = R.mu_a + R.mu_s;
         const double albedo = mu_t > 0.0 ? R.mu_s / mu_t : 0.0;
-        double *d = &reg64[(size_t)8 * r];
-        d[0] = R.mu_a; d[1] = R.mu_s; d[2] = R.g; d[3] = R.n; d[4] = mu_t; d[5] = albedo;
+        fill_reg64(R, &reg64[(size_t)kReg64 * r]);
         reg32[2 * r] = make_float4((float)mu_t, mu_t > 0 ? (float)(1.0 / mu_t) : 0.f, (float)albedo, (float)R.g);
         reg32[2 * r + 1] = make_float4((float)R.n, (float)R.mu_a, (float)R.mu_s, 0.f);
     }
@@ -464,7 +464,7 @@ int build_plan(smcrt_ctx *ctx, const smcrt_scene *sc, const smcrt_source *src, c
     const size_t o_p64 = take(sizeof(double) * 8 * np);
     const size_t o_p32 = take(sizeof(float4) * 2 * np);
     const size_t o_rr = take(sizeof(int2) * nr);
-    const size_t o_r64 = take(sizeof(double) * 8 * nr);
+    const size_t o_r64 = take(sizeof(double) * kReg64 * nr);
     const size_t o_r32 = take(sizeof(float4) * 2 * nr);
     CullGrid cg;
     if (precision == SMCRT_MIXED) build_cull(sc, cg);
@@ -482,6 +482,7 @@ int build_plan(smcrt_ctx *ctx, const smcrt_scene *sc, const smcrt_source *src, c
     const size_t o_segm32 = take(sizeof(float) * nseg);
     const size_t o_xf64 = take(sizeof(double) * xf64.size());
     const size_t o_xf32 = take(sizeof(float4) * xf32.size());
+    const size_t o_planes = take(precision == SMCRT_FP64 ? sizeof(double) * plane_count(g) : 0);
     const size_t total = off;
 
     std::unique_ptr<smcrt_plan> pl(new smcrt_plan());
@@ -580,7 +581,10 @@ int build_plan(smcrt_ctx *ctx, const smcrt_scene *sc, const smcrt_source *src, c
     }
     H.src_radius = src->radius;
     H.src_radius32 = (float)src->radius;
-    if (precision == SMCRT_FP64) fill_screen(H, sc, src, g, ins.data(), rr.data());
+    if (precision == SMCRT_FP64) {
+        fill_screen(H, sc, src, g, ins.data(), rr.data());
+        H.planes = (const double *)(base + o_planes);
+    }
 
     std::vector<char> hb(total, 0);
     std::memcpy(hb.data() + o_scene, &H, sizeof H);
@@ -590,7 +594,8 @@ int build_plan(smcrt_ctx *ctx, const smcrt_scene *sc, const smcrt_source *src, c
     std::memcpy(hb.data() + o_p64, p64.data(), sizeof(double) * 8 * np);
     std::memcpy(hb.data() + o_p32, p32.data(), sizeof(float4) * 2 * np);
     std::memcpy(hb.data() + o_rr, rr.data(), sizeof(int2) * nr);
-    std::memcpy(hb.data() + o_r64, reg64.data(), sizeof(double) * 8 * nr);
+    std::memcpy(hb.data() + o_r64, reg64.data(), sizeof(double) * kReg64 * nr);
+    if (precision == SMCRT_FP64) fill_planes(g, (double *)(hb.data() + o_planes));
     std::memcpy(hb.data() + o_r32, reg32.data(), sizeof(float4) * 2 * nr);
     if (!cg.off.empty()) std::memcpy(hb.data() + o_coff, cg.off.data(), sizeof(int32_t) * cg.off.size());
     if (!cg.list.empty()) std::memcpy(hb.data() + o_clist, cg.list.data(), sizeof(int32_t) * cg.list.size());
@@ -637,6 +642,7 @@ int build_plan(smcrt_ctx *ctx, const smcrt_scene *sc, const smcrt_source *src, c
             pl->blocks = it->second.blocks;
             pl->threads = it->second.threads;
             pl->variant = it->second.variant % kNumVariants;
+            pl->chosen = true;
             pl->stage = it->second.variant / kNumVariants;
         }
     }
@@ -644,18 +650,21 @@ int build_plan(smcrt_ctx *ctx, const smcrt_scene *sc, const smcrt_source *src, c
     return SMCRT_OK;
 }
 
-void default_launch(const smcrt_plan *pl, int &blocks, int &threads)
+void default_launch(const smcrt_plan *pl, uint64_t npackets, int &blocks, int &threads, int &variant)
 {
+    const bool few = pl->precision == SMCRT_FP64 && !pl->chosen && npackets < kFewFp64Packets;
+    variant = few ? kFewFp64Variant : pl->variant;
     threads = pl->threads > 0 ? pl->threads : 128;
     blocks = pl->blocks;
     if (blocks <= 0) {
-        const int occ = std::max(1, occupancy(pl->precision, threads, kvariant(pl)));
-        blocks = pl->ctx->sm_count * occ;
+        const int occ = std::max(1, occupancy(pl->precision, threads, kvariant(pl, variant)));
+        blocks = pl->ctx->sm_count * (few ? 1 : occ);
     }
 }
 
 int plan_launch_impl(smcrt_plan *pl, uint64_t id_begin, uint64_t n, uint64_t seed, int64_t *flu,
-                     smcrt_totals *tot, smcrt_packet_record *rec, cudaStream_t s, int blocks, int threads)
+                     smcrt_totals *tot, smcrt_packet_record *rec, cudaStream_t s, int blocks, int threads,
+                     int variant)
 {
     JobWork jw{};
     jw.next = id_begin;
@@ -673,7 +682,8 @@ int plan_launch_impl(smcrt_plan *pl, uint64_t id_begin, uint64_t n, uint64_t see
     JobWork *slot = pl->djobs + pl->ring_pos;
     pl->ring_pos = (pl->ring_pos + 1) % pl->ring;
     if (launch_set_job(slot, jw, s) != cudaSuccess) return SMCRT_ERR_CUDA;
-    if (launch_kernel(pl->precision, slot, 1, pl->dstatus, blocks, threads, s, kvariant(pl)) != cudaSuccess)
+    if (launch_kernel(pl->precision, slot, 1, pl->dstatus, blocks, threads, s, kvariant(pl, variant)) !=
+        cudaSuccess)
         return SMCRT_ERR_CUDA;
     return SMCRT_OK;
 }
@@ -1371,10 +1381,10 @@ int smcrt_plan_launch(smcrt_plan *pl, uint64_t id_begin, uint64_t npackets, uint
     if (!pl || !totals_dev) return SMCRT_ERR_BAD_ARG;
     if (npackets == 0) return SMCRT_OK;
     if (id_begin + npackets < id_begin) return SMCRT_ERR_BAD_ARG;
-    int blocks, threads;
-    default_launch(pl, blocks, threads);
+    int blocks, threads, variant;
+    default_launch(pl, npackets, blocks, threads, variant);
     return plan_launch_impl(pl, id_begin, npackets, seed, fluence_dev, totals_dev, records_dev,
-                            (cudaStream_t)stream, blocks, threads);
+                            (cudaStream_t)stream, blocks, threads, variant);
 }
 
 int smcrt_plan_set_variant(smcrt_plan *pl, int32_t variant)
@@ -1382,6 +1392,7 @@ int smcrt_plan_set_variant(smcrt_plan *pl, int32_t variant)
     const int nv = pl && pl->precision == SMCRT_MIXED ? 2 * kNumVariants : kNumVariants;
     if (!pl || variant < 0 || variant >= nv) return SMCRT_ERR_BAD_ARG;
     pl->variant = variant % kNumVariants;
+    pl->chosen = true;
     pl->stage = variant / kNumVariants;
     return SMCRT_OK;
 }
@@ -1440,14 +1451,15 @@ int smcrt_plan_autotune(smcrt_plan *pl, uint64_t trial, int32_t *blocks_out, int
         for (int t : thread_opts) {
             const int occ = occupancy(pl->precision, t, v);
             if (occ < 1) continue;
-            for (int mult : {1, 2}) {
-                const int b = pl->ctx->sm_count * occ * mult;
+            for (int mult : {0, 1, 2}) {
+                if (mult == 0 && pl->precision != SMCRT_FP64) continue;
+                const int b = pl->ctx->sm_count * (mult == 0 ? 1 : occ * mult);   // FP64: one block per SM too
                 float ms_best = 1e30f;
                 for (int rep = 0; rep < 2; ++rep) {
                     cudaMemsetAsync(flu, 0, pl->cells * 8, 0);
                     cudaMemsetAsync(tot, 0, sizeof(smcrt_totals), 0);
                     cudaEventRecord(e0, 0);
-                    rc = plan_launch_impl(pl, 0, trial, 12345, flu, tot, nullptr, 0, b, t);
+                    rc = plan_launch_impl(pl, 0, trial, 12345, flu, tot, nullptr, 0, b, t, v);
                     cudaEventRecord(e1, 0);
                     if (rc != SMCRT_OK || cudaEventSynchronize(e1) != cudaSuccess) {
                         rc = SMCRT_ERR_CUDA;
@@ -1479,6 +1491,7 @@ int smcrt_plan_autotune(smcrt_plan *pl, uint64_t trial, int32_t *blocks_out, int
     pl->blocks = bb;
     pl->threads = bt;
     pl->variant = bv % kNumVariants;
+    pl->chosen = true;
     pl->stage = bv / kNumVariants;
     {
         std::lock_guard<std::mutex> lk(pl->ctx->tune_mu);
@@ -1512,9 +1525,9 @@ int smcrt_run(smcrt_ctx *ctx, const smcrt_scene *scene, const smcrt_source *sour
         if (cudaMemsetAsync(dtot, 0, sizeof(smcrt_totals), 0) != cudaSuccess) rc = SMCRT_ERR_CUDA;
     }
     if (rc == SMCRT_OK && npackets > 0) {
-        int blocks, threads;
-        default_launch(pl, blocks, threads);
-        rc = plan_launch_impl(pl, 0, npackets, seed, dflu, dtot, nullptr, 0, blocks, threads);
+        int blocks, threads, variant;
+        default_launch(pl, npackets, blocks, threads, variant);
+        rc = plan_launch_impl(pl, 0, npackets, seed, dflu, dtot, nullptr, 0, blocks, threads, variant);
     }
     smcrt_totals t{};
     if (rc == SMCRT_OK) {

@@ -152,6 +152,36 @@ inline int seg_entries(const smcrt_scene *sc, int32_t *out, double *margin, int 
     return n;
 }
 
+// FP64 optics of a region: mu_a, mu_s, g, n, mu_t, albedo, and the constants of
+// its scattering: 1 / mu_t, 1 - g g, 1 - g, 2 g, 1 + g g, 1 / (2 g).
+constexpr int kReg64 = 12;
+
+inline void fill_reg64(const smcrt_region &R, double *d)
+{
+    const double mu_t = R.mu_a + R.mu_s;
+    d[0] = R.mu_a; d[1] = R.mu_s; d[2] = R.g; d[3] = R.n;
+    d[4] = mu_t;
+    d[5] = mu_t > 0.0 ? R.mu_s / mu_t : 0.0;
+    d[6] = mu_t > 0.0 ? 1.0 / mu_t : 0.0;
+    d[7] = 1.0 - R.g * R.g;
+    d[8] = 1.0 - R.g;
+    d[9] = 2.0 * R.g;
+    d[10] = 1.0 + R.g * R.g;
+    d[11] = R.g != 0.0 ? 1.0 / (2.0 * R.g) : 0.0;
+}
+
+// The grid's planes lo + i dl of the three axes in turn (nx + 1, ny + 1,
+// nz + 1 of them).
+inline size_t plane_count(const smcrt_grid *g) { return (size_t)g->n[0] + g->n[1] + g->n[2] + 3; }
+
+inline void fill_planes(const smcrt_grid *g, double *d)
+{
+    for (int a = 0; a < 3; ++a) {
+        const double dl = (g->hi[a] - g->lo[a]) / (double)g->n[a];
+        for (int i = 0; i <= g->n[a]; ++i) *d++ = g->lo[a] + (double)i * dl;
+    }
+}
+
 // Device instruction (compiled CSG program).  op: 0 push primitive;
 // 1 union, 2 smooth union, 3 intersect, 4 subtract.  prim >= 0 with a
 // binary op means "combine the stack top (left) with this primitive
@@ -178,7 +208,7 @@ struct DevScene {
     const double *p64;        // 8 per primitive (capsule: a, b-a, r, |b-a|^2)
     const float4 *p32;        // 2 per primitive (capsule: a|r, b-a|1/|b-a|^2)
     const int2 *rrange;       // per region: instruction [begin, end)
-    const double *reg64;      // 8 per region: mu_a, mu_s, g, n, mu_t, albedo, 0, 0
+    const double *reg64;      // kReg64 per region (fill_reg64)
     const float4 *reg32;      // per region: mu_t, albedo, g, n
     int32_t ninstr, nregions, nprims, precision;
     // bounding box as centre / half extent
@@ -226,7 +256,10 @@ struct DevScene {
     uint64_t fold_mask;       // regions that are left folds of unions and smooth unions
     uint64_t soft_mask;       // soft regions (segment stepping)
     float feps;               // error bound of an FP32 distance
-    float gm32[3];            // error bound of an FP32 position in voxels, per axis
+    float gm32[3];            // error bound of an FP32 position in voxels from an FP64 difference, per axis
+    float gr32[3];            // ... from FP32 coordinates
+    int32_t pad2;
+    const double *planes;     // fill_planes; null: computed
 };
 
 // The screening fields of a compiled scene without general shapes: the error
@@ -251,7 +284,7 @@ inline void fill_screen(DevScene &H, const smcrt_scene *sc, const smcrt_source *
     R = R + 4.0 * sc->delta;
     H.screen_mask = H.fold_mask = H.soft_mask = 0;
     H.feps = 0.f;
-    for (int a = 0; a < 3; ++a) H.gm32[a] = INFINITY;
+    for (int a = 0; a < 3; ++a) H.gm32[a] = H.gr32[a] = INFINITY;
     if (H.general || !(R > 1e-6 && R < 1e12)) return;   // FP32 squares stay in range
     H.feps = (float)(R / 65536.0);
     for (int r = 0; r < sc->nregions; ++r) {
@@ -267,7 +300,12 @@ inline void fill_screen(DevScene &H, const smcrt_scene *sc, const smcrt_source *
         if (fold || smooth <= 8) H.screen_mask |= bit;
         if (region_is_soft(sc, r)) H.soft_mask |= bit;
     }
-    for (int a = 0; a < 3; ++a) H.gm32[a] = (float)(g->n[a] * (16.0 / 16777216.0));
+    for (int a = 0; a < 3; ++a) {
+        const double Rg = std::fmax(R, std::fmax(std::fabs(g->lo[a]), std::fabs(g->hi[a])));
+        const double dl = (g->hi[a] - g->lo[a]) / (double)g->n[a];
+        H.gm32[a] = (float)(g->n[a] * (16.0 / 16777216.0));
+        H.gr32[a] = (float)((Rg / dl + (double)g->n[a]) * (16.0 / 16777216.0));
+    }
 }
 
 // A packet parked between serving rounds: its complete state at a trace
@@ -332,6 +370,17 @@ int occupancy_mixed(int threads, int variant = 0);
 cudaError_t launch_mixed_multi(JobWork *jobs, int njobs, int *status, int blocks, int threads,
                                cudaStream_t stream, int variant = 0);
 int occupancy_mixed_multi(int threads, int variant = 0);
+// FP64 plan launches of fewer packets than this run, unless the caller or the
+// autotuner chose a shape, one block of 128 threads per SM with the largest
+// register budget (variant 2): one warp per scheduler nearly fills the FP64
+// pipe, and four warps disturb one another's instruction fetch less than
+// twelve.  Measured, 1 x 128 against 3 x 128: layered slab 1e4 packets 17.0
+// / 24.7 ms, 1e5 61 / 73 ms, 1e6 501 / 522 ms; glass container 3e4 49 / 58
+// ms, 5e5 237 / 232 ms; sphere 1e5, sphere tracing, 77 / 80 ms, 1e6 324 /
+// 285 ms.
+constexpr uint64_t kFewFp64Packets = 1u << 19;
+constexpr int kFewFp64Variant = 2;
+
 // Lanes of a warp that carry packets in a plan launch (JobWork.lanes; 0 =
 // all).  A launch with fewer packets than lanes is bound by the latency of
 // one loop iteration, which grows with the number of different branches a

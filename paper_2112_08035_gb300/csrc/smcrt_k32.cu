@@ -111,7 +111,7 @@ __device__ __forceinline__ float region_n32(const DevScene &S, int r)
 
 __device__ __forceinline__ double region_n64(const DevScene &S, int r)
 {
-    return r < 0 ? S.ambient_n : __ldg(S.reg64 + 8 * r + 3);
+    return r < 0 ? S.ambient_n : __ldg(S.reg64 + kReg64 * r + 3);
 }
 
 // FP64 interface localisation for a crossing whose normal must be accurate:

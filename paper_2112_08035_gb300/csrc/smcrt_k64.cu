@@ -10,37 +10,100 @@ namespace smcrt {
 
 namespace {
 
-__device__ __forceinline__ double hg_cos64(double g, double xi)
+// a / b given y = 1 / b rounded to nearest: two corrections of a y, each
+// with the remainder from a fused multiply-add.  The result is the quotient
+// rounded to nearest if its remainder is below half an ulp of it times b,
+// which is compared exactly; otherwise (and near the range's ends) divides.
+__device__ __forceinline__ double div_by64(double a, double b, double y)
+{
+    const double q0 = a * y;
+    const double q = __fma_rn(__fma_rn(-b, q0, a), y, q0);
+    const double r = __fma_rn(-b, q, a);
+    const long long qb = __double_as_longlong(q) & 0x7fffffffffffffffLL, bb = __double_as_longlong(b) & 0x7fffffffffffffffLL;
+    const int eq = (int)(qb >> 52), eb = (int)(bb >> 52);
+    const long long half = bb + ((long long)(eq - 1076) << 52);
+    const bool ok = eq > 700 && eq < 1400 && eb > 700 && eb < 1400 && (qb & 0x000FFFFFFFFFFFFFLL) != 0 &&
+                    (__double_as_longlong(r) & 0x7fffffffffffffffLL) < half;
+    return ok ? q : div64(a, b);
+}
+
+__device__ __forceinline__ double hg_cos64(const double *RG, double xi)
 {   // Henyey-Greenstein inverse CDF (Sec. 3.1); isotropic for |g| < 1e-6
+    const double g = __ldg(RG + 2);
     double c;
     if (fabs(g) < 1e-6) {
         c = 2.0 * xi - 1.0;
     } else {
-        const double t = div64(1.0 - g * g, 1.0 - g + 2.0 * g * xi);
-        c = div64(1.0 + g * g - t * t, 2.0 * g);
+        const double t = div64(__ldg(RG + 7), __ldg(RG + 8) + __ldg(RG + 9) * xi);
+        c = div_by64(__ldg(RG + 10) - t * t, __ldg(RG + 9), __ldg(RG + 11));
     }
-    return fmin(fmax(c, -1.0), 1.0);
+    return min64(max64(c, -1.0), 1.0);
 }
 
+// x / l for l = 1 + e, |e| < 2^-20: x - x e is the quotient but for a
+// relative 2^-40, and its remainder tells exactly whether it is the one
+// rounded to nearest (as in div_by64).
+__device__ __forceinline__ double unit_div64(double x, double l, double e)
+{
+    const double q = __fma_rn(-x, e, x);
+    const double r = __fma_rn(-l, q, x);
+    const long long qb = __double_as_longlong(q) & 0x7fffffffffffffffLL;
+    const int eq = (int)(qb >> 52);
+    const long long half = __double_as_longlong(l) + ((long long)(eq - 1076) << 52);
+    const bool ok = eq > 700 && (qb & 0x000FFFFFFFFFFFFFLL) != 0 &&
+                    (__double_as_longlong(r) & 0x7fffffffffffffffLL) < half;
+    return ok ? q : div64(x, l);
+}
+
+// x, y, z over their norm.  Directions are unit vectors up to rounding, so
+// the square s of the norm is 1 + f with a tiny f.  For |f| < 2^-27 the root
+// is 1 + f / 2 - f f / 8 + ..., below h = 1 + f / 2 by less than 2^-57; h is
+// a floating-point number or lies halfway between two, so the root rounded
+// to nearest is h rounded down: one fused multiply-add.  14 FP64 operations
+// in place of 41.
 __device__ __forceinline__ void normalise64(double &x, double &y, double &z)
 {
-    const double l = sqrt64(x * x + y * y + z * z);
-    x = div64(x, l);
-    y = div64(y, l);
-    z = div64(z, l);
+    const double s = x * x + y * y + z * z;
+    const int hs = __double2hiint(s);
+    double l;
+    if (hs >= 0x3fefffff && hs <= 0x3ff00000 && (hs == 0x3ff00000 ? (unsigned)__double2loint(s) < (1u << 25)
+                                                                     : (unsigned)__double2loint(s) > 0xfc000000u))
+        l = __fma_rd(s - 1.0, 0.5, 1.0);
+    else
+        l = sqrt64(s);
+    const double e = l - 1.0;
+    if ((__double2hiint(e) & 0x7fffffff) < 0x3eb00000) {   // |e| < 2^-20
+        x = unit_div64(x, l, e);
+        y = unit_div64(y, l, e);
+        z = unit_div64(z, l, e);
+    } else {
+        x = div64(x, l);
+        y = div64(y, l);
+        z = div64(z, l);
+    }
 }
 
-__device__ __forceinline__ void scatter64(double &ux, double &uy, double &uz, double ct, double xi_phi)
+__device__ __forceinline__ double flip64(double x, double s)   // x times the sign of s
+{
+    return __longlong_as_double(__double_as_longlong(x) ^ (__double_as_longlong(s) & (long long)0x8000000000000000ULL));
+}
+
+// Rotation by the scattering angle; the azimuth from a Philox word.  The
+// basis is onb64's, its products with the sign of uz (+-1) as sign flips.
+__device__ __forceinline__ void scatter64(double &ux, double &uy, double &uz, double ct, uint32_t wphi)
 {
     const double st = sqrt64((1.0 - ct) * (1.0 + ct));
     double sp, cp;
-    sincos2pi64(xi_phi, &sp, &cp);
-    double b1[3], b2[3];
-    onb64(ux, uy, uz, b1, b2);
+    sincos2pi_word(wphi, &sp, &cp);
+    const double a = div64(-1.0, copysign(1.0, uz) + uz);
+    const double b = ux * uy * a;
+    const double sx = flip64(ux, uz);
+    const double b1x = 1.0 + sx * ux * a, b1y = flip64(b, uz), b1z = -sx;
+    const double b2y = copysign(1.0, uz) + uy * uy * a, b2z = -uy;
     const double a1 = st * cp, a2 = st * sp;
-    double vx = a1 * b1[0] + a2 * b2[0] + ct * ux;
-    double vy = a1 * b1[1] + a2 * b2[1] + ct * uy;
-    double vz = a1 * b1[2] + a2 * b2[2] + ct * uz;
+    double vx = a1 * b1x + a2 * b + ct * ux;
+    double vy = a1 * b1y + a2 * b2y + ct * uy;
+    double vz = a1 * b1z + a2 * b2z + ct * uz;
     normalise64(vx, vy, vz);
     ux = vx; uy = vy; uz = vz;
 }
@@ -54,7 +117,7 @@ struct Launched64 {
 static __device__ __noinline__ Launched64 launch64(const DevScene &S, uint4 r)
 {
     Launched64 o;
-    const double x0 = u01_64(r.x), x1 = u01_64(r.y), x3 = u01_64(r.w);
+    const double x0 = u01_64(r.x), x3 = u01_64(r.w);
     o.px = S.src_pos[0]; o.py = S.src_pos[1]; o.pz = S.src_pos[2];
     o.ux = S.src_dir[0]; o.uy = S.src_dir[1]; o.uz = S.src_dir[2];
     if (S.src_kind == 1 || S.src_kind == 2) {
@@ -62,12 +125,12 @@ static __device__ __noinline__ Launched64 launch64(const DevScene &S, uint4 r)
         if (S.src_kind == 1) {
             const double rho = S.src_radius * sqrt64(x0);
             double sn, cs;
-            sincos2pi64(x1, &sn, &cs);
+            sincos2pi_word(r.y, &sn, &cs);
             c1 = rho * cs;
             c2 = rho * sn;
         } else {
             c1 = S.src_radius * (2.0 * x0 - 1.0);
-            c2 = S.src_radius * (2.0 * x1 - 1.0);
+            c2 = S.src_radius * (2.0 * u01_64(r.y) - 1.0);
         }
         o.px = S.src_pos[0] + c1 * S.src_b1[0] + c2 * S.src_b2[0];
         o.py = S.src_pos[1] + c1 * S.src_b1[1] + c2 * S.src_b2[1];
@@ -76,7 +139,7 @@ static __device__ __noinline__ Launched64 launch64(const DevScene &S, uint4 r)
         const double ctt = 2.0 * x0 - 1.0;
         const double st = sqrt64((1.0 - ctt) * (1.0 + ctt));
         double sn, cs;
-        sincos2pi64(x1, &sn, &cs);
+        sincos2pi_word(r.y, &sn, &cs);
         o.ux = st * cs; o.uy = st * sn; o.uz = ctt;
     }
     o.tau = -ln64(x3);
@@ -113,6 +176,13 @@ static __device__ __noinline__ Crossed64 cross64(double ux, double uy, double uz
     return o;
 }
 
+// Waiting packets are served when the lane iterations that they have waited
+// reach the live lanes / kWaitExact (distances, about 100 FP64 operations)
+// or / kWaitArrive (interfaces, about 250), against about 165 for an
+// interaction.  Layered slab 1e5 packets: 60.9 ms with 3 and 2, 59.1 with 1
+// for interfaces, 64.0 with 4; distances at once 62.7.
+constexpr int kWaitExact = 3, kWaitArrive = 1;
+
 struct WarpShared {
     DevScene S;
     WarpAcc acc;
@@ -137,7 +207,12 @@ __device__ bool run_job_fp64(const DevScene &S, WarpAcc *wa, const volatile JobC
     int phase = kTrace, istar = -1, reg = -1;
     int nsteps = 0;
     unsigned pscat = 0, npieces = 0, nev = 0;
-    int waited = 0;                      // lane iterations that arrived packets have waited (warp-uniform)
+    // lane iterations that packets have waited for FP64 distances and at
+    // surfaces (warp-uniform), and a waiting packet's screening
+    int wait_x = 0, wait_i = 0;
+    unsigned long long kneg = 0ull, kmask = 0ull, klist = 0ull;
+    float ksoft = 0.f, kdb = 0.f;
+    int kfold = 0;
     long long pA = 0, pG = 0;
     uint32_t id_lo = 0, id_hi = 0, event = 0;
     uint32_t t_acq = 0;
@@ -205,69 +280,105 @@ __device__ bool run_job_fp64(const DevScene &S, WarpAcc *wa, const volatile JobC
             if (__all_sync(SMCRT_FULL, retired)) break;
         }
 
-        // ---- 2. the scene evaluation of this iteration
-        Eval64 E{};
+        // ---- 2. the scene in FP32: where that shows that the packet
+        // interacts before it can reach anything, no FP64 distance is needed
+        Screen64 C;
+        bool interact = false;
         const bool evals = alive && phase == kTrace;
-        if (G)
-            E = scene_eval64<G>(S, px, py, pz, -2);
-        else if (evals)
-            E = scene_eval64_screened(S, px, py, pz, -2, kForTrace);
+        if (G) {
+            if (evals) phase = kExact;
+        } else if (evals) {
+            C = scene_screen(S, (float)px, (float)py, (float)pz, kForTrace);
+            kneg = C.neg; kmask = C.mask; klist = C.list; kfold = C.flr << 8 | (C.cnt & 0xff);
+            ksoft = C.soft; kdb = C.db;
+            phase = kExact;
+            if (C.lo > (float)delta * kScrUp) {          // clear of every surface, region known
+                reg = C.neg != 0ull ? 63 - __clzll((long long)C.neg) : -1;
+                const float m = reg >= 0 ? (float)__ldg(S.reg64 + kReg64 * reg + 4) : 0.f;
+                const float need = (float)tau * (kScrUp * kScrUp);
+                interact = m > 0.f && need < m * (C.lo - (float)delta);
+                if (!interact && S.stepping == SMCRT_STEP_SEGMENT) {
+                    const float p[3] = {(float)px, (float)py, (float)pz}, u[3] = {(float)ux, (float)uy, (float)uz};
+                    interact = m > 0.f && need < m * segment_screen(S, C.soft, p, u);
+                }
+            }
+        }
         nev += evals;
 
-        // ---- 3. classify
-        bool move = false, fresnel = false, iter_done = false;
-        bool seg_step = false;                 // a tracing move that segment stepping may lengthen
+        // ---- 3. FP64: the packets for which FP32 did not do, once enough of
+        // them wait (an FP64 operation costs the same for one lane as for
+        // all); moves, arrivals at a surface, escapes
+        bool move = interact, fresnel = false, iter_done = false;
         bool fin = false;                      // the packet ends this iteration
         bool out = false;                      // ... leaving the volume: R or T
         long long fin_R = 0, fin_T = 0, fin_K = 0;
         double L = 0.0;
-        if (evals) {
-            if (E.dbox > 0.0) {                          // outside the volume of interest
-                out = true;
-            } else {
-                reg = E.region;
-                if (E.dmin < delta) {                    // on a boundary
-                    istar = E.istar;
-                    dstar = E.dstar;
-                    phase = kArrive;
+        const unsigned here = __ballot_sync(SMCRT_FULL, alive);
+        const bool none = __ballot_sync(SMCRT_FULL, alive && (interact || phase == kLaunch)) == 0u;   // no other lane moves
+        const unsigned exact = __ballot_sync(SMCRT_FULL, alive && phase == kExact && !interact);
+        wait_x += __popc(exact);
+        if (exact != 0u && (G || none || kWaitExact * wait_x >= __popc(here))) {
+            wait_x = 0;
+            if (alive && phase == kExact && !interact) {
+                Eval64 E;
+                if (G) {
+                    E = scene_eval64<G>(S, px, py, pz, -2);
                 } else {
-                    L = E.dmin - 0.5 * delta;            // stop short of the surface
-                    move = true;
-                    seg_step = S.stepping == SMCRT_STEP_SEGMENT;
+                    C.neg = kneg; C.mask = kmask; C.list = klist; C.flr = kfold >> 8; C.cnt = (int)(int8_t)(kfold & 0xff);
+                    C.soft = ksoft; C.db = kdb;
+                    E = scene_exact(S, px, py, pz, C, kForTrace);
+                }
+                if (E.dbox > 0.0) {                      // outside the volume of interest
+                    out = true;
+                } else {
+                    reg = E.region;
+                    if (E.dmin < delta) {                // on a boundary
+                        istar = E.istar;
+                        dstar = E.dstar;
+                        phase = kArrive;
+                    } else {
+                        const double mu_t = reg >= 0 ? __ldg(S.reg64 + kReg64 * reg + 4) : 0.0;
+                        L = E.dmin - 0.5 * delta;        // stop short of the surface
+                        move = true;
+                        interact = mu_t > 0.0 && tau < mu_t * L;
+                        if (!interact && S.stepping == SMCRT_STEP_SEGMENT) {   // a longer move along u
+                            if (G) L = fmax(L, segment_bound64<G>(S, E.dsoft, E.dbox, px, py, pz, ux, uy, uz));
+                            else L = max64(L, segment_bound64_screened(S, E.dsoft, E.dbox, px, py, pz, ux, uy, uz));
+                            interact = mu_t > 0.0 && tau < mu_t * L;
+                        }
+                    }
                 }
             }
         }
 
-        // ---- 3b. the packets at a surface, once enough of them wait: the
-        // routine costs as much for one lane as for all, about ten times
-        // what a waiting lane loses per iteration
+        // ---- 3b. the packets at a surface, once enough of them wait
         Interface64 I;
         I.R = 1.0;
         const unsigned arrived = __ballot_sync(SMCRT_FULL, alive && phase == kArrive);
-        if (arrived != 0u) {
-            waited += __popc(arrived);
-            const unsigned here = __ballot_sync(SMCRT_FULL, alive);
-            if (3 * waited >= __popc(here) || here == arrived) {
-                waited = 0;
-                if (alive && phase == kArrive) {
-                    I = interface64<G>(S, px, py, pz, ux, uy, uz, istar, dstar);
-                    nev += I.evals;
-                    phase = kTrace;
-                    if (I.what == kIntfForced) {
-                        L = delta;                       // forced step along u
-                        move = true;
-                    } else if (I.what == kIntfEscape) {
-                        out = true;                      // outward through the bounding box
+        wait_i += __popc(arrived);
+        if (arrived != 0u && (kWaitArrive * wait_i >= __popc(here) ||
+                              __ballot_sync(SMCRT_FULL, alive && (move || phase == kLaunch)) == 0u)) {
+            wait_i = 0;
+            if (alive && phase == kArrive) {
+                I = interface64<G>(S, px, py, pz, ux, uy, uz, istar, dstar);
+                nev += I.evals;
+                phase = kTrace;
+                if (I.what == kIntfForced) {
+                    L = delta;                           // forced step along u
+                    move = true;
+                    const double mu_t = reg >= 0 ? __ldg(S.reg64 + kReg64 * reg + 4) : 0.0;
+                    interact = mu_t > 0.0 && tau < mu_t * L;
+                } else if (I.what == kIntfEscape) {
+                    out = true;                          // outward through the bounding box
+                } else {
+                    wadd(wa, kIntf, 1);
+                    if (I.what == kIntfMatched) {
+                        const double ee = 2.0 * delta * (I.cdot > 0.0 ? 1.0 : -1.0);
+                        px = I.qx + ee * I.nx; py = I.qy + ee * I.ny; pz = I.qz + ee * I.nz;
+                        iter_done = true;
                     } else {
-                        wadd(wa, kIntf, 1);
-                        if (I.what == kIntfMatched) {
-                            const double ee = 2.0 * delta * (I.cdot > 0.0 ? 1.0 : -1.0);
-                            px = I.qx + ee * I.nx; py = I.qy + ee * I.ny; pz = I.qz + ee * I.nz;
-                            iter_done = true;
-                        } else {
-                            wadd(wa, kFres, 1);
-                            fresnel = true;
-                        }
+                        wadd(wa, kFres, 1);
+                        fresnel = true;
                     }
                 }
             }
@@ -280,28 +391,9 @@ __device__ bool run_job_fp64(const DevScene &S, WarpAcc *wa, const volatile JobC
         }
 
         // ---- 4. move: interaction point or sphere-trace step, one tally site
-        bool interact = false;
         if (move) {
-            double mu_t = 0.0;
-            if (reg >= 0) mu_t = __ldg(S.reg64 + 8 * reg + 4);
-            interact = mu_t > 0.0 && tau < mu_t * L;
-            if (seg_step && !interact) {           // segment stepping: a longer move along u
-                if (G) {
-                    L = fmax(L, segment_bound64<G>(S, E.dsoft, E.dbox, px, py, pz, ux, uy, uz));
-                    interact = mu_t > 0.0 && tau < mu_t * L;
-                } else {
-                    // FP32 first: most of these packets interact before the
-                    // bound, whose value then does not matter
-                    const float p[3] = {(float)px, (float)py, (float)pz}, u[3] = {(float)ux, (float)uy, (float)uz};
-                    const float lo = segment_screen(S, (float)E.dsoft, p, u);
-                    interact = mu_t > 0.0 && (float)tau * kScrUp < (float)mu_t * lo * kScrDown;
-                    if (!interact) {
-                        L = fmax(L, segment_bound64_screened(S, E.dsoft, E.dbox, px, py, pz, ux, uy, uz));
-                        interact = mu_t > 0.0 && tau < mu_t * L;
-                    }
-                }
-            }
-            const double seg = interact ? div64(tau, mu_t) : L;
+            const double mu_t = reg >= 0 ? __ldg(S.reg64 + kReg64 * reg + 4) : 0.0;
+            const double seg = interact ? div_by64(tau, mu_t, __ldg(S.reg64 + kReg64 * reg + 6)) : L;
             long long *const flu = (long long *)jc->flu;
             if (flu) {
                 if (G) npieces += tally64(S, flu, px, py, pz, ux, uy, uz, seg, w);
@@ -332,11 +424,11 @@ __device__ bool run_job_fp64(const DevScene &S, WarpAcc *wa, const volatile JobC
             phase = kTrace;
         }
         if (interact) {                                  // implicit capture, HG, roulette
-            const double *RG = S.reg64 + 8 * reg;
+            const double *RG = S.reg64 + kReg64 * reg;
             const double wn = w * __ldg(RG + 5);
             pA += fx64(w - wn);
             w = wn;
-            scatter64(ux, uy, uz, hg_cos64(__ldg(RG + 2), u01_64(r.x)), u01_64(r.y));
+            scatter64(ux, uy, uz, hg_cos64(RG, u01_64(r.x)), r.y);
             pscat += 1u;
             if (w < kWRoulette) {
                 if (u01_64(r.z) <= 1.0 / kRouletteM) {

@@ -72,8 +72,16 @@ struct Rng {
     }
 };
 
+// v 2^e for 0 < v < 2^53, put together from its bits (exact): an integer
+// conversion takes the FP64 pipe as long as an addition.
+__device__ __forceinline__ double scaled64(unsigned long long v, int e)
+{
+    const int z = __clzll((long long)v);
+    return __longlong_as_double((long long)(((v << z) << 1 >> 12) | (unsigned long long)(1023 + 63 - z + e) << 52));
+}
+
 // Uniforms in (0, 1]: FP64 uses the whole 32-bit word, FP32 its top 24 bits.
-__device__ __forceinline__ double u01_64(uint32_t w) { return ((double)w + 1.0) * (1.0 / 4294967296.0); }
+__device__ __forceinline__ double u01_64(uint32_t w) { return scaled64((unsigned long long)w + 1ull, -32); }
 // FP32: the top 23 bits mapped to bin midpoints, (k + 1/2) 2^-23, strictly
 // inside (0, 1) and unbiased (24 bits would not do: (2^24 - 1/2) 2^-24
 // rounds to 1 in FP32).  The value 1 would put a square or disc source's
@@ -100,8 +108,8 @@ __device__ __forceinline__ double ln64(double x)
     const long long b = __double_as_longlong(x);
     int e = (int)((b >> 52) & 0x7ff) - 1023;
     double m = __longlong_as_double((b & 0x000FFFFFFFFFFFFFLL) | 0x3FF0000000000000LL);
-    if (m > 1.4142135623730951) {
-        m = m * 0.5;
+    if (__double_as_longlong(m) > 0x3FF6A09E667F3BCDLL) {   // sqrt(2)
+        m = __longlong_as_double(__double_as_longlong(m) - 0x0010000000000000LL);
         e = e + 1;
     }
     const double s = div64(m - 1.0, m + 1.0);
@@ -117,14 +125,13 @@ __device__ __forceinline__ double ln64(double x)
     t = t * z + 1.0 / 5.0;
     t = t * z + 1.0 / 3.0;
     t = t * z + 1.0;
-    return (double)e * 0.6931471805599453 + (2.0 * s) * t;
+    const double ed = e == 0 ? 0.0 : scaled64((unsigned long long)abs(e), 0);
+    return (e < 0 ? -ed : ed) * 0.6931471805599453 + (2.0 * s) * t;
 }
 
-__device__ __forceinline__ void sincos2pi64(double t, double *sn, double *cs)
+// sin and cos of a + (q quarter turns), |a| <= pi/4.
+__device__ __forceinline__ void sincos_quarter64(double a, int q, double *sn, double *cs)
 {
-    const double q = floor(t * 4.0 + 0.5);
-    const double f = t - q * 0.25;
-    const double a = f * 6.283185307179586;
     const double z = a * a;
     double ps = 1.0 / 355687428096000.0;
     ps = ps * z - 1.0 / 1307674368000.0;
@@ -144,16 +151,41 @@ __device__ __forceinline__ void sincos2pi64(double t, double *sn, double *cs)
     pc = pc * z + 1.0 / 24.0;
     pc = pc * z - 0.5;
     const double c = 1.0 + z * pc;
-    switch (((int)q) & 3) {
-    case 0: *sn = s; *cs = c; break;
-    case 1: *sn = c; *cs = -s; break;
-    case 2: *sn = -s; *cs = -c; break;
-    default: *sn = -c; *cs = s; break;
-    }
+    const double x = (q & 1) ? c : s, y = (q & 1) ? s : c;
+    *sn = (q & 2) ? -x : x;
+    *cs = ((q + 1) & 2) ? -y : y;
 }
 
-// Fixed point: 2^-32 weight units.  FP64: round half to even like llrint.
-__device__ __forceinline__ long long fx64(double x) { return __double2ll_rn(x * 4294967296.0); }
+__device__ __forceinline__ void sincos2pi64(double t, double *sn, double *cs)
+{
+    const double q = floor(t * 4.0 + 0.5);
+    const double f = t - q * 0.25;
+    sincos_quarter64(f * 6.283185307179586, (int)q, sn, cs);
+}
+
+// The same for t = u01_64(w), whose reduction is exact: in integers.
+__device__ __forceinline__ void sincos2pi_word(uint32_t w, double *sn, double *cs)
+{
+    const unsigned long long v = (unsigned long long)w + 1ull;
+    const int q = (int)((v + (1ull << 29)) >> 30);
+    const long long i = (long long)v - ((long long)q << 30);   // f 2^32
+    double f = 0.0;
+    if (i != 0) f = scaled64((unsigned long long)(i < 0 ? -i : i), -32);
+    sincos_quarter64((i < 0 ? -f : f) * 6.283185307179586, q, sn, cs);
+}
+
+// Fixed point: 2^-32 weight units.  FP64: round half to even like llrint, in
+// integers for x >= 0 (the conversion takes the FP64 pipe as long as an add).
+__device__ __forceinline__ long long fx64(double x)
+{
+    const long long b = __double_as_longlong(x);
+    const int s = 1043 - (int)(b >> 52);     // shift to the units: 52 - 32 - (exponent - 1023)
+    if (b < 0 || s <= 0) return __double2ll_rn(x * 4294967296.0);
+    if (s > 54) return 0;
+    const unsigned long long m = ((unsigned long long)b & 0x000FFFFFFFFFFFFFull) | 0x0010000000000000ull;
+    const unsigned long long q = m >> s, rem = m << (64 - s);
+    return (long long)(q + (rem > 0x8000000000000000ull || (rem == 0x8000000000000000ull && (q & 1ull)) ? 1ull : 0ull));
+}
 // FP32 (0 <= x < 2^31): x * 2^32 is exact (a power-of-two scale), then one
 // hardware conversion to int64, round half to even (cheaper than shifting
 // the mantissa in integer code, which cost the tally 7 % of the kernel).
@@ -170,13 +202,22 @@ __device__ __forceinline__ long long fx32(float x) { return __float2ll_rn(x * 42
 struct Eval64 { double dmin, dstar, dsel, dbox, dsoft; int istar, region; };
 struct Eval32 { float dmin, dstar, dsel, dbox, dsoft; int istar, region; };
 
-// The larger of two numbers (not NaN), compared as integers.
+// The larger / smaller of two numbers (not NaN), compared as integers: an
+// FP64 fmax takes the FP64 pipe 2.4 times as long as an addition.
 __device__ __forceinline__ double max64(double a, double b)
 {
     long long x = __double_as_longlong(a), y = __double_as_longlong(b);
     x ^= (long long)((unsigned long long)(x >> 63) >> 1);
     y ^= (long long)((unsigned long long)(y >> 63) >> 1);
     return x > y ? a : b;
+}
+
+__device__ __forceinline__ double min64(double a, double b)
+{
+    long long x = __double_as_longlong(a), y = __double_as_longlong(b);
+    x ^= (long long)((unsigned long long)(x >> 63) >> 1);
+    y ^= (long long)((unsigned long long)(y >> 63) >> 1);
+    return x < y ? a : b;
 }
 
 // a < b for numbers that are not negative (nor NaN).
@@ -196,10 +237,9 @@ __device__ __forceinline__ double box64(double x, double y, double z, double cx,
     const int one = (__double2hiint(qx) >= 0) + (__double2hiint(qy) >= 0) + (__double2hiint(qz) >= 0);
     const int hq = __double2hiint(q);
     if (one == 0 || (one == 1 && hq > 0x20000000 && hq < 0x5f000000)) return q;
-    const double mx = fmax(qx, 0.0), my = fmax(qy, 0.0), mz = fmax(qz, 0.0);
-    const double outside = sqrt64(mx * mx + my * my + mz * mz);
-    const double inside = fmin(fmax(qx, fmax(qy, qz)), 0.0);
-    return outside + inside;
+    // here some q is positive: the inside part is zero
+    const double mx = max64(qx, 0.0), my = max64(qy, 0.0), mz = max64(qz, 0.0);
+    return sqrt64(mx * mx + my * my + mz * mz);
 }
 
 __device__ __forceinline__ float box32(float x, float y, float z, float cx, float cy, float cz,
@@ -245,7 +285,7 @@ __device__ __forceinline__ double base64(int kind, const double *P, double x, do
         const double pax = x - __ldg(P), pay = y - __ldg(P + 1), paz = z - __ldg(P + 2);
         const double bax = __ldg(P + 3), bay = __ldg(P + 4), baz = __ldg(P + 5);
         double t = div64(pax * bax + pay * bay + paz * baz, __ldg(P + 7));
-        t = fmin(fmax(t, 0.0), 1.0);
+        t = min64(max64(t, 0.0), 1.0);
         const double dx = pax - bax * t, dy = pay - bay * t, dz = paz - baz * t;
         return sqrt64(dx * dx + dy * dy + dz * dz) - __ldg(P + 6);
     }
@@ -370,11 +410,11 @@ __device__ __forceinline__ float prim32(const DevScene &S, int kind, int i, floa
 // minimum (the SDF literature cited with Fig. 1 e).
 __device__ __forceinline__ double csg64(int op, double a, double b, double k)
 {
-    if (op == 1) return fmin(a, b);
-    if (op == 3) return fmax(a, b);
-    if (op == 4) return fmax(a, -b);
+    if (op == 1) return min64(a, b);
+    if (op == 3) return max64(a, b);
+    if (op == 4) return max64(a, -b);
     double h = 0.5 + div64(0.5 * (b - a), k);
-    h = fmin(fmax(h, 0.0), 1.0);
+    h = min64(max64(h, 0.0), 1.0);
     const double m = b * (1.0 - h) + a * h;
     return m - k * h * (1.0 - h);
 }
@@ -746,8 +786,8 @@ static __device__ __noinline__ double seg_box64(double cx, double cy, double cz,
         const double lo = c[a] - (h[a] + e), hi = c[a] + (h[a] + e);
         if (u[a] != 0.0) {
             const double t0 = div64(lo - p[a], u[a]), t1 = div64(hi - p[a], u[a]);
-            tn = fmax(tn, fmin(t0, t1));
-            tf = fmin(tf, fmax(t0, t1));
+            tn = max64(tn, min64(t0, t1));
+            tf = min64(tf, max64(t0, t1));
         } else if (p[a] < lo || p[a] > hi) {
             return d > 0.0 ? inf : 0.0;
         }
@@ -1255,8 +1295,8 @@ __device__ __forceinline__ bool clip64(double lo, double hi, double p, double u,
     if (u != 0.0) {
         const double t0 = div64(lo - p, u);
         const double t1 = div64(hi - p, u);
-        tin = fmax(tin, fmin(t0, t1));
-        tout = fmin(tout, fmax(t0, t1));
+        tin = max64(tin, min64(t0, t1));
+        tout = min64(tout, max64(t0, t1));
         return true;
     }
     return !(p < lo || p > hi);
@@ -1410,15 +1450,6 @@ __device__ __forceinline__ void tally32(const DevScene &S, long long *flu, float
 // Orthonormal basis perpendicular to a unit vector: branchless construction
 // of Duff et al., "Building an Orthonormal Basis, Revisited", JCGT 2017.
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ void onb64(double nx, double ny, double nz, double b1[3], double b2[3])
-{
-    const double sg = copysign(1.0, nz);
-    const double a = div64(-1.0, sg + nz);
-    const double b = nx * ny * a;
-    b1[0] = 1.0 + sg * nx * nx * a; b1[1] = sg * b; b1[2] = -sg * nx;
-    b2[0] = b; b2[1] = sg + ny * ny * a; b2[2] = -ny;
-}
-
 __device__ __forceinline__ void onb32(float nx, float ny, float nz, float b1[3], float b2[3])
 {
     const float sg = copysignf(1.f, nz);
@@ -1527,7 +1558,7 @@ __device__ __forceinline__ void jobconst_fill(volatile JobConst *jc, const JobWo
     jc->deadline = J->time_limit_ns > 0ull ? globaltimer_ns() + J->time_limit_ns : 0ull;
 }
 
-enum Phase { kTrace = 0, kNrm = 1, kFar = 3, kNear = 4, kLaunch = 5, kArrive = 6 };
+enum Phase { kTrace = 0, kNrm = 1, kFar = 3, kNear = 4, kLaunch = 5, kArrive = 6, kExact = 7 };
 
 constexpr double kWRoulette = 1e-4;   // roulette threshold (MCML convention)
 constexpr double kRouletteM = 10.0;   // survival 1/m, weight x m

@@ -151,7 +151,7 @@ int build_image(const smcrt_scene *sc, const smcrt_source *src, const smcrt_grid
     const size_t o_p64 = take(sizeof(double) * 8 * np);
     const size_t o_p32 = take(sizeof(float4) * 2 * np);
     const size_t o_rr = take(sizeof(int2) * nr);
-    const size_t o_r64 = take(sizeof(double) * 8 * nr);
+    const size_t o_r64 = take(sizeof(double) * kReg64 * nr);
     const size_t o_r32 = take(sizeof(float4) * 2 * nr);
     int32_t segp[kMaxPrims];
     double segm[kMaxPrims];
@@ -163,6 +163,10 @@ int build_image(const smcrt_scene *sc, const smcrt_source *src, const smcrt_grid
     const size_t o_xf64 = take(has_xf ? sizeof(double) * kXf64 * np : 0);
     const size_t o_xf32 = take(has_xf ? sizeof(float4) * kXf32 * np : 0);
     if (kImageOff + off > kNoAllocScratchBytes) return SMCRT_ERR_NO_MEMORY;
+    // the grid's planes where they fit (else the kernel computes them)
+    const size_t plane_bytes = sizeof(double) * plane_count(g);
+    const bool with_planes = precision == SMCRT_FP64 && kImageOff + a16(off + plane_bytes) <= kNoAllocScratchBytes;
+    const size_t o_planes = take(with_planes ? plane_bytes : 0);
     std::memset(img, 0, off);
 
     int32_t *pkind = (int32_t *)(img + o_kind);
@@ -181,8 +185,7 @@ int build_image(const smcrt_scene *sc, const smcrt_source *src, const smcrt_grid
         const smcrt_region &R = sc->regions[r];
         const double mu_t = R.mu_a + R.mu_s;
         const double albedo = mu_t > 0.0 ? R.mu_s / mu_t : 0.0;
-        double *d = reg64 + 8 * r;
-        d[0] = R.mu_a; d[1] = R.mu_s; d[2] = R.g; d[3] = R.n; d[4] = mu_t; d[5] = albedo;
+        fill_reg64(R, reg64 + kReg64 * r);
         reg32[2 * r] = make_float4((float)mu_t, mu_t > 0 ? (float)(1.0 / mu_t) : 0.f, (float)albedo, (float)R.g);
         reg32[2 * r + 1] = make_float4((float)R.n, (float)R.mu_a, (float)R.mu_s, 0.f);
     }
@@ -277,6 +280,10 @@ int build_image(const smcrt_scene *sc, const smcrt_source *src, const smcrt_grid
     H.src_radius = src->radius;
     H.src_radius32 = (float)src->radius;
     if (precision == SMCRT_FP64) fill_screen(H, sc, src, g, ins, rr);
+    if (with_planes) {
+        fill_planes(g, (double *)(img + o_planes));
+        H.planes = (const double *)(base + o_planes);
+    }
     std::memcpy(img + o_scene, &H, sizeof H);
     *used = off;
     return SMCRT_OK;
@@ -350,9 +357,10 @@ extern "C" int smcrt_run_noalloc(const smcrt_scene *scene, const smcrt_source *s
     cudaGetDevice(&dev);
     if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return SMCRT_ERR_CUDA;
     const int threads = 128;
-    const int variant = (precision == SMCRT_FP64 ? 1 : 0) + (general ? kNumVariants : 0);
+    const bool few = precision == SMCRT_FP64 && npackets < kFewFp64Packets;
+    const int variant = (precision == SMCRT_FP64 ? (few ? kFewFp64Variant : 1) : 0) + (general ? kNumVariants : 0);
     const int occ = precision == SMCRT_FP64 ? occupancy_fp64(threads, variant) : occupancy_mixed(threads, variant);
-    const int blocks = sms * (occ > 0 ? occ : 1);
+    const int blocks = sms * (occ > 0 && !few ? occ : 1);
     jw.lanes = spread_lanes(npackets, blocks, threads);
     JobWork *dj = (JobWork *)(base + kJobOff);
     if (launch_set_job(dj, jw, s) != cudaSuccess) return SMCRT_ERR_CUDA;

@@ -21,6 +21,8 @@
 // errors do not grow).  DevScene.feps = 2^-16 R = 256 u R exceeds the sum.
 #pragma once
 
+#include <cstddef>
+
 #include "smcrt_kernel.cuh"
 
 namespace smcrt {
@@ -156,90 +158,103 @@ __device__ __forceinline__ void fold_list(const DevScene &S, int r, double x, do
     if (rr.y - rr.x > kFoldList) fold_screen(S, rr.x, rr.y, (float)x, (float)y, (float)z, list, cnt, err);
 }
 
-// What an evaluation is for: a trace position (region, nearest surface), one
-// surface's value (normal probes, projection), or the region at a point.
-enum EvalFor { kForTrace = 0, kForSurface = 1, kForRegion = 2 };
+// What an evaluation is for: a trace position (region, nearest surface) or the
+// region at a point.
+enum EvalFor { kForTrace = 0, kForRegion = 1 };
 
-// Scene evaluation in which only the values that count are FP64: the
-// regions that may be nearest (trace), whose sign FP32 cannot tell, or the
-// one surface asked for.  dsoft: a lower bound (FP32) over the soft regions;
-// dbox: FP64 where it may be nearest, else an FP32 value of the right sign.
-// Layered slab: 1.1 of 4 surfaces are left per trace evaluation; without the
-// square root where at most one axis is outside (box_exact).
-static __device__ __noinline__ Eval64 scene_eval64_screened(const DevScene &S, double x, double y, double z, int sel,
-                                                        int mode)
+// The scene in FP32.
+struct Screen64 {
+    unsigned long long neg;  // regions with a negative value
+    unsigned long long mask; // regions whose FP64 value counts (nearest, sign, or unscreened)
+    unsigned long long list; // the list of fold flr, cnt entries
+    int flr, cnt;
+    float soft;              // lower bound of |d| over the soft regions
+    float lo;                // lower bound of |d| over all surfaces; <= 0: some sign is open
+    float db;                // bounding box
+};
+
+static __device__ __noinline__ Screen64 scene_screen(const DevScene &S, float x, float y, float z, int mode)
+{
+    Screen64 C;
+    const float inf = __int_as_float(0x7f800000), eps = S.feps;
+    C.neg = C.mask = C.list = 0ull;
+    C.flr = -1; C.cnt = 0;
+    float mlo = inf, mhi = inf, soft = inf, all = inf;   // bounds of the smallest |d|
+    for (int r = 0; r < S.nregions; ++r) {
+        const unsigned long long bit = 1ull << r;
+        if (!(S.screen_mask & bit)) {            // FP32 says nothing about this one
+            C.mask |= bit;
+            if (S.soft_mask & bit) soft = 0.f;
+            all = -1.f;
+            continue;
+        }
+        const int2 rr = __ldg(S.rrange + r);
+        float d, err = eps;
+        unsigned long long li = 0ull;
+        int n = 0;
+        if (S.fold_mask & bit) d = fold_screen(S, rr.x, rr.y, x, y, z, li, n, err);
+        else d = prog_screen(S, rr.x, rr.y, x, y, z);
+        if (d < 0.f) C.neg |= bit;
+        const float lo = fabsf(d) - err, hi = fabsf(d) + err;
+        if (S.soft_mask & bit) soft = fminf(soft, lo);
+        all = fminf(all, lo);
+        bool in;
+        if (mode == kForRegion) {
+            in = !(lo > 0.f);
+        } else {
+            in = !(lo > mhi);
+            if (hi < mlo) {                      // nearer than all so far: they are out
+                C.mask &= ~S.screen_mask;
+                mlo = lo;
+            } else if (in) {
+                mlo = fminf(mlo, lo);
+            }
+            mhi = fminf(mhi, hi);
+        }
+        if (in) {
+            C.mask |= bit;
+            if (S.fold_mask & bit) { C.flr = r; C.list = li; C.cnt = min(n, kFoldList + 1); }
+        }
+    }
+    C.soft = soft;
+    const float db = scr_box(x, y, z, S.bbc32[0], S.bbc32[1], S.bbc32[2], S.bbh32[0], S.bbh32[1], S.bbh32[2]);
+    // db = 0: the box's FP64 value counts (it may be nearest, or its sign is open)
+    C.db = !(fabsf(db) - eps > mhi) || !(fabsf(db) > eps) ? 0.f : db;
+    C.lo = eps > 0.f ? fminf(all, -db - eps) : -1.f;
+    return C;
+}
+
+// The scene evaluation from its screening, in which only the values that
+// count are FP64.  dsoft: a lower bound (FP32) over the soft regions; dbox:
+// FP64 where it may be nearest, else an FP32 value of the right sign.  1.1
+// of the layered slab's 4 surfaces are left per trace evaluation, and no
+// square root where at most one axis is outside (box64).
+static __device__ __noinline__ Eval64 scene_exact(const DevScene &S, double x, double y, double z, const Screen64 &C,
+                                                  int mode)
 {
     Eval64 E;
     E.dmin = __longlong_as_double(0x7ff0000000000000LL);
-    E.dsoft = E.dmin;
-    E.dstar = 0.0; E.dsel = 0.0; E.dbox = -1.0; E.istar = -1; E.region = -1;
-    const float inf = __int_as_float(0x7f800000), eps = S.feps;
-    const float fx = (float)x, fy = (float)y, fz = (float)z;
-    unsigned long long neg = 0ull, mask = 0ull, list = 0ull;
-    int flr = -1, cnt = 0;                       // the fold whose list is at hand
-    float mlo = inf, mhi = inf, soft = inf;      // bounds of the smallest |d|
-    if (mode == kForSurface) {
-        if (sel >= 0) mask = 1ull << sel;
-    } else {
-        for (int r = 0; r < S.nregions; ++r) {
-            const unsigned long long bit = 1ull << r;
-            if (!(S.screen_mask & bit)) {        // FP32 says nothing about this one
-                mask |= bit;
-                if (S.soft_mask & bit) soft = 0.f;
-                continue;
-            }
-            const int2 rr = __ldg(S.rrange + r);
-            float d, err = eps;
-            unsigned long long li = 0ull;
-            int n = 0;
-            if (S.fold_mask & bit) d = fold_screen(S, rr.x, rr.y, fx, fy, fz, li, n, err);
-            else d = prog_screen(S, rr.x, rr.y, fx, fy, fz);
-            if (d < 0.f) neg |= bit;
-            const float lo = fabsf(d) - err, hi = fabsf(d) + err;
-            if (S.soft_mask & bit) soft = fminf(soft, lo);
-            bool in;
-            if (mode == kForRegion) {
-                in = !(lo > 0.f);
-            } else {
-                in = !(lo > mhi);
-                if (hi < mlo) {                  // nearer than all so far: they are out
-                    mask &= ~S.screen_mask;
-                    mlo = lo;
-                } else if (in) {
-                    mlo = fminf(mlo, lo);
-                }
-                mhi = fminf(mhi, hi);
-            }
-            if (in) {
-                mask |= bit;
-                if (S.fold_mask & bit) { flr = r; list = li; cnt = n; }
-            }
-        }
-    }
+    E.dstar = 0.0; E.dsel = 0.0; E.istar = -1; E.region = -1;
+    E.dsoft = (double)C.soft;
+    E.dbox = (double)C.db;
+    unsigned long long neg = C.neg, mask = C.mask;
     while (mask != 0ull) {
         const int r = __ffsll((long long)mask) - 1;
         const unsigned long long bit = 1ull << r;
         mask ^= bit;
-        unsigned long long li = list;
-        int n = cnt;
-        if (r != flr) fold_list(S, r, x, y, z, li, n);
+        unsigned long long li = C.list;
+        int n = C.cnt;
+        if (r != C.flr) fold_list(S, r, x, y, z, li, n);
         const double d = region_exact(S, r, x, y, z, li, n);
         if (d < 0.0) neg |= bit; else neg &= ~bit;
         const double ad = fabs(d);
         if (less64(ad, E.dmin)) { E.dmin = ad; E.istar = r; E.dstar = d; }
-        if (r == sel) E.dsel = d;
     }
     if (neg != 0ull) E.region = 63 - __clzll((long long)neg);
-    E.dsoft = (double)soft;
-    const float db = mode == kForTrace ? scr_box(fx, fy, fz, S.bbc32[0], S.bbc32[1], S.bbc32[2], S.bbh32[0],
-                                                 S.bbh32[1], S.bbh32[2])
-                                       : 0.f;
-    if (mode == kForTrace) E.dbox = (double)db;
-    if ((mode == kForTrace && (!(fabsf(db) - eps > mhi) || !(fabsf(db) > eps))) || (mode == kForSurface && sel == -1)) {
+    if (mode == kForTrace && C.db == 0.f) {
         const double d = box64(x, y, z, S.bbc[0], S.bbc[1], S.bbc[2], S.bbh[0], S.bbh[1], S.bbh[2]);
         E.dbox = d;
-        if (fabs(d) < E.dmin) { E.dmin = fabs(d); E.istar = -1; E.dstar = d; }
-        if (sel == -1) E.dsel = d;
+        if (less64(fabs(d), E.dmin)) { E.dmin = fabs(d); E.istar = -1; E.dstar = d; }
     }
     return E;
 }
@@ -269,12 +284,14 @@ static __device__ __noinline__ double surface_at64(const DevScene &S, int r, dou
 template <bool G>
 static __device__ __noinline__ int region_at64(const DevScene &S, double x, double y, double z)
 {
-    return (G ? scene_eval64<G>(S, x, y, z, -2) : scene_eval64_screened(S, x, y, z, -2, kForRegion)).region;
+    if (G) return scene_eval64<G>(S, x, y, z, -2).region;
+    const Screen64 C = scene_screen(S, (float)x, (float)y, (float)z, kForRegion);
+    return scene_exact(S, x, y, z, C, kForRegion).region;
 }
 
 __device__ __forceinline__ double region_n64(const DevScene &S, int r)
 {
-    return r < 0 ? S.ambient_n : __ldg(S.reg64 + 8 * r + 3);
+    return r < 0 ? S.ambient_n : __ldg(S.reg64 + kReg64 * r + 3);
 }
 
 template <bool G>
@@ -413,35 +430,48 @@ static __device__ __noinline__ float segment_screen(const DevScene &S, float sof
     return t;
 }
 
-// Exit from inside a box shrunk by e, where FP32 finds the axes that may come
-// first and only their quotients are taken (the reference takes the larger of
-// an axis' two quotients, which is the one of the plane ahead: rounding is
-// monotone).
-static __device__ __noinline__ double seg_exit64(double cx, double cy, double cz, double hx, double hy, double hz,
-                                             double d, double px, double py, double pz, double ux, double uy,
-                                             double uz, double e, float eps)
+// seg_box64 of the box P (centre, half extents), with the quotients of the
+// axes that FP32 shows to count.  The reference takes an axis' smaller and
+// larger quotient, which are those of the plane behind and ahead (rounding
+// is monotone): from inside, the bound is the first plane ahead; from
+// outside, the last plane behind, if it certainly lies before the first one
+// ahead and ahead of the packet.
+static __device__ __noinline__ double seg_face64(const double *P, double d, double px, double py, double pz,
+                                                 double ux, double uy, double uz, double e, float eps)
 {
-    const double c[3] = {cx, cy, cz}, h[3] = {hx, hy, hz}, p[3] = {px, py, pz}, u[3] = {ux, uy, uz};
-    float lo[3], first = __int_as_float(0x7f800000);
+    const double c[3] = {P[0], P[1], P[2]}, h[3] = {P[3], P[4], P[5]}, p[3] = {px, py, pz}, u[3] = {ux, uy, uz};
+    const bool inside = !(d > 0.0);
+    const double eo = inside ? -e : e;
+    const float inf = __int_as_float(0x7f800000);
+    float at[3], lo[3], hi[3];               // the face that counts: bounds of its distance
+    float ahead = inf, behind = -inf, last = -inf;
     bool odd = false;                        // a direction component of zero, a box thinner than 2 e
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
-        const float uf = (float)u[a], hf = (float)h[a] - (float)e;
+        const float uf = (float)u[a], g = (float)h[a] + (float)eo;
         const float q = uf > 0.f ? (float)p[a] - (float)c[a] : (float)c[a] - (float)p[a];
-        odd = odd || uf == 0.f || !(hf > eps);
+        odd = odd || uf == 0.f || !(g > eps);
         const float iu = __fdividef(1.f, fabsf(uf));
-        lo[a] = fmaxf(hf - q - eps, 0.f) * iu * kScrDown;
-        first = fminf(first, fmaxf(hf - q + eps, 0.f) * iu * kScrUp);
+        at[a] = (inside ? g : -g) - q;
+        const float x = (at[a] - eps) * iu, y = (at[a] + eps) * iu;
+        lo[a] = x - 1e-5f * fabsf(x); hi[a] = y + 1e-5f * fabsf(y);
+        ahead = fminf(ahead, inside ? hi[a] : (g - q - eps) * iu * kScrDown);
+        behind = fmaxf(behind, lo[a]);
+        last = fmaxf(last, hi[a]);
     }
-    if (eps == 0.f || odd || !(first < 1e30f)) return seg_box64(cx, cy, cz, hx, hy, hz, d, px, py, pz, ux, uy, uz, e);
-    double tf = __longlong_as_double(0x7ff0000000000000LL);
+    // from outside: certainly hit (the last plane behind before the first ahead) and ahead
+    if (eps == 0.f || odd || !(fabsf(ahead) < 1e30f) || (!inside && !(behind > 0.f && last < ahead)))
+        return seg_box64(P[0], P[1], P[2], P[3], P[4], P[5], d, px, py, pz, ux, uy, uz, e);
+    double t = __longlong_as_double(inside ? 0x7ff0000000000000LL : (long long)0xfff0000000000000ULL);
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
-        if (lo[a] > first) continue;
-        const double he = h[a] + (-e);
-        tf = fmin(tf, div64((u[a] > 0.0 ? c[a] + he : c[a] - he) - p[a], u[a]));
+        if (inside ? lo[a] > ahead : hi[a] < behind) continue;
+        const double he = h[a] + eo;
+        const bool plus = (u[a] > 0.0) == inside;
+        const double x = div64((plus ? c[a] + he : c[a] - he) - p[a], u[a]);
+        t = inside ? min64(t, x) : max64(t, x);
     }
-    return tf > 0.0 ? tf : 0.0;
+    return t > 0.0 ? t : 0.0;
 }
 
 // The move bound of segment_bound64, leaving out what cannot lower it.
@@ -451,10 +481,9 @@ static __device__ __noinline__ double segment_bound64_screened(const DevScene &S
     const float eps = S.feps;
     const float p[3] = {(float)px, (float)py, (float)pz}, u[3] = {(float)ux, (float)uy, (float)uz};
     const double dh = 0.5 * S.delta;
-    double t = dbox > 0.0 ? seg_box64(S.bbc[0], S.bbc[1], S.bbc[2], S.bbh[0], S.bbh[1], S.bbh[2], dbox, px, py, pz,
-                                      ux, uy, uz, dh)
-                          : seg_exit64(S.bbc[0], S.bbc[1], S.bbc[2], S.bbh[0], S.bbh[1], S.bbh[2], dbox, px, py, pz,
-                                       ux, uy, uz, dh, eps);
+    static_assert(offsetof(DevScene, bbh) == offsetof(DevScene, bbc) + 3 * sizeof(double), "centre, half extents");
+    const double *box = reinterpret_cast<const double *>(reinterpret_cast<const char *>(&S) + offsetof(DevScene, bbc));
+    double t = seg_face64(box, dbox, px, py, pz, ux, uy, uz, dh, eps);
     if (S.soft_mask != 0ull && soft - dh <= t) {
         double ds = __longlong_as_double(0x7ff0000000000000LL);
         for (unsigned long long m = S.soft_mask; m != 0ull; m &= m - 1ull) {
@@ -462,9 +491,9 @@ static __device__ __noinline__ double segment_bound64_screened(const DevScene &S
             unsigned long long list = 0ull;
             int cnt;
             fold_list(S, r, px, py, pz, list, cnt);
-            ds = fmin(ds, fabs(region_exact(S, r, px, py, pz, list, cnt)));
+            ds = min64(ds, fabs(region_exact(S, r, px, py, pz, list, cnt)));
         }
-        t = fmin(t, ds - dh);
+        t = min64(t, ds - dh);
     }
     for (int j = 0; j < S.nseg; ++j) {
         const int i = __ldg(S.seg_prims + j);
@@ -482,21 +511,23 @@ static __device__ __noinline__ double segment_bound64_screened(const DevScene &S
                 continue;
             if (kind == 0 && scr_sphere(A, df, ef, p, u, eps) > tu) continue;
         }
-        const double d = prim64<false>(S, kind, i, px, py, pz);
-        if (!(fabs(d) > e)) return 0.0;
-        if (fabs(d) - e >= t) continue;
+        // FP64 where FP32 leaves it open whether the primitive is passed over
+        // (|d| within its margin, or |d| - e not below the bound so far)
+        double d = (double)df;
+        if (!(eps > 0.f && iso > 0.f && fabsf(df) + eps - ef * kScrDown * kScrDown < tu * kScrDown * kScrDown)) {
+            d = prim64<false>(S, kind, i, px, py, pz);
+            if (!(fabs(d) > e)) return 0.0;
+            if (fabs(d) - e >= t) continue;
+        }
         const double *P = S.p64 + 8 * i;
         double b;
         if (kind == 0)
             b = seg_sphere64(P, d, px, py, pz, ux, uy, uz, e);
         else if (kind == 1)
-            b = d > 0.0 ? seg_box64(__ldg(P), __ldg(P + 1), __ldg(P + 2), __ldg(P + 3), __ldg(P + 4), __ldg(P + 5), d,
-                                    px, py, pz, ux, uy, uz, e)
-                        : seg_exit64(__ldg(P), __ldg(P + 1), __ldg(P + 2), __ldg(P + 3), __ldg(P + 4), __ldg(P + 5),
-                                     d, px, py, pz, ux, uy, uz, e, eps);
+            b = seg_face64(P, d, px, py, pz, ux, uy, uz, e, eps);
         else
             b = seg_capsule64(P, d, px, py, pz, ux, uy, uz, e);
-        t = fmin(t, b);
+        t = min64(t, b);
     }
     return t;
 }
@@ -504,39 +535,67 @@ static __device__ __noinline__ double segment_bound64_screened(const DevScene &S
 // ---------------------------------------------------------------------------
 // Track-length tally: tally64 with the grid clip left out where the segment
 // starts inside the grid, the voxel index taken from FP32 where its fraction
-// is clear of a voxel boundary, and one plane's quotient taken per voxel
-// crossing (the axis that certainly comes first) in place of three and of a
-// comparison of three.  Positions are in voxels from the grid's corner (one
-// FP64 subtraction per axis); the FP32 error of one is below
-// DevScene.gm32 = 16 u n.  A segment inside one voxel (most of them) takes
-// five FP64 operations, a crossing 16.
+// is clear of a voxel face, and one plane's quotient taken per voxel crossing
+// (the axis that certainly comes first) in place of three and of a
+// comparison of three.  Positions are in voxels from the grid's corner; the
+// error of one is below DevScene.gr32 = 16 u (R / dl + n), or gm32 = 16 u n
+// from an FP64 difference.  A segment inside one voxel (most of them) takes
+// one FP64 operation, a crossing 12.
 // ---------------------------------------------------------------------------
+// The rest of a walk of a segment that starts inside the grid, in FP64 (clipped at the grid's far faces).
+static __device__ __noinline__ unsigned walk_rest64(const DevScene &S, long long *flu, double px, double py, double pz,
+                                                    double ux, double uy, double uz, int ix, int iy, int iz, double t,
+                                                    double len, double w)
+{
+    double tin = 0.0, tout = len;
+    clip64(S.g_lo[0], S.g_hi[0], px, ux, tin, tout);
+    clip64(S.g_lo[1], S.g_hi[1], py, uy, tin, tout);
+    clip64(S.g_lo[2], S.g_hi[2], pz, uz, tin, tout);
+    return walk64(S, flu, px, py, pz, ux, uy, uz, ix, iy, iz, t, tout, w);
+}
+
 static __device__ __noinline__ unsigned tally64_screened(const DevScene &S, long long *flu, double px, double py,
                                                          double pz, double ux, double uy, double uz, double len,
                                                          double w)
 {
     if (!(len > 0.0) || !(w > 0.0)) return 0u;
     const float lf = (float)len;
-    const float mx = S.gm32[0], my = S.gm32[1], mz = S.gm32[2];
     const int nx = S.g_n[0], ny = S.g_n[1], nz = S.g_n[2];
-    const float gx = (float)(px - S.g_lo[0]) * S.g_idl32[0], ax = lf * (float)ux * S.g_idl32[0], hx = gx + ax;
-    const float gy = (float)(py - S.g_lo[1]) * S.g_idl32[1], ay = lf * (float)uy * S.g_idl32[1], hy = gy + ay;
-    const float gz = (float)(pz - S.g_lo[2]) * S.g_idl32[2], az = lf * (float)uz * S.g_idl32[2], hz = gz + az;
-    // both ends beyond one side of the grid: no voxel
-    const float ex = mx + 1e-6f * (fabsf(gx) + fabsf(ax)), ey = my + 1e-6f * (fabsf(gy) + fabsf(ay)),
-                ez = mz + 1e-6f * (fabsf(gz) + fabsf(az));
-    if (fminf(gx, hx) > (float)nx + ex || fmaxf(gx, hx) < -ex || fminf(gy, hy) > (float)ny + ey ||
-        fmaxf(gy, hy) < -ey || fminf(gz, hz) > (float)nz + ez || fmaxf(gz, hz) < -ez)
-        return 0u;
-    const float bx = floorf(gx), by = floorf(gy), bz = floorf(gz);
-    float sx = gx - bx, sy = gy - by, sz = gz - bz;          // position in the voxel
-    const bool clear = gx > mx && gx < (float)nx - mx && gy > my && gy < (float)ny - my && gz > mz &&
-                       gz < (float)nz - mz && fminf(sx, 1.f - sx) > 2.f * mx && fminf(sy, 1.f - sy) > 2.f * my &&
-                       fminf(sz, 1.f - sz) > 2.f * mz;
-    if (!clear) return tally64(S, flu, px, py, pz, ux, uy, uz, len, w);
+    const float ax = lf * (float)ux * S.g_idl32[0], ay = lf * (float)uy * S.g_idl32[1], az = lf * (float)uz * S.g_idl32[2];
+    float mx = S.gr32[0], my = S.gr32[1], mz = S.gr32[2];
+    float gx = ((float)px - S.g_lo32[0]) * S.g_idl32[0], gy = ((float)py - S.g_lo32[1]) * S.g_idl32[1],
+          gz = ((float)pz - S.g_lo32[2]) * S.g_idl32[2];
+    float bx = floorf(gx), by = floorf(gy), bz = floorf(gz);
+    // starts inside the grid, clear of the voxel's faces?
+    const auto within = [&]() {
+        return gx > mx && gx < (float)nx - mx && gy > my && gy < (float)ny - my && gz > mz && gz < (float)nz - mz;
+    };
+    const auto clear = [](float g, float b, float m) { return fminf(g - b, b + 1.f - g) > 2.f * m; };
+    if (!(within() && clear(gx, bx, mx) && clear(gy, by, my) && clear(gz, bz, mz))) {
+        // both ends beyond one side of the grid: no voxel
+        const float hx = gx + ax, hy = gy + ay, hz = gz + az;
+        const float ex = mx + 1e-6f * (fabsf(gx) + fabsf(ax)), ey = my + 1e-6f * (fabsf(gy) + fabsf(ay)),
+                    ez = mz + 1e-6f * (fabsf(gz) + fabsf(az));
+        if (fminf(gx, hx) > (float)nx + ex || fmaxf(gx, hx) < -ex || fminf(gy, hy) > (float)ny + ey ||
+            fmaxf(gy, hy) < -ey || fminf(gz, hz) > (float)nz + ez || fmaxf(gz, hz) < -ez)
+            return 0u;
+        // FP64 differences, and the index itself where that is not enough
+        mx = S.gm32[0]; my = S.gm32[1]; mz = S.gm32[2];
+        const double ox = px - S.g_lo[0], oy = py - S.g_lo[1], oz = pz - S.g_lo[2];
+        gx = (float)ox * S.g_idl32[0]; gy = (float)oy * S.g_idl32[1]; gz = (float)oz * S.g_idl32[2];
+        if (!within()) return tally64(S, flu, px, py, pz, ux, uy, uz, len, w);
+        bx = floorf(gx); by = floorf(gy); bz = floorf(gz);
+        if (!clear(gx, bx, mx)) bx = (float)floor(div64(ox, S.g_dl[0]));
+        if (!clear(gy, by, my)) by = (float)floor(div64(oy, S.g_dl[1]));
+        if (!clear(gz, bz, mz)) bz = (float)floor(div64(oz, S.g_dl[2]));
+    }
     int ix = (int)bx, iy = (int)by, iz = (int)bz;
+    float sx = gx - bx, sy = gy - by, sz = gz - bz;          // position in the voxel
     // voxels to the plane ahead of each axis, and 1 / (voxels the segment advances)
-    sx = ax > 0.f ? 1.f - sx : sx; sy = ay > 0.f ? 1.f - sy : sy; sz = az > 0.f ? 1.f - sz : sz;
+    // (a direction of zero has none)
+    sx = ax > 0.f ? 1.f - sx : ux == 0.0 ? 1e6f : sx;
+    sy = ay > 0.f ? 1.f - sy : uy == 0.0 ? 1e6f : sy;
+    sz = az > 0.f ? 1.f - sz : uz == 0.0 ? 1e6f : sz;
     const float vx = __fdividef(1.f, fmaxf(fabsf(ax), 1e-30f)), vy = __fdividef(1.f, fmaxf(fabsf(ay), 1e-30f)),
                 vz = __fdividef(1.f, fmaxf(fabsf(az), 1e-30f));
     double t = 0.0;
@@ -550,19 +609,26 @@ static __device__ __noinline__ unsigned tally64_screened(const DevScene &S, long
                     oz = (sz + 2.f * mz) * vz * kScrUp;
         const bool cx = ox < fminf(ly, lz), cy = oy < fminf(lx, lz), cz = oz < fminf(lx, ly);
         if (!ends && (!(cx || cy || cz) || !(fminf(ox, fminf(oy, oz)) < kScrDown)))   // a tie, for FP32
-            return npieces + walk64(S, flu, px, py, pz, ux, uy, uz, ix, iy, iz, t, len, w);
+            return npieces + walk_rest64(S, flu, px, py, pz, ux, uy, uz, ix, iy, iz, t, len, w);
         const bool up = (cx ? ax : cy ? ay : az) > 0.f;
         const int i = cx ? ix : cy ? iy : iz, n = cx ? nx : cy ? ny : nz;
         const bool leaves = !ends && (up ? i + 1 >= n : i == 0);
         double tend = len;
         if (!ends) {
-            const double lo = cx ? S.g_lo[0] : cy ? S.g_lo[1] : S.g_lo[2];
-            const double dl = cx ? S.g_dl[0] : cy ? S.g_dl[1] : S.g_dl[2];
             const double p = cx ? px : cy ? py : pz, u = cx ? ux : cy ? uy : uz;
-            tend = div64((lo + (double)(i + up) * dl) - p, u);
+            double plane;
+            if (S.planes != nullptr) {
+                plane = __ldg(S.planes + (cx ? 0 : cy ? nx + 1 : nx + ny + 2) + i + up);
+            } else {
+                const double lo = cx ? S.g_lo[0] : cy ? S.g_lo[1] : S.g_lo[2];
+                const double dl = cx ? S.g_dl[0] : cy ? S.g_dl[1] : S.g_dl[2];
+                plane = lo + (double)(i + up) * dl;
+            }
+            tend = div64(plane - p, u);
             if (leaves) {                        // the grid's own face clips the segment
-                const double hi = cx ? S.g_hi[0] : cy ? S.g_hi[1] : S.g_hi[2];
-                tend = fmin(tend, div64((up ? hi : lo) - p, u));
+                const double face = up ? (cx ? S.g_hi[0] : cy ? S.g_hi[1] : S.g_hi[2])
+                                       : (cx ? S.g_lo[0] : cy ? S.g_lo[1] : S.g_lo[2]);
+                tend = min64(tend, div64(face - p, u));
             }
         }
         const double piece = tend - t;
