@@ -285,9 +285,9 @@ cudaError_t launch_kernel(int precision, JobWork *jobs, int njobs, int *status, 
                                    : launch_mixed(jobs, njobs, status, blocks, threads, s, variant);
 }
 
-// Register budgets measured fastest at full size on GB300 (see the design
-// notes): mixed 96 registers x 5 blocks/SM, FP64 146 registers x 3 blocks/SM.
-int default_variant(int precision) { return precision == SMCRT_FP64 ? 1 : 0; }
+// Register budgets of served rounds: mixed 96 registers x 5 blocks/SM until the
+// trials on the first mixed job, FP64 3 blocks/SM.
+int serving_variant(int precision) { return precision == SMCRT_FP64 ? 1 : 0; }
 
 uint64_t shape_key(const smcrt_scene *sc, int precision, const smcrt_grid *g)
 {
@@ -488,7 +488,6 @@ int build_plan(smcrt_ctx *ctx, const smcrt_scene *sc, const smcrt_source *src, c
     std::unique_ptr<smcrt_plan> pl(new smcrt_plan());
     pl->ctx = ctx;
     pl->precision = precision;
-    pl->variant = default_variant(precision);
     if (cudaSetDevice(ctx->device) != cudaSuccess) return SMCRT_ERR_CUDA;
     if (serving_stream) {
         if (cudaMallocAsync(&pl->dbuf, total, serving_stream) != cudaSuccess) return SMCRT_ERR_NO_MEMORY;
@@ -653,7 +652,7 @@ int build_plan(smcrt_ctx *ctx, const smcrt_scene *sc, const smcrt_source *src, c
 void default_launch(const smcrt_plan *pl, uint64_t npackets, int &blocks, int &threads, int &variant)
 {
     const bool few = pl->precision == SMCRT_FP64 && !pl->chosen && npackets < kFewFp64Packets;
-    variant = few ? kFewFp64Variant : pl->variant;
+    variant = pl->chosen ? pl->variant : default_variant(pl->precision, npackets, pl->host);
     threads = pl->threads > 0 ? pl->threads : 128;
     blocks = pl->blocks;
     if (blocks <= 0) {
@@ -835,7 +834,7 @@ void scheduler(smcrt_ctx *ctx)
     int threads_m = 128, variant_m = 0;
     int blocks_m = ctx->sm_count * std::max(1, occupancy_mixed_multi(threads_m, variant_m));
     const int threads_d = 128;
-    const int blocks_d = ctx->sm_count * std::max(1, occupancy_fp64(threads_d, default_variant(SMCRT_FP64)));
+    const int blocks_d = ctx->sm_count * std::max(1, occupancy_fp64(threads_d, serving_variant(SMCRT_FP64)));
     bool tuned_served = false;
     int clk_khz = 1900000;
     cudaDeviceGetAttribute(&clk_khz, cudaDevAttrClockRate, ctx->device);
@@ -892,7 +891,7 @@ void scheduler(smcrt_ctx *ctx)
                 cudaStreamWaitEvent(st2, ev_fork, 0);
                 launch_mixed_multi(b.d_tab, kMaxSlots, d_status + bi, blocks_m, threads_m, st, variant_m + off);
                 launch_fp64(b.d_tab + kMaxSlots, kMaxSlots, d_status + bi, blocks_d, threads_d, st2,
-                            default_variant(SMCRT_FP64) + off);
+                            serving_variant(SMCRT_FP64) + off);
                 cudaEventRecord(ev_join, st2);
                 cudaStreamWaitEvent(st, ev_join, 0);
                 cudaMemcpyAsync(b.h_tot, d_tot, sizeof(smcrt_totals) * kMaxSlots, cudaMemcpyDeviceToHost, st);

@@ -381,6 +381,23 @@ int occupancy_mixed_multi(int threads, int variant = 0);
 constexpr uint64_t kFewFp64Packets = 1u << 19;
 constexpr int kFewFp64Variant = 2;
 
+// Mixed plan launches run 4 blocks of 128 threads per SM with 128 registers
+// (variant 1) unless the caller or the autotuner chose a shape, and 5 blocks
+// with 96 registers (variant 0) from this many packets on in scenes without
+// general shapes or a cell list.  Measured, variant 0 / 1: layered slab 1e5
+// packets 3.97 / 3.70 ms, 5e5 9.86 / 9.58, 1e6 17.01 / 17.08, 2e6 31.3 /
+// 31.7; glass container 5e5 16.95 / 16.18 ms, 1e6 23.7 / 23.4; thick slab 1e5
+// 30.0 / 26.7 ms, 1e6 70.6 / 72.2; vessel tree 4e6 135 / 130 ms; shape
+// gallery 5e5 165 / 158 ms.
+constexpr uint64_t kManyMixedPackets = 3u << 18;
+
+// Variant of a plan launch whose shape nobody chose.
+inline int default_variant(int precision, uint64_t npackets, const DevScene &S)
+{
+    if (precision == SMCRT_FP64) return npackets < kFewFp64Packets ? kFewFp64Variant : 1;
+    return npackets < kManyMixedPackets || S.general || S.cull_region >= 0 ? 1 : 0;
+}
+
 // Lanes of a warp that carry packets in a plan launch (JobWork.lanes; 0 =
 // all).  A launch with fewer packets than lanes is bound by the latency of
 // one loop iteration, which grows with the number of different branches a

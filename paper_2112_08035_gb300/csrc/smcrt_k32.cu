@@ -183,7 +183,7 @@ __device__ __noinline__ void refine64(const DevScene &S, int istar, int rnear, i
     pz = (float)(qz + s * vz + rest * nz);
 }
 
-// A crossing of a surface (Sec. 2.3), out of line: Fresnel reflection or
+// A crossing of a surface (Sec. 2.3): Fresnel reflection or
 // Snell refraction when the refractive index changes (FP32 on planar faces,
 // refine64 where the cosines are ill-conditioned or the normal is noisy),
 // or a straight crossing when it does not (matched); the line-preserving
@@ -261,6 +261,97 @@ static __device__ __noinline__ Crossed cross32(const DevScene &S, float ux, floa
     return o;
 }
 
+// Value of one surface (region program, or the bounding box for r = -1).
+template <bool G>
+static __device__ __noinline__ float surface32(const DevScene &S, int r, float x, float y, float z)
+{
+    if (r < 0) return box32(x, y, z, S.bbc32[0], S.bbc32[1], S.bbc32[2], S.bbh32[0], S.bbh32[1], S.bbh32[2]);
+    if (r == S.cull_region) return culled_region32(S, x, y, z);
+    const int2 rr = (*(S.rrange + r));
+    return run_prog32<G>(S, rr.x, rr.y, x, y, z);
+}
+
+// A packet within delta32 of a surface (Sec. 2.3), all of it at once, out of
+// line: normal (analytic, or six probes of the one surface), approach test,
+// the regions on both sides, Fresnel / Snell and the landing.  Taken step by
+// step in the packet loop it ran for 1.5 lanes of 32 in nearly every
+// iteration, a quarter of the time (layered slab); a warp's packets wait for
+// each other (kWaitArrive), since the routine costs as much for one lane as
+// for all.  Layered slab 1e7 packets 157 -> 148 ms, glass container 4e6 73.5
+// -> 64.2 ms, shape gallery (six full evaluations per normal before) 2e5
+// packets 407 -> 138 ms.
+struct Interface32 {
+    float px, py, pz, ux, uy, uz, tau, pend;   // after a crossing
+    int what;
+    int refined;
+};
+enum { kIntfForced = 0, kIntfEscape = 1, kIntfInteract = 2, kIntfMatched = 3, kIntfFresnel = 4 };
+
+template <bool G>
+static __device__ __noinline__ Interface32 interface32(const DevScene &S, float px, float py, float pz, float ux,
+                                                       float uy, float uz, float tau, int reg, int istar,
+                                                       float dstar, uint32_t event, uint32_t id_lo, uint32_t id_hi,
+                                                       uint32_t k0, uint32_t k1)
+{
+    Interface32 o;
+    o.refined = 0;
+    float nx, ny, nz;
+    if (!G || S.analytic_nrm) {              // gradient of a short program
+        grad_surface32(S, istar, px, py, pz, nx, ny, nz);
+    } else {                                 // central differences
+        const float h = S.h32;
+        float g[3];
+        for (int a = 0; a < 3; ++a) {
+            const float fp = surface32<G>(S, istar, a == 0 ? px + h : px, a == 1 ? py + h : py, a == 2 ? pz + h : pz);
+            const float fm = surface32<G>(S, istar, a == 0 ? px - h : px, a == 1 ? py - h : py, a == 2 ? pz - h : pz);
+            g[0] = a == 0 ? fp - fm : g[0];
+            g[1] = a == 1 ? fp - fm : g[1];
+            g[2] = a == 2 ? fp - fm : g[2];
+        }
+        nx = g[0]; ny = g[1]; nz = g[2];
+    }
+    o.what = kIntfForced;
+    const float l2 = nx * nx + ny * ny + nz * nz;
+    if (!(l2 > 0.f)) return o;
+    const float il = rsqrtf(l2);
+    nx *= il; ny *= il; nz *= il;
+    const float cdot = ux * nx + uy * ny + uz * nz;
+    if (!((cdot > 0.f && dstar < 0.f) || (cdot < 0.f && dstar >= 0.f))) return o;
+    o.what = kIntfEscape;
+    if (istar < 0) return o;
+    // the optical depth runs out before the surface: interact here, at the
+    // arrival point (inside this region by evaluation).  Moving on by tau /
+    // mu_t could round the point across the surface, and a packet scattered
+    // just inside a clear glass wall can take a direction that total internal
+    // reflection traps at both walls.
+    o.what = kIntfInteract;
+    if (tau < __fmul_rn(reg >= 0 ? (*(S.reg32 + 2 * reg)).x : 0.f, approach_len32(dstar, cdot))) return o;
+    const float qx = px - dstar * nx, qy = py - dstar * ny, qz = pz - dstar * nz;
+    const float sg = cdot > 0.f ? 1.f : -1.f;
+    int rfar = -1, rnear = -1;
+    for (int side = 0; side < 2; ++side) {   // the regions beyond and before the surface
+        const float e = (side == 0 ? 2.f : -2.f) * S.delta32 * sg;
+        rnear = scene_eval32<G>(S, qx + e * nx, qy + e * ny, qz + e * nz).region;
+        if (side == 0) rfar = rnear;
+    }
+    // matched indices cross on the ray, as a Fresnel landing does.  A push
+    // along n alone never advances along u, and where the normal turns
+    // between the two sides (a smooth union's crease) a packet moving along
+    // the wall was pushed back and forth across it until the step cap.
+    const bool matched = region_n32(S, rnear) == region_n32(S, rfar);
+    uint32_t xiw = 0u;
+    if (!matched) xiw = philox4x32_10(make_uint4(event, 0u, id_lo, id_hi), k0, k1).x;
+    const Crossed c = cross32<G>(S, ux, uy, uz, qx, qy, qz, nx, ny, nz, tau, dstar, cdot, istar, rnear, rfar, xiw,
+                                 matched);
+    o.what = matched ? kIntfMatched : kIntfFresnel;
+    o.refined = c.refined;
+    o.px = c.px; o.py = c.py; o.pz = c.pz;
+    o.ux = c.ux; o.uy = c.uy; o.uz = c.uz;
+    o.tau = c.tau;
+    o.pend = c.pend;
+    return o;
+}
+
 // Photon release (Sec. 2.1), out of line: position and direction from the
 // source (pencil, disc, square, isotropic point) and the first optical depth
 // (Eq. 1), from one Philox call's words.
@@ -299,6 +390,15 @@ static __device__ __noinline__ Launched launch32(const DevScene &S, uint4 r)
     o.tau = -__logf(u01_32(r.w));
     return o;
 }
+
+// Packets at a surface are served when the lane iterations that they have
+// waited reach kWaitArrive times the live lanes, or when no other lane can
+// move.  Layered slab 2e6 packets: served at once 41.6 ms, factor 1/2 33.3, 1
+// 31.9, 2 31.4, 5 31.3; glass container 1e6 29.3, 24.8, 23.7, 23.7, 23.8.
+// Setting them aside in shared memory, so that their lanes go on with other
+// packets, measured slower (33.4 and 24.4 ms): the traffic of 24 words each
+// way, and a longer tail with 56 packets per warp.
+constexpr int kWaitArrive = 2;
 
 // Per-warp shared state: the staged scene and the warp's tally slots.
 // Scene-table staging (a launch option the autotuner tries): the warp copies
@@ -425,15 +525,14 @@ __device__ __forceinline__ void multi_stage(JobSlot *sl, JobWork *J, int lane)
 }
 
 // One warp works through packet ids of job J until the job's cursor passes
-// its end.  Iteration structure (all lanes execute every stage; a lane's
-// phase only selects operands or predicates a short update):
+// its end.  Iteration structure:
 //   1 refill dead lanes (one atomicAdd per warp),
-//   2 one FP32 scene evaluation at the lane's phase point,
-//   3 classify: escape / start interface / move / normal bookkeeping /
-//     far-near regions / Fresnel,
+//   2 one FP32 scene evaluation for the lanes that trace,
+//   3 classify: escape / arrive at a surface (and wait) / move; the interface
+//     routine for the waiting lanes, once enough of them wait,
 //   4 the track-length tally of this iteration's move (one call site),
-//   5 one Philox call serving launch, interaction and Fresnel draws,
-//   6 the consumers: release a packet, scatter (HG + roulette), Fresnel.
+//   5 one Philox call serving release and interaction draws,
+//   6 the consumers: release a packet, scatter (HG + roulette).
 //
 // MULTI = false (plan launches): one job, jobs[0], in slots[0].  MULTI =
 // true (served rounds): the warp works through the table jobs[0, njobs)
@@ -443,7 +542,7 @@ template <bool G, bool MULTI>
 __device__ bool run_job_mixed(JobSlot *slots, JobWork *jobs, int njobs, int first, int *status, int lane)
 {
     const DevScene &S0 = slots[0].S;
-    const float delta0 = S0.delta32, hstep0 = S0.h32;
+    const float delta0 = S0.delta32;
     const volatile JobConst *const jc0 = &slots[0].jc;
     JobWork *const J = jobs;
     int js = 0;                          // the lane's job slot
@@ -472,7 +571,7 @@ __device__ bool run_job_mixed(JobSlot *slots, JobWork *jobs, int njobs, int firs
     // a small plan launch spreads its packets over all warps
     bool alive = false, retired = !MULTI && J->lanes > 0 && lane >= J->lanes;
     float px = 0, py = 0, pz = 0, ux = 0, uy = 0, uz = 0, w = 0, tau = 0;
-    float qx = 0, qy = 0, qz = 0;        // FAR / NEAR: surface point; TRACE: crawl anchor
+    float qx = 0, qy = 0, qz = 0;        // crawl anchor
     // Crawl: a packet within delta32 of a surface that it is leaving takes
     // forced steps of delta32 along u.  Adding the same small step to an
     // FP32 position again and again rounds the same way every time, and over
@@ -482,14 +581,16 @@ __device__ bool run_job_mixed(JobSlot *slots, JobWork *jobs, int njobs, int firs
     // q + cs u (one rounding, whatever the step count).  cs < 0: no crawl.
     float cs = -1.f;
     float pend = 0.f;                    // track length of a crossing's shortcut, tallied with the next move
-    float nx = 0, ny = 0, nz = 0, cdot = 0, fplus = 0, dstar = 0;
-    int phase = kTrace, sub = 0, istar = -1, reg = -1, rfar = -1;
+    float dstar = 0;                     // at a surface
+    int phase = kTrace, istar = -1, reg = -1;
+    int waited = 0;                      // lane iterations that packets at a surface have waited (warp-uniform)
     int nsteps = 0;
     unsigned pscat = 0, npieces = 0;
     long long pA = 0, pG = 0;
     uint32_t id_lo = 0, id_hi = 0, event = 0;
     uint32_t t_acq = 0;
     bool timed_out = false;              // the launch's time limit stopped the refills
+    unsigned long long nev = 0ull;       // scene evaluations of the warp (plan launches)
 
     for (;;) {
         // ---- 1. refill: this job's parked packets first, then new ids
@@ -629,137 +730,97 @@ __device__ bool run_job_mixed(JobSlot *slots, JobWork *jobs, int njobs, int firs
         // the lane's job: its scene, constants and accumulator (one job in a
         // plan launch; compile-time slot 0 there)
         const DevScene &S = MULTI ? slots[js].S : S0;
-        const float delta = MULTI ? S.delta32 : delta0, hstep = MULTI ? S.h32 : hstep0;
+        const float delta = MULTI ? S.delta32 : delta0;
         const volatile JobConst *const jc = MULTI ? &slots[js].jc : jc0;
         WarpAcc *const wa = MULTI ? &slots[js].acc : &slots[0].acc;
 
         // ---- 2. the scene evaluation of this iteration
-        const float sg = cdot > 0.f ? 1.f : -1.f;
-        float ex = px, ey = py, ez = pz;
-        int sel = -2;
-        if (G && SMCRT_RARE(phase == kNrm)) {   // probe normals: general instantiation only
-            const float hh = (sub & 1) ? -hstep : hstep;
-            const int a = sub >> 1;
-            if (a == 0) ex = px + hh; else if (a == 1) ey = py + hh; else ez = pz + hh;
-            sel = istar;
-        } else if (SMCRT_RARE(phase == kFar || phase == kNear)) {
-            const float e = (phase == kFar ? 2.f : -2.f) * delta * sg;
-            ex = qx + e * nx; ey = qy + e * ny; ez = qz + e * nz;
-        }
-        const Eval32 E = scene_eval32<G>(S, ex, ey, ez, sel);
+        const bool evals = alive && phase == kTrace;
+        Eval32 E{};
+        if (evals) E = scene_eval32<G>(S, px, py, pz);
         if (MULTI) {                           // evaluations counted per job slot
             for (int k = 0; k < kMultiSlots; ++k) {
-                const unsigned ev = __ballot_sync(SMCRT_FULL, alive && phase != kLaunch && js == k);
+                const unsigned ev = __ballot_sync(SMCRT_FULL, evals && js == k);
                 if (lane == 0 && ev != 0u) wadd(&slots[k].acc, kEvals, __popc(ev));
             }
         } else {
-            const unsigned ev = __ballot_sync(SMCRT_FULL, alive && phase != kLaunch);
-            if (lane == 0) wadd(wa, kEvals, __popc(ev));
+            nev += __popc(__ballot_sync(SMCRT_FULL, evals));
         }
 
         // ---- 3. classify
-        bool move = false, fresnel = false, iter_done = false, nrm_ready = false;
+        bool move = false, iter_done = false;
         bool seg_step = false;                 // a tracing move that segment stepping may lengthen
         bool crawl = false;                    // a forced step away from a surface
+        bool out = false;                      // leaves the volume: R or T
         bool fin = false;                      // the packet ends this iteration
-        bool near_hit = false;                 // interacts before reaching the surface
-        bool matched = false;                  // a crossing without an index change
+        bool interact = false;
         long long fin_R = 0, fin_T = 0, fin_K = 0;
         float L = 0.f;
-        int rnear = -1;
-        if (alive) {
-            if (phase == kTrace) {
-                if (SMCRT_RARE(E.dbox > 0.f)) {
-                    {                                          // leaves the volume: R or T
-                        const long long v = fx32(w);
-                        if (ux * S.src_dir32[0] + uy * S.src_dir32[1] + uz * S.src_dir32[2] < 0.f) fin_R = v; else fin_T = v;
-                        fin = true;
-                        alive = false;
-                    }
+        if (evals) {
+            if (SMCRT_RARE(E.dbox > 0.f)) {
+                out = true;
+            } else {
+                reg = E.region;
+                if (SMCRT_RARE(E.dmin < delta)) {
+                    istar = E.istar;
+                    dstar = E.dstar;
+                    phase = kArrive;
                 } else {
-                    reg = E.region;
-                    if (SMCRT_RARE(E.dmin < delta)) {
-                        istar = E.istar;
-                        dstar = E.dstar;
-                        if (!G || S.analytic_nrm) {        // gradient of a short program, now
-                            grad_surface32(S, istar, px, py, pz, nx, ny, nz);
-                            nrm_ready = true;
-                        } else {                           // six probes in the next iterations
-                            phase = kNrm;
-                            sub = 0;
-                        }
-                    } else {
-                        L = E.dmin - 0.5f * delta;
-                        move = true;
-                        seg_step = S.stepping == SMCRT_STEP_SEGMENT;
-                    }
+                    L = E.dmin - 0.5f * delta;
+                    move = true;
+                    seg_step = S.stepping == SMCRT_STEP_SEGMENT;
                 }
-            } else if (G && SMCRT_RARE(phase == kNrm)) {
-                const float f = E.dsel;
-                if ((sub & 1) == 0) {
-                    fplus = f;
-                } else {
-                    const float gg = fplus - f;
-                    const int a = sub >> 1;
-                    if (a == 0) nx = gg; else if (a == 1) ny = gg; else nz = gg;
-                }
-                if (++sub >= 6) nrm_ready = true;
-            } else if (phase == kFar) {
-                rfar = E.region;
-                phase = kNear;
-            } else if (phase == kNear) {
-                rnear = E.region;
-                // matched indices cross on the ray, as a Fresnel landing does
-                // (cross32).  A push along n alone never advances along u, and
-                // where the normal turns between the two sides (a smooth
-                // union's crease) a packet moving along the wall was pushed
-                // back and forth across it until the step cap.
-                matched = region_n32(S, rnear) == region_n32(S, rfar);
-                fresnel = true;
             }
         }
 
-        // ---- 3b. a normal is ready (analytic, or after the sixth probe)
-        if (SMCRT_RARE(nrm_ready)) {
-            const float l2 = nx * nx + ny * ny + nz * nz;
-            bool approaching = false;
-            if (l2 > 0.f) {
-                const float il = rsqrtf(l2);
-                nx *= il; ny *= il; nz *= il;
-                cdot = ux * nx + uy * ny + uz * nz;
-                approaching = (cdot > 0.f && dstar < 0.f) || (cdot < 0.f && dstar >= 0.f);
+        // ---- 3b. the packets at a surface, once enough of them wait
+        const unsigned arrived = __ballot_sync(SMCRT_FULL, alive && phase == kArrive);
+        if (SMCRT_RARE(arrived != 0u)) {
+            waited += __popc(arrived);
+            if (waited >= kWaitArrive * __popc(__ballot_sync(SMCRT_FULL, alive)) ||
+                __ballot_sync(SMCRT_FULL, alive && (move || phase == kLaunch)) == 0u) {
+                waited = 0;
+                if (alive && phase == kArrive) {
+                    const Interface32 I = interface32<G>(S, px, py, pz, ux, uy, uz, tau, reg, istar, dstar, event,
+                                                         id_lo, id_hi, jc->k0, jc->k1);
+                    phase = kTrace;
+                    if (G && !S.analytic_nrm) wadd(wa, kEvals, 6);   // the probes
+                    if (I.what == kIntfForced) {
+                        L = delta;                          // forced step along u
+                        move = true;
+                        crawl = true;
+                    } else if (I.what == kIntfEscape) {
+                        out = true;
+                    } else if (I.what == kIntfInteract) {
+                        interact = true;
+                        cs = -1.f;
+                        iter_done = true;
+                    } else {
+                        wadd(wa, kIntf, 1);
+                        wadd(wa, kEvals, 2);
+                        if (I.what == kIntfFresnel) {
+                            wadd(wa, kFres, 1);
+                            event += 1u;
+                        }
+                        if (I.refined) wadd(wa, kRefined, 1);
+                        px = I.px; py = I.py; pz = I.pz;
+                        ux = I.ux; uy = I.uy; uz = I.uz;
+                        tau = I.tau;
+                        pend = I.pend;
+                        cs = -1.f;
+                        iter_done = true;
+                    }
+                }
             }
-            if (!approaching) {
-                L = delta;                          // forced step along u
-                move = true;
-                crawl = true;
-            } else if (istar < 0) {                 // leaves the volume: R or T
-                const long long v = fx32(w);
-                if (ux * S.src_dir32[0] + uy * S.src_dir32[1] + uz * S.src_dir32[2] < 0.f) fin_R = v; else fin_T = v;
-                fin = true;
-                alive = false;
-            } else if (tau < __fmul_rn(reg >= 0 ? (*(S.reg32 + 2 * reg)).x : 0.f, approach_len32(dstar, cdot))) {
-                // the optical depth runs out before the surface: interact here,
-                // at the arrival point (inside this region by evaluation).  Moving
-                // on by tau / mu_t could round the point across the surface, and
-                // a packet scattered just inside a clear glass wall can take a
-                // direction that total internal reflection traps at both walls.
-                near_hit = true;
-            } else {
-                wadd(wa, kIntf, 1);
-                qx = px - dstar * nx; qy = py - dstar * ny; qz = pz - dstar * nz;
-                cs = -1.f;
-                phase = kFar;
-            }
+        }
+        if (SMCRT_RARE(out)) {
+            const long long v = fx32(w);
+            if (ux * S.src_dir32[0] + uy * S.src_dir32[1] + uz * S.src_dir32[2] < 0.f) fin_R = v; else fin_T = v;
+            fin = true;
+            alive = false;
         }
 
         // ---- 4. move: interaction point or sphere-trace step, one tally site
-        bool interact = near_hit;
-        if (SMCRT_RARE(near_hit)) {
-            cs = -1.f;
-            phase = kTrace;                        // also after the sixth probe
-            iter_done = true;
-        }
         if (move) {
             float mu_t = 0.f, imu_t = 0.f;
             if (reg >= 0) {
@@ -768,7 +829,7 @@ __device__ bool run_job_mixed(JobSlot *slots, JobWork *jobs, int njobs, int firs
             }
             interact = mu_t > 0.f && tau < mu_t * L;
             if (SMCRT_RARE(seg_step && !interact)) {           // segment stepping: a longer move along u
-                L = fmaxf(L, segment_bound32<G>(S, E.dsoft, E.dbox, px, py, pz, ux, uy, uz));
+                L = fmaxf(L, segment_bound32<G>(S, L, E.dsoft, E.dbox, px, py, pz, ux, uy, uz));
                 interact = mu_t > 0.f && tau < mu_t * L;
             }
             const float seg = interact ? tau * imu_t : L;
@@ -791,7 +852,7 @@ __device__ bool run_job_mixed(JobSlot *slots, JobWork *jobs, int njobs, int firs
         }
 
         // ---- 5. one Philox call for every lane that draws this iteration
-        const bool draws = alive && (phase == kLaunch || interact || (fresnel && !matched));
+        const bool draws = alive && (phase == kLaunch || interact);
         uint4 r = make_uint4(0u, 0u, 0u, 0u);
         if (__any_sync(SMCRT_FULL, draws)) {
             r = philox4x32_10(make_uint4(event, 0u, id_lo, id_hi), jc->k0, jc->k1);
@@ -829,18 +890,6 @@ __device__ bool run_job_mixed(JobSlot *slots, JobWork *jobs, int njobs, int firs
                     alive = false;
                 }
             }
-        }
-        if (SMCRT_RARE(fresnel)) {                             // reflect, refract or cross (Sec. 2.3)
-            const Crossed c = cross32<G>(S, ux, uy, uz, qx, qy, qz, nx, ny, nz, tau, dstar, cdot, istar, rnear, rfar,
-                                         r.x, matched);
-            if (!matched) wadd(wa, kFres, 1);
-            if (c.refined) wadd(wa, kRefined, 1);
-            px = c.px; py = c.py; pz = c.pz;
-            ux = c.ux; uy = c.uy; uz = c.uz;
-            tau = c.tau;
-            pend = c.pend;
-            phase = kTrace;
-            iter_done = true;
         }
         if (iter_done && alive) {
             nsteps += 1;
@@ -913,7 +962,10 @@ __device__ bool run_job_mixed(JobSlot *slots, JobWork *jobs, int njobs, int firs
         return false;
     }
     const long long pc = warp_sum((long long)npieces);
-    if (lane == 0) wadd(&slots[0].acc, kPieces, pc);
+    if (lane == 0) {
+        wadd(&slots[0].acc, kPieces, pc);
+        wadd(&slots[0].acc, kEvals, (long long)nev);
+    }
     return timed_out;
 }
 

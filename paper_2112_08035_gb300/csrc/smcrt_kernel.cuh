@@ -5,20 +5,14 @@
 // from a ballot), so a lane whose packet terminates is refilled at the
 // next iteration and the warp stays full until the job runs dry.
 //
-// Every loop iteration performs exactly ONE full scene SDF evaluation per
-// lane (the dominant cost, Sec. 4 "having to evaluate every SDF each time
-// the photon needs to be moved").  What the lane does with it depends on
-// its phase:
-//   TRACE  evaluate at p: bounding box exit, interaction or sphere-trace
-//          step (Sec. 2.3, Fig. 2 right, Fig. 3; Eq. 1 for tau),
-//   NRM    six probes p +/- h e_a of the nearest surface's SDF: central
-//          differences for the normal (Sec. 1 "numerical differentiation"),
-//   PROJ   (FP64) Newton projection onto the surface along the normal,
-//   FAR    region on the far side of the surface,
-//   NEAR   region on the near side; then Fresnel reflection or Snell
-//          refraction if the refractive index changes (Sec. 2.3).
-// Lanes at an interface therefore share the scene evaluation with lanes
-// that are tracing, instead of running a divergent interface routine.
+// Every loop iteration performs one scene SDF evaluation per tracing lane
+// (Sec. 4 "having to evaluate every SDF each time the photon needs to be
+// moved"): bounding box exit, interaction or sphere-trace step (Sec. 2.3,
+// Fig. 2 right, Fig. 3; Eq. 1 for tau).  A lane within delta of a surface
+// waits until several do, and then takes the interface routine with them:
+// the normal (Sec. 1 "numerical differentiation", or the analytic gradient
+// in the mixed kernel), the regions on both sides, Fresnel reflection or
+// Snell refraction if the refractive index changes (Sec. 2.3).
 //
 // The FP64 instantiation performs the same IEEE operations in the same
 // order as the FP64 reference algorithm (compiled with -fmad=false), with
@@ -200,7 +194,7 @@ __device__ __forceinline__ long long fx32(float x) { return __float2ll_rn(x * 42
 // ---------------------------------------------------------------------------
 // dsoft: min |d| over soft regions (segment stepping), +inf if none.
 struct Eval64 { double dmin, dstar, dsel, dbox, dsoft; int istar, region; };
-struct Eval32 { float dmin, dstar, dsel, dbox, dsoft; int istar, region; };
+struct Eval32 { float dmin, dstar, dbox, dsoft; int istar, region; };
 
 // The larger / smaller of two numbers (not NaN), compared as integers: an
 // FP64 fmax takes the FP64 pipe 2.4 times as long as an addition.
@@ -466,9 +460,8 @@ __device__ __forceinline__ double run_prog64(const DevScene &S, int i0, int i1, 
     return s0;
 }
 
-template <bool kFull, bool G>
-__device__ __forceinline__ float run_prog32(const DevScene &S, int i0, int i1, float x, float y, float z,
-                                            int sel, Eval32 *E)
+template <bool G>
+__device__ __forceinline__ float run_prog32(const DevScene &S, int i0, int i1, float x, float y, float z)
 {
     float s0 = 0.f, s1 = 0.f, s2 = 0.f, s3 = 0.f;
     for (int i = i0; i < i1; ++i) {
@@ -486,14 +479,6 @@ __device__ __forceinline__ float run_prog32(const DevScene &S, int i0, int i1, f
                 s0 = csg32(op, s1, s0, kinv);
                 s1 = s2; s2 = s3;
             }
-        }
-        if (kFull && ins.z >= 0) {
-            const float d = s0;
-            if (d < 0.f) E->region = ins.z;
-            const float ad = fabsf(d);
-            if (ad < E->dmin) { E->dmin = ad; E->istar = ins.z; E->dstar = d; }
-            if ((ins.x & kSoftRegionEnd) && ad < E->dsoft) E->dsoft = ad;
-            if (ins.z == sel) E->dsel = d;
         }
     }
     return s0;
@@ -538,13 +523,12 @@ __device__ __forceinline__ float culled_region32(const DevScene &S, float x, flo
     return fminf(acc, S.cull_rmax);
 }
 
-__device__ __forceinline__ void region_end32(Eval32 *E, int r, float d, int sel, bool soft)
+__device__ __forceinline__ void region_end32(Eval32 *E, int r, float d, bool soft)
 {
     if (d < 0.f) E->region = r;
     const float ad = fabsf(d);
     if (ad < E->dmin) { E->dmin = ad; E->istar = r; E->dstar = d; }
     if (soft && ad < E->dsoft) E->dsoft = ad;
-    if (r == sel) E->dsel = d;
 }
 
 // One copy of the interpreter in the packet loop: the culled region's
@@ -554,12 +538,13 @@ __device__ __forceinline__ void region_end32(Eval32 *E, int r, float d, int sel,
 // close to the instruction cache's capacity (measured on the layered slab:
 // three interpreter copies 203.6 ms per 1e7 packets, one copy 184.4 ms).
 template <bool G>
-__device__ __forceinline__ Eval32 scene_eval32(const DevScene &S, float x, float y, float z, int sel)
+__device__ __forceinline__ Eval32 scene_eval32(const DevScene &S, float x, float y, float z)
 {
+
     Eval32 E;
     E.dmin = __int_as_float(0x7f800000);
     E.dsoft = E.dmin;
-    E.dstar = 0.f; E.dsel = 0.f; E.istar = -1; E.region = -1;
+    E.dstar = 0.f; E.istar = -1; E.region = -1;
     int cb = S.ninstr, ce = S.ninstr;
     if (S.cull_region >= 0) {
         const int2 rr = (*(S.rrange + S.cull_region));
@@ -571,7 +556,7 @@ __device__ __forceinline__ Eval32 scene_eval32(const DevScene &S, float x, float
         if (i == cb) {
             // the culled region's distance bounds segment moves
             // isotropically (its primitives are not in seg_prims)
-            region_end32(&E, S.cull_region, culled_region32(S, x, y, z), sel, true);
+            region_end32(&E, S.cull_region, culled_region32(S, x, y, z), true);
             i = ce - 1;
             continue;
         }
@@ -590,12 +575,11 @@ __device__ __forceinline__ Eval32 scene_eval32(const DevScene &S, float x, float
                 s1 = s2; s2 = s3;
             }
         }
-        if (ins.z >= 0) region_end32(&E, ins.z, s0, sel, (ins.x & kSoftRegionEnd) != 0);
+        if (ins.z >= 0) region_end32(&E, ins.z, s0, (ins.x & kSoftRegionEnd) != 0);
     }
     const float db = box32(x, y, z, S.bbc32[0], S.bbc32[1], S.bbc32[2], S.bbh32[0], S.bbh32[1], S.bbh32[2]);
     E.dbox = db;
     if (fabsf(db) < E.dmin) { E.dmin = fabsf(db); E.istar = -1; E.dstar = db; }
-    if (sel == -1) E.dsel = db;
     return E;
 }
 
@@ -693,23 +677,13 @@ __device__ __forceinline__ float grad_culled32(const DevScene &S, float x, float
     return acc;
 }
 
-static __device__ __noinline__ float grad_surface32(const DevScene &S, int r, float x, float y, float z, float &gx,
-                                             float &gy, float &gz)
+// Value and gradient of a region's program.
+static __device__ __noinline__ float grad_program32(const DevScene &S, int i0, int i1, float x, float y, float z,
+                                                    float &gx, float &gy, float &gz)
 {
-    if (r >= 0 && r == S.cull_region) return grad_culled32(S, x, y, z, gx, gy, gz);
-    if (r < 0) {
-        const float px = x - S.bbc32[0], py = y - S.bbc32[1], pz = z - S.bbc32[2];
-        const float qx = fabsf(px) - S.bbh32[0], qy = fabsf(py) - S.bbh32[1], qz = fabsf(pz) - S.bbh32[2];
-        gx = gy = gz = 0.f;
-        if (qx >= qy && qx >= qz) { gx = copysignf(1.f, px); return qx; }
-        if (qy >= qz) { gy = copysignf(1.f, py); return qy; }
-        gz = copysignf(1.f, pz);
-        return qz;
-    }
-    const int2 rr = (*(S.rrange + r));
     float v[kMaxStack], vx[kMaxStack], vy[kMaxStack], vz[kMaxStack];
     int sp = 0;
-    for (int i = rr.x; i < rr.y; ++i) {
+    for (int i = i0; i < i1; ++i) {
         const int4 ins = (*(reinterpret_cast<const int4 *>(S.instr) + i));
         const int op = ins.x & 0xff, kind = (ins.x >> 8) & 0xff;
         float a = 0.f, ax = 0.f, ay = 0.f, az = 0.f;
@@ -727,6 +701,27 @@ static __device__ __noinline__ float grad_surface32(const DevScene &S, int r, fl
     }
     gx = vx[0]; gy = vy[0]; gz = vz[0];
     return v[0];
+}
+
+static __device__ __noinline__ float grad_surface32(const DevScene &S, int r, float x, float y, float z, float &gx,
+                                             float &gy, float &gz)
+{
+    if (r >= 0 && r == S.cull_region) return grad_culled32(S, x, y, z, gx, gy, gz);
+    if (r < 0) {
+        const float px = x - S.bbc32[0], py = y - S.bbc32[1], pz = z - S.bbc32[2];
+        const float qx = fabsf(px) - S.bbh32[0], qy = fabsf(py) - S.bbh32[1], qz = fabsf(pz) - S.bbh32[2];
+        gx = gy = gz = 0.f;
+        if (qx >= qy && qx >= qz) { gx = copysignf(1.f, px); return qx; }
+        if (qy >= qz) { gy = copysignf(1.f, py); return qy; }
+        gz = copysignf(1.f, pz);
+        return qz;
+    }
+    const int2 rr = (*(S.rrange + r));
+    if (rr.y - rr.x == 1) {              // a primitive
+        const int4 ins = (*(reinterpret_cast<const int4 *>(S.instr) + rr.x));
+        return prim_grad32(S, (ins.x >> 8) & 0xff, ins.y, x, y, z, gx, gy, gz);
+    }
+    return grad_program32(S, rr.x, rr.y, x, y, z, gx, gy, gz);
 }
 
 // SDF of one surface in FP64 (region program, or the bounding box for -1).
@@ -1045,12 +1040,11 @@ __device__ __forceinline__ float seg_sphere32(float4 A, float d, float px, float
     return t > 0.f ? t : 0.f;
 }
 
-__device__ __forceinline__ float seg_box32(float cx, float cy, float cz, float hx, float hy, float hz, float d,
-                                           float px, float py, float pz, float ux, float uy, float uz, float iux,
-                                           float iuy, float iuz, float dh)
+static __device__ __noinline__ float seg_box_any32(float cx, float cy, float cz, float hx, float hy, float hz, float d,
+                                                   float px, float py, float pz, float ux, float uy, float uz,
+                                                   float iux, float iuy, float iuz, float e)
 {
     const float inf = __int_as_float(0x7f800000);
-    const float e = d > 0.f ? dh : -dh;
     const float c[3] = {cx, cy, cz}, h[3] = {hx, hy, hz}, p[3] = {px, py, pz}, u[3] = {ux, uy, uz};
     const float iu[3] = {iux, iuy, iuz};
     float tn = -inf, tf = inf;
@@ -1066,6 +1060,29 @@ __device__ __forceinline__ float seg_box32(float cx, float cy, float cz, float h
         }
     }
     if (d > 0.f) {
+        if (tn > tf || tf < 0.f) return inf;
+        return tn > 0.f ? tn : 0.f;
+    }
+    return tf > 0.f ? tf : 0.f;
+}
+
+// Of an axis' two planes, the one behind gives the smaller product and the
+// one ahead the larger (rounding is monotone), so from inside only the planes
+// ahead are needed.  Directions with a zero component and boxes that shrink
+// to nothing take the routine with both planes.
+__device__ __forceinline__ float seg_box32(float cx, float cy, float cz, float hx, float hy, float hz, float d,
+                                           float px, float py, float pz, float ux, float uy, float uz, float iux,
+                                           float iuy, float iuz, float dh)
+{
+    const float inf = __int_as_float(0x7f800000);
+    const float e = d > 0.f ? dh : -dh;
+    const float gx = hx + e, gy = hy + e, gz = hz + e;
+    if (SMCRT_RARE(ux == 0.f || uy == 0.f || uz == 0.f || !(fminf(gx, fminf(gy, gz)) >= 0.f)))
+        return seg_box_any32(cx, cy, cz, hx, hy, hz, d, px, py, pz, ux, uy, uz, iux, iuy, iuz, e);
+    const float sx = copysignf(gx, ux), sy = copysignf(gy, uy), sz = copysignf(gz, uz);
+    const float tf = fminf(fminf((cx + sx - px) * iux, (cy + sy - py) * iuy), (cz + sz - pz) * iuz);
+    if (d > 0.f) {
+        const float tn = fmaxf(fmaxf((cx - sx - px) * iux, (cy - sy - py) * iuy), (cz - sz - pz) * iuz);
         if (tn > tf || tf < 0.f) return inf;
         return tn > 0.f ? tn : 0.f;
     }
@@ -1243,8 +1260,10 @@ static __device__ __noinline__ float seg_xprim32(const DevScene &S, int kind, in
 // candidates); most of the loss came with the longer, more uneven moves'
 // tally (without a fluence grid the cell's exit alone cost 4 %).  The
 // isotropic bound is kept.
+// The caller's move is at least L: once the bound is not above it, what is
+// left cannot matter.
 template <bool G>
-static __device__ __noinline__ float segment_bound32(const DevScene &S, float dsoft, float dbox, float px,
+static __device__ __noinline__ float segment_bound32(const DevScene &S, float L, float dsoft, float dbox, float px,
                                                      float py, float pz, float ux, float uy, float uz)
 {
     const float dh = 0.5f * S.delta32;
@@ -1252,7 +1271,7 @@ static __device__ __noinline__ float segment_bound32(const DevScene &S, float ds
     float t = fminf(seg_box32(S.bbc32[0], S.bbc32[1], S.bbc32[2], S.bbh32[0], S.bbh32[1], S.bbh32[2], dbox, px, py,
                               pz, ux, uy, uz, iux, iuy, iuz, dh),
                     dsoft - dh);
-    for (int j = 0; j < S.nseg; ++j) {
+    for (int j = 0; j < S.nseg && t > L; ++j) {
         const int i = __ldg(S.seg_prims + j);
         const int kind = (*(S.pkind + i));
         const float e = __ldg(S.seg_m32 + j) + dh;
@@ -1558,7 +1577,9 @@ __device__ __forceinline__ void jobconst_fill(volatile JobConst *jc, const JobWo
     jc->deadline = J->time_limit_ns > 0ull ? globaltimer_ns() + J->time_limit_ns : 0ull;
 }
 
-enum Phase { kTrace = 0, kNrm = 1, kFar = 3, kNear = 4, kLaunch = 5, kArrive = 6, kExact = 7 };
+// What a packet does next: trace, release, wait at a surface, or (FP64) wait
+// for FP64 distances.
+enum Phase { kTrace = 0, kLaunch = 1, kArrive = 2, kExact = 3 };
 
 constexpr double kWRoulette = 1e-4;   // roulette threshold (MCML convention)
 constexpr double kRouletteM = 10.0;   // survival 1/m, weight x m
