@@ -1436,13 +1436,14 @@ __device__ __forceinline__ void tally32(const DevScene &S, long long *flu, float
     const float tdx = ux != 0.f ? dx * fabsf(iux) : inf;
     const float tdy = uy != 0.f ? dy * fabsf(iuy) : inf;
     const float tdz = uz != 0.f ? dz * fabsf(iuz) : inf;
-    long long off = ((long long)iz * ny + iy) * nx + ix;
-    const long long ox = sx, oy = sy > 0 ? nx : -nx, oz = sz > 0 ? (long long)nx * ny : -(long long)nx * ny;
-    // remaining planes along each axis before the grid ends
-    const int rx = sx > 0 ? nx - 1 - ix : ix, ry = sy > 0 ? ny - 1 - iy : iy, rz = sz > 0 ? nz - 1 - iz : iz;
-    int cx = 0, cy = 0, cz = 0;
+    // a grid has at most 2^30 voxels
+    int off = (iz * ny + iy) * nx + ix;
+    const int ox = sx, oy = sy > 0 ? nx : -nx, oz = sz > 0 ? nx * ny : -nx * ny;
+    // planes left along each axis before the grid ends
+    int rx = sx > 0 ? nx - 1 - ix : ix, ry = sy > 0 ? ny - 1 - iy : iy, rz = sz > 0 ? nz - 1 - iz : iz;
+    const float ws = w * 4294967296.f;   // in units: the same products but for the scale
     float t = tin;
-    for (int guard = nx + ny + nz + 3; guard > 0; --guard) {
+    for (;;) {
         const bool bx = tx <= ty && tx <= tz;
         const bool by = !bx && ty <= tz;
         const bool bz = !bx && !by;
@@ -1450,18 +1451,18 @@ __device__ __forceinline__ void tally32(const DevScene &S, long long *flu, float
         const float tend = fminf(ta, tout);
         const float piece = tend - t;
         if (piece > 0.f) {
-            red_add(flu + off, fx32(w * piece));
+            red_add(flu + off, __float2ll_rn(ws * piece));
             *npieces += 1u;
             t = tend;
         }
         if (ta >= tout) break;
         // step to the next voxel along the axis whose plane came first
-        cx += bx; cy += by; cz += bz;
-        if (cx > rx || cy > ry || cz > rz) break;
-        off += bx ? ox : (by ? oy : oz);
-        tx += bx ? tdx : 0.f;
-        ty += by ? tdy : 0.f;
-        tz += bz ? tdz : 0.f;
+        rx -= bx; ry -= by; rz -= bz;
+        off += bx ? ox : by ? oy : oz;
+        tx = bx ? __fadd_rn(tx, tdx) : tx;
+        ty = by ? __fadd_rn(ty, tdy) : ty;
+        tz = bz ? __fadd_rn(tz, tdz) : tz;
+        if ((rx | ry | rz) < 0) break;
     }
 }
 
