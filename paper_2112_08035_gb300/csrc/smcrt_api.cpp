@@ -387,24 +387,50 @@ void build_cull(const smcrt_scene *sc, CullGrid &cg)
     }
     const double smax = std::max(s[0], std::max(s[1], s[2]));
     const double Rl = 1.05 * std::max(R, smax) + 0.01 * smax;
+    // Per primitive, the squared gaps of the G cells of each axis; only the
+    // cells within Rl on every axis are looked at.  One pass counts, one
+    // fills, primitive by primitive, so a cell's list is in fold order.
+    // (Testing every cell against every primitive took 15 ms of a 64-capsule
+    // plan, and of each such run and served job.)
     cg.off.assign((size_t)G * G * G + 1, 0);
-    cg.list.clear();
-    for (int cz = 0; cz < G; ++cz)
-        for (int cy = 0; cy < G; ++cy)
-            for (int cx = 0; cx < G; ++cx) {
-                const int c = (cz * G + cy) * G + cx;
-                const double clo[3] = {glo[0] + cx * s[0], glo[1] + cy * s[1], glo[2] + cz * s[2]};
-                cg.off[c] = (int32_t)cg.list.size();
-                for (int j = 0; j < n; ++j) {
-                    double d2 = 0.0;
-                    for (int a = 0; a < 3; ++a) {
-                        const double gap = std::max(0.0, std::max(clo[a] - phi[3 * j + a], plo[3 * j + a] - (clo[a] + s[a])));
-                        d2 += gap * gap;
-                    }
-                    if (d2 <= Rl * Rl) cg.list.push_back(bprims[j]);
+    std::vector<double> gap2((size_t)3 * G * n);
+    std::vector<int> from((size_t)3 * n), to((size_t)3 * n);
+    for (int j = 0; j < n; ++j)
+        for (int a = 0; a < 3; ++a) {
+            double *g2 = &gap2[((size_t)3 * j + a) * G];
+            int lo = G, hi = -1;
+            for (int c = 0; c < G; ++c) {
+                const double clo = glo[a] + c * s[a];
+                const double gap = std::max(0.0, std::max(clo - phi[3 * j + a], plo[3 * j + a] - (clo + s[a])));
+                g2[c] = gap * gap;
+                if (g2[c] <= Rl * Rl) {
+                    lo = std::min(lo, c);
+                    hi = c;
                 }
             }
-    cg.off[(size_t)G * G * G] = (int32_t)cg.list.size();
+            from[3 * j + a] = lo;
+            to[3 * j + a] = hi;
+        }
+    std::vector<int32_t> next;
+    for (int pass = 0; pass < 2; ++pass) {
+        for (int j = 0; j < n; ++j) {
+            const double *gx = &gap2[((size_t)3 * j) * G], *gy = gx + G, *gz = gy + G;
+            for (int cz = from[3 * j + 2]; cz <= to[3 * j + 2]; ++cz)
+                for (int cy = from[3 * j + 1]; cy <= to[3 * j + 1]; ++cy)
+                    for (int cx = from[3 * j]; cx <= to[3 * j]; ++cx) {
+                        const double d2 = gx[cx] + gy[cy] + gz[cz];
+                        if (!(d2 <= Rl * Rl)) continue;
+                        const int c = (cz * G + cy) * G + cx;
+                        if (pass == 0) ++cg.off[c + 1];
+                        else cg.list[next[c]++] = bprims[j];
+                    }
+        }
+        if (pass == 0) {
+            for (int c = 0; c < G * G * G; ++c) cg.off[c + 1] += cg.off[c];
+            cg.list.assign((size_t)cg.off[(size_t)G * G * G], 0);
+            next.assign(cg.off.begin(), cg.off.end() - 1);
+        }
+    }
     cg.region = best;
     cg.g = G;
     cg.op = bop;

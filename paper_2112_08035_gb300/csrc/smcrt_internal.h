@@ -124,29 +124,23 @@ inline double region_margin(const smcrt_scene *sc, int r)
 // the culling).  Writes at most kMaxPrims entries; no allocation.
 inline int seg_entries(const smcrt_scene *sc, int32_t *out, double *margin, int skip_region = -1)
 {
-    uint64_t seen[kMaxPrims / 64] = {};
+    int16_t at[kMaxPrims];   // entry of a primitive + 1 (kMaxPrims fits)
+    for (int i = 0; i < sc->nprims && i < kMaxPrims; ++i) at[i] = 0;
     int n = 0;
     for (int r = 0; r < sc->nregions; ++r) {
         if (r == skip_region || region_is_soft(sc, r)) continue;
         const smcrt_region &R = sc->regions[r];
+        const double m = region_margin(sc, r);
         for (int i = 0; i < R.node_count; ++i) {
             const smcrt_csg_node &nd = sc->nodes[R.node_begin + i];
-            if (nd.op != SMCRT_OP_PRIM || nd.prim < 0 || nd.prim >= kMaxPrims) continue;
-            const uint64_t bit = 1ull << (nd.prim & 63);
-            if (seen[nd.prim >> 6] & bit) continue;
-            seen[nd.prim >> 6] |= bit;
-            double m = 0.0;
-            for (int r2 = 0; r2 < sc->nregions; ++r2) {
-                if (r2 == skip_region || region_is_soft(sc, r2)) continue;
-                const smcrt_region &Q = sc->regions[r2];
-                for (int j = 0; j < Q.node_count; ++j)
-                    if (sc->nodes[Q.node_begin + j].op == SMCRT_OP_PRIM && sc->nodes[Q.node_begin + j].prim == nd.prim) {
-                        m = std::fmax(m, region_margin(sc, r2));
-                        break;
-                    }
+            if (nd.op != SMCRT_OP_PRIM || nd.prim < 0 || nd.prim >= sc->nprims || nd.prim >= kMaxPrims) continue;
+            if (at[nd.prim] == 0) {
+                margin[n] = 0.0;
+                out[n] = nd.prim;
+                at[nd.prim] = (int16_t)++n;
             }
-            margin[n] = m;
-            out[n++] = nd.prim;
+            double &e = margin[at[nd.prim] - 1];
+            e = std::fmax(e, m);
         }
     }
     return n;
