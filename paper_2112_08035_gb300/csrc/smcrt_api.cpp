@@ -269,9 +269,11 @@ struct smcrt_plan {
 
 namespace {
 
-// Kernel instantiation of a plan: its register variant, in the general-shape
-// family when the scene has tori, cylinders or primitive frames.
-int kvariant(const smcrt_plan *pl, int variant) { return variant + (pl->host.general ? kNumVariants : 0); }
+// Kernel instantiation of a plan: its register variant, in its scene's family.
+int kvariant(const smcrt_plan *pl, int variant)
+{
+    return variant + kNumVariants * scene_family(pl->precision, pl->host);
+}
 
 int occupancy(int precision, int threads, int variant)
 {
@@ -551,6 +553,8 @@ int build_plan(smcrt_ctx *ctx, const smcrt_scene *sc, const smcrt_source *src, c
     H.cull_region = cg.region;
     H.cull_g = cg.g;
     H.cull_op = cg.op;
+    H.cull_capsules = cg.region >= 0;
+    for (int32_t i : cg.list) H.cull_capsules = H.cull_capsules && pkind[i] == SMCRT_CAPSULE;
     for (int a = 0; a < 3; ++a) {
         H.cull_lo[a] = cg.lo[a];
         H.cull_inv_s[a] = cg.inv_s[a];

@@ -218,6 +218,7 @@ struct DevScene {
     int32_t cull_region;      // -1: none
     int32_t cull_g;
     int32_t cull_op;          // 1 union, 2 smooth union
+    int32_t cull_capsules;    // all listed primitives are capsules
     float cull_lo[3], cull_inv_s[3];
     float cull_rmax;          // R (union) or R - k/4 (smooth union)
     float cull_kinv;
@@ -360,7 +361,8 @@ int occupancy_fp64(int threads, int variant = 0);
 int occupancy_mixed(int threads, int variant = 0);
 // Served rounds' mixed kernel, whose warps hold two jobs at a time (lanes
 // refill from the next job instead of draining each): variant 0 / 1 = 5 / 4
-// resident blocks of 128 threads, + kNumVariants for general shapes.
+// resident blocks of 128 threads, for scenes with and without a cell list,
+// + kNumVariants for general shapes.
 cudaError_t launch_mixed_multi(JobWork *jobs, int njobs, int *status, int blocks, int threads,
                                cudaStream_t stream, int variant = 0);
 int occupancy_mixed_multi(int threads, int variant = 0);
@@ -390,6 +392,24 @@ inline int default_variant(int precision, uint64_t npackets, const DevScene &S)
 {
     if (precision == SMCRT_FP64) return npackets < kFewFp64Packets ? kFewFp64Variant : 1;
     return npackets < kManyMixedPackets || S.general || S.cull_region >= 0 ? 1 : 0;
+}
+
+// Kernel family of a scene: its register variants start at kNumVariants
+// times this.  A plain scene's mixed kernel carries neither the general
+// shapes' code nor the cell lists': the packet loop is close to the
+// instruction cache's size, so code that a scene does not use costs it time
+// all the same.  Measured, cell lists in the plain kernel / in a family of
+// their own: layered slab 1e7 packets 138.2 / 134.4 ms, 1e6 with sphere
+// tracing 30.8 / 28.7; glass container 4e6 59.9 / 58.4 ms; the vessel tree
+// 4e6, with the capsule loop of culled_region32, 128.8 / 117.0 ms (with that
+// loop in the shared kernel 117.3, but the slab 149.5).  The FP64 kernels
+// have no cell lists; the served kernels have no plain family of their own
+// (a round holds scenes of both kinds).
+enum : int { kPlainScene = 0, kGeneralScene = 1, kCulledScene = 2 };
+inline int scene_family(int precision, const DevScene &S)
+{
+    if (S.general) return kGeneralScene;
+    return precision == SMCRT_MIXED && S.cull_region >= 0 ? kCulledScene : kPlainScene;
 }
 
 // Lanes of a warp that carry packets in a plan launch (JobWork.lanes; 0 =

@@ -262,13 +262,13 @@ static __device__ __noinline__ Crossed cross32(const DevScene &S, float ux, floa
 }
 
 // Value of one surface (region program, or the bounding box for r = -1).
-template <bool G>
+template <int K>
 static __device__ __noinline__ float surface32(const DevScene &S, int r, float x, float y, float z)
 {
     if (r < 0) return box32(x, y, z, S.bbc32[0], S.bbc32[1], S.bbc32[2], S.bbh32[0], S.bbh32[1], S.bbh32[2]);
-    if (r == S.cull_region) return culled_region32(S, x, y, z);
+    if (K != kPlainScene && r == S.cull_region) return culled_region32(S, x, y, z);
     const int2 rr = (*(S.rrange + r));
-    return run_prog32<G>(S, rr.x, rr.y, x, y, z);
+    return run_prog32<K == kGeneralScene>(S, rr.x, rr.y, x, y, z);
 }
 
 // A packet within delta32 of a surface (Sec. 2.3), all of it at once, out of
@@ -287,7 +287,7 @@ struct Interface32 {
 };
 enum { kIntfForced = 0, kIntfEscape = 1, kIntfInteract = 2, kIntfMatched = 3, kIntfFresnel = 4 };
 
-template <bool G>
+template <int K>
 static __device__ __noinline__ Interface32 interface32(const DevScene &S, float px, float py, float pz, float ux,
                                                        float uy, float uz, float tau, int reg, int istar,
                                                        float dstar, uint32_t event, uint32_t id_lo, uint32_t id_hi,
@@ -296,14 +296,14 @@ static __device__ __noinline__ Interface32 interface32(const DevScene &S, float 
     Interface32 o;
     o.refined = 0;
     float nx, ny, nz;
-    if (!G || S.analytic_nrm) {              // gradient of a short program
+    if (K != kGeneralScene || S.analytic_nrm) {   // gradient of a short program
         grad_surface32(S, istar, px, py, pz, nx, ny, nz);
     } else {                                 // central differences
         const float h = S.h32;
         float g[3];
         for (int a = 0; a < 3; ++a) {
-            const float fp = surface32<G>(S, istar, a == 0 ? px + h : px, a == 1 ? py + h : py, a == 2 ? pz + h : pz);
-            const float fm = surface32<G>(S, istar, a == 0 ? px - h : px, a == 1 ? py - h : py, a == 2 ? pz - h : pz);
+            const float fp = surface32<K>(S, istar, a == 0 ? px + h : px, a == 1 ? py + h : py, a == 2 ? pz + h : pz);
+            const float fm = surface32<K>(S, istar, a == 0 ? px - h : px, a == 1 ? py - h : py, a == 2 ? pz - h : pz);
             g[0] = a == 0 ? fp - fm : g[0];
             g[1] = a == 1 ? fp - fm : g[1];
             g[2] = a == 2 ? fp - fm : g[2];
@@ -331,7 +331,7 @@ static __device__ __noinline__ Interface32 interface32(const DevScene &S, float 
     int rfar = -1, rnear = -1;
     for (int side = 0; side < 2; ++side) {   // the regions beyond and before the surface
         const float e = (side == 0 ? 2.f : -2.f) * S.delta32 * sg;
-        rnear = scene_eval32<G>(S, qx + e * nx, qy + e * ny, qz + e * nz).region;
+        rnear = scene_eval32<K>(S, qx + e * nx, qy + e * ny, qz + e * nz).region;
         if (side == 0) rfar = rnear;
     }
     // matched indices cross on the ray, as a Fresnel landing does.  A push
@@ -341,8 +341,8 @@ static __device__ __noinline__ Interface32 interface32(const DevScene &S, float 
     const bool matched = region_n32(S, rnear) == region_n32(S, rfar);
     uint32_t xiw = 0u;
     if (!matched) xiw = philox4x32_10(make_uint4(event, 0u, id_lo, id_hi), k0, k1).x;
-    const Crossed c = cross32<G>(S, ux, uy, uz, qx, qy, qz, nx, ny, nz, tau, dstar, cdot, istar, rnear, rfar, xiw,
-                                 matched);
+    const Crossed c = cross32<K == kGeneralScene>(S, ux, uy, uz, qx, qy, qz, nx, ny, nz, tau, dstar, cdot, istar,
+                                                  rnear, rfar, xiw, matched);
     o.what = matched ? kIntfMatched : kIntfFresnel;
     o.refined = c.refined;
     o.px = c.px; o.py = c.py; o.pz = c.pz;
@@ -460,10 +460,10 @@ __device__ __forceinline__ void stage_tables(WarpShared *ws, int lane)
 // Served rounds: the first job of jobs[start, ...) (cyclically) with work
 // for a warp -- new ids or parked packets -- other than `exclude`; -1 if
 // none.  The lanes look at 32 entries at a time.  A descriptor without
-// scene or totals, or a scene that needs the general-shape kernel in the
-// plain one, is flagged in the launch's and the job's status words and
+// scene or totals, or a scene of a family that this instantiation does not
+// run, is flagged in the launch's and the job's status words and
 // skipped from then on.  Warp-collective; the result is warp-uniform.
-template <bool G>
+template <int K>
 __device__ int multi_find(JobWork *jobs, int njobs, int start, int exclude, unsigned long long &skip, int *status,
                           int lane)
 {
@@ -484,7 +484,7 @@ __device__ int multi_find(JobWork *jobs, int njobs, int start, int exclude, unsi
             // a cancelled job's ids are no work (its parked packets still are)
             const bool fresh = nxt < J->end && *(volatile int32_t *)&J->cancelled == 0;
             if (fresh || parked) {
-                if (J->scene == nullptr || J->totals == nullptr || (!G && J->scene->general)) {
+                if (J->scene == nullptr || J->totals == nullptr || !scene_runs<K>(*J->scene)) {
                     bad = true;
                     atomicOr(status, kStatusBadJob);
                     if (J->jstat != nullptr) atomicOr(J->jstat, kStatusBadJob);
@@ -538,7 +538,7 @@ __device__ __forceinline__ void multi_stage(JobSlot *sl, JobWork *J, int lane)
 // true (served rounds): the warp works through the table jobs[0, njobs)
 // starting at `first`, holding up to two jobs in slots[0..1] (see
 // WarpSharedMulti); each lane's packet belongs to the job of its slot js.
-template <bool G, bool MULTI>
+template <int K, bool MULTI>
 __device__ bool run_job_mixed(JobSlot *slots, JobWork *jobs, int njobs, int first, int *status, int lane)
 {
     const DevScene &S0 = slots[0].S;
@@ -561,7 +561,7 @@ __device__ bool run_job_mixed(JobSlot *slots, JobWork *jobs, int njobs, int firs
     // so idle lanes retire without asking again
     bool nomore = false;
     if (MULTI) {
-        const int nj = multi_find<G>(jobs, njobs, scan, -1, skip, status, lane);
+        const int nj = multi_find<K>(jobs, njobs, scan, -1, skip, status, lane);
         if (nj < 0) return false;
         multi_stage(slots, jobs + nj, lane);
         sj0 = nj;
@@ -679,7 +679,7 @@ __device__ bool run_job_mixed(JobSlot *slots, JobWork *jobs, int njobs, int firs
                 if (__ballot_sync(SMCRT_FULL, alive && js == o) != 0u) break;
                 const int oj = o ? sj1 : sj0;
                 if (oj >= 0) wacc_flush(&slots[o].acc, jobs[oj].totals, lane);
-                const int nj = multi_find<G>(jobs, njobs, scan, feed ? sj1 : sj0, skip, status, lane);
+                const int nj = multi_find<K>(jobs, njobs, scan, feed ? sj1 : sj0, skip, status, lane);
                 if (o) sj1 = -1; else sj0 = -1;
                 if (nj < 0) {                  // no job has work left: idle lanes retire
                     if (!alive) retired = true;
@@ -737,7 +737,7 @@ __device__ bool run_job_mixed(JobSlot *slots, JobWork *jobs, int njobs, int firs
         // ---- 2. the scene evaluation of this iteration
         const bool evals = alive && phase == kTrace;
         Eval32 E{};
-        if (evals) E = scene_eval32<G>(S, px, py, pz);
+        if (evals) E = scene_eval32<K>(S, px, py, pz);
         if (MULTI) {                           // evaluations counted per job slot
             for (int k = 0; k < kMultiSlots; ++k) {
                 const unsigned ev = __ballot_sync(SMCRT_FULL, evals && js == k);
@@ -781,10 +781,10 @@ __device__ bool run_job_mixed(JobSlot *slots, JobWork *jobs, int njobs, int firs
                 __ballot_sync(SMCRT_FULL, alive && (move || phase == kLaunch)) == 0u) {
                 waited = 0;
                 if (alive && phase == kArrive) {
-                    const Interface32 I = interface32<G>(S, px, py, pz, ux, uy, uz, tau, reg, istar, dstar, event,
+                    const Interface32 I = interface32<K>(S, px, py, pz, ux, uy, uz, tau, reg, istar, dstar, event,
                                                          id_lo, id_hi, jc->k0, jc->k1);
                     phase = kTrace;
-                    if (G && !S.analytic_nrm) wadd(wa, kEvals, 6);   // the probes
+                    if (K == kGeneralScene && !S.analytic_nrm) wadd(wa, kEvals, 6);   // the probes
                     if (I.what == kIntfForced) {
                         L = delta;                          // forced step along u
                         move = true;
@@ -829,7 +829,7 @@ __device__ bool run_job_mixed(JobSlot *slots, JobWork *jobs, int njobs, int firs
             }
             interact = mu_t > 0.f && tau < mu_t * L;
             if (SMCRT_RARE(seg_step && !interact)) {           // segment stepping: a longer move along u
-                L = fmaxf(L, segment_bound32<G>(S, L, E.dsoft, E.dbox, px, py, pz, ux, uy, uz));
+                L = fmaxf(L, segment_bound32<K == kGeneralScene>(S, L, E.dsoft, E.dbox, px, py, pz, ux, uy, uz));
                 interact = mu_t > 0.f && tau < mu_t * L;
             }
             const float seg = interact ? tau * imu_t : L;
@@ -969,7 +969,7 @@ __device__ bool run_job_mixed(JobSlot *slots, JobWork *jobs, int njobs, int firs
     return timed_out;
 }
 
-template <int kMinBlocks, bool G>
+template <int kMinBlocks, int K>
 __global__ void __launch_bounds__(128, kMinBlocks) packets_mixed(JobWork *jobs, int njobs, int *status)
 {
     extern __shared__ __align__(16) unsigned char smem[];
@@ -1008,7 +1008,7 @@ __global__ void __launch_bounds__(128, kMinBlocks) packets_mixed(JobWork *jobs, 
         for (int i = lane; i < (int)(sizeof(DevScene) / 8); i += 32) d8[i] = s8[i];
         __syncwarp();
         if (J->stage) stage_tables(ws, lane);
-        if (!G && ws->slot.S.general) {      // a scene with general shapes needs the G instantiation
+        if (!scene_runs<K>(ws->slot.S)) {    // a scene of another kind than this instantiation's
             if (lane == 0) {
                 atomicOr(status, kStatusBadJob);
                 if (J->jstat != nullptr) atomicOr(J->jstat, kStatusBadJob);
@@ -1018,7 +1018,7 @@ __global__ void __launch_bounds__(128, kMinBlocks) packets_mixed(JobWork *jobs, 
         if (lane == 0) jobconst_fill(&ws->slot.jc, J);
         wacc_clear(&ws->slot.acc, lane);
         const long long t0 = clock64();
-        const bool timed_out = run_job_mixed<G, false>(&ws->slot, J, 1, 0, status, lane);
+        const bool timed_out = run_job_mixed<K, false>(&ws->slot, J, 1, 0, status, lane);
         __syncwarp();
         if (lane == 0) wadd(&ws->slot.acc, kBusy, clock64() - t0);
         wacc_flush(&ws->slot.acc, J->totals, lane);
@@ -1033,9 +1033,9 @@ __global__ void __launch_bounds__(128, kMinBlocks) packets_mixed(JobWork *jobs, 
 }
 
 // Served rounds: every warp works through the whole job table, two jobs at a
-// time (run_job_mixed<G, true>), starting at a job of its own so that the
+// time (run_job_mixed<K, true>), starting at a job of its own so that the
 // warps spread over the table.
-template <int kMinBlocks, bool G>
+template <int kMinBlocks, int K>
 __global__ void __launch_bounds__(128, kMinBlocks) packets_mixed_multi(JobWork *jobs, int njobs, int *status)
 {
     extern __shared__ __align__(16) unsigned char smem[];
@@ -1043,7 +1043,7 @@ __global__ void __launch_bounds__(128, kMinBlocks) packets_mixed_multi(JobWork *
     const int gw = blockIdx.x * (blockDim.x >> 5) + warp;
     WarpSharedMulti *ws = reinterpret_cast<WarpSharedMulti *>(smem) + warp;
     if (njobs <= 0) return;
-    run_job_mixed<G, true>(ws->slot, jobs, njobs, gw % njobs, status, lane);
+    run_job_mixed<K, true>(ws->slot, jobs, njobs, gw % njobs, status, lane);
 }
 
 }  // namespace
@@ -1052,7 +1052,8 @@ __global__ void __launch_bounds__(128, kMinBlocks) packets_mixed_multi(JobWork *
 // blocks of 128 threads resident per SM (more blocks = fewer registers per
 // thread, possibly spilled); the autotuner picks per scene.  Variants
 // kNumVariants .. 2 kNumVariants - 1 are the same budgets for scenes with
-// general shapes (tori, cylinders, primitive frames).
+// general shapes (tori, cylinders, primitive frames), 2 kNumVariants .. for
+// plain scenes with a cell list.
 constexpr int kVariantBlocks[kNumVariants] = {5, 4, 3};
 
 cudaError_t launch_mixed(JobWork *jobs, int njobs, int *status, int blocks, int threads, cudaStream_t stream,
@@ -1060,27 +1061,30 @@ cudaError_t launch_mixed(JobWork *jobs, int njobs, int *status, int blocks, int 
 {
     const size_t sm = (size_t)(threads / 32) * sizeof(WarpShared);
     switch (variant) {
-    case 1: packets_mixed<4, false><<<blocks, threads, sm, stream>>>(jobs, njobs, status); break;
-    case 2: packets_mixed<3, false><<<blocks, threads, sm, stream>>>(jobs, njobs, status); break;
-    case 3: packets_mixed<5, true><<<blocks, threads, sm, stream>>>(jobs, njobs, status); break;
-    case 4: packets_mixed<4, true><<<blocks, threads, sm, stream>>>(jobs, njobs, status); break;
-    case 5: packets_mixed<3, true><<<blocks, threads, sm, stream>>>(jobs, njobs, status); break;
-    default: packets_mixed<5, false><<<blocks, threads, sm, stream>>>(jobs, njobs, status); break;
+    case 1: packets_mixed<4, kPlainScene><<<blocks, threads, sm, stream>>>(jobs, njobs, status); break;
+    case 2: packets_mixed<3, kPlainScene><<<blocks, threads, sm, stream>>>(jobs, njobs, status); break;
+    case 3: packets_mixed<5, kGeneralScene><<<blocks, threads, sm, stream>>>(jobs, njobs, status); break;
+    case 4: packets_mixed<4, kGeneralScene><<<blocks, threads, sm, stream>>>(jobs, njobs, status); break;
+    case 5: packets_mixed<3, kGeneralScene><<<blocks, threads, sm, stream>>>(jobs, njobs, status); break;
+    case 6: packets_mixed<5, kCulledScene><<<blocks, threads, sm, stream>>>(jobs, njobs, status); break;
+    case 7: packets_mixed<4, kCulledScene><<<blocks, threads, sm, stream>>>(jobs, njobs, status); break;
+    case 8: packets_mixed<3, kCulledScene><<<blocks, threads, sm, stream>>>(jobs, njobs, status); break;
+    default: packets_mixed<5, kPlainScene><<<blocks, threads, sm, stream>>>(jobs, njobs, status); break;
     }
     return cudaGetLastError();
 }
 
-// The served kernel: variant 0 / 1 = 5 / 4 resident blocks, plain shapes;
-// 3 / 4 = the same for general shapes (the index space of launch_mixed).
+// The served kernel: variant 0 / 1 = 5 / 4 resident blocks, plain shapes,
+// with or without a cell list; 3 / 4 = the same for general shapes (the index space of launch_mixed).
 cudaError_t launch_mixed_multi(JobWork *jobs, int njobs, int *status, int blocks, int threads, cudaStream_t stream,
                                int variant)
 {
     const size_t sm = (size_t)(threads / 32) * sizeof(WarpSharedMulti);
     switch (variant) {
-    case 1: packets_mixed_multi<4, false><<<blocks, threads, sm, stream>>>(jobs, njobs, status); break;
-    case 3: packets_mixed_multi<5, true><<<blocks, threads, sm, stream>>>(jobs, njobs, status); break;
-    case 4: packets_mixed_multi<4, true><<<blocks, threads, sm, stream>>>(jobs, njobs, status); break;
-    default: packets_mixed_multi<5, false><<<blocks, threads, sm, stream>>>(jobs, njobs, status); break;
+    case 1: packets_mixed_multi<4, kCulledScene><<<blocks, threads, sm, stream>>>(jobs, njobs, status); break;
+    case 3: packets_mixed_multi<5, kGeneralScene><<<blocks, threads, sm, stream>>>(jobs, njobs, status); break;
+    case 4: packets_mixed_multi<4, kGeneralScene><<<blocks, threads, sm, stream>>>(jobs, njobs, status); break;
+    default: packets_mixed_multi<5, kCulledScene><<<blocks, threads, sm, stream>>>(jobs, njobs, status); break;
     }
     return cudaGetLastError();
 }
@@ -1090,10 +1094,10 @@ int occupancy_mixed_multi(int threads, int variant)
     int n = 0;
     const size_t sm = (size_t)(threads / 32) * sizeof(WarpSharedMulti);
     switch (variant) {
-    case 1: cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, packets_mixed_multi<4, false>, threads, sm); break;
-    case 3: cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, packets_mixed_multi<5, true>, threads, sm); break;
-    case 4: cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, packets_mixed_multi<4, true>, threads, sm); break;
-    default: cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, packets_mixed_multi<5, false>, threads, sm); break;
+    case 1: cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, packets_mixed_multi<4, kCulledScene>, threads, sm); break;
+    case 3: cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, packets_mixed_multi<5, kGeneralScene>, threads, sm); break;
+    case 4: cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, packets_mixed_multi<4, kGeneralScene>, threads, sm); break;
+    default: cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, packets_mixed_multi<5, kCulledScene>, threads, sm); break;
     }
     return n;
 }
@@ -1103,12 +1107,15 @@ int occupancy_mixed(int threads, int variant)
     int n = 0;
     const size_t sm = (size_t)(threads / 32) * sizeof(WarpShared);
     switch (variant) {
-    case 1: cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, packets_mixed<4, false>, threads, sm); break;
-    case 2: cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, packets_mixed<3, false>, threads, sm); break;
-    case 3: cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, packets_mixed<5, true>, threads, sm); break;
-    case 4: cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, packets_mixed<4, true>, threads, sm); break;
-    case 5: cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, packets_mixed<3, true>, threads, sm); break;
-    default: cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, packets_mixed<5, false>, threads, sm); break;
+    case 1: cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, packets_mixed<4, kPlainScene>, threads, sm); break;
+    case 2: cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, packets_mixed<3, kPlainScene>, threads, sm); break;
+    case 3: cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, packets_mixed<5, kGeneralScene>, threads, sm); break;
+    case 4: cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, packets_mixed<4, kGeneralScene>, threads, sm); break;
+    case 5: cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, packets_mixed<3, kGeneralScene>, threads, sm); break;
+    case 6: cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, packets_mixed<5, kCulledScene>, threads, sm); break;
+    case 7: cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, packets_mixed<4, kCulledScene>, threads, sm); break;
+    case 8: cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, packets_mixed<3, kCulledScene>, threads, sm); break;
+    default: cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, packets_mixed<5, kPlainScene>, threads, sm); break;
     }
     return n;
 }

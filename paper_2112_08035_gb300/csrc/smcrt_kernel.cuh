@@ -484,6 +484,13 @@ __device__ __forceinline__ float run_prog32(const DevScene &S, int i0, int i1, f
     return s0;
 }
 
+// Whether the mixed instantiation K can run scene S.
+template <int K>
+__device__ __forceinline__ bool scene_runs(const DevScene &S)
+{
+    return K == kGeneralScene || (!S.general && (K == kCulledScene || S.cull_region < 0));
+}
+
 // Full scene evaluation (Sec. 2.3): every region, then the bounding box.
 template <bool G>
 __device__ __forceinline__ Eval64 scene_eval64(const DevScene &S, double x, double y, double z, int sel)
@@ -503,6 +510,8 @@ __device__ __forceinline__ Eval64 scene_eval64(const DevScene &S, double x, doub
 // Value of the culled fold region at p: the fold over the primitives listed
 // for p's cell, bounded by cull_rmax (every unlisted primitive is farther
 // than R from the cell, so it cannot change the value below that bound).
+// A vessel tree's list holds capsules only, so the loop over them looks at
+// no kind: vessel tree 4e6 packets 128.8 -> 117.0 ms.
 __device__ __forceinline__ float culled_region32(const DevScene &S, float x, float y, float z)
 {
     const int g = S.cull_g;
@@ -514,6 +523,16 @@ __device__ __forceinline__ float culled_region32(const DevScene &S, float x, flo
     const int c = (cz * g + cy) * g + cx;
     const int o0 = __ldg(S.cull_off + c), o1 = __ldg(S.cull_off + c + 1);
     if (o1 <= o0) return S.cull_rmax;
+    if (S.cull_capsules) {
+        const bool smooth = S.cull_op == 2;
+        const float kinv = S.cull_kinv;
+        float acc = base32<false>(2, S.p32 + 2 * __ldg(S.cull_list + o0), x, y, z);
+        for (int j = o0 + 1; j < o1; ++j) {
+            const float d = base32<false>(2, S.p32 + 2 * __ldg(S.cull_list + j), x, y, z);
+            acc = smooth ? csg32(2, acc, d, kinv) : fminf(acc, d);
+        }
+        return fminf(acc, S.cull_rmax);
+    }
     int i = __ldg(S.cull_list + o0);
     float acc = prim32<false>(S, (*(S.pkind + i)), i, x, y, z);   // culled regions are plain
     for (int j = o0 + 1; j < o1; ++j) {
@@ -534,26 +553,26 @@ __device__ __forceinline__ void region_end32(Eval32 *E, int r, float d, bool sof
 // One copy of the interpreter in the packet loop: the culled region's
 // instructions [cb, ce) are replaced by its culled distance inside the same
 // loop (each region's program is self-contained, so the stack left by the
-// regions before it does not matter).  Code size counts here: the loop runs
+// regions before it does not matter); a plain scene's instantiation has no
+// cell list.  Code size counts here: the loop runs
 // close to the instruction cache's capacity (measured on the layered slab:
 // three interpreter copies 203.6 ms per 1e7 packets, one copy 184.4 ms).
-template <bool G>
+template <int K>   // kPlainScene, kGeneralScene or kCulledScene
 __device__ __forceinline__ Eval32 scene_eval32(const DevScene &S, float x, float y, float z)
 {
-
     Eval32 E;
     E.dmin = __int_as_float(0x7f800000);
     E.dsoft = E.dmin;
     E.dstar = 0.f; E.istar = -1; E.region = -1;
     int cb = S.ninstr, ce = S.ninstr;
-    if (S.cull_region >= 0) {
+    if (K != kPlainScene && S.cull_region >= 0) {
         const int2 rr = (*(S.rrange + S.cull_region));
         cb = rr.x;
         ce = rr.y;
     }
     float s0 = 0.f, s1 = 0.f, s2 = 0.f, s3 = 0.f;
     for (int i = 0; i < S.ninstr; ++i) {
-        if (i == cb) {
+        if (K != kPlainScene && i == cb) {
             // the culled region's distance bounds segment moves
             // isotropically (its primitives are not in seg_prims)
             region_end32(&E, S.cull_region, culled_region32(S, x, y, z), true);
@@ -563,7 +582,7 @@ __device__ __forceinline__ Eval32 scene_eval32(const DevScene &S, float x, float
         const int4 ins = (*(reinterpret_cast<const int4 *>(S.instr) + i));
         const int op = ins.x & 0xff, kind = (ins.x >> 8) & 0xff;
         float v = 0.f;
-        if (ins.y >= 0) v = prim32<G>(S, kind, ins.y, x, y, z);
+        if (ins.y >= 0) v = prim32<K == kGeneralScene>(S, kind, ins.y, x, y, z);
         if (op == 0) {
             s3 = s2; s2 = s1; s1 = s0; s0 = v;
         } else {
