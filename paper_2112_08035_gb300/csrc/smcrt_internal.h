@@ -188,6 +188,15 @@ struct Instr {
     int32_t pad;
 };
 
+// Whether every region is one box in scene coordinates (a compiled program:
+// one instruction per region).
+inline bool box_regions(const Instr *ins, int ninstr, int nregions)
+{
+    bool all = ninstr == nregions && nregions > 0;
+    for (int i = 0; all && i < ninstr; ++i) all = (ins[i].op & 0xff) == 0 && ((ins[i].op >> 8) & 0xff) == SMCRT_BOX;
+    return all;
+}
+
 // Scene + source + grid of one plan as the kernels read them.  Lives in
 // device memory; each warp stages a copy in shared memory when it starts
 // on a job.  All double fields are computed on the host with the same
@@ -235,7 +244,7 @@ struct DevScene {
     const double *xf64;
     const float4 *xf32;
     int32_t general;          // some primitive is a torus or cylinder or has a frame
-    int32_t general_pad;
+    int32_t boxes;            // every region is one box in scene coordinates
     float h32;                // FP32 central-difference step for normals
     int64_t max_steps;
     // source
@@ -402,14 +411,19 @@ inline int default_variant(int precision, uint64_t npackets, const DevScene &S)
 // their own: layered slab 1e7 packets 138.2 / 134.4 ms, 1e6 with sphere
 // tracing 30.8 / 28.7; glass container 4e6 59.9 / 58.4 ms; the vessel tree
 // 4e6, with the capsule loop of culled_region32, 128.8 / 117.0 ms (with that
-// loop in the shared kernel 117.3, but the slab 149.5).  The FP64 kernels
+// loop in the shared kernel 117.3, but the slab 149.5).  Scenes whose every
+// region is one box (layered tissue, block phantoms) run a kernel without the
+// CSG interpreter and the other shapes: layered slab 1e7 packets 134.4 ->
+// 111.0 ms, 1e4 2.05 -> 1.77 ms, with sphere tracing 1e6 28.8 -> 25.1; thick
+// slab 1e6 67.7 -> 65.3 ms (its loop is mostly scattering).  The FP64 kernels
 // have no cell lists; the served kernels have no plain family of their own
 // (a round holds scenes of both kinds).
-enum : int { kPlainScene = 0, kGeneralScene = 1, kCulledScene = 2 };
+enum : int { kPlainScene = 0, kGeneralScene = 1, kCulledScene = 2, kBoxScene = 3 };
 inline int scene_family(int precision, const DevScene &S)
 {
     if (S.general) return kGeneralScene;
-    return precision == SMCRT_MIXED && S.cull_region >= 0 ? kCulledScene : kPlainScene;
+    if (precision == SMCRT_FP64) return kPlainScene;
+    return S.cull_region >= 0 ? kCulledScene : S.boxes ? kBoxScene : kPlainScene;
 }
 
 // Lanes of a warp that carry packets in a plan launch (JobWork.lanes; 0 =

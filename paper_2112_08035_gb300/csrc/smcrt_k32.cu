@@ -266,7 +266,7 @@ template <int K>
 static __device__ __noinline__ float surface32(const DevScene &S, int r, float x, float y, float z)
 {
     if (r < 0) return box32(x, y, z, S.bbc32[0], S.bbc32[1], S.bbc32[2], S.bbh32[0], S.bbh32[1], S.bbh32[2]);
-    if (K != kPlainScene && r == S.cull_region) return culled_region32(S, x, y, z);
+    if ((K == kGeneralScene || K == kCulledScene) && r == S.cull_region) return culled_region32(S, x, y, z);
     const int2 rr = (*(S.rrange + r));
     return run_prog32<K == kGeneralScene>(S, rr.x, rr.y, x, y, z);
 }
@@ -297,7 +297,7 @@ static __device__ __noinline__ Interface32 interface32(const DevScene &S, float 
     o.refined = 0;
     float nx, ny, nz;
     if (K != kGeneralScene || S.analytic_nrm) {   // gradient of a short program
-        grad_surface32(S, istar, px, py, pz, nx, ny, nz);
+        grad_surface32<K>(S, istar, px, py, pz, nx, ny, nz);
     } else {                                 // central differences
         const float h = S.h32;
         float g[3];
@@ -829,7 +829,7 @@ __device__ bool run_job_mixed(JobSlot *slots, JobWork *jobs, int njobs, int firs
             }
             interact = mu_t > 0.f && tau < mu_t * L;
             if (SMCRT_RARE(seg_step && !interact)) {           // segment stepping: a longer move along u
-                L = fmaxf(L, segment_bound32<K == kGeneralScene>(S, L, E.dsoft, E.dbox, px, py, pz, ux, uy, uz));
+                L = fmaxf(L, segment_bound32<K>(S, L, E.dsoft, E.dbox, px, py, pz, ux, uy, uz));
                 interact = mu_t > 0.f && tau < mu_t * L;
             }
             const float seg = interact ? tau * imu_t : L;
@@ -1053,7 +1053,8 @@ __global__ void __launch_bounds__(128, kMinBlocks) packets_mixed_multi(JobWork *
 // thread, possibly spilled); the autotuner picks per scene.  Variants
 // kNumVariants .. 2 kNumVariants - 1 are the same budgets for scenes with
 // general shapes (tori, cylinders, primitive frames), 2 kNumVariants .. for
-// plain scenes with a cell list.
+// plain scenes with a cell list, 3 kNumVariants .. for scenes of boxes
+// (scene_family).
 constexpr int kVariantBlocks[kNumVariants] = {5, 4, 3};
 
 cudaError_t launch_mixed(JobWork *jobs, int njobs, int *status, int blocks, int threads, cudaStream_t stream,
@@ -1069,6 +1070,9 @@ cudaError_t launch_mixed(JobWork *jobs, int njobs, int *status, int blocks, int 
     case 6: packets_mixed<5, kCulledScene><<<blocks, threads, sm, stream>>>(jobs, njobs, status); break;
     case 7: packets_mixed<4, kCulledScene><<<blocks, threads, sm, stream>>>(jobs, njobs, status); break;
     case 8: packets_mixed<3, kCulledScene><<<blocks, threads, sm, stream>>>(jobs, njobs, status); break;
+    case 9: packets_mixed<5, kBoxScene><<<blocks, threads, sm, stream>>>(jobs, njobs, status); break;
+    case 10: packets_mixed<4, kBoxScene><<<blocks, threads, sm, stream>>>(jobs, njobs, status); break;
+    case 11: packets_mixed<3, kBoxScene><<<blocks, threads, sm, stream>>>(jobs, njobs, status); break;
     default: packets_mixed<5, kPlainScene><<<blocks, threads, sm, stream>>>(jobs, njobs, status); break;
     }
     return cudaGetLastError();
@@ -1115,6 +1119,9 @@ int occupancy_mixed(int threads, int variant)
     case 6: cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, packets_mixed<5, kCulledScene>, threads, sm); break;
     case 7: cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, packets_mixed<4, kCulledScene>, threads, sm); break;
     case 8: cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, packets_mixed<3, kCulledScene>, threads, sm); break;
+    case 9: cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, packets_mixed<5, kBoxScene>, threads, sm); break;
+    case 10: cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, packets_mixed<4, kBoxScene>, threads, sm); break;
+    case 11: cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, packets_mixed<3, kBoxScene>, threads, sm); break;
     default: cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, packets_mixed<5, kPlainScene>, threads, sm); break;
     }
     return n;

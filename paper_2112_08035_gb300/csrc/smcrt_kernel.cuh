@@ -488,7 +488,8 @@ __device__ __forceinline__ float run_prog32(const DevScene &S, int i0, int i1, f
 template <int K>
 __device__ __forceinline__ bool scene_runs(const DevScene &S)
 {
-    return K == kGeneralScene || (!S.general && (K == kCulledScene || S.cull_region < 0));
+    return K == kGeneralScene ||
+           (!S.general && (K == kCulledScene || S.cull_region < 0) && (K != kBoxScene || S.boxes));
 }
 
 // Full scene evaluation (Sec. 2.3): every region, then the bounding box.
@@ -557,21 +558,27 @@ __device__ __forceinline__ void region_end32(Eval32 *E, int r, float d, bool sof
 // cell list.  Code size counts here: the loop runs
 // close to the instruction cache's capacity (measured on the layered slab:
 // three interpreter copies 203.6 ms per 1e7 packets, one copy 184.4 ms).
-template <int K>   // kPlainScene, kGeneralScene or kCulledScene
+template <int K>   // the scene family
 __device__ __forceinline__ Eval32 scene_eval32(const DevScene &S, float x, float y, float z)
 {
     Eval32 E;
     E.dmin = __int_as_float(0x7f800000);
     E.dsoft = E.dmin;
     E.dstar = 0.f; E.istar = -1; E.region = -1;
+    if (K == kBoxScene) {                // one instruction, one box per region
+        for (int i = 0; i < S.ninstr; ++i) {
+            const int4 ins = (*(reinterpret_cast<const int4 *>(S.instr) + i));
+            region_end32(&E, ins.z, base32<false>(1, S.p32 + 2 * ins.y, x, y, z), false);
+        }
+    }
     int cb = S.ninstr, ce = S.ninstr;
-    if (K != kPlainScene && S.cull_region >= 0) {
+    if ((K == kGeneralScene || K == kCulledScene) && S.cull_region >= 0) {
         const int2 rr = (*(S.rrange + S.cull_region));
         cb = rr.x;
         ce = rr.y;
     }
     float s0 = 0.f, s1 = 0.f, s2 = 0.f, s3 = 0.f;
-    for (int i = 0; i < S.ninstr; ++i) {
+    for (int i = 0; K != kBoxScene && i < S.ninstr; ++i) {
         if (K != kPlainScene && i == cb) {
             // the culled region's distance bounds segment moves
             // isotropically (its primitives are not in seg_prims)
@@ -722,10 +729,12 @@ static __device__ __noinline__ float grad_program32(const DevScene &S, int i0, i
     return v[0];
 }
 
+template <int K>
 static __device__ __noinline__ float grad_surface32(const DevScene &S, int r, float x, float y, float z, float &gx,
                                              float &gy, float &gz)
 {
-    if (r >= 0 && r == S.cull_region) return grad_culled32(S, x, y, z, gx, gy, gz);
+    if ((K == kGeneralScene || K == kCulledScene) && r >= 0 && r == S.cull_region)
+        return grad_culled32(S, x, y, z, gx, gy, gz);
     if (r < 0) {
         const float px = x - S.bbc32[0], py = y - S.bbc32[1], pz = z - S.bbc32[2];
         const float qx = fabsf(px) - S.bbh32[0], qy = fabsf(py) - S.bbh32[1], qz = fabsf(pz) - S.bbh32[2];
@@ -736,9 +745,9 @@ static __device__ __noinline__ float grad_surface32(const DevScene &S, int r, fl
         return qz;
     }
     const int2 rr = (*(S.rrange + r));
-    if (rr.y - rr.x == 1) {              // a primitive
+    if (K == kBoxScene || rr.y - rr.x == 1) {   // a primitive
         const int4 ins = (*(reinterpret_cast<const int4 *>(S.instr) + rr.x));
-        return prim_grad32(S, (ins.x >> 8) & 0xff, ins.y, x, y, z, gx, gy, gz);
+        return prim_grad32(S, K == kBoxScene ? 1 : (ins.x >> 8) & 0xff, ins.y, x, y, z, gx, gy, gz);
     }
     return grad_program32(S, rr.x, rr.y, x, y, z, gx, gy, gz);
 }
@@ -1281,7 +1290,7 @@ static __device__ __noinline__ float seg_xprim32(const DevScene &S, int kind, in
 // isotropic bound is kept.
 // The caller's move is at least L: once the bound is not above it, what is
 // left cannot matter.
-template <bool G>
+template <int K>
 static __device__ __noinline__ float segment_bound32(const DevScene &S, float L, float dsoft, float dbox, float px,
                                                      float py, float pz, float ux, float uy, float uz)
 {
@@ -1292,9 +1301,9 @@ static __device__ __noinline__ float segment_bound32(const DevScene &S, float L,
                     dsoft - dh);
     for (int j = 0; j < S.nseg && t > L; ++j) {
         const int i = __ldg(S.seg_prims + j);
-        const int kind = (*(S.pkind + i));
+        const int kind = K == kBoxScene ? 1 : (*(S.pkind + i));
         const float e = __ldg(S.seg_m32 + j) + dh;
-        const float d = prim32<G>(S, kind, i, px, py, pz);
+        const float d = prim32<K == kGeneralScene>(S, kind, i, px, py, pz);
         if (!(fabsf(d) > e)) return 0.f;
         if (fabsf(d) - e >= t) continue;
         float b;
@@ -1303,7 +1312,7 @@ static __device__ __noinline__ float segment_bound32(const DevScene &S, float L,
         } else if (kind == 1) {
             const float4 A = (*(S.p32 + 2 * i)), B = (*(S.p32 + 2 * i + 1));
             b = seg_box32(A.x, A.y, A.z, B.x, B.y, B.z, d, px, py, pz, ux, uy, uz, iux, iuy, iuz, e);
-        } else if (!G || kind == 2) {
+        } else if (K != kGeneralScene || kind == 2) {
             b = seg_capsule32((*(S.p32 + 2 * i)), (*(S.p32 + 2 * i + 1)), d, px, py, pz, ux, uy, uz, e);
         } else if (kind & kXformFlag) {
             b = seg_xprim32(S, kind & 0xf, i, d, px, py, pz, ux, uy, uz, e);

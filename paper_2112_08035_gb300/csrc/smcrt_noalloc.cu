@@ -242,6 +242,7 @@ int build_image(const smcrt_scene *sc, const smcrt_source *src, const smcrt_grid
         if (!plain) longest = kAnalyticNormalMaxInstr + 1;   // probe normals for other shapes and frames
         H.analytic_nrm = longest <= kAnalyticNormalMaxInstr ? 1 : 0;
     }
+    H.boxes = box_regions(ins, ni, nr);
     // probe normals run in the general mixed instantiation (the plain one
     // leaves them out)
     if (precision == SMCRT_MIXED && !H.analytic_nrm) H.general = 1;
@@ -321,17 +322,15 @@ extern "C" int smcrt_run_noalloc(const smcrt_scene *scene, const smcrt_source *s
     int rc = scratch_address(&base);
     if (rc != SMCRT_OK) return rc;
     cudaStream_t s = (cudaStream_t)stream;
-    // tori, cylinders, frames (and, in mixed precision, probe normals): the
-    // general instantiation, as the image's scene header records
-    bool general = false;
-    int base_variant = 0;
+    // the scene's family and default shape, from the image's scene header
+    int variant = 0;
     {
         std::lock_guard<std::mutex> lk(g_image_mu);
         size_t used = 0;
         rc = build_image(scene, source, grid, precision, base, g_image, &used);
         if (rc != SMCRT_OK) return rc;
-        general = reinterpret_cast<const DevScene *>(g_image)->general != 0;
-        base_variant = default_variant(precision, npackets, *reinterpret_cast<const DevScene *>(g_image));
+        const DevScene &H = *reinterpret_cast<const DevScene *>(g_image);
+        variant = default_variant(precision, npackets, H) + kNumVariants * scene_family(precision, H);
         if (npackets == 0) return SMCRT_OK;
         // the image (a multiple of 16 bytes), chunk by chunk, in the copy
         // kernels' launch arguments
@@ -360,7 +359,6 @@ extern "C" int smcrt_run_noalloc(const smcrt_scene *scene, const smcrt_source *s
     if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return SMCRT_ERR_CUDA;
     const int threads = 128;
     const bool few = precision == SMCRT_FP64 && npackets < kFewFp64Packets;
-    const int variant = base_variant + (general ? kNumVariants : 0);
     const int occ = precision == SMCRT_FP64 ? occupancy_fp64(threads, variant) : occupancy_mixed(threads, variant);
     const int blocks = sms * (occ > 0 && !few ? occ : 1);
     jw.lanes = spread_lanes(npackets, blocks, threads);

@@ -1,0 +1,62 @@
+"""Scenes whose every region is one box run mixed-kernel instantiations that
+know no other shape.  The same scene with one region written as the union of
+its box with itself runs the plain ones, whose arithmetic is the same, so
+every tally must be equal."""
+import pytest
+
+import paper_2112_08035_gb300 as smc
+import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+# centre and half extents of the regions' boxes
+SCENES = {
+    "one": [(0.0, 0.0, 0.0, 0.5, 0.4, 0.3)],
+    "layers": [(0.0, 0.0, 0.45, 4.0, 4.0, 0.05), (0.0, 0.0, 0.2, 4.0, 4.0, 0.2), (0.0, 0.0, -0.3, 4.0, 4.0, 0.3)],
+    "nested": [(0.0, 0.0, 0.0, 0.5, 0.5, 0.5), (0.1, -0.1, 0.0, 0.3, 0.2, 0.25), (0.1, -0.1, 0.05, 0.1, 0.1, 0.1)],
+    "edges": [(-0.2, 0.0, 0.0, 0.2, 0.5, 0.5), (0.2, 0.2, 0.0, 0.2, 0.3, 0.5), (0.2, -0.3, 0.0, 0.2, 0.2, 0.5),
+              (0.0, 0.0, 0.0, 0.01, 0.01, 0.6)],
+    "many": [(0.2 * (i % 4) - 0.3, 0.2 * (i // 4 % 4) - 0.3, 0.25 * (i // 16) - 0.2, 0.07, 0.08, 0.09)
+             for i in range(16)],
+}
+
+
+def _workload(name, doubled, stepping):
+    prims = tuple(W.Prim(W.BOX, tuple(float(v) for v in b)) for b in SCENES[name])
+    regions = []
+    for i in range(len(prims)):
+        prog = W.prim_program([0, 0]) if doubled and i == 0 else W.prim_program([i])
+        regions.append(W.Region(prog, 0.3 + 0.1 * (i % 5), 5.0 + 10.0 * (i % 3), 0.8, (1.4, 1.33, 1.5)[i % 3]))
+    b = 0.7
+    scene = W.Scene(prims, tuple(regions), 1.0, (-b, -b, -b), (b, b, b))
+    return W.Workload("boxes", scene, W.Source(W.SQUARE, (0.0, 0.0, 0.65), (0.0, 0.0, -1.0), 0.5),
+                      W.Grid((-0.5, -0.5, -0.5), (0.5, 0.5, 0.5), (17, 16, 15)), 20_000, 3,
+                      "mixed").with_stepping(stepping)
+
+
+@pytest.mark.parametrize("stepping", [W.SPHERE_TRACING, W.SEGMENT])
+@pytest.mark.parametrize("name", list(SCENES))
+def test_box_scenes_equal_plain(name, stepping):
+    import torch
+    ctx = smc.Context(0)
+    got = []
+    for doubled, alloc in ((True, True), (False, True), (False, False)):
+        wl = _workload(name, doubled, stepping)
+        flu = torch.zeros(wl.grid.size, dtype=torch.int64, device="cuda")
+        tot = smc.totals_tensor()
+        if alloc:
+            plan = ctx.plan(wl, "mixed")
+            plan.launch(0, wl.npackets, wl.seed, flu, tot)
+            torch.cuda.synchronize()
+            assert plan.status() == 0
+            plan.close()
+        else:
+            smc.run_noalloc(wl, 0, wl.npackets, wl.seed, flu, tot, "mixed")
+            torch.cuda.synchronize()
+        t = smc.totals_from_tensor(tot)
+        got.append((flu, {k: t[k] for k in ("R", "T", "A", "killed", "gain", "packets", "scatters", "steps")}))
+    ctx.close()
+    assert got[0][1]["packets"] == 20_000
+    for flu, t in got[1:]:
+        assert t == got[0][1]
+        assert torch.equal(flu, got[0][0])
