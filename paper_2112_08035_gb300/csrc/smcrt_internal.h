@@ -415,15 +415,16 @@ inline int default_variant(int precision, uint64_t npackets, const DevScene &S)
 // region is one box (layered tissue, block phantoms) run a kernel without the
 // CSG interpreter and the other shapes: layered slab 1e7 packets 134.4 ->
 // 111.0 ms, 1e4 2.05 -> 1.77 ms, with sphere tracing 1e6 28.8 -> 25.1; thick
-// slab 1e6 67.7 -> 65.3 ms (its loop is mostly scattering).  The FP64 kernels
-// have no cell lists; the served kernels have no plain family of their own
-// (a round holds scenes of both kinds).
+// slab 1e6 67.7 -> 65.3 ms (its loop is mostly scattering); in FP64, layered
+// slab 1e5 58.9 -> 46.2 ms, 1e4 16.4 -> 13.4, 1e6 485 -> 342, thick slab 3e3
+// 114.6 -> 110.9.  The FP64 kernels have no cell lists; served rounds hold
+// scenes of all kinds and have two families, general and not.
 enum : int { kPlainScene = 0, kGeneralScene = 1, kCulledScene = 2, kBoxScene = 3 };
 inline int scene_family(int precision, const DevScene &S)
 {
     if (S.general) return kGeneralScene;
-    if (precision == SMCRT_FP64) return kPlainScene;
-    return S.cull_region >= 0 ? kCulledScene : S.boxes ? kBoxScene : kPlainScene;
+    if (precision == SMCRT_MIXED && S.cull_region >= 0) return kCulledScene;
+    return S.boxes ? kBoxScene : kPlainScene;
 }
 
 // Lanes of a warp that carry packets in a plan launch (JobWork.lanes; 0 =

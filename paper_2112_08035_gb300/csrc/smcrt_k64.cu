@@ -194,7 +194,7 @@ struct WarpShared {
 // every floating-point operation the reference algorithm's, in its order:
 // the oracle's run of a packet is a sequence of the same IEEE operations on
 // the same values, so its tallies come out bit for bit.
-template <bool G>
+template <int K>
 __device__ bool run_job_fp64(const DevScene &S, WarpAcc *wa, const volatile JobConst *jc, JobWork *J,
                              int lane)
 {
@@ -285,10 +285,10 @@ __device__ bool run_job_fp64(const DevScene &S, WarpAcc *wa, const volatile JobC
         Screen64 C;
         bool interact = false;
         const bool evals = alive && phase == kTrace;
-        if (G) {
+        if (K == kGeneralScene) {
             if (evals) phase = kExact;
         } else if (evals) {
-            C = scene_screen(S, (float)px, (float)py, (float)pz, kForTrace);
+            C = scene_screen<K>(S, (float)px, (float)py, (float)pz, kForTrace);
             kneg = C.neg; kmask = C.mask; klist = C.list; kfold = C.flr << 8 | (C.cnt & 0xff);
             ksoft = C.soft; kdb = C.db;
             phase = kExact;
@@ -299,7 +299,7 @@ __device__ bool run_job_fp64(const DevScene &S, WarpAcc *wa, const volatile JobC
                 interact = m > 0.f && need < m * (C.lo - (float)delta);
                 if (!interact && S.stepping == SMCRT_STEP_SEGMENT) {
                     const float p[3] = {(float)px, (float)py, (float)pz}, u[3] = {(float)ux, (float)uy, (float)uz};
-                    interact = m > 0.f && need < m * segment_screen(S, C.soft, p, u);
+                    interact = m > 0.f && need < m * segment_screen<K>(S, C.soft, p, u);
                 }
             }
         }
@@ -317,16 +317,16 @@ __device__ bool run_job_fp64(const DevScene &S, WarpAcc *wa, const volatile JobC
         const bool none = __ballot_sync(SMCRT_FULL, alive && (interact || phase == kLaunch)) == 0u;   // no other lane moves
         const unsigned exact = __ballot_sync(SMCRT_FULL, alive && phase == kExact && !interact);
         wait_x += __popc(exact);
-        if (exact != 0u && (G || none || kWaitExact * wait_x >= __popc(here))) {
+        if (exact != 0u && (K == kGeneralScene || none || kWaitExact * wait_x >= __popc(here))) {
             wait_x = 0;
             if (alive && phase == kExact && !interact) {
                 Eval64 E;
-                if (G) {
-                    E = scene_eval64<G>(S, px, py, pz, -2);
+                if (K == kGeneralScene) {
+                    E = scene_eval64<true>(S, px, py, pz, -2);
                 } else {
                     C.neg = kneg; C.mask = kmask; C.list = klist; C.flr = kfold >> 8; C.cnt = (int)(int8_t)(kfold & 0xff);
                     C.soft = ksoft; C.db = kdb;
-                    E = scene_exact(S, px, py, pz, C, kForTrace);
+                    E = scene_exact<K>(S, px, py, pz, C, kForTrace);
                 }
                 if (E.dbox > 0.0) {                      // outside the volume of interest
                     out = true;
@@ -342,8 +342,8 @@ __device__ bool run_job_fp64(const DevScene &S, WarpAcc *wa, const volatile JobC
                         move = true;
                         interact = mu_t > 0.0 && tau < mu_t * L;
                         if (!interact && S.stepping == SMCRT_STEP_SEGMENT) {   // a longer move along u
-                            if (G) L = fmax(L, segment_bound64<G>(S, E.dsoft, E.dbox, px, py, pz, ux, uy, uz));
-                            else L = max64(L, segment_bound64_screened(S, E.dsoft, E.dbox, px, py, pz, ux, uy, uz));
+                            if (K == kGeneralScene) L = fmax(L, segment_bound64<true>(S, E.dsoft, E.dbox, px, py, pz, ux, uy, uz));
+                            else L = max64(L, segment_bound64_screened<K>(S, E.dsoft, E.dbox, px, py, pz, ux, uy, uz));
                             interact = mu_t > 0.0 && tau < mu_t * L;
                         }
                     }
@@ -360,7 +360,7 @@ __device__ bool run_job_fp64(const DevScene &S, WarpAcc *wa, const volatile JobC
                               __ballot_sync(SMCRT_FULL, alive && (move || phase == kLaunch)) == 0u)) {
             wait_i = 0;
             if (alive && phase == kArrive) {
-                I = interface64<G>(S, px, py, pz, ux, uy, uz, istar, dstar);
+                I = interface64<K>(S, px, py, pz, ux, uy, uz, istar, dstar);
                 nev += I.evals;
                 phase = kTrace;
                 if (I.what == kIntfForced) {
@@ -396,7 +396,7 @@ __device__ bool run_job_fp64(const DevScene &S, WarpAcc *wa, const volatile JobC
             const double seg = interact ? div_by64(tau, mu_t, __ldg(S.reg64 + kReg64 * reg + 6)) : L;
             long long *const flu = (long long *)jc->flu;
             if (flu) {
-                if (G) npieces += tally64(S, flu, px, py, pz, ux, uy, uz, seg, w);
+                if (K == kGeneralScene) npieces += tally64(S, flu, px, py, pz, ux, uy, uz, seg, w);
                 else npieces += tally64_screened(S, flu, px, py, pz, ux, uy, uz, seg, w);
             }
             px = px + seg * ux; py = py + seg * uy; pz = pz + seg * uz;
@@ -503,7 +503,7 @@ __device__ bool run_job_fp64(const DevScene &S, WarpAcc *wa, const volatile JobC
     return timed_out;
 }
 
-template <int kMinBlocks, bool G>
+template <int kMinBlocks, int K>
 __global__ void __launch_bounds__(128, kMinBlocks) packets_fp64(JobWork *jobs, int njobs, int *status)
 {
     extern __shared__ __align__(16) unsigned char smem[];
@@ -540,7 +540,7 @@ __global__ void __launch_bounds__(128, kMinBlocks) packets_fp64(JobWork *jobs, i
         const long long *s8 = reinterpret_cast<const long long *>(src);
         long long *d8 = reinterpret_cast<long long *>(&ws->S);
         for (int i = lane; i < (int)(sizeof(DevScene) / 8); i += 32) d8[i] = s8[i];
-        if (!G && ws->S.general) {           // a scene with general shapes needs the G instantiation
+        if (!scene_runs64<K>(ws->S)) {       // a scene of another family than this instantiation's
             if (lane == 0) {
                 atomicOr(status, kStatusBadJob);
                 if (J->jstat != nullptr) atomicOr(J->jstat, kStatusBadJob);
@@ -550,7 +550,7 @@ __global__ void __launch_bounds__(128, kMinBlocks) packets_fp64(JobWork *jobs, i
         if (lane == 0) jobconst_fill(&ws->jc, J);
         wacc_clear(&ws->acc, lane);
         const long long t0 = clock64();
-        const bool timed_out = run_job_fp64<G>(ws->S, &ws->acc, &ws->jc, J, lane);
+        const bool timed_out = run_job_fp64<K>(ws->S, &ws->acc, &ws->jc, J, lane);
         __syncwarp();
         if (lane == 0) wadd(&ws->acc, kBusy, clock64() - t0);
         wacc_flush(&ws->acc, J->totals, lane);
@@ -575,13 +575,16 @@ cudaError_t launch_fp64(JobWork *jobs, int njobs, int *status, int blocks, int t
                         int variant)
 {
     const size_t sm = (size_t)(threads / 32) * sizeof(WarpShared);
-    switch (variant) {   // kNumVariants and up: the same budgets for scenes with general shapes
-    case 1: packets_fp64<3, false><<<blocks, threads, sm, stream>>>(jobs, njobs, status); break;
-    case 2: packets_fp64<2, false><<<blocks, threads, sm, stream>>>(jobs, njobs, status); break;
-    case 3: packets_fp64<4, true><<<blocks, threads, sm, stream>>>(jobs, njobs, status); break;
-    case 4: packets_fp64<3, true><<<blocks, threads, sm, stream>>>(jobs, njobs, status); break;
-    case 5: packets_fp64<2, true><<<blocks, threads, sm, stream>>>(jobs, njobs, status); break;
-    default: packets_fp64<4, false><<<blocks, threads, sm, stream>>>(jobs, njobs, status); break;
+    switch (variant) {   // kNumVariants and up: the same budgets for the other scene families
+    case 1: packets_fp64<3, kPlainScene><<<blocks, threads, sm, stream>>>(jobs, njobs, status); break;
+    case 2: packets_fp64<2, kPlainScene><<<blocks, threads, sm, stream>>>(jobs, njobs, status); break;
+    case 3: packets_fp64<4, kGeneralScene><<<blocks, threads, sm, stream>>>(jobs, njobs, status); break;
+    case 4: packets_fp64<3, kGeneralScene><<<blocks, threads, sm, stream>>>(jobs, njobs, status); break;
+    case 5: packets_fp64<2, kGeneralScene><<<blocks, threads, sm, stream>>>(jobs, njobs, status); break;
+    case 9: packets_fp64<4, kBoxScene><<<blocks, threads, sm, stream>>>(jobs, njobs, status); break;
+    case 10: packets_fp64<3, kBoxScene><<<blocks, threads, sm, stream>>>(jobs, njobs, status); break;
+    case 11: packets_fp64<2, kBoxScene><<<blocks, threads, sm, stream>>>(jobs, njobs, status); break;
+    default: packets_fp64<4, kPlainScene><<<blocks, threads, sm, stream>>>(jobs, njobs, status); break;
     }
     return cudaGetLastError();
 }
@@ -591,12 +594,15 @@ int occupancy_fp64(int threads, int variant)
     int n = 0;
     const size_t sm = (size_t)(threads / 32) * sizeof(WarpShared);
     switch (variant) {
-    case 1: cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, packets_fp64<3, false>, threads, sm); break;
-    case 2: cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, packets_fp64<2, false>, threads, sm); break;
-    case 3: cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, packets_fp64<4, true>, threads, sm); break;
-    case 4: cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, packets_fp64<3, true>, threads, sm); break;
-    case 5: cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, packets_fp64<2, true>, threads, sm); break;
-    default: cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, packets_fp64<4, false>, threads, sm); break;
+    case 1: cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, packets_fp64<3, kPlainScene>, threads, sm); break;
+    case 2: cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, packets_fp64<2, kPlainScene>, threads, sm); break;
+    case 3: cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, packets_fp64<4, kGeneralScene>, threads, sm); break;
+    case 4: cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, packets_fp64<3, kGeneralScene>, threads, sm); break;
+    case 5: cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, packets_fp64<2, kGeneralScene>, threads, sm); break;
+    case 9: cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, packets_fp64<4, kBoxScene>, threads, sm); break;
+    case 10: cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, packets_fp64<3, kBoxScene>, threads, sm); break;
+    case 11: cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, packets_fp64<2, kBoxScene>, threads, sm); break;
+    default: cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, packets_fp64<4, kPlainScene>, threads, sm); break;
     }
     return n;
 }

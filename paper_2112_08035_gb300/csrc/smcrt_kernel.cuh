@@ -492,6 +492,13 @@ __device__ __forceinline__ bool scene_runs(const DevScene &S)
            (!S.general && (K == kCulledScene || S.cull_region < 0) && (K != kBoxScene || S.boxes));
 }
 
+// The same for the FP64 kernels, which have no cell lists.
+template <int K>
+__device__ __forceinline__ bool scene_runs64(const DevScene &S)
+{
+    return K == kGeneralScene || (!S.general && (K != kBoxScene || S.boxes));
+}
+
 // Full scene evaluation (Sec. 2.3): every region, then the bounding box.
 template <bool G>
 __device__ __forceinline__ Eval64 scene_eval64(const DevScene &S, double x, double y, double z, int sel)

@@ -118,13 +118,19 @@ static __device__ __noinline__ float prog_screen(const DevScene &S, int i0, int 
     return s0;
 }
 
+// The functions below are instantiated per scene family (K), as the kernels.
 // The FP64 value of region r: of a fold the listed instructions (cnt >= 0), or
 // the whole program.  Out of line, with the one copy of the primitives: code
 // size counts (see div64).
+template <int K>
 static __device__ __noinline__ double region_exact(const DevScene &S, int r, double x, double y, double z,
                                                    unsigned long long list, int cnt)
 {
     const int2 rr = __ldg(S.rrange + r);
+    if (K == kBoxScene) {                // its one box
+        const int4 ins = __ldg(reinterpret_cast<const int4 *>(S.instr) + rr.x);
+        return base64<false>(1, S.p64 + 8 * ins.y, x, y, z);
+    }
     const bool listed = cnt >= 0 && cnt <= kFoldList;
     const int n = listed ? cnt : rr.y - rr.x;
     double s0 = 0.0, s1 = 0.0, s2 = 0.0, s3 = 0.0;
@@ -147,12 +153,13 @@ static __device__ __noinline__ double region_exact(const DevScene &S, int r, dou
 }
 
 // The list of region r where it is a fold worth one (cnt = -1: none).
+template <int K>
 __device__ __forceinline__ void fold_list(const DevScene &S, int r, double x, double y, double z,
                                           unsigned long long &list, int &cnt)
 {
     cnt = -1;
     list = 0ull;
-    if (!((S.fold_mask >> r) & 1ull)) return;
+    if (K == kBoxScene || !((S.fold_mask >> r) & 1ull)) return;
     const int2 rr = __ldg(S.rrange + r);
     float err;
     if (rr.y - rr.x > kFoldList) fold_screen(S, rr.x, rr.y, (float)x, (float)y, (float)z, list, cnt, err);
@@ -173,6 +180,7 @@ struct Screen64 {
     float db;                // bounding box
 };
 
+template <int K>
 static __device__ __noinline__ Screen64 scene_screen(const DevScene &S, float x, float y, float z, int mode)
 {
     Screen64 C;
@@ -192,8 +200,14 @@ static __device__ __noinline__ Screen64 scene_screen(const DevScene &S, float x,
         float d, err = eps;
         unsigned long long li = 0ull;
         int n = 0;
-        if (S.fold_mask & bit) d = fold_screen(S, rr.x, rr.y, x, y, z, li, n, err);
-        else d = prog_screen(S, rr.x, rr.y, x, y, z);
+        if (K == kBoxScene) {
+            const int4 ins = __ldg(reinterpret_cast<const int4 *>(S.instr) + rr.x);
+            d = scr_prim(S, 1, ins.y, x, y, z);
+        } else if (S.fold_mask & bit) {
+            d = fold_screen(S, rr.x, rr.y, x, y, z, li, n, err);
+        } else {
+            d = prog_screen(S, rr.x, rr.y, x, y, z);
+        }
         if (d < 0.f) C.neg |= bit;
         const float lo = fabsf(d) - err, hi = fabsf(d) + err;
         if (S.soft_mask & bit) soft = fminf(soft, lo);
@@ -213,7 +227,7 @@ static __device__ __noinline__ Screen64 scene_screen(const DevScene &S, float x,
         }
         if (in) {
             C.mask |= bit;
-            if (S.fold_mask & bit) { C.flr = r; C.list = li; C.cnt = min(n, kFoldList + 1); }
+            if (K != kBoxScene && (S.fold_mask & bit)) { C.flr = r; C.list = li; C.cnt = min(n, kFoldList + 1); }
         }
     }
     C.soft = soft;
@@ -229,6 +243,7 @@ static __device__ __noinline__ Screen64 scene_screen(const DevScene &S, float x,
 // FP64 where it may be nearest, else an FP32 value of the right sign.  1.1
 // of the layered slab's 4 surfaces are left per trace evaluation, and no
 // square root where at most one axis is outside (box64).
+template <int K>
 static __device__ __noinline__ Eval64 scene_exact(const DevScene &S, double x, double y, double z, const Screen64 &C,
                                                   int mode)
 {
@@ -244,8 +259,8 @@ static __device__ __noinline__ Eval64 scene_exact(const DevScene &S, double x, d
         mask ^= bit;
         unsigned long long li = C.list;
         int n = C.cnt;
-        if (r != C.flr) fold_list(S, r, x, y, z, li, n);
-        const double d = region_exact(S, r, x, y, z, li, n);
+        if (K != kBoxScene && r != C.flr) fold_list<K>(S, r, x, y, z, li, n);
+        const double d = region_exact<K>(S, r, x, y, z, li, n);
         if (d < 0.0) neg |= bit; else neg &= ~bit;
         const double ad = fabs(d);
         if (less64(ad, E.dmin)) { E.dmin = ad; E.istar = r; E.dstar = d; }
@@ -271,22 +286,22 @@ struct Interface64 {
 };
 enum { kIntfForced = 0, kIntfEscape = 1, kIntfMatched = 2, kIntfFresnel = 3 };
 
-template <bool G>
+template <int K>
 static __device__ __noinline__ double surface_at64(const DevScene &S, int r, double x, double y, double z)
 {
-    if (G || r < 0) return surface64<G>(S, r, x, y, z);
+    if (K == kGeneralScene || r < 0) return surface64<K == kGeneralScene>(S, r, x, y, z);
     unsigned long long list = 0ull;
     int cnt;
-    fold_list(S, r, x, y, z, list, cnt);
-    return region_exact(S, r, x, y, z, list, cnt);
+    fold_list<K>(S, r, x, y, z, list, cnt);
+    return region_exact<K>(S, r, x, y, z, list, cnt);
 }
 
-template <bool G>
+template <int K>
 static __device__ __noinline__ int region_at64(const DevScene &S, double x, double y, double z)
 {
-    if (G) return scene_eval64<G>(S, x, y, z, -2).region;
-    const Screen64 C = scene_screen(S, (float)x, (float)y, (float)z, kForRegion);
-    return scene_exact(S, x, y, z, C, kForRegion).region;
+    if (K == kGeneralScene) return scene_eval64<K == kGeneralScene>(S, x, y, z, -2).region;
+    const Screen64 C = scene_screen<K>(S, (float)x, (float)y, (float)z, kForRegion);
+    return scene_exact<K>(S, x, y, z, C, kForRegion).region;
 }
 
 __device__ __forceinline__ double region_n64(const DevScene &S, int r)
@@ -294,7 +309,7 @@ __device__ __forceinline__ double region_n64(const DevScene &S, int r)
     return r < 0 ? S.ambient_n : __ldg(S.reg64 + kReg64 * r + 3);
 }
 
-template <bool G>
+template <int K>
 static __device__ __noinline__ Interface64 interface64(const DevScene &S, double px, double py, double pz, double ux,
                                                        double uy, double uz, int istar, double dstar)
 {
@@ -307,8 +322,8 @@ static __device__ __noinline__ Interface64 interface64(const DevScene &S, double
     double gx = 0.0, gy = 0.0, gz = 0.0;
     for (int a = 0; a < 3; ++a) {            // central differences
         const double ex = a == 0 ? delta : 0.0, ey = a == 1 ? delta : 0.0, ez = a == 2 ? delta : 0.0;
-        const double fp = surface_at64<G>(S, istar, px + ex, py + ey, pz + ez);
-        const double fm = surface_at64<G>(S, istar, px - ex, py - ey, pz - ez);
+        const double fp = surface_at64<K>(S, istar, px + ex, py + ey, pz + ez);
+        const double fm = surface_at64<K>(S, istar, px - ex, py - ey, pz - ez);
         gx = gy; gy = gz; gz = fp - fm;      // after three turns: x, y, z
     }
     const double l2 = gx * gx + gy * gy + gz * gz;
@@ -323,15 +338,15 @@ static __device__ __noinline__ Interface64 interface64(const DevScene &S, double
     if (istar < 0) return o;
     double qx = px, qy = py, qz = pz;        // Newton projection
     for (int k = 0; k < 3; ++k) {
-        const double dq = surface_at64<G>(S, istar, qx, qy, qz);
+        const double dq = surface_at64<K>(S, istar, qx, qy, qz);
         o.evals += 1;
         if (fabs(dq) <= delta * 1e-3) break;
         qx = qx - dq * nx; qy = qy - dq * ny; qz = qz - dq * nz;
     }
     o.qx = qx; o.qy = qy; o.qz = qz;
     const double ee = 2.0 * delta * (cdot > 0.0 ? 1.0 : -1.0);
-    o.n2 = region_n64(S, region_at64<G>(S, qx + ee * nx, qy + ee * ny, qz + ee * nz));
-    o.n1 = region_n64(S, region_at64<G>(S, qx - ee * nx, qy - ee * ny, qz - ee * nz));
+    o.n2 = region_n64(S, region_at64<K>(S, qx + ee * nx, qy + ee * ny, qz + ee * nz));
+    o.n1 = region_n64(S, region_at64<K>(S, qx - ee * nx, qy - ee * ny, qz - ee * nz));
     o.evals += 2;
     o.what = kIntfMatched;
     if (o.n1 == o.n2) return o;
@@ -409,13 +424,14 @@ __device__ __forceinline__ float scr_sphere(float4 A, float d, float e, const fl
 
 // A lower bound of the move bound (segment_bound64), or a value <= 0 when
 // FP32 cannot tell.
+template <int K>
 static __device__ __noinline__ float segment_screen(const DevScene &S, float soft, const float *p, const float *u)
 {
     const float eps = S.feps, dh = (float)(0.5 * S.delta) * kScrUp;
     if (eps == 0.f) return 0.f;
     float t = fminf(scr_box_exit(S.bbc32, S.bbh32, dh, p, u, eps), soft - dh);
     for (int j = 0; j < S.nseg; ++j) {
-        const int i = __ldg(S.seg_prims + j), kind = __ldg(S.pkind + i);
+        const int i = __ldg(S.seg_prims + j), kind = K == kBoxScene ? 1 : __ldg(S.pkind + i);
         const float e = __ldg(S.seg_m32 + j) * kScrUp + dh;
         const float d = scr_prim(S, kind, i, p[0], p[1], p[2]);
         float b = fabsf(d) - eps - e;
@@ -475,6 +491,7 @@ static __device__ __noinline__ double seg_face64(const double *P, double d, doub
 }
 
 // The move bound of segment_bound64, leaving out what cannot lower it.
+template <int K>
 static __device__ __noinline__ double segment_bound64_screened(const DevScene &S, double soft, double dbox, double px,
                                                                double py, double pz, double ux, double uy, double uz)
 {
@@ -484,20 +501,20 @@ static __device__ __noinline__ double segment_bound64_screened(const DevScene &S
     static_assert(offsetof(DevScene, bbh) == offsetof(DevScene, bbc) + 3 * sizeof(double), "centre, half extents");
     const double *box = reinterpret_cast<const double *>(reinterpret_cast<const char *>(&S) + offsetof(DevScene, bbc));
     double t = seg_face64(box, dbox, px, py, pz, ux, uy, uz, dh, eps);
-    if (S.soft_mask != 0ull && soft - dh <= t) {
+    if (K != kBoxScene && S.soft_mask != 0ull && soft - dh <= t) {
         double ds = __longlong_as_double(0x7ff0000000000000LL);
         for (unsigned long long m = S.soft_mask; m != 0ull; m &= m - 1ull) {
             const int r = __ffsll((long long)m) - 1;
             unsigned long long list = 0ull;
             int cnt;
-            fold_list(S, r, px, py, pz, list, cnt);
-            ds = min64(ds, fabs(region_exact(S, r, px, py, pz, list, cnt)));
+            fold_list<K>(S, r, px, py, pz, list, cnt);
+            ds = min64(ds, fabs(region_exact<K>(S, r, px, py, pz, list, cnt)));
         }
         t = min64(t, ds - dh);
     }
     for (int j = 0; j < S.nseg; ++j) {
         const int i = __ldg(S.seg_prims + j);
-        const int kind = __ldg(S.pkind + i);
+        const int kind = K == kBoxScene ? 1 : __ldg(S.pkind + i);
         const double e = __ldg(S.seg_m64 + j) + dh;
         const float ef = (float)e * kScrUp, tu = (float)t * kScrUp;
         const float df = scr_prim(S, kind, i, p[0], p[1], p[2]);

@@ -1,5 +1,5 @@
-"""Scenes whose every region is one box run mixed-kernel instantiations that
-know no other shape.  The same scene with one region written as the union of
+"""Scenes whose every region is one box run kernel instantiations that know no
+other shape.  The same scene with one region written as the union of
 its box with itself runs the plain ones, whose arithmetic is the same, so
 every tally must be equal."""
 import pytest
@@ -34,9 +34,10 @@ def _workload(name, doubled, stepping):
                       "mixed").with_stepping(stepping)
 
 
+@pytest.mark.parametrize("precision", ["mixed", "fp64"])
 @pytest.mark.parametrize("stepping", [W.SPHERE_TRACING, W.SEGMENT])
 @pytest.mark.parametrize("name", list(SCENES))
-def test_box_scenes_equal_plain(name, stepping):
+def test_box_scenes_equal_plain(name, stepping, precision):
     import torch
     ctx = smc.Context(0)
     got = []
@@ -45,13 +46,13 @@ def test_box_scenes_equal_plain(name, stepping):
         flu = torch.zeros(wl.grid.size, dtype=torch.int64, device="cuda")
         tot = smc.totals_tensor()
         if alloc:
-            plan = ctx.plan(wl, "mixed")
+            plan = ctx.plan(wl, precision)
             plan.launch(0, wl.npackets, wl.seed, flu, tot)
             torch.cuda.synchronize()
             assert plan.status() == 0
             plan.close()
         else:
-            smc.run_noalloc(wl, 0, wl.npackets, wl.seed, flu, tot, "mixed")
+            smc.run_noalloc(wl, 0, wl.npackets, wl.seed, flu, tot, precision)
             torch.cuda.synchronize()
         t = smc.totals_from_tensor(tot)
         got.append((flu, {k: t[k] for k in ("R", "T", "A", "killed", "gain", "packets", "scatters", "steps")}))
