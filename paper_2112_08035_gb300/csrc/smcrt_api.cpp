@@ -287,10 +287,6 @@ cudaError_t launch_kernel(int precision, JobWork *jobs, int njobs, int *status, 
                                    : launch_mixed(jobs, njobs, status, blocks, threads, s, variant);
 }
 
-// Register budgets of served rounds: mixed 96 registers x 5 blocks/SM until the
-// trials on the first mixed job, FP64 3 blocks/SM.
-int serving_variant(int precision) { return precision == SMCRT_FP64 ? 1 : 0; }
-
 uint64_t shape_key(const smcrt_scene *sc, int precision, const smcrt_grid *g)
 {
     uint64_t h = 1469598103934665603ull;
@@ -865,7 +861,7 @@ void scheduler(smcrt_ctx *ctx)
     int threads_m = 128, variant_m = 0;
     int blocks_m = ctx->sm_count * std::max(1, occupancy_mixed_multi(threads_m, variant_m));
     const int threads_d = 128;
-    const int blocks_d = ctx->sm_count * std::max(1, occupancy_fp64(threads_d, serving_variant(SMCRT_FP64)));
+    const int blocks_d = ctx->sm_count * std::max(1, occupancy_fp64_served(threads_d));
     bool tuned_served = false;
     int clk_khz = 1900000;
     cudaDeviceGetAttribute(&clk_khz, cudaDevAttrClockRate, ctx->device);
@@ -921,8 +917,7 @@ void scheduler(smcrt_ctx *ctx)
                 cudaEventRecord(ev_fork, st);
                 cudaStreamWaitEvent(st2, ev_fork, 0);
                 launch_mixed_multi(b.d_tab, kMaxSlots, d_status + bi, blocks_m, threads_m, st, variant_m + off);
-                launch_fp64(b.d_tab + kMaxSlots, kMaxSlots, d_status + bi, blocks_d, threads_d, st2,
-                            serving_variant(SMCRT_FP64) + off);
+                launch_fp64_served(b.d_tab + kMaxSlots, kMaxSlots, d_status + bi, blocks_d, threads_d, st2, gen != 0);
                 cudaEventRecord(ev_join, st2);
                 cudaStreamWaitEvent(st, ev_join, 0);
                 cudaMemcpyAsync(b.h_tot, d_tot, sizeof(smcrt_totals) * kMaxSlots, cudaMemcpyDeviceToHost, st);

@@ -367,6 +367,10 @@ cudaError_t launch_fp64(JobWork *jobs, int njobs, int *status, int blocks, int t
 cudaError_t launch_mixed(JobWork *jobs, int njobs, int *status, int blocks, int threads,
                          cudaStream_t stream, int variant = 0);
 int occupancy_fp64(int threads, int variant = 0);
+// Served rounds' FP64 kernel (3 blocks of 128 threads per SM).
+cudaError_t launch_fp64_served(JobWork *jobs, int njobs, int *status, int blocks, int threads, cudaStream_t stream,
+                               bool general);
+int occupancy_fp64_served(int threads);
 int occupancy_mixed(int threads, int variant = 0);
 // Served rounds' mixed kernel, whose warps hold two jobs at a time (lanes
 // refill from the next job instead of draining each): variant 0 / 1 = 5 / 4

@@ -194,7 +194,7 @@ struct WarpShared {
 // every floating-point operation the reference algorithm's, in its order:
 // the oracle's run of a packet is a sequence of the same IEEE operations on
 // the same values, so its tallies come out bit for bit.
-template <int K>
+template <int K, bool SERVED>
 __device__ bool run_job_fp64(const DevScene &S, WarpAcc *wa, const volatile JobConst *jc, JobWork *J,
                              int lane)
 {
@@ -224,7 +224,7 @@ __device__ bool run_job_fp64(const DevScene &S, WarpAcc *wa, const volatile JobC
             unsigned need = __ballot_sync(SMCRT_FULL, !alive && !retired);
             JobDefer *const dfr = (JobDefer *)jc->dfr;
             const int din = jc->din;
-            if (need && dfr != nullptr) {
+            if (SERVED && need && dfr != nullptr) {
                 const int leader = __ffs(need) - 1;
                 unsigned base = 0u, avail = 0u;
                 if (lane == leader) {
@@ -468,7 +468,7 @@ __device__ bool run_job_fp64(const DevScene &S, WarpAcc *wa, const volatile JobC
             wadd(wa, kPackets, 1); wadd(wa, kEvals, nev);
             nev = 0;
             smcrt_packet_record *const recs = (smcrt_packet_record *)jc->recs;
-            if (recs) {
+            if (!SERVED && recs) {
                 smcrt_packet_record r;
                 r.R = fin_R; r.T = fin_T; r.A = pA; r.killed = fin_K; r.gain = pG;
                 r.scatters = pscat; r.steps = nsteps; r.reserved = 0;
@@ -477,7 +477,7 @@ __device__ bool run_job_fp64(const DevScene &S, WarpAcc *wa, const volatile JobC
             }
         }
         // ---- park a straggler at a trace boundary (serving rounds only)
-        if (SMCRT_RARE(alive && phase == kTrace && jc->budget > 0u && (uint32_t)clock() - t_acq > jc->budget)) {
+        if (SERVED && SMCRT_RARE(alive && phase == kTrace && jc->budget > 0u && (uint32_t)clock() - t_acq > jc->budget)) {
             JobDefer *const dfr = (JobDefer *)jc->dfr;
             const int din = jc->din;
             const unsigned k = atomicAdd(&dfr->count[1 - din], 1u);
@@ -503,7 +503,7 @@ __device__ bool run_job_fp64(const DevScene &S, WarpAcc *wa, const volatile JobC
     return timed_out;
 }
 
-template <int kMinBlocks, int K>
+template <int kMinBlocks, int K, bool SERVED>
 __global__ void __launch_bounds__(128, kMinBlocks) packets_fp64(JobWork *jobs, int njobs, int *status)
 {
     extern __shared__ __align__(16) unsigned char smem[];
@@ -520,7 +520,7 @@ __global__ void __launch_bounds__(128, kMinBlocks) packets_fp64(JobWork *jobs, i
             src = J->scene;
         }
         int parked = 0;
-        if (lane == 0 && J->defer != nullptr) {
+        if (SERVED && lane == 0 && J->defer != nullptr) {
             const int in = J->defer_in & 1;
             parked = min(*(volatile unsigned *)&J->defer->count[in], J->defer->cap) >
                      *(volatile unsigned *)&J->defer->cursor[in];
@@ -550,7 +550,7 @@ __global__ void __launch_bounds__(128, kMinBlocks) packets_fp64(JobWork *jobs, i
         if (lane == 0) jobconst_fill(&ws->jc, J);
         wacc_clear(&ws->acc, lane);
         const long long t0 = clock64();
-        const bool timed_out = run_job_fp64<K>(ws->S, &ws->acc, &ws->jc, J, lane);
+        const bool timed_out = run_job_fp64<K, SERVED>(ws->S, &ws->acc, &ws->jc, J, lane);
         __syncwarp();
         if (lane == 0) wadd(&ws->acc, kBusy, clock64() - t0);
         wacc_flush(&ws->acc, J->totals, lane);
@@ -576,17 +576,37 @@ cudaError_t launch_fp64(JobWork *jobs, int njobs, int *status, int blocks, int t
 {
     const size_t sm = (size_t)(threads / 32) * sizeof(WarpShared);
     switch (variant) {   // kNumVariants and up: the same budgets for the other scene families
-    case 1: packets_fp64<3, kPlainScene><<<blocks, threads, sm, stream>>>(jobs, njobs, status); break;
-    case 2: packets_fp64<2, kPlainScene><<<blocks, threads, sm, stream>>>(jobs, njobs, status); break;
-    case 3: packets_fp64<4, kGeneralScene><<<blocks, threads, sm, stream>>>(jobs, njobs, status); break;
-    case 4: packets_fp64<3, kGeneralScene><<<blocks, threads, sm, stream>>>(jobs, njobs, status); break;
-    case 5: packets_fp64<2, kGeneralScene><<<blocks, threads, sm, stream>>>(jobs, njobs, status); break;
-    case 9: packets_fp64<4, kBoxScene><<<blocks, threads, sm, stream>>>(jobs, njobs, status); break;
-    case 10: packets_fp64<3, kBoxScene><<<blocks, threads, sm, stream>>>(jobs, njobs, status); break;
-    case 11: packets_fp64<2, kBoxScene><<<blocks, threads, sm, stream>>>(jobs, njobs, status); break;
-    default: packets_fp64<4, kPlainScene><<<blocks, threads, sm, stream>>>(jobs, njobs, status); break;
+    case 1: packets_fp64<3, kPlainScene, false><<<blocks, threads, sm, stream>>>(jobs, njobs, status); break;
+    case 2: packets_fp64<2, kPlainScene, false><<<blocks, threads, sm, stream>>>(jobs, njobs, status); break;
+    case 3: packets_fp64<4, kGeneralScene, false><<<blocks, threads, sm, stream>>>(jobs, njobs, status); break;
+    case 4: packets_fp64<3, kGeneralScene, false><<<blocks, threads, sm, stream>>>(jobs, njobs, status); break;
+    case 5: packets_fp64<2, kGeneralScene, false><<<blocks, threads, sm, stream>>>(jobs, njobs, status); break;
+    case 9: packets_fp64<4, kBoxScene, false><<<blocks, threads, sm, stream>>>(jobs, njobs, status); break;
+    case 10: packets_fp64<3, kBoxScene, false><<<blocks, threads, sm, stream>>>(jobs, njobs, status); break;
+    case 11: packets_fp64<2, kBoxScene, false><<<blocks, threads, sm, stream>>>(jobs, njobs, status); break;
+    default: packets_fp64<4, kPlainScene, false><<<blocks, threads, sm, stream>>>(jobs, njobs, status); break;
     }
     return cudaGetLastError();
+}
+
+// Served rounds: packets park, no packet records, and a round holds scenes of
+// all families.  Plan launches leave the parking out (layered slab 1e5
+// packets 46.2 -> 44.5 ms, thick slab 3e3 110.5 -> 108.0 ms).
+cudaError_t launch_fp64_served(JobWork *jobs, int njobs, int *status, int blocks, int threads, cudaStream_t stream,
+                               bool general)
+{
+    const size_t sm = (size_t)(threads / 32) * sizeof(WarpShared);
+    if (general) packets_fp64<3, kGeneralScene, true><<<blocks, threads, sm, stream>>>(jobs, njobs, status);
+    else packets_fp64<3, kPlainScene, true><<<blocks, threads, sm, stream>>>(jobs, njobs, status);
+    return cudaGetLastError();
+}
+
+int occupancy_fp64_served(int threads)
+{
+    int n = 0;
+    const size_t sm = (size_t)(threads / 32) * sizeof(WarpShared);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, packets_fp64<3, kPlainScene, true>, threads, sm);
+    return n;
 }
 
 int occupancy_fp64(int threads, int variant)
@@ -594,15 +614,15 @@ int occupancy_fp64(int threads, int variant)
     int n = 0;
     const size_t sm = (size_t)(threads / 32) * sizeof(WarpShared);
     switch (variant) {
-    case 1: cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, packets_fp64<3, kPlainScene>, threads, sm); break;
-    case 2: cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, packets_fp64<2, kPlainScene>, threads, sm); break;
-    case 3: cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, packets_fp64<4, kGeneralScene>, threads, sm); break;
-    case 4: cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, packets_fp64<3, kGeneralScene>, threads, sm); break;
-    case 5: cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, packets_fp64<2, kGeneralScene>, threads, sm); break;
-    case 9: cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, packets_fp64<4, kBoxScene>, threads, sm); break;
-    case 10: cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, packets_fp64<3, kBoxScene>, threads, sm); break;
-    case 11: cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, packets_fp64<2, kBoxScene>, threads, sm); break;
-    default: cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, packets_fp64<4, kPlainScene>, threads, sm); break;
+    case 1: cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, packets_fp64<3, kPlainScene, false>, threads, sm); break;
+    case 2: cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, packets_fp64<2, kPlainScene, false>, threads, sm); break;
+    case 3: cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, packets_fp64<4, kGeneralScene, false>, threads, sm); break;
+    case 4: cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, packets_fp64<3, kGeneralScene, false>, threads, sm); break;
+    case 5: cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, packets_fp64<2, kGeneralScene, false>, threads, sm); break;
+    case 9: cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, packets_fp64<4, kBoxScene, false>, threads, sm); break;
+    case 10: cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, packets_fp64<3, kBoxScene, false>, threads, sm); break;
+    case 11: cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, packets_fp64<2, kBoxScene, false>, threads, sm); break;
+    default: cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, packets_fp64<4, kPlainScene, false>, threads, sm); break;
     }
     return n;
 }
