@@ -188,13 +188,18 @@ struct Instr {
     int32_t pad;
 };
 
-// Whether every region is one box in scene coordinates (a compiled program:
-// one instruction per region).
-inline bool box_regions(const Instr *ins, int ninstr, int nregions)
+// Whether every region is one sphere, box or capsule in scene coordinates (a
+// compiled program: one instruction per region), or even one box.
+enum : int { kSinglePrims = 1, kSingleBoxes = 2 };
+inline int single_regions(const Instr *ins, int ninstr, int nregions)
 {
-    bool all = ninstr == nregions && nregions > 0;
-    for (int i = 0; all && i < ninstr; ++i) all = (ins[i].op & 0xff) == 0 && ((ins[i].op >> 8) & 0xff) == SMCRT_BOX;
-    return all;
+    bool one = ninstr == nregions && nregions > 0, box = true;
+    for (int i = 0; one && i < ninstr; ++i) {
+        const int kind = (ins[i].op >> 8) & 0xff;
+        one = (ins[i].op & 0xff) == 0 && kind <= SMCRT_CAPSULE;
+        box = box && kind == SMCRT_BOX;
+    }
+    return !one ? 0 : box ? kSingleBoxes : kSinglePrims;
 }
 
 // Scene + source + grid of one plan as the kernels read them.  Lives in
@@ -244,7 +249,7 @@ struct DevScene {
     const double *xf64;
     const float4 *xf32;
     int32_t general;          // some primitive is a torus or cylinder or has a frame
-    int32_t boxes;            // every region is one box in scene coordinates
+    int32_t singles;          // single_regions: kSingleBoxes, kSinglePrims or 0
     float h32;                // FP32 central-difference step for normals
     int64_t max_steps;
     // source
@@ -421,14 +426,18 @@ inline int default_variant(int precision, uint64_t npackets, const DevScene &S)
 // 111.0 ms, 1e4 2.05 -> 1.77 ms, with sphere tracing 1e6 28.8 -> 25.1; thick
 // slab 1e6 67.7 -> 65.3 ms (its loop is mostly scattering); in FP64, layered
 // slab 1e5 58.9 -> 46.2 ms, 1e4 16.4 -> 13.4, 1e6 485 -> 342, thick slab 3e3
-// 114.6 -> 110.9.  The FP64 kernels have no cell lists; served rounds hold
-// scenes of all kinds and have two families, general and not.
-enum : int { kPlainScene = 0, kGeneralScene = 1, kCulledScene = 2, kBoxScene = 3 };
+// 114.6 -> 110.9.  In FP64 scenes of one primitive per region have a family
+// too (sphere 1e5, sphere tracing, 73.4 -> 65.1 ms, segments 13.1 -> 11.3);
+// in mixed precision it gained nothing (homogeneous sphere 2e6 24.8 -> 25.2
+// ms).  The FP64 kernels have no cell lists; served rounds hold scenes of all
+// kinds and have two families, general and not.
+enum : int { kPlainScene = 0, kGeneralScene = 1, kCulledScene = 2, kBoxScene = 3, kSingleScene = 4 };
 inline int scene_family(int precision, const DevScene &S)
 {
     if (S.general) return kGeneralScene;
     if (precision == SMCRT_MIXED && S.cull_region >= 0) return kCulledScene;
-    return S.boxes ? kBoxScene : kPlainScene;
+    if (S.singles == kSingleBoxes) return kBoxScene;
+    return precision == SMCRT_FP64 && S.singles != 0 ? kSingleScene : kPlainScene;
 }
 
 // Lanes of a warp that carry packets in a plan launch (JobWork.lanes; 0 =

@@ -584,6 +584,9 @@ cudaError_t launch_fp64(JobWork *jobs, int njobs, int *status, int blocks, int t
     case 9: packets_fp64<4, kBoxScene, false><<<blocks, threads, sm, stream>>>(jobs, njobs, status); break;
     case 10: packets_fp64<3, kBoxScene, false><<<blocks, threads, sm, stream>>>(jobs, njobs, status); break;
     case 11: packets_fp64<2, kBoxScene, false><<<blocks, threads, sm, stream>>>(jobs, njobs, status); break;
+    case 12: packets_fp64<4, kSingleScene, false><<<blocks, threads, sm, stream>>>(jobs, njobs, status); break;
+    case 13: packets_fp64<3, kSingleScene, false><<<blocks, threads, sm, stream>>>(jobs, njobs, status); break;
+    case 14: packets_fp64<2, kSingleScene, false><<<blocks, threads, sm, stream>>>(jobs, njobs, status); break;
     default: packets_fp64<4, kPlainScene, false><<<blocks, threads, sm, stream>>>(jobs, njobs, status); break;
     }
     return cudaGetLastError();
@@ -622,6 +625,9 @@ int occupancy_fp64(int threads, int variant)
     case 9: cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, packets_fp64<4, kBoxScene, false>, threads, sm); break;
     case 10: cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, packets_fp64<3, kBoxScene, false>, threads, sm); break;
     case 11: cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, packets_fp64<2, kBoxScene, false>, threads, sm); break;
+    case 12: cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, packets_fp64<4, kSingleScene, false>, threads, sm); break;
+    case 13: cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, packets_fp64<3, kSingleScene, false>, threads, sm); break;
+    case 14: cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, packets_fp64<2, kSingleScene, false>, threads, sm); break;
     default: cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, packets_fp64<4, kPlainScene, false>, threads, sm); break;
     }
     return n;

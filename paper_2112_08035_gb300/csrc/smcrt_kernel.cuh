@@ -489,14 +489,15 @@ template <int K>
 __device__ __forceinline__ bool scene_runs(const DevScene &S)
 {
     return K == kGeneralScene ||
-           (!S.general && (K == kCulledScene || S.cull_region < 0) && (K != kBoxScene || S.boxes));
+           (!S.general && (K == kCulledScene || S.cull_region < 0) && (K != kBoxScene || S.singles == kSingleBoxes));
 }
 
 // The same for the FP64 kernels, which have no cell lists.
 template <int K>
 __device__ __forceinline__ bool scene_runs64(const DevScene &S)
 {
-    return K == kGeneralScene || (!S.general && (K != kBoxScene || S.boxes));
+    return K == kGeneralScene ||
+           (!S.general && (K != kBoxScene || S.singles == kSingleBoxes) && (K != kSingleScene || S.singles != 0));
 }
 
 // Full scene evaluation (Sec. 2.3): every region, then the bounding box.

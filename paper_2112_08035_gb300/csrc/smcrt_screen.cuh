@@ -119,6 +119,12 @@ static __device__ __noinline__ float prog_screen(const DevScene &S, int i0, int 
 }
 
 // The functions below are instantiated per scene family (K), as the kernels.
+template <int K>
+__device__ constexpr bool one_each()     // one primitive per region
+{
+    return K == kBoxScene || K == kSingleScene;
+}
+
 // The FP64 value of region r: of a fold the listed instructions (cnt >= 0), or
 // the whole program.  Out of line, with the one copy of the primitives: code
 // size counts (see div64).
@@ -127,9 +133,9 @@ static __device__ __noinline__ double region_exact(const DevScene &S, int r, dou
                                                    unsigned long long list, int cnt)
 {
     const int2 rr = __ldg(S.rrange + r);
-    if (K == kBoxScene) {                // its one box
+    if (one_each<K>()) {                 // its one primitive
         const int4 ins = __ldg(reinterpret_cast<const int4 *>(S.instr) + rr.x);
-        return base64<false>(1, S.p64 + 8 * ins.y, x, y, z);
+        return base64<false>(K == kBoxScene ? 1 : (ins.x >> 8) & 0xff, S.p64 + 8 * ins.y, x, y, z);
     }
     const bool listed = cnt >= 0 && cnt <= kFoldList;
     const int n = listed ? cnt : rr.y - rr.x;
@@ -159,7 +165,7 @@ __device__ __forceinline__ void fold_list(const DevScene &S, int r, double x, do
 {
     cnt = -1;
     list = 0ull;
-    if (K == kBoxScene || !((S.fold_mask >> r) & 1ull)) return;
+    if (one_each<K>() || !((S.fold_mask >> r) & 1ull)) return;
     const int2 rr = __ldg(S.rrange + r);
     float err;
     if (rr.y - rr.x > kFoldList) fold_screen(S, rr.x, rr.y, (float)x, (float)y, (float)z, list, cnt, err);
@@ -200,9 +206,9 @@ static __device__ __noinline__ Screen64 scene_screen(const DevScene &S, float x,
         float d, err = eps;
         unsigned long long li = 0ull;
         int n = 0;
-        if (K == kBoxScene) {
+        if (one_each<K>()) {
             const int4 ins = __ldg(reinterpret_cast<const int4 *>(S.instr) + rr.x);
-            d = scr_prim(S, 1, ins.y, x, y, z);
+            d = scr_prim(S, K == kBoxScene ? 1 : (ins.x >> 8) & 0xff, ins.y, x, y, z);
         } else if (S.fold_mask & bit) {
             d = fold_screen(S, rr.x, rr.y, x, y, z, li, n, err);
         } else {
@@ -227,7 +233,11 @@ static __device__ __noinline__ Screen64 scene_screen(const DevScene &S, float x,
         }
         if (in) {
             C.mask |= bit;
-            if (K != kBoxScene && (S.fold_mask & bit)) { C.flr = r; C.list = li; C.cnt = min(n, kFoldList + 1); }
+            if (!one_each<K>() && (S.fold_mask & bit)) {
+                C.flr = r;
+                C.list = li;
+                C.cnt = min(n, kFoldList + 1);
+            }
         }
     }
     C.soft = soft;
@@ -259,7 +269,7 @@ static __device__ __noinline__ Eval64 scene_exact(const DevScene &S, double x, d
         mask ^= bit;
         unsigned long long li = C.list;
         int n = C.cnt;
-        if (K != kBoxScene && r != C.flr) fold_list<K>(S, r, x, y, z, li, n);
+        if (!one_each<K>() && r != C.flr) fold_list<K>(S, r, x, y, z, li, n);
         const double d = region_exact<K>(S, r, x, y, z, li, n);
         if (d < 0.0) neg |= bit; else neg &= ~bit;
         const double ad = fabs(d);
@@ -501,7 +511,7 @@ static __device__ __noinline__ double segment_bound64_screened(const DevScene &S
     static_assert(offsetof(DevScene, bbh) == offsetof(DevScene, bbc) + 3 * sizeof(double), "centre, half extents");
     const double *box = reinterpret_cast<const double *>(reinterpret_cast<const char *>(&S) + offsetof(DevScene, bbc));
     double t = seg_face64(box, dbox, px, py, pz, ux, uy, uz, dh, eps);
-    if (K != kBoxScene && S.soft_mask != 0ull && soft - dh <= t) {
+    if (!one_each<K>() && S.soft_mask != 0ull && soft - dh <= t) {
         double ds = __longlong_as_double(0x7ff0000000000000LL);
         for (unsigned long long m = S.soft_mask; m != 0ull; m &= m - 1ull) {
             const int r = __ffsll((long long)m) - 1;

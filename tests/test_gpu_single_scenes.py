@@ -1,6 +1,7 @@
-"""Scenes whose every region is one box run kernel instantiations that know no
-other shape.  The same scene with one region written as the union of
-its box with itself runs the plain ones, whose arithmetic is the same, so
+"""Scenes whose every region is one box, or one primitive, run kernel
+instantiations without the interpreter (boxes: in both precisions; any
+primitives: FP64).  The same scene with one region written as the union of its
+primitive with itself runs the plain ones, whose arithmetic is the same, so
 every tally must be equal."""
 import pytest
 
@@ -9,7 +10,7 @@ import workloads as W
 
 pytestmark = pytest.mark.gpu
 
-# centre and half extents of the regions' boxes
+# boxes: centre and half extents; spheres: centre and radius; capsules: ends and radius
 SCENES = {
     "one": [(0.0, 0.0, 0.0, 0.5, 0.4, 0.3)],
     "layers": [(0.0, 0.0, 0.45, 4.0, 4.0, 0.05), (0.0, 0.0, 0.2, 4.0, 4.0, 0.2), (0.0, 0.0, -0.3, 4.0, 4.0, 0.3)],
@@ -18,18 +19,22 @@ SCENES = {
               (0.0, 0.0, 0.0, 0.01, 0.01, 0.6)],
     "many": [(0.2 * (i % 4) - 0.3, 0.2 * (i // 4 % 4) - 0.3, 0.25 * (i // 16) - 0.2, 0.07, 0.08, 0.09)
              for i in range(16)],
+    "sphere": [(0.0, 0.0, 0.0, 0.5)],
+    "inclusions": [(0.0, 0.0, 0.0, 0.5, 0.5, 0.5), (0.1, 0.1, 0.1, 0.3), (-0.3, -0.2, -0.4, 0.2, 0.3, 0.4, 0.08),
+                   (0.0, 0.0, -0.2, 0.2, 0.2, 0.05), (0.1, 0.1, 0.1, 0.25)],
 }
 
 
 def _workload(name, doubled, stepping):
-    prims = tuple(W.Prim(W.BOX, tuple(float(v) for v in b)) for b in SCENES[name])
+    kinds = {4: W.SPHERE, 6: W.BOX, 7: W.CAPSULE}
+    prims = tuple(W.Prim(kinds[len(b)], tuple(float(v) for v in b)) for b in SCENES[name])
     regions = []
     for i in range(len(prims)):
         prog = W.prim_program([0, 0]) if doubled and i == 0 else W.prim_program([i])
         regions.append(W.Region(prog, 0.3 + 0.1 * (i % 5), 5.0 + 10.0 * (i % 3), 0.8, (1.4, 1.33, 1.5)[i % 3]))
     b = 0.7
     scene = W.Scene(prims, tuple(regions), 1.0, (-b, -b, -b), (b, b, b))
-    return W.Workload("boxes", scene, W.Source(W.SQUARE, (0.0, 0.0, 0.65), (0.0, 0.0, -1.0), 0.5),
+    return W.Workload("singles", scene, W.Source(W.SQUARE, (0.0, 0.0, 0.65), (0.0, 0.0, -1.0), 0.5),
                       W.Grid((-0.5, -0.5, -0.5), (0.5, 0.5, 0.5), (17, 16, 15)), 20_000, 3,
                       "mixed").with_stepping(stepping)
 
@@ -37,7 +42,7 @@ def _workload(name, doubled, stepping):
 @pytest.mark.parametrize("precision", ["mixed", "fp64"])
 @pytest.mark.parametrize("stepping", [W.SPHERE_TRACING, W.SEGMENT])
 @pytest.mark.parametrize("name", list(SCENES))
-def test_box_scenes_equal_plain(name, stepping, precision):
+def test_single_scenes_equal_plain(name, stepping, precision):
     import torch
     ctx = smc.Context(0)
     got = []
