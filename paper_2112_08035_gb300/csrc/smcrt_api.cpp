@@ -549,8 +549,11 @@ int build_plan(smcrt_ctx *ctx, const smcrt_scene *sc, const smcrt_source *src, c
     H.cull_region = cg.region;
     H.cull_g = cg.g;
     H.cull_op = cg.op;
-    H.cull_capsules = cg.region >= 0;
-    for (int32_t i : cg.list) H.cull_capsules = H.cull_capsules && pkind[i] == SMCRT_CAPSULE;
+    bool capsules = cg.region >= 0, tree = true;
+    for (int32_t i : cg.list) capsules = capsules && pkind[i] == SMCRT_CAPSULE;
+    for (int r = 0; r < nr; ++r)
+        if (r != cg.region) tree = tree && rr[r].y - rr[r].x == 1 && (ins[rr[r].x].op >> 8 & 0xff) == SMCRT_BOX;
+    H.cull_kind = !capsules ? 0 : tree ? kListTree : kListCapsules;
     for (int a = 0; a < 3; ++a) {
         H.cull_lo[a] = cg.lo[a];
         H.cull_inv_s[a] = cg.inv_s[a];

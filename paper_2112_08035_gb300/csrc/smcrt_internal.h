@@ -232,7 +232,7 @@ struct DevScene {
     int32_t cull_region;      // -1: none
     int32_t cull_g;
     int32_t cull_op;          // 1 union, 2 smooth union
-    int32_t cull_capsules;    // all listed primitives are capsules
+    int32_t cull_kind;        // kListCapsules: only capsules listed; kListTree: and every other region is one box
     float cull_lo[3], cull_inv_s[3];
     float cull_rmax;          // R (union) or R - k/4 (smooth union)
     float cull_kinv;
@@ -413,29 +413,34 @@ inline int default_variant(int precision, uint64_t npackets, const DevScene &S)
 }
 
 // Kernel family of a scene: its register variants start at kNumVariants
-// times this.  A plain scene's mixed kernel carries neither the general
-// shapes' code nor the cell lists': the packet loop is close to the
-// instruction cache's size, so code that a scene does not use costs it time
-// all the same.  Measured, cell lists in the plain kernel / in a family of
+// times this.  The packet loop is close to the instruction cache's size, so
+// code that a scene does not use costs it time all the same; a family's
+// kernels leave out what its scenes cannot need:
+//   general        tori, cylinders, frames, long programs (mixed: probe normals)
+//   cell lists     mixed only; with general shapes or without
+//   tree           a cell list of capsules among regions of one box each
+//   boxes          every region one box: no other shape, no CSG interpreter
+//   singles        FP64: every region one sphere, box or capsule
+//   plain          the rest: spheres, boxes and capsules, any CSG
+// Measured, without and with the family.  Cell lists in the plain kernel / in
 // their own: layered slab 1e7 packets 138.2 / 134.4 ms, 1e6 with sphere
-// tracing 30.8 / 28.7; glass container 4e6 59.9 / 58.4 ms; the vessel tree
-// 4e6, with the capsule loop of culled_region32, 128.8 / 117.0 ms (with that
-// loop in the shared kernel 117.3, but the slab 149.5).  Scenes whose every
-// region is one box (layered tissue, block phantoms) run a kernel without the
-// CSG interpreter and the other shapes: layered slab 1e7 packets 134.4 ->
-// 111.0 ms, 1e4 2.05 -> 1.77 ms, with sphere tracing 1e6 28.8 -> 25.1; thick
-// slab 1e6 67.7 -> 65.3 ms (its loop is mostly scattering); in FP64, layered
-// slab 1e5 58.9 -> 46.2 ms, 1e4 16.4 -> 13.4, 1e6 485 -> 342, thick slab 3e3
-// 114.6 -> 110.9.  In FP64 scenes of one primitive per region have a family
-// too (sphere 1e5, sphere tracing, 73.4 -> 65.1 ms, segments 13.1 -> 11.3);
-// in mixed precision it gained nothing (homogeneous sphere 2e6 24.8 -> 25.2
-// ms).  The FP64 kernels have no cell lists; served rounds hold scenes of all
-// kinds and have two families, general and not.
-enum : int { kPlainScene = 0, kGeneralScene = 1, kCulledScene = 2, kBoxScene = 3, kSingleScene = 4 };
+// tracing 30.8 / 28.7, glass container 4e6 59.9 / 58.4; out of the general
+// one: shape gallery 5e5 157 / 147 ms.  Tree: vessel tree 4e6 116 / 96 ms, 1e4
+// 6.4 / 5.8.  Boxes: layered slab 1e7 134.4 / 111.0 ms, 1e4 2.05 / 1.77, with
+// sphere tracing 1e6 28.8 / 25.1, thick slab 1e6 67.7 / 65.3 (its loop is
+// mostly scattering); FP64 layered slab 1e5 58.9 / 46.2 ms, 1e4 16.4 / 13.4,
+// 1e6 485 / 342, thick slab 3e3 114.6 / 110.9.  Singles: FP64 sphere 1e5, with
+// sphere tracing, 73.7 / 64.0 ms, segments 13.1 / 11.2; in mixed precision
+// nothing (homogeneous sphere 2e6 24.8 / 25.2).  Served rounds hold scenes of
+// all kinds and have two families, general with cell lists and plain with.
+enum : int { kPlainScene = 0, kGeneralScene = 1, kCulledScene = 2, kBoxScene = 3, kSingleScene = 4,
+             kGeneralCulledScene = 5, kTreeScene = 6 };
+enum : int { kListCapsules = 1, kListTree = 2 };   // DevScene.cull_kind
 inline int scene_family(int precision, const DevScene &S)
 {
-    if (S.general) return kGeneralScene;
-    if (precision == SMCRT_MIXED && S.cull_region >= 0) return kCulledScene;
+    const bool cells = precision == SMCRT_MIXED && S.cull_region >= 0;
+    if (S.general) return cells ? kGeneralCulledScene : kGeneralScene;
+    if (cells) return S.cull_kind == kListTree ? kTreeScene : kCulledScene;
     if (S.singles == kSingleBoxes) return kBoxScene;
     return precision == SMCRT_FP64 && S.singles != 0 ? kSingleScene : kPlainScene;
 }

@@ -266,9 +266,9 @@ template <int K>
 static __device__ __noinline__ float surface32(const DevScene &S, int r, float x, float y, float z)
 {
     if (r < 0) return box32(x, y, z, S.bbc32[0], S.bbc32[1], S.bbc32[2], S.bbh32[0], S.bbh32[1], S.bbh32[2]);
-    if ((K == kGeneralScene || K == kCulledScene) && r == S.cull_region) return culled_region32(S, x, y, z);
+    if (has_cells<K>() && r == S.cull_region) return culled_region32<K>(S, x, y, z);
     const int2 rr = (*(S.rrange + r));
-    return run_prog32<K == kGeneralScene>(S, rr.x, rr.y, x, y, z);
+    return run_prog32<has_shapes<K>()>(S, rr.x, rr.y, x, y, z);
 }
 
 // A packet within delta32 of a surface (Sec. 2.3), all of it at once, out of
@@ -296,7 +296,7 @@ static __device__ __noinline__ Interface32 interface32(const DevScene &S, float 
     Interface32 o;
     o.refined = 0;
     float nx, ny, nz;
-    if (K != kGeneralScene || S.analytic_nrm) {   // gradient of a short program
+    if (!has_shapes<K>() || S.analytic_nrm) {   // gradient of a short program
         grad_surface32<K>(S, istar, px, py, pz, nx, ny, nz);
     } else {                                 // central differences
         const float h = S.h32;
@@ -341,7 +341,7 @@ static __device__ __noinline__ Interface32 interface32(const DevScene &S, float 
     const bool matched = region_n32(S, rnear) == region_n32(S, rfar);
     uint32_t xiw = 0u;
     if (!matched) xiw = philox4x32_10(make_uint4(event, 0u, id_lo, id_hi), k0, k1).x;
-    const Crossed c = cross32<K == kGeneralScene>(S, ux, uy, uz, qx, qy, qz, nx, ny, nz, tau, dstar, cdot, istar,
+    const Crossed c = cross32<has_shapes<K>()>(S, ux, uy, uz, qx, qy, qz, nx, ny, nz, tau, dstar, cdot, istar,
                                                   rnear, rfar, xiw, matched);
     o.what = matched ? kIntfMatched : kIntfFresnel;
     o.refined = c.refined;
@@ -784,7 +784,7 @@ __device__ bool run_job_mixed(JobSlot *slots, JobWork *jobs, int njobs, int firs
                     const Interface32 I = interface32<K>(S, px, py, pz, ux, uy, uz, tau, reg, istar, dstar, event,
                                                          id_lo, id_hi, jc->k0, jc->k1);
                     phase = kTrace;
-                    if (K == kGeneralScene && !S.analytic_nrm) wadd(wa, kEvals, 6);   // the probes
+                    if (has_shapes<K>() && !S.analytic_nrm) wadd(wa, kEvals, 6);   // the probes
                     if (I.what == kIntfForced) {
                         L = delta;                          // forced step along u
                         move = true;
@@ -1051,10 +1051,7 @@ __global__ void __launch_bounds__(128, kMinBlocks) packets_mixed_multi(JobWork *
 // Register budgets of the instantiations: variant v keeps kMinBlocks
 // blocks of 128 threads resident per SM (more blocks = fewer registers per
 // thread, possibly spilled); the autotuner picks per scene.  Variants
-// kNumVariants .. 2 kNumVariants - 1 are the same budgets for scenes with
-// general shapes (tori, cylinders, primitive frames), 2 kNumVariants .. for
-// plain scenes with a cell list, 3 kNumVariants .. for scenes of boxes
-// (scene_family).
+// kNumVariants * k .. are the same budgets for scene family k (scene_family).
 constexpr int kVariantBlocks[kNumVariants] = {5, 4, 3};
 
 cudaError_t launch_mixed(JobWork *jobs, int njobs, int *status, int blocks, int threads, cudaStream_t stream,
@@ -1073,6 +1070,12 @@ cudaError_t launch_mixed(JobWork *jobs, int njobs, int *status, int blocks, int 
     case 9: packets_mixed<5, kBoxScene><<<blocks, threads, sm, stream>>>(jobs, njobs, status); break;
     case 10: packets_mixed<4, kBoxScene><<<blocks, threads, sm, stream>>>(jobs, njobs, status); break;
     case 11: packets_mixed<3, kBoxScene><<<blocks, threads, sm, stream>>>(jobs, njobs, status); break;
+    case 15: packets_mixed<5, kGeneralCulledScene><<<blocks, threads, sm, stream>>>(jobs, njobs, status); break;
+    case 16: packets_mixed<4, kGeneralCulledScene><<<blocks, threads, sm, stream>>>(jobs, njobs, status); break;
+    case 17: packets_mixed<3, kGeneralCulledScene><<<blocks, threads, sm, stream>>>(jobs, njobs, status); break;
+    case 18: packets_mixed<5, kTreeScene><<<blocks, threads, sm, stream>>>(jobs, njobs, status); break;
+    case 19: packets_mixed<4, kTreeScene><<<blocks, threads, sm, stream>>>(jobs, njobs, status); break;
+    case 20: packets_mixed<3, kTreeScene><<<blocks, threads, sm, stream>>>(jobs, njobs, status); break;
     default: packets_mixed<5, kPlainScene><<<blocks, threads, sm, stream>>>(jobs, njobs, status); break;
     }
     return cudaGetLastError();
@@ -1086,8 +1089,8 @@ cudaError_t launch_mixed_multi(JobWork *jobs, int njobs, int *status, int blocks
     const size_t sm = (size_t)(threads / 32) * sizeof(WarpSharedMulti);
     switch (variant) {
     case 1: packets_mixed_multi<4, kCulledScene><<<blocks, threads, sm, stream>>>(jobs, njobs, status); break;
-    case 3: packets_mixed_multi<5, kGeneralScene><<<blocks, threads, sm, stream>>>(jobs, njobs, status); break;
-    case 4: packets_mixed_multi<4, kGeneralScene><<<blocks, threads, sm, stream>>>(jobs, njobs, status); break;
+    case 3: packets_mixed_multi<5, kGeneralCulledScene><<<blocks, threads, sm, stream>>>(jobs, njobs, status); break;
+    case 4: packets_mixed_multi<4, kGeneralCulledScene><<<blocks, threads, sm, stream>>>(jobs, njobs, status); break;
     default: packets_mixed_multi<5, kCulledScene><<<blocks, threads, sm, stream>>>(jobs, njobs, status); break;
     }
     return cudaGetLastError();
@@ -1099,8 +1102,8 @@ int occupancy_mixed_multi(int threads, int variant)
     const size_t sm = (size_t)(threads / 32) * sizeof(WarpSharedMulti);
     switch (variant) {
     case 1: cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, packets_mixed_multi<4, kCulledScene>, threads, sm); break;
-    case 3: cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, packets_mixed_multi<5, kGeneralScene>, threads, sm); break;
-    case 4: cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, packets_mixed_multi<4, kGeneralScene>, threads, sm); break;
+    case 3: cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, packets_mixed_multi<5, kGeneralCulledScene>, threads, sm); break;
+    case 4: cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, packets_mixed_multi<4, kGeneralCulledScene>, threads, sm); break;
     default: cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, packets_mixed_multi<5, kCulledScene>, threads, sm); break;
     }
     return n;
@@ -1122,6 +1125,12 @@ int occupancy_mixed(int threads, int variant)
     case 9: cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, packets_mixed<5, kBoxScene>, threads, sm); break;
     case 10: cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, packets_mixed<4, kBoxScene>, threads, sm); break;
     case 11: cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, packets_mixed<3, kBoxScene>, threads, sm); break;
+    case 15: cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, packets_mixed<5, kGeneralCulledScene>, threads, sm); break;
+    case 16: cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, packets_mixed<4, kGeneralCulledScene>, threads, sm); break;
+    case 17: cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, packets_mixed<3, kGeneralCulledScene>, threads, sm); break;
+    case 18: cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, packets_mixed<5, kTreeScene>, threads, sm); break;
+    case 19: cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, packets_mixed<4, kTreeScene>, threads, sm); break;
+    case 20: cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, packets_mixed<3, kTreeScene>, threads, sm); break;
     default: cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, packets_mixed<5, kPlainScene>, threads, sm); break;
     }
     return n;

@@ -484,12 +484,20 @@ __device__ __forceinline__ float run_prog32(const DevScene &S, int i0, int i1, f
     return s0;
 }
 
+// What a mixed instantiation of scene family K carries.
+template <int K>
+__device__ constexpr bool has_shapes() { return K == kGeneralScene || K == kGeneralCulledScene; }
+template <int K>
+__device__ constexpr bool has_cells() { return K == kCulledScene || K == kGeneralCulledScene || K == kTreeScene; }
+template <int K>                         // outside the cell list, one box per region
+__device__ constexpr bool has_boxes_only() { return K == kBoxScene || K == kTreeScene; }
+
 // Whether the mixed instantiation K can run scene S.
 template <int K>
 __device__ __forceinline__ bool scene_runs(const DevScene &S)
 {
-    return K == kGeneralScene ||
-           (!S.general && (K == kCulledScene || S.cull_region < 0) && (K != kBoxScene || S.singles == kSingleBoxes));
+    return (has_shapes<K>() || !S.general) && (has_cells<K>() || S.cull_region < 0) &&
+           (K != kBoxScene || S.singles == kSingleBoxes) && (K != kTreeScene || S.cull_kind == kListTree);
 }
 
 // The same for the FP64 kernels, which have no cell lists.
@@ -520,7 +528,9 @@ __device__ __forceinline__ Eval64 scene_eval64(const DevScene &S, double x, doub
 // for p's cell, bounded by cull_rmax (every unlisted primitive is farther
 // than R from the cell, so it cannot change the value below that bound).
 // A vessel tree's list holds capsules only, so the loop over them looks at
-// no kind: vessel tree 4e6 packets 128.8 -> 117.0 ms.
+// no kind: vessel tree 4e6 packets 128.8 -> 117.0 ms (then tree scenes got
+// kernels of their own).
+template <int K>
 __device__ __forceinline__ float culled_region32(const DevScene &S, float x, float y, float z)
 {
     const int g = S.cull_g;
@@ -532,7 +542,7 @@ __device__ __forceinline__ float culled_region32(const DevScene &S, float x, flo
     const int c = (cz * g + cy) * g + cx;
     const int o0 = __ldg(S.cull_off + c), o1 = __ldg(S.cull_off + c + 1);
     if (o1 <= o0) return S.cull_rmax;
-    if (S.cull_capsules) {
+    if (K == kTreeScene || S.cull_kind != 0) {
         const bool smooth = S.cull_op == 2;
         const float kinv = S.cull_kinv;
         float acc = base32<false>(2, S.p32 + 2 * __ldg(S.cull_list + o0), x, y, z);
@@ -542,6 +552,7 @@ __device__ __forceinline__ float culled_region32(const DevScene &S, float x, flo
         }
         return fminf(acc, S.cull_rmax);
     }
+    if (K == kTreeScene) return S.cull_rmax;     // not reached
     int i = __ldg(S.cull_list + o0);
     float acc = prim32<false>(S, (*(S.pkind + i)), i, x, y, z);   // culled regions are plain
     for (int j = o0 + 1; j < o1; ++j) {
@@ -573,31 +584,42 @@ __device__ __forceinline__ Eval32 scene_eval32(const DevScene &S, float x, float
     E.dmin = __int_as_float(0x7f800000);
     E.dsoft = E.dmin;
     E.dstar = 0.f; E.istar = -1; E.region = -1;
-    if (K == kBoxScene) {                // one instruction, one box per region
+    if (has_boxes_only<K>()) {           // one instruction, one box per region
+        int cb = -1, ce = 0;
+        if (K == kTreeScene) {
+            const int2 rr = (*(S.rrange + S.cull_region));
+            cb = rr.x;
+            ce = rr.y;
+        }
         for (int i = 0; i < S.ninstr; ++i) {
+            if (K == kTreeScene && i == cb) {
+                region_end32(&E, S.cull_region, culled_region32<K>(S, x, y, z), true);
+                i = ce - 1;
+                continue;
+            }
             const int4 ins = (*(reinterpret_cast<const int4 *>(S.instr) + i));
             region_end32(&E, ins.z, base32<false>(1, S.p32 + 2 * ins.y, x, y, z), false);
         }
     }
     int cb = S.ninstr, ce = S.ninstr;
-    if ((K == kGeneralScene || K == kCulledScene) && S.cull_region >= 0) {
+    if (has_cells<K>() && K != kTreeScene && S.cull_region >= 0) {
         const int2 rr = (*(S.rrange + S.cull_region));
         cb = rr.x;
         ce = rr.y;
     }
     float s0 = 0.f, s1 = 0.f, s2 = 0.f, s3 = 0.f;
-    for (int i = 0; K != kBoxScene && i < S.ninstr; ++i) {
-        if (K != kPlainScene && i == cb) {
+    for (int i = 0; !has_boxes_only<K>() && i < S.ninstr; ++i) {
+        if (has_cells<K>() && i == cb) {
             // the culled region's distance bounds segment moves
             // isotropically (its primitives are not in seg_prims)
-            region_end32(&E, S.cull_region, culled_region32(S, x, y, z), true);
+            region_end32(&E, S.cull_region, culled_region32<K>(S, x, y, z), true);
             i = ce - 1;
             continue;
         }
         const int4 ins = (*(reinterpret_cast<const int4 *>(S.instr) + i));
         const int op = ins.x & 0xff, kind = (ins.x >> 8) & 0xff;
         float v = 0.f;
-        if (ins.y >= 0) v = prim32<K == kGeneralScene>(S, kind, ins.y, x, y, z);
+        if (ins.y >= 0) v = prim32<has_shapes<K>()>(S, kind, ins.y, x, y, z);
         if (op == 0) {
             s3 = s2; s2 = s1; s1 = s0; s0 = v;
         } else {
@@ -686,6 +708,7 @@ __device__ __forceinline__ void csg_grad32(int op, float &a, float &ax, float &a
 // over the cell's candidates, as culled_region32): the gradient of a smooth
 // minimum is the h-weighted blend of its operands' gradients.  Only called
 // within delta of the region's surface, where the fold is below the clamp.
+template <int K>
 __device__ __forceinline__ float grad_culled32(const DevScene &S, float x, float y, float z, float &gx, float &gy,
                                                float &gz)
 {
@@ -700,11 +723,11 @@ __device__ __forceinline__ float grad_culled32(const DevScene &S, float x, float
     const int o0 = __ldg(S.cull_off + c), o1 = __ldg(S.cull_off + c + 1);
     if (o1 <= o0) return S.cull_rmax;
     int i = __ldg(S.cull_list + o0);
-    float acc = prim_grad32(S, (*(S.pkind + i)), i, x, y, z, gx, gy, gz);
+    float acc = prim_grad32(S, K == kTreeScene ? 2 : (*(S.pkind + i)), i, x, y, z, gx, gy, gz);
     for (int j = o0 + 1; j < o1; ++j) {
         i = __ldg(S.cull_list + j);
         float bx, by, bz;
-        const float b = prim_grad32(S, (*(S.pkind + i)), i, x, y, z, bx, by, bz);
+        const float b = prim_grad32(S, K == kTreeScene ? 2 : (*(S.pkind + i)), i, x, y, z, bx, by, bz);
         csg_grad32(S.cull_op, acc, gx, gy, gz, b, bx, by, bz, S.cull_kinv);
     }
     if (!(acc < S.cull_rmax)) { gx = gy = gz = 0.f; return S.cull_rmax; }
@@ -741,8 +764,7 @@ template <int K>
 static __device__ __noinline__ float grad_surface32(const DevScene &S, int r, float x, float y, float z, float &gx,
                                              float &gy, float &gz)
 {
-    if ((K == kGeneralScene || K == kCulledScene) && r >= 0 && r == S.cull_region)
-        return grad_culled32(S, x, y, z, gx, gy, gz);
+    if (has_cells<K>() && r >= 0 && r == S.cull_region) return grad_culled32<K>(S, x, y, z, gx, gy, gz);
     if (r < 0) {
         const float px = x - S.bbc32[0], py = y - S.bbc32[1], pz = z - S.bbc32[2];
         const float qx = fabsf(px) - S.bbh32[0], qy = fabsf(py) - S.bbh32[1], qz = fabsf(pz) - S.bbh32[2];
@@ -753,9 +775,9 @@ static __device__ __noinline__ float grad_surface32(const DevScene &S, int r, fl
         return qz;
     }
     const int2 rr = (*(S.rrange + r));
-    if (K == kBoxScene || rr.y - rr.x == 1) {   // a primitive
+    if (has_boxes_only<K>() || rr.y - rr.x == 1) {   // a primitive
         const int4 ins = (*(reinterpret_cast<const int4 *>(S.instr) + rr.x));
-        return prim_grad32(S, K == kBoxScene ? 1 : (ins.x >> 8) & 0xff, ins.y, x, y, z, gx, gy, gz);
+        return prim_grad32(S, has_boxes_only<K>() ? 1 : (ins.x >> 8) & 0xff, ins.y, x, y, z, gx, gy, gz);
     }
     return grad_program32(S, rr.x, rr.y, x, y, z, gx, gy, gz);
 }
@@ -1309,9 +1331,9 @@ static __device__ __noinline__ float segment_bound32(const DevScene &S, float L,
                     dsoft - dh);
     for (int j = 0; j < S.nseg && t > L; ++j) {
         const int i = __ldg(S.seg_prims + j);
-        const int kind = K == kBoxScene ? 1 : (*(S.pkind + i));
+        const int kind = has_boxes_only<K>() ? 1 : (*(S.pkind + i));
         const float e = __ldg(S.seg_m32 + j) + dh;
-        const float d = prim32<K == kGeneralScene>(S, kind, i, px, py, pz);
+        const float d = prim32<has_shapes<K>()>(S, kind, i, px, py, pz);
         if (!(fabsf(d) > e)) return 0.f;
         if (fabsf(d) - e >= t) continue;
         float b;
@@ -1320,7 +1342,7 @@ static __device__ __noinline__ float segment_bound32(const DevScene &S, float L,
         } else if (kind == 1) {
             const float4 A = (*(S.p32 + 2 * i)), B = (*(S.p32 + 2 * i + 1));
             b = seg_box32(A.x, A.y, A.z, B.x, B.y, B.z, d, px, py, pz, ux, uy, uz, iux, iuy, iuz, e);
-        } else if (K != kGeneralScene || kind == 2) {
+        } else if (!has_shapes<K>() || kind == 2) {
             b = seg_capsule32((*(S.p32 + 2 * i)), (*(S.p32 + 2 * i + 1)), d, px, py, pz, ux, uy, uz, e);
         } else if (kind & kXformFlag) {
             b = seg_xprim32(S, kind & 0xf, i, d, px, py, pz, ux, uy, uz, e);
