@@ -581,7 +581,7 @@ int build_plan(smcrt_ctx *ctx, const smcrt_scene *sc, const smcrt_source *src, c
         for (int i = 0; i < np; ++i) plain = plain && plain_prim(sc->prims[i]);
         H.analytic_nrm = longest <= kAnalyticNormalMaxInstr && plain ? 1 : 0;
     }
-    H.singles = single_regions(ins.data(), (int)ins.size(), nr);
+    H.singles = single_regions(ins.data(), rr.data(), nr);
     // The plain mixed instantiation leaves the six-probe normal out of its
     // loop (smaller loop: 4.6 % on the layered slab); a mixed scene whose
     // normals need the probes runs the general one, whose plain-shape

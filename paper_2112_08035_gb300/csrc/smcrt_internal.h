@@ -188,18 +188,25 @@ struct Instr {
     int32_t pad;
 };
 
-// Whether every region is one sphere, box or capsule in scene coordinates (a
-// compiled program: one instruction per region), or even one box.
-enum : int { kSinglePrims = 1, kSingleBoxes = 2 };
-inline int single_regions(const Instr *ins, int ninstr, int nregions)
+// Scenes of simple regions (a compiled program): every region one box; one
+// sphere, box or capsule; or one box or a left fold of unions and smooth
+// unions of two or more capsules.  All in scene coordinates.
+enum : int { kSinglePrims = 1, kSingleBoxes = 2, kSingleTree = 3 };
+inline int single_regions(const Instr *ins, const int2 *rr, int nregions)
 {
-    bool one = ninstr == nregions && nregions > 0, box = true;
-    for (int i = 0; one && i < ninstr; ++i) {
-        const int kind = (ins[i].op >> 8) & 0xff;
-        one = (ins[i].op & 0xff) == 0 && kind <= SMCRT_CAPSULE;
-        box = box && kind == SMCRT_BOX;
+    bool one = true, box = true, tree = true;
+    for (int r = 0; r < nregions; ++r) {
+        const bool alone = rr[r].y - rr[r].x == 1;
+        for (int i = rr[r].x; i < rr[r].y; ++i) {
+            const int op = ins[i].op & 0xff, kind = (ins[i].op >> 8) & 0xff;
+            one = one && alone && kind <= SMCRT_CAPSULE;
+            box = box && alone && kind == SMCRT_BOX;
+            tree = tree && ins[i].prim >= 0 &&
+                   (alone ? kind == SMCRT_BOX
+                          : kind == SMCRT_CAPSULE && (i == rr[r].x || op == SMCRT_OP_UNION || op == SMCRT_OP_SMOOTH_UNION));
+        }
     }
-    return !one ? 0 : box ? kSingleBoxes : kSinglePrims;
+    return box ? kSingleBoxes : one ? kSinglePrims : tree ? kSingleTree : 0;
 }
 
 // Scene + source + grid of one plan as the kernels read them.  Lives in
@@ -249,7 +256,7 @@ struct DevScene {
     const double *xf64;
     const float4 *xf32;
     int32_t general;          // some primitive is a torus or cylinder or has a frame
-    int32_t singles;          // single_regions: kSingleBoxes, kSinglePrims or 0
+    int32_t singles;          // single_regions
     float h32;                // FP32 central-difference step for normals
     int64_t max_steps;
     // source
@@ -418,7 +425,8 @@ inline int default_variant(int precision, uint64_t npackets, const DevScene &S)
 // kernels leave out what its scenes cannot need:
 //   general        tori, cylinders, frames, long programs (mixed: probe normals)
 //   cell lists     mixed only; with general shapes or without
-//   tree           a cell list of capsules among regions of one box each
+//   tree           a fold of capsules (mixed: a cell list) among regions of one
+//                  box each
 //   boxes          every region one box: no other shape, no CSG interpreter
 //   singles        FP64: every region one sphere, box or capsule
 //   plain          the rest: spheres, boxes and capsules, any CSG
@@ -426,7 +434,7 @@ inline int default_variant(int precision, uint64_t npackets, const DevScene &S)
 // their own: layered slab 1e7 packets 138.2 / 134.4 ms, 1e6 with sphere
 // tracing 30.8 / 28.7, glass container 4e6 59.9 / 58.4; out of the general
 // one: shape gallery 5e5 157 / 147 ms.  Tree: vessel tree 4e6 116 / 96 ms, 1e4
-// 6.4 / 5.8.  Boxes: layered slab 1e7 134.4 / 111.0 ms, 1e4 2.05 / 1.77, with
+// 6.4 / 5.8; FP64 1e4 53.1 / 36.2, 4e4 80.4 / 56.5.  Boxes: layered slab 1e7 134.4 / 111.0 ms, 1e4 2.05 / 1.77, with
 // sphere tracing 1e6 28.8 / 25.1, thick slab 1e6 67.7 / 65.3 (its loop is
 // mostly scattering); FP64 layered slab 1e5 58.9 / 46.2 ms, 1e4 16.4 / 13.4,
 // 1e6 485 / 342, thick slab 3e3 114.6 / 110.9.  Singles: FP64 sphere 1e5, with
@@ -442,7 +450,8 @@ inline int scene_family(int precision, const DevScene &S)
     if (S.general) return cells ? kGeneralCulledScene : kGeneralScene;
     if (cells) return S.cull_kind == kListTree ? kTreeScene : kCulledScene;
     if (S.singles == kSingleBoxes) return kBoxScene;
-    return precision == SMCRT_FP64 && S.singles != 0 ? kSingleScene : kPlainScene;
+    if (precision == SMCRT_MIXED) return kPlainScene;
+    return S.singles == kSinglePrims ? kSingleScene : S.singles == kSingleTree ? kTreeScene : kPlainScene;
 }
 
 // Lanes of a warp that carry packets in a plan launch (JobWork.lanes; 0 =

@@ -587,6 +587,9 @@ cudaError_t launch_fp64(JobWork *jobs, int njobs, int *status, int blocks, int t
     case 12: packets_fp64<4, kSingleScene, false><<<blocks, threads, sm, stream>>>(jobs, njobs, status); break;
     case 13: packets_fp64<3, kSingleScene, false><<<blocks, threads, sm, stream>>>(jobs, njobs, status); break;
     case 14: packets_fp64<2, kSingleScene, false><<<blocks, threads, sm, stream>>>(jobs, njobs, status); break;
+    case 18: packets_fp64<4, kTreeScene, false><<<blocks, threads, sm, stream>>>(jobs, njobs, status); break;
+    case 19: packets_fp64<3, kTreeScene, false><<<blocks, threads, sm, stream>>>(jobs, njobs, status); break;
+    case 20: packets_fp64<2, kTreeScene, false><<<blocks, threads, sm, stream>>>(jobs, njobs, status); break;
     default: packets_fp64<4, kPlainScene, false><<<blocks, threads, sm, stream>>>(jobs, njobs, status); break;
     }
     return cudaGetLastError();
@@ -628,6 +631,9 @@ int occupancy_fp64(int threads, int variant)
     case 12: cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, packets_fp64<4, kSingleScene, false>, threads, sm); break;
     case 13: cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, packets_fp64<3, kSingleScene, false>, threads, sm); break;
     case 14: cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, packets_fp64<2, kSingleScene, false>, threads, sm); break;
+    case 18: cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, packets_fp64<4, kTreeScene, false>, threads, sm); break;
+    case 19: cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, packets_fp64<3, kTreeScene, false>, threads, sm); break;
+    case 20: cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, packets_fp64<2, kTreeScene, false>, threads, sm); break;
     default: cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, packets_fp64<4, kPlainScene, false>, threads, sm); break;
     }
     return n;

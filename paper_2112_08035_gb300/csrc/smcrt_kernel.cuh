@@ -505,7 +505,9 @@ template <int K>
 __device__ __forceinline__ bool scene_runs64(const DevScene &S)
 {
     return K == kGeneralScene ||
-           (!S.general && (K != kBoxScene || S.singles == kSingleBoxes) && (K != kSingleScene || S.singles != 0));
+           (!S.general && (K == kPlainScene || S.singles == (K == kBoxScene    ? kSingleBoxes
+                                                             : K == kTreeScene ? kSingleTree
+                                                                               : kSinglePrims)));
 }
 
 // Full scene evaluation (Sec. 2.3): every region, then the bounding box.

@@ -242,7 +242,7 @@ int build_image(const smcrt_scene *sc, const smcrt_source *src, const smcrt_grid
         if (!plain) longest = kAnalyticNormalMaxInstr + 1;   // probe normals for other shapes and frames
         H.analytic_nrm = longest <= kAnalyticNormalMaxInstr ? 1 : 0;
     }
-    H.singles = single_regions(ins, ni, nr);
+    H.singles = single_regions(ins, rr, nr);
     // probe normals run in the general mixed instantiation (the plain one
     // leaves them out)
     if (precision == SMCRT_MIXED && !H.analytic_nrm) H.general = 1;
