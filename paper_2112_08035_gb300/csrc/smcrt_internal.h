@@ -274,6 +274,8 @@ struct DevScene {
     float feps;               // error bound of an FP32 distance
     float gm32[3];            // error bound of an FP32 position in voxels from an FP64 difference, per axis
     float gr32[3];            // ... from FP32 coordinates
+    float tq[3];              // fixed-point walk: error of a plane's distance times |u|, in units, per axis
+    int32_t tfix;             // ... its unit is 2^-tfix (0: no fixed-point walk)
     int32_t pad2;
     const double *planes;     // fill_planes; null: computed
 };
@@ -300,6 +302,7 @@ inline void fill_screen(DevScene &H, const smcrt_scene *sc, const smcrt_source *
     R = R + 4.0 * sc->delta;
     H.screen_mask = H.fold_mask = H.soft_mask = 0;
     H.feps = 0.f;
+    H.tfix = 0;
     for (int a = 0; a < 3; ++a) H.gm32[a] = H.gr32[a] = INFINITY;
     if (H.general || !(R > 1e-6 && R < 1e12)) return;   // FP32 squares stay in range
     H.feps = (float)(R / 65536.0);
@@ -316,9 +319,14 @@ inline void fill_screen(DevScene &H, const smcrt_scene *sc, const smcrt_source *
         if (fold || smooth <= 8) H.screen_mask |= bit;
         if (region_is_soft(sc, r)) H.soft_mask |= bit;
     }
+    int k;
+    std::frexp(R, &k);                           // R < 2^k: a move is shorter than 4 R <= 2^(k + 2)
+    H.tfix = 58 - k >= 40 ? 58 - k : 0;
     for (int a = 0; a < 3; ++a) {
         const double Rg = std::fmax(R, std::fmax(std::fabs(g->lo[a]), std::fabs(g->hi[a])));
         const double dl = (g->hi[a] - g->lo[a]) / (double)g->n[a];
+        const double span = g->hi[a] - g->lo[a], far = std::fmax(std::fabs(g->lo[a]), std::fabs(g->hi[a]));
+        H.tq[a] = (float)std::ldexp(6.1 * span + 2.1 * far, H.tfix - 53);
         H.gm32[a] = (float)(g->n[a] * (16.0 / 16777216.0));
         H.gr32[a] = (float)((Rg / dl + (double)g->n[a]) * (16.0 / 16777216.0));
     }

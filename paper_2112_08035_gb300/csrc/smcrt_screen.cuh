@@ -607,13 +607,31 @@ static __device__ __noinline__ double segment_bound64_screened(const DevScene &S
 
 // ---------------------------------------------------------------------------
 // Track-length tally: tally64 with the grid clip left out where the segment
-// starts inside the grid, the voxel index taken from FP32 where its fraction
-// is clear of a voxel face, and one plane's quotient taken per voxel crossing
-// (the axis that certainly comes first) in place of three and of a
-// comparison of three.  Positions are in voxels from the grid's corner; the
-// error of one is below DevScene.gr32 = 16 u (R / dl + n), or gm32 = 16 u n
-// from an FP64 difference.  A segment inside one voxel (most of them) takes
-// one FP64 operation, a crossing 12.
+// starts inside the grid, and the voxel index taken from FP32 where its
+// fraction is clear of a voxel face.  Positions are in voxels from the grid's
+// corner; the error of one is below DevScene.gr32 = 16 u (R / dl + n), or gm32
+// = 16 u n from an FP64 difference.  A segment inside one voxel (most of them)
+// takes one FP64 operation.
+//
+// A longer one walks in fixed point.  What a voxel gets is the integer nearest
+// to 2^32 w times a piece's length, so the pieces need no more digits than
+// decide that: distances along the segment are 64-bit integers in units of
+// 2^-tfix, at least 2^-58 of the scene's size, 26 bits below the tally's own
+// unit.  They come from one approximate reciprocal per axis (5 FP64 operations
+// per axis, all told) and are stepped by additions; the reference takes 12 FP64
+// operations per crossing, a rounded quotient each.
+//
+// Error.  With p exact, the reference's quotient fl(fl(plane_k - p) / u), where
+// plane_k = fl(lo + fl(k dl)), and the integer fl(plane_k0 - p) r + (k - k0)
+// fl(dl r), |r u - 1| < 2^-51, differ by less than 2^-53 / |u| times 2 (hi - lo)
+// + 2 max(|lo|, |hi|) (the rounded planes k0 and k) + (hi - lo) + dl (the
+// differences), on the grid's last plane 2 (hi - lo) more (its own face clips
+// the segment there): DevScene.tq, an axis' e; by 2^-50 t for r and the
+// products; and by one unit per addition: slack.  Where an order of planes, a
+// piece's sign or its rounding is closer than the errors, the FP64 walk goes on
+// from the last plane.  Homogeneous sphere 3e4 packets (200^3 grid) 16.9 -> 9.0
+// ms, glass sphere in a beam 3e5 16.8 -> 5.8 ms, vessel tree 1e4 35.2 -> 33.3
+// ms, layered slab 1e6 332 -> 325 ms.
 // ---------------------------------------------------------------------------
 // The rest of a walk of a segment that starts inside the grid, in FP64 (clipped at the grid's far faces).
 static __device__ __noinline__ unsigned walk_rest64(const DevScene &S, long long *flu, double px, double py, double pz,
@@ -625,6 +643,58 @@ static __device__ __noinline__ unsigned walk_rest64(const DevScene &S, long long
     clip64(S.g_lo[1], S.g_hi[1], py, uy, tin, tout);
     clip64(S.g_lo[2], S.g_hi[2], pz, uz, tin, tout);
     return walk64(S, flu, px, py, pz, ux, uy, uz, ix, iy, iz, t, tout, w);
+}
+
+// A number >= 0 in units of 2^-e, rounded down; those from 2^64 units on: 2^62.
+__device__ __forceinline__ unsigned long long fixed64(double x, int e)
+{
+    const unsigned long long b = (unsigned long long)__double_as_longlong(x);
+    const unsigned long long m = (b & 0x000FFFFFFFFFFFFFull) | 0x0010000000000000ull;
+    const int s = (int)(b >> 52) - 1075 + e;
+    return s >= 0 ? s > 11 ? 1ull << 62 : m << s : s < -63 ? 0ull : m >> -s;
+}
+
+// The plane i of one axis.
+__device__ __forceinline__ double grid_plane(const DevScene &S, int a, int i)
+{
+    if (S.planes != nullptr)
+        return __ldg(S.planes + (a == 0 ? 0 : a == 1 ? S.g_n[0] + 1 : S.g_n[0] + S.g_n[1] + 2) + i);
+    return S.g_lo[a] + (double)i * S.g_dl[a];
+}
+
+// One axis of a fixed-point walk: the distance of the plane ahead along the
+// segment, its step from plane to plane, and the error of any of them (see
+// below).  far: the plane lies certainly beyond the end.  False: the error
+// is too large (a direction almost along the planes).
+struct FixAxis {
+    long long t, dt, e;
+};
+
+__device__ __forceinline__ bool fix_axis(const DevScene &S, int a, int &i, double p, double u, bool far, FixAxis &o)
+{
+    o.t = 1ll << 62;
+    o.dt = 0;
+    o.e = 0;
+    if (far || u == 0.0) return true;
+    const float iu = __fdividef(1.f, fabsf((float)u)), e = S.tq[a] * iu * kScrUp;
+    if (!(e < 1e9f) || !(iu > 0.5f)) return false;
+    o.e = (long long)(int)e + 1;
+    // 1 / |u| from the FP32 reciprocal (relative error f below 2^-21): f^3 is
+    // beyond FP64
+    const double ua = fabs(u);
+    const double r0 = __longlong_as_double(((long long)__float_as_int(iu) << 29) + (896ll << 52));
+    const double f = __fma_rn(-ua, r0, 1.0);
+    const double r = __fma_rn(r0, __fma_rn(f, f, f), r0);
+    const unsigned long long most = 1ull << 62;
+    const bool up = __double2hiint(u) >= 0;
+    const double way = grid_plane(S, a, i + up) - p;
+    o.dt = (long long)min(most, fixed64(S.g_dl[a] * r, S.tfix));
+    o.t = (long long)min(most, fixed64(fabs(way) * r, S.tfix));
+    if ((__double_as_longlong(way) << 1) == 0) {     // on the plane: a crossing of no length
+        i += up ? 1 : -1;
+        o.t = o.dt;
+    }
+    return true;
 }
 
 static __device__ __noinline__ unsigned tally64_screened(const DevScene &S, long long *flu, double px, double py,
@@ -643,19 +713,22 @@ static __device__ __noinline__ unsigned tally64_screened(const DevScene &S, long
     const auto within = [&]() {
         return gx > mx && gx < (float)nx - mx && gy > my && gy < (float)ny - my && gz > mz && gz < (float)nz - mz;
     };
-    const auto clear = [](float g, float b, float m) { return fminf(g - b, b + 1.f - g) > 2.f * m; };
-    if (!(within() && clear(gx, bx, mx) && clear(gy, by, my) && clear(gz, bz, mz))) {
-        // both ends beyond one side of the grid: no voxel
+    // both ends beyond one side of the grid: no voxel
+    const auto outside = [&]() {
         const float hx = gx + ax, hy = gy + ay, hz = gz + az;
         const float ex = mx + 1e-6f * (fabsf(gx) + fabsf(ax)), ey = my + 1e-6f * (fabsf(gy) + fabsf(ay)),
                     ez = mz + 1e-6f * (fabsf(gz) + fabsf(az));
-        if (fminf(gx, hx) > (float)nx + ex || fmaxf(gx, hx) < -ex || fminf(gy, hy) > (float)ny + ey ||
-            fmaxf(gy, hy) < -ey || fminf(gz, hz) > (float)nz + ez || fmaxf(gz, hz) < -ez)
-            return 0u;
+        return fminf(gx, hx) > (float)nx + ex || fmaxf(gx, hx) < -ex || fminf(gy, hy) > (float)ny + ey ||
+               fmaxf(gy, hy) < -ey || fminf(gz, hz) > (float)nz + ez || fmaxf(gz, hz) < -ez;
+    };
+    const auto clear = [](float g, float b, float m) { return fminf(g - b, b + 1.f - g) > 2.f * m; };
+    if (!(within() && clear(gx, bx, mx) && clear(gy, by, my) && clear(gz, bz, mz))) {
+        if (outside()) return 0u;
         // FP64 differences, and the index itself where that is not enough
         mx = S.gm32[0]; my = S.gm32[1]; mz = S.gm32[2];
         const double ox = px - S.g_lo[0], oy = py - S.g_lo[1], oz = pz - S.g_lo[2];
         gx = (float)ox * S.g_idl32[0]; gy = (float)oy * S.g_idl32[1]; gz = (float)oz * S.g_idl32[2];
+        if (outside()) return 0u;
         if (!within()) return tally64(S, flu, px, py, pz, ux, uy, uz, len, w);
         bx = floorf(gx); by = floorf(gy); bz = floorf(gz);
         if (!clear(gx, bx, mx)) bx = (float)floor(div64(ox, S.g_dl[0]));
@@ -671,50 +744,75 @@ static __device__ __noinline__ unsigned tally64_screened(const DevScene &S, long
     sz = az > 0.f ? 1.f - sz : uz == 0.0 ? 1e6f : sz;
     const float vx = __fdividef(1.f, fmaxf(fabsf(ax), 1e-30f)), vy = __fdividef(1.f, fmaxf(fabsf(ay), 1e-30f)),
                 vz = __fdividef(1.f, fmaxf(fabsf(az), 1e-30f));
-    double t = 0.0;
+    // where the planes ahead certainly do not lie before, along the segment
+    // (1 = its end)
+    const float lx = (sx - 2.f * mx) * vx * kScrDown, ly = (sy - 2.f * my) * vy * kScrDown,
+                lz = (sz - 2.f * mz) * vz * kScrDown;
+    if (fminf(lx, fminf(ly, lz)) > kScrUp) {                 // all of it in this voxel
+        red_add(flu + ((long long)iz * ny + iy) * nx + ix, fx64(w * len));
+        return 1u;
+    }
+    // the walk in fixed point
+    FixAxis X, Y, Z;
+    bool ok = S.tfix != 0 && w <= 1.0;
+    ok = ok && fix_axis(S, 0, ix, px, ux, lx > kScrUp, X);
+    ok = ok && fix_axis(S, 1, iy, py, uy, ly > kScrUp, Y);
+    ok = ok && fix_axis(S, 2, iz, pz, uz, lz > kScrUp, Z);
+    if (!ok) return walk_rest64(S, flu, px, py, pz, ux, uy, uz, (int)bx, (int)by, (int)bz, 0.0, len, w);
+    if ((unsigned)ix >= (unsigned)nx || (unsigned)iy >= (unsigned)ny || (unsigned)iz >= (unsigned)nz) return 0u;
+    const int shift = S.tfix - 33;
+    const unsigned long long half = 1ull << (shift - 1);
+    const unsigned long long wf = fixed64(w, 63);
+    const long long tl = (long long)min(1ull << 60, fixed64(len, S.tfix));
+    long long slack = (tl >> 49) + 16;
+    long long *at = flu + ((long long)iz * ny + iy) * nx + ix;
+    const long long row = nx, sheet = (long long)nx * ny;
+    long long t = 0, et = 0;
+    int last = -1;                           // the axis of the plane at t
     unsigned npieces = 0u;
     for (;;) {
-        // where the planes ahead lie along the segment (1 = its end)
-        const float lx = (sx - 2.f * mx) * vx * kScrDown, ly = (sy - 2.f * my) * vy * kScrDown,
-                    lz = (sz - 2.f * mz) * vz * kScrDown;
-        const bool ends = fminf(lx, fminf(ly, lz)) > kScrUp;  // in this voxel
-        const float ox = (sx + 2.f * mx) * vx * kScrUp, oy = (sy + 2.f * my) * vy * kScrUp,
-                    oz = (sz + 2.f * mz) * vz * kScrUp;
-        const bool cx = ox < fminf(ly, lz), cy = oy < fminf(lx, lz), cz = oz < fminf(lx, ly);
-        if (!ends && (!(cx || cy || cz) || !(fminf(ox, fminf(oy, oz)) < kScrDown)))   // a tie, for FP32
-            return npieces + walk_rest64(S, flu, px, py, pz, ux, uy, uz, ix, iy, iz, t, len, w);
-        const bool up = (cx ? ax : cy ? ay : az) > 0.f;
-        const int i = cx ? ix : cy ? iy : iz, n = cx ? nx : cy ? ny : nz;
-        const bool leaves = !ends && (up ? i + 1 >= n : i == 0);
-        double tend = len;
-        if (!ends) {
-            const double p = cx ? px : cy ? py : pz, u = cx ? ux : cy ? uy : uz;
-            double plane;
-            if (S.planes != nullptr) {
-                plane = __ldg(S.planes + (cx ? 0 : cy ? nx + 1 : nx + ny + 2) + i + up);
-            } else {
-                const double lo = cx ? S.g_lo[0] : cy ? S.g_lo[1] : S.g_lo[2];
-                const double dl = cx ? S.g_dl[0] : cy ? S.g_dl[1] : S.g_dl[2];
-                plane = lo + (double)(i + up) * dl;
+        const bool cx = X.t <= Y.t && X.t <= Z.t, cy = !cx && Y.t <= Z.t;
+        const long long tn = cx ? X.t : cy ? Y.t : Z.t, en = (cx ? X.e : cy ? Y.e : Z.e) + slack;
+        const long long o1 = cx ? Y.t - Y.e : X.t - X.e, o2 = cx || cy ? Z.t - Z.e : Y.t - Y.e;
+        const long long other = min(o1, o2);
+        const bool ends = min(tn - en, other) > tl + slack;
+        const long long p = (ends ? tl : tn) - t, err = et + (ends ? 0 : en) + slack;
+        const unsigned long long v = __umul64hi(wf, (unsigned long long)p) + half;
+        const long long ev = (long long)__umul64hi(wf, (unsigned long long)err) + 16;
+        const long long frac = (long long)(v & (2ull * half - 1ull));
+        if (!((ends || (tn + en < other && tn + en < tl)) && p > err && frac > ev &&
+              frac + ev < (long long)(2ull * half))) {
+            // too close to call: FP64 from the plane at t on
+            double te = 0.0;
+            if (last >= 0) {
+                const int i = last == 0 ? ix : last == 1 ? iy : iz;
+                const double u = last == 0 ? ux : last == 1 ? uy : uz, q = last == 0 ? px : last == 1 ? py : pz;
+                te = div64(grid_plane(S, last, u > 0.0 ? i : i + 1) - q, u);
             }
-            tend = div64(plane - p, u);
-            if (leaves) {                        // the grid's own face clips the segment
-                const double face = up ? (cx ? S.g_hi[0] : cy ? S.g_hi[1] : S.g_hi[2])
-                                       : (cx ? S.g_lo[0] : cy ? S.g_lo[1] : S.g_lo[2]);
-                tend = min64(tend, div64(face - p, u));
-            }
+            return npieces + walk_rest64(S, flu, px, py, pz, ux, uy, uz, ix, iy, iz, te, len, w);
         }
-        const double piece = tend - t;
-        if (piece > 0.0) {
-            red_add(flu + ((long long)iz * ny + iy) * nx + ix, fx64(w * piece));
-            npieces += 1u;
-            t = tend;
+        red_add(at, (long long)(v >> shift));
+        npieces += 1u;
+        if (ends) return npieces;
+        t = tn;
+        et = en;
+        slack += 2;
+        if (cx) {
+            last = 0;
+            X.t += X.dt;
+            if (ux > 0.0 ? ++ix >= nx : --ix < 0) return npieces;
+            at += ux > 0.0 ? 1 : -1;
+        } else if (cy) {
+            last = 1;
+            Y.t += Y.dt;
+            if (uy > 0.0 ? ++iy >= ny : --iy < 0) return npieces;
+            at += uy > 0.0 ? row : -row;
+        } else {
+            last = 2;
+            Z.t += Z.dt;
+            if (uz > 0.0 ? ++iz >= nz : --iz < 0) return npieces;
+            at += uz > 0.0 ? sheet : -sheet;
         }
-        if (ends || leaves) return npieces;
-        const int s = up ? 1 : -1;
-        if (cx) { ix += s; sx += 1.f; }
-        else if (cy) { iy += s; sy += 1.f; }
-        else { iz += s; sz += 1.f; }
     }
 }
 
