@@ -343,7 +343,7 @@ __device__ bool run_job_fp64(const DevScene &S, WarpAcc *wa, const volatile JobC
                         interact = mu_t > 0.0 && tau < mu_t * L;
                         if (!interact && S.stepping == SMCRT_STEP_SEGMENT) {   // a longer move along u
                             if (K == kGeneralScene) L = fmax(L, segment_bound64<true>(S, E.dsoft, E.dbox, px, py, pz, ux, uy, uz));
-                            else L = max64(L, segment_bound64_screened<K>(S, E.dsoft, E.dbox, px, py, pz, ux, uy, uz));
+                            else L = max64(L, segment_bound64_screened<K>(S, E, C, px, py, pz, ux, uy, uz));
                             interact = mu_t > 0.0 && tau < mu_t * L;
                         }
                     }

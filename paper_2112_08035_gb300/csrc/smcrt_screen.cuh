@@ -263,11 +263,11 @@ static __device__ __noinline__ Screen64 scene_screen(const DevScene &S, float x,
         }
         if (in) {
             C.mask |= bit;
-            if (!one_each<K>() && (S.fold_mask & bit) && (mode == kForTrace || flr < 0)) {
-                C.flr = r;
-                C.list = li;
-                C.cnt = min(n, kFoldList + 1);
-            }
+        }
+        if (!one_each<K>() && (S.fold_mask & bit) && (mode == kForTrace ? in || C.flr < 0 : in && flr < 0)) {
+            C.flr = r;
+            C.list = li;
+            C.cnt = min(n, kFoldList + 1);
         }
     }
     C.soft = soft;
@@ -502,69 +502,119 @@ static __device__ __noinline__ float segment_screen(const DevScene &S, float sof
     return t;
 }
 
-// seg_box64 of the box P (centre, half extents), with the quotients of the
+// A packet's ray in FP32.
+struct Ray32 {
+    float p[3], u[3], iu[3];                 // iu: 1 / |u|
+};
+
+// seg_box64 of the box P (centre, half extents; FP32: c, h), with the quotients of the
 // axes that FP32 shows to count.  The reference takes an axis' smaller and
 // larger quotient, which are those of the plane behind and ahead (rounding
 // is monotone): from inside, the bound is the first plane ahead; from
 // outside, the last plane behind, if it certainly lies before the first one
 // ahead and ahead of the packet.
-static __device__ __noinline__ double seg_face64(const double *P, double d, double px, double py, double pz,
-                                                 double ux, double uy, double uz, double e, float eps)
+static __device__ __noinline__ double seg_face64(const double *P, const Ray32 &r, const float *c, const float *h,
+                                                 bool inside, double px, double py, double pz, double ux, double uy,
+                                                 double uz, double e, float ef, float eps)
 {
-    const double c[3] = {P[0], P[1], P[2]}, h[3] = {P[3], P[4], P[5]}, p[3] = {px, py, pz}, u[3] = {ux, uy, uz};
-    const bool inside = !(d > 0.0);
-    const double eo = inside ? -e : e;
     const float inf = __int_as_float(0x7f800000);
-    float at[3], lo[3], hi[3];               // the face that counts: bounds of its distance
+    float lo[3], hi[3];                      // bounds of the distance of the face that counts
     float ahead = inf, behind = -inf, last = -inf;
     bool odd = false;                        // a direction component of zero, a box thinner than 2 e
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
-        const float uf = (float)u[a], g = (float)h[a] + (float)eo;
-        const float q = uf > 0.f ? (float)p[a] - (float)c[a] : (float)c[a] - (float)p[a];
-        odd = odd || uf == 0.f || !(g > eps);
-        const float iu = __fdividef(1.f, fabsf(uf));
-        at[a] = (inside ? g : -g) - q;
-        const float x = (at[a] - eps) * iu, y = (at[a] + eps) * iu;
+        const float g = inside ? h[a] - ef : h[a] + ef;
+        const float q = r.u[a] > 0.f ? r.p[a] - c[a] : c[a] - r.p[a];
+        odd = odd || r.u[a] == 0.f || !(g > eps);
+        const float at = (inside ? g : -g) - q;
+        const float x = (at - eps) * r.iu[a], y = (at + eps) * r.iu[a];
         lo[a] = x - 1e-5f * fabsf(x); hi[a] = y + 1e-5f * fabsf(y);
-        ahead = fminf(ahead, inside ? hi[a] : (g - q - eps) * iu * kScrDown);
+        ahead = fminf(ahead, inside ? hi[a] : (g - q - eps) * r.iu[a] * kScrDown);
         behind = fmaxf(behind, lo[a]);
         last = fmaxf(last, hi[a]);
     }
     // from outside: certainly hit (the last plane behind before the first ahead) and ahead
     if (eps == 0.f || odd || !(fabsf(ahead) < 1e30f) || (!inside && !(behind > 0.f && last < ahead)))
-        return seg_box64(P[0], P[1], P[2], P[3], P[4], P[5], d, px, py, pz, ux, uy, uz, e);
+        return seg_box64(P[0], P[1], P[2], P[3], P[4], P[5], inside ? -1.0 : 1.0, px, py, pz, ux, uy, uz, e);
     double t = __longlong_as_double(inside ? 0x7ff0000000000000LL : (long long)0xfff0000000000000ULL);
-#pragma unroll
+#pragma unroll 1
     for (int a = 0; a < 3; ++a) {
-        if (inside ? lo[a] > ahead : hi[a] < behind) continue;
-        const double he = h[a] + eo;
-        const bool plus = (u[a] > 0.0) == inside;
-        const double x = div64((plus ? c[a] + he : c[a] - he) - p[a], u[a]);
+        if (a == 0 ? (inside ? lo[0] > ahead : hi[0] < behind)
+                   : a == 1 ? (inside ? lo[1] > ahead : hi[1] < behind) : (inside ? lo[2] > ahead : hi[2] < behind))
+            continue;
+        const double p = a == 0 ? px : a == 1 ? py : pz, u = a == 0 ? ux : a == 1 ? uy : uz;
+        const double he = inside ? P[3 + a] - e : P[3 + a] + e;
+        const bool plus = (__double2hiint(u) >= 0) == inside;
+        const double x = div64((plus ? P[a] + he : P[a] - he) - p, u);
         t = inside ? min64(t, x) : max64(t, x);
     }
-    return t > 0.0 ? t : 0.0;
+    return __double2hiint(t) >= 0 ? t : 0.0;
 }
 
-// The move bound of segment_bound64, leaving out what cannot lower it.
+// An upper bound of the exit from a box certainly around p (else inf).
+__device__ __forceinline__ float scr_exit_most(const Ray32 &r, const float *c, const float *h, float e, float eps)
+{
+    float t = __int_as_float(0x7f800000);
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        const float q = r.u[a] > 0.f ? r.p[a] - c[a] : c[a] - r.p[a];
+        if (!(fabsf(q) + e + eps < h[a])) return __int_as_float(0x7f800000);
+        if (r.u[a] != 0.f) t = fminf(t, (h[a] - q + eps) * r.iu[a] * kScrUp);
+    }
+    return t;
+}
+
+// The move bound of segment_bound64, leaving out what cannot lower it: first
+// an FP32 upper bound of the result (cap), then, in the reference's order, the
+// surfaces that FP32 does not show to lie beyond it or beyond the smallest so
+// far.  E and C: the evaluation at p and its screening, which know the nearest
+// surface's distance and a fold's list.  A call took 26000 to 43000 cycles
+// (layered slab, vessel tree), most of it for surfaces that did not count, for
+// conversions of FP64 tables that FP32 copies exist of (64 cycles each, as any
+// FP64 operation), and for the tree's fold a second time: vessel tree 1e4
+// packets 33.9 -> 26.2 ms, 4e4 51.4 -> 39.0, layered slab 1e5 44.7 -> 42.5.
 template <int K>
-static __device__ __noinline__ double segment_bound64_screened(const DevScene &S, double soft, double dbox, double px,
-                                                               double py, double pz, double ux, double uy, double uz)
+static __device__ __noinline__ double segment_bound64_screened(const DevScene &S, const Eval64 &E, const Screen64 &C,
+                                                               double px, double py, double pz, double ux, double uy,
+                                                               double uz)
 {
     const float eps = S.feps;
-    const float p[3] = {(float)px, (float)py, (float)pz}, u[3] = {(float)ux, (float)uy, (float)uz};
+    Ray32 r;
+    r.p[0] = (float)px; r.p[1] = (float)py; r.p[2] = (float)pz;
+    r.u[0] = (float)ux; r.u[1] = (float)uy; r.u[2] = (float)uz;
+    for (int a = 0; a < 3; ++a) r.iu[a] = __fdividef(1.f, fabsf(r.u[a]));
+    const float *const p = r.p, *const u = r.u;
     const double dh = 0.5 * S.delta;
+    const float dhf = (float)dh;
     static_assert(offsetof(DevScene, bbh) == offsetof(DevScene, bbc) + 3 * sizeof(double), "centre, half extents");
     const double *box = reinterpret_cast<const double *>(reinterpret_cast<const char *>(&S) + offsetof(DevScene, bbc));
-    double t = seg_face64(box, dbox, px, py, pz, ux, uy, uz, dh, eps);
-    if (!one_each<K>() && S.soft_mask != 0ull && soft - dh <= t) {
+    float cap = __int_as_float(0x7f800000);
+    if (eps > 0.f) {
+        cap = scr_exit_most(r, S.bbc32, S.bbh32, dhf * kScrUp, eps);
+        for (int j = 0; j < S.nseg; ++j) {
+            const int i = __ldg(S.seg_prims + j);
+            if (K != kBoxScene && __ldg(S.pkind + i) != 1) continue;
+            const float4 A = __ldg(S.p32 + 2 * i), B = __ldg(S.p32 + 2 * i + 1);
+            const float c[3] = {A.x, A.y, A.z}, h[3] = {B.x, B.y, B.z};
+            cap = fminf(cap, scr_exit_most(r, c, h, __ldg(S.seg_m32 + j) * kScrUp + dhf * kScrUp, eps));
+        }
+        cap *= kScrUp;
+    }
+    double t = __longlong_as_double(0x7ff0000000000000LL);
+    if (!(eps > 0.f && scr_box_exit(S.bbc32, S.bbh32, dhf * kScrUp, p, u, eps) > cap))
+        t = seg_face64(box, r, S.bbc32, S.bbh32, true, px, py, pz, ux, uy, uz, dh, dhf, eps);
+    if (!one_each<K>() && S.soft_mask != 0ull && !(C.soft - dhf * kScrUp > fminf(cap, (float)t * kScrUp))) {
         double ds = __longlong_as_double(0x7ff0000000000000LL);
         for (unsigned long long m = S.soft_mask; m != 0ull; m &= m - 1ull) {
-            const int r = __ffsll((long long)m) - 1;
-            unsigned long long list = 0ull;
-            int cnt;
-            fold_list<K>(S, r, px, py, pz, 0.f, list, cnt);
-            ds = min64(ds, fabs(region_exact<K>(S, r, px, py, pz, list, cnt)));
+            const int k = __ffsll((long long)m) - 1;
+            double d = E.dmin;                   // the nearest surface's is known
+            if (k != E.istar) {
+                unsigned long long list = C.list;
+                int cnt = C.cnt;
+                if (k != C.flr) fold_list<K>(S, k, px, py, pz, 0.f, list, cnt);
+                d = fabs(region_exact<K>(S, k, px, py, pz, list, cnt));
+            }
+            ds = min64(ds, d);
         }
         t = min64(t, ds - dh);
     }
@@ -572,7 +622,7 @@ static __device__ __noinline__ double segment_bound64_screened(const DevScene &S
         const int i = __ldg(S.seg_prims + j);
         const int kind = K == kBoxScene ? 1 : __ldg(S.pkind + i);
         const double e = __ldg(S.seg_m64 + j) + dh;
-        const float ef = (float)e * kScrUp, tu = (float)t * kScrUp;
+        const float e32 = __ldg(S.seg_m32 + j) + dhf, ef = e32 * kScrUp, tu = fminf((float)t * kScrUp, cap);
         const float df = scr_prim(S, kind, i, p[0], p[1], p[2]);
         const float iso = fabsf(df) - eps - ef;
         const float4 A = __ldg(S.p32 + 2 * i), B = __ldg(S.p32 + 2 * i + 1);
@@ -597,7 +647,7 @@ static __device__ __noinline__ double segment_bound64_screened(const DevScene &S
         if (kind == 0)
             b = seg_sphere64(P, d, px, py, pz, ux, uy, uz, e);
         else if (kind == 1)
-            b = seg_face64(P, d, px, py, pz, ux, uy, uz, e, eps);
+            b = seg_face64(P, r, c, h, !(d > 0.0), px, py, pz, ux, uy, uz, e, e32, eps);
         else
             b = seg_capsule64(P, d, px, py, pz, ux, uy, uz, e);
         t = min64(t, b);
