@@ -403,10 +403,11 @@ int occupancy_mixed_multi(int threads, int variant = 0);
 // autotuner chose a shape, one block of 128 threads per SM with the largest
 // register budget (variant 2): one warp per scheduler nearly fills the FP64
 // pipe, and four warps disturb one another's instruction fetch less than
-// twelve.  Measured, 1 x 128 against 3 x 128: layered slab 1e4 packets 17.0
-// / 24.7 ms, 1e5 61 / 73 ms, 1e6 501 / 522 ms; glass container 3e4 49 / 58
-// ms, 5e5 237 / 232 ms; sphere 1e5, sphere tracing, 77 / 80 ms, 1e6 324 /
-// 285 ms.
+// twelve.  Measured, 1 x 128 against 3 x 128: layered slab 1e4 packets 13.3
+// / 17.6 ms, 1e5 42.6 / 45.1; vessel tree 1e4 25.7 / 34.0; glass container
+// 3e4 48.6 / 58.3; thick slab 3e3 109.9 / 117.0; sphere 1e5, sphere tracing,
+// 65.4 / 62.2 ms.  From the limit on the wider launch won (before the scene
+// families: glass container 5e5 237 / 232 ms, sphere 1e6 324 / 285).
 constexpr uint64_t kFewFp64Packets = 1u << 19;
 constexpr int kFewFp64Variant = 2;
 
@@ -414,10 +415,12 @@ constexpr int kFewFp64Variant = 2;
 // (variant 1) unless the caller or the autotuner chose a shape, and 5 blocks
 // with 96 registers (variant 0) from this many packets on in scenes without
 // general shapes or a cell list.  Measured, variant 0 / 1: layered slab 1e5
-// packets 3.97 / 3.70 ms, 5e5 9.86 / 9.58, 1e6 17.01 / 17.08, 2e6 31.3 /
-// 31.7; glass container 5e5 16.95 / 16.18 ms, 1e6 23.7 / 23.4; thick slab 1e5
-// 30.0 / 26.7 ms, 1e6 70.6 / 72.2; vessel tree 4e6 135 / 130 ms; shape
-// gallery 5e5 165 / 158 ms.
+// packets 3.22 / 3.03 ms, 5e5 7.36 / 7.83, 1e6 12.9 / 14.0, 1e7 111 / 124;
+// with sphere tracing 4e5 15.0 / 14.7, 1e6 25.3 / 25.6; glass container 5e5
+// 15.4 / 15.0, 1e6 21.4 / 21.6; thick slab 1e5 27.3 / 24.2, 4e5 37.6 / 35.3,
+// 1e6 65.7 / 66.5; vessel tree 1e5 21.1 / 19.7, 4e6 98 / 96 ms; shape gallery
+// 1e4 16.9 / 17.1, 5e5 126 / 126.  (Layered slabs alone would cross over at
+// 2e5; thick ones and sphere tracing near 1e6.)
 constexpr uint64_t kManyMixedPackets = 3u << 18;
 
 // Variant of a plan launch whose shape nobody chose.
