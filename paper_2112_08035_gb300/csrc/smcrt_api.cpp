@@ -883,8 +883,7 @@ void scheduler(smcrt_ctx *ctx)
         JobWork *h_tab = nullptr, *d_tab = nullptr;   // [2 * kMaxSlots]: mixed table, then FP64 table
         smcrt_totals *h_tot = nullptr;                // totals snapshot taken at the end of the round
         int32_t *h_stat = nullptr;                    // [1 + kMaxSlots]: the round's status, then each slot's
-        cudaGraphExec_t graph = nullptr;     // plain scenes only
-        cudaGraphExec_t graph_g = nullptr;   // kernels for scenes with general shapes
+        cudaGraphExec_t graph[3] = {};       // by served_family
         cudaEvent_t ev = nullptr, ev0 = nullptr;
         bool busy = false;
         int64_t idx = -1;
@@ -910,8 +909,7 @@ void scheduler(smcrt_ctx *ctx)
     auto capture = [&]() -> int {
         for (int bi = 0; bi < kRoundsInFlight; ++bi) {
             Buf &b = buf[bi];
-            for (int gen = 0; gen < 2; ++gen) {
-                const int off = gen ? kNumVariants : 0;
+            for (int family = 0; family < 3; ++family) {
                 cudaGraph_t g;
                 if (cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal) != cudaSuccess) return SMCRT_ERR_CUDA;
                 cudaMemsetAsync(d_status + bi, 0, sizeof(int), st);
@@ -919,15 +917,17 @@ void scheduler(smcrt_ctx *ctx)
                 launch_round_prologue(b.d_tab, 2 * kMaxSlots, st);
                 cudaEventRecord(ev_fork, st);
                 cudaStreamWaitEvent(st2, ev_fork, 0);
-                launch_mixed_multi(b.d_tab, kMaxSlots, d_status + bi, blocks_m, threads_m, st, variant_m + off);
-                launch_fp64_served(b.d_tab + kMaxSlots, kMaxSlots, d_status + bi, blocks_d, threads_d, st2, gen != 0);
+                launch_mixed_multi(b.d_tab, kMaxSlots, d_status + bi, blocks_m, threads_m, st,
+                                   variant_m + kNumVariants * family);
+                launch_fp64_served(b.d_tab + kMaxSlots, kMaxSlots, d_status + bi, blocks_d, threads_d, st2,
+                                   family == kGeneralScene);
                 cudaEventRecord(ev_join, st2);
                 cudaStreamWaitEvent(st, ev_join, 0);
                 cudaMemcpyAsync(b.h_tot, d_tot, sizeof(smcrt_totals) * kMaxSlots, cudaMemcpyDeviceToHost, st);
                 cudaMemcpyAsync(b.h_stat, d_status + bi, sizeof(int32_t), cudaMemcpyDeviceToHost, st);
                 cudaMemcpyAsync(b.h_stat + 1, d_jstat, sizeof(int32_t) * kMaxSlots, cudaMemcpyDeviceToHost, st);
                 if (cudaStreamEndCapture(st, &g) != cudaSuccess) return SMCRT_ERR_CUDA;
-                cudaGraphExec_t &ge = gen ? b.graph_g : b.graph;
+                cudaGraphExec_t &ge = b.graph[family];
                 if (ge) cudaGraphExecDestroy(ge);
                 ge = nullptr;
                 const cudaError_t e = cudaGraphInstantiate(&ge, g, 0);
@@ -956,7 +956,7 @@ void scheduler(smcrt_ctx *ctx)
                   cudaMallocAsync(&tab, sizeof(JobWork), st) == cudaSuccess &&
                   cudaMallocAsync(&tst, sizeof(int), st) == cudaSuccess &&
                   cudaEventCreate(&e0) == cudaSuccess && cudaEventCreate(&e1) == cudaSuccess;
-        const int off = j.plan->host.general ? kNumVariants : 0;
+        const int off = kNumVariants * served_family(j.plan->host.general, j.plan->host.cull_region >= 0);
         float best = 1e30f;
         for (int v = 0; ok && v < 2; ++v) {
             for (int t : {64, 128}) {
@@ -1208,9 +1208,10 @@ void scheduler(smcrt_ctx *ctx)
         const long long budget = nfresh == 0 && !waiting ? tail_cycles : park_cycles;
         const double share = round_cycles() / (double)std::max(1, nfresh);
         int nm = 0, nd = 0;
-        bool general = false;
+        bool general = false, cells = false;
         for (auto &j : runnable) {
             general = general || j->plan->host.general;
+            cells = cells || j->plan->host.cull_region >= 0;
             const double c = j->cost > 0 ? j->cost : dflt;
             uint64_t q = (uint64_t)std::max(2048.0, share / c);
             if (!(j->cost > 0)) q = std::min<uint64_t>(q, 16384);   // unmeasured: a short first quantum
@@ -1244,7 +1245,7 @@ void scheduler(smcrt_ctx *ctx)
         for (int k = 0; k < nd; ++k) B.quanta += B.h_tab[kMaxSlots + k].end - B.h_tab[kMaxSlots + k].next;
         B.t_launch = now_s();
         cudaEventRecord(B.ev0, st);
-        cudaGraphLaunch(general ? B.graph_g : B.graph, st);
+        cudaGraphLaunch(B.graph[served_family(general, cells)], st);
         cudaEventRecord(B.ev, st);
         B.busy = true;
         B.idx = issued++;
@@ -1278,8 +1279,8 @@ void scheduler(smcrt_ctx *ctx)
     }
     if (st) cudaStreamSynchronize(st);
     for (auto &b : buf) {
-        if (b.graph) cudaGraphExecDestroy(b.graph);
-        if (b.graph_g) cudaGraphExecDestroy(b.graph_g);
+        for (cudaGraphExec_t g : b.graph)
+            if (g) cudaGraphExecDestroy(g);
         if (b.ev) cudaEventDestroy(b.ev);
         if (b.ev0) cudaEventDestroy(b.ev0);
         if (b.h_tab) cudaFreeHost(b.h_tab);

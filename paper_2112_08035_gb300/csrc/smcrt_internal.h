@@ -394,8 +394,7 @@ int occupancy_fp64_served(int threads);
 int occupancy_mixed(int threads, int variant = 0);
 // Served rounds' mixed kernel, whose warps hold two jobs at a time (lanes
 // refill from the next job instead of draining each): variant 0 / 1 = 5 / 4
-// resident blocks of 128 threads, for scenes with and without a cell list,
-// + kNumVariants for general shapes.
+// resident blocks of 128 threads, + kNumVariants * served_family.
 cudaError_t launch_mixed_multi(JobWork *jobs, int njobs, int *status, int blocks, int threads,
                                cudaStream_t stream, int variant = 0);
 int occupancy_mixed_multi(int threads, int variant = 0);
@@ -451,7 +450,7 @@ inline int default_variant(int precision, uint64_t npackets, const DevScene &S)
 // 1e6 485 / 342, thick slab 3e3 114.6 / 110.9.  Singles: FP64 sphere 1e5, with
 // sphere tracing, 73.7 / 64.0 ms, segments 13.1 / 11.2; in mixed precision
 // nothing (homogeneous sphere 2e6 24.8 / 25.2).  Served rounds hold scenes of
-// all kinds and have two families, general with cell lists and plain with.
+// several kinds and have three families (served_family).
 enum : int { kPlainScene = 0, kGeneralScene = 1, kCulledScene = 2, kBoxScene = 3, kSingleScene = 4,
              kGeneralCulledScene = 5, kTreeScene = 6 };
 enum : int { kListCapsules = 1, kListTree = 2 };   // DevScene.cull_kind
@@ -463,6 +462,13 @@ inline int scene_family(int precision, const DevScene &S)
     if (S.singles == kSingleBoxes) return kBoxScene;
     if (precision == SMCRT_MIXED) return kPlainScene;
     return S.singles == kSinglePrims ? kSingleScene : S.singles == kSingleTree ? kTreeScene : kPlainScene;
+}
+
+// Families of the served rounds' kernels, of which a round takes the one that
+// runs all its scenes: plain, plain with cell lists, general with cell lists.
+inline int served_family(bool general, bool cells)
+{
+    return general ? kGeneralScene : cells ? kCulledScene : kPlainScene;
 }
 
 // Lanes of a warp that carry packets in a plan launch (JobWork.lanes; 0 =

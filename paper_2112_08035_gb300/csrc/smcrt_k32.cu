@@ -1113,17 +1113,19 @@ cudaError_t launch_mixed(JobWork *jobs, int njobs, int *status, int blocks, int 
     return cudaGetLastError();
 }
 
-// The served kernel: variant 0 / 1 = 5 / 4 resident blocks, plain shapes,
-// with or without a cell list; 3 / 4 = the same for general shapes (the index space of launch_mixed).
+// The served kernel: variant 0 / 1 = 5 / 4 resident blocks, plain shapes;
+// 6 / 7 = with cell lists as well; 3 / 4 = the same for general shapes (the index space of launch_mixed).
 cudaError_t launch_mixed_multi(JobWork *jobs, int njobs, int *status, int blocks, int threads, cudaStream_t stream,
                                int variant)
 {
     const size_t sm = (size_t)(threads / 32) * sizeof(WarpSharedMulti);
     switch (variant) {
-    case 1: packets_mixed_multi<4, kCulledScene><<<blocks, threads, sm, stream>>>(jobs, njobs, status); break;
+    case 1: packets_mixed_multi<4, kPlainScene><<<blocks, threads, sm, stream>>>(jobs, njobs, status); break;
+    case 6: packets_mixed_multi<5, kCulledScene><<<blocks, threads, sm, stream>>>(jobs, njobs, status); break;
+    case 7: packets_mixed_multi<4, kCulledScene><<<blocks, threads, sm, stream>>>(jobs, njobs, status); break;
     case 3: packets_mixed_multi<5, kGeneralCulledScene><<<blocks, threads, sm, stream>>>(jobs, njobs, status); break;
     case 4: packets_mixed_multi<4, kGeneralCulledScene><<<blocks, threads, sm, stream>>>(jobs, njobs, status); break;
-    default: packets_mixed_multi<5, kCulledScene><<<blocks, threads, sm, stream>>>(jobs, njobs, status); break;
+    default: packets_mixed_multi<5, kPlainScene><<<blocks, threads, sm, stream>>>(jobs, njobs, status); break;
     }
     return cudaGetLastError();
 }
@@ -1133,10 +1135,12 @@ int occupancy_mixed_multi(int threads, int variant)
     int n = 0;
     const size_t sm = (size_t)(threads / 32) * sizeof(WarpSharedMulti);
     switch (variant) {
-    case 1: cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, packets_mixed_multi<4, kCulledScene>, threads, sm); break;
+    case 1: cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, packets_mixed_multi<4, kPlainScene>, threads, sm); break;
+    case 6: cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, packets_mixed_multi<5, kCulledScene>, threads, sm); break;
+    case 7: cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, packets_mixed_multi<4, kCulledScene>, threads, sm); break;
     case 3: cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, packets_mixed_multi<5, kGeneralCulledScene>, threads, sm); break;
     case 4: cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, packets_mixed_multi<4, kGeneralCulledScene>, threads, sm); break;
-    default: cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, packets_mixed_multi<5, kCulledScene>, threads, sm); break;
+    default: cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, packets_mixed_multi<5, kPlainScene>, threads, sm); break;
     }
     return n;
 }
