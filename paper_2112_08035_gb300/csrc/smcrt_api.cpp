@@ -546,6 +546,7 @@ int build_plan(smcrt_ctx *ctx, const smcrt_scene *sc, const smcrt_source *src, c
     H.delta = sc->delta;
     H.ambient_n = sc->ambient_n;
     H.ambient_n32 = (float)sc->ambient_n;
+    H.matched = matched_regions(sc);
     H.cull_region = cg.region;
     H.cull_g = cg.g;
     H.cull_op = cg.op;

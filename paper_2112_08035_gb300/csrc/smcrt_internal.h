@@ -276,7 +276,7 @@ struct DevScene {
     float gr32[3];            // ... from FP32 coordinates
     float tq[3];              // fixed-point walk: error of a plane's distance times |u|, in units, per axis
     int32_t tfix;             // ... its unit is 2^-tfix (0: no fixed-point walk)
-    int32_t pad2;
+    int32_t matched;          // every region has the ambient index (default_variant)
     const double *planes;     // fill_planes; null: computed
 };
 
@@ -423,14 +423,25 @@ constexpr int kFewFp64Variant = 2;
 // variants 0 / 1 / 2, 3e4 26.8 / 25.4 / 23.9, 5e5 126 / 127 / 122, 1e6 172 /
 // 178 / 171, with sphere tracing 5e5 316 / 312 / 300.  (Layered slabs alone would cross over at
 // 2e5; thick ones and sphere tracing near 1e6.)
+//
+// Scenes without an index step, whose packets meet no Fresnel surface, cross
+// over earlier: homogeneous sphere (isotropic, optical radius 10) 6e4 packets
+// 2.80 / 2.66 ms, 1e5 2.88 / 3.04, 6e5 8.80 / 10.16.
 constexpr uint64_t kManyMixedPackets = 3u << 18;
+constexpr uint64_t kManyMatchedPackets = 5u << 14;
+inline bool matched_regions(const smcrt_scene *sc)
+{
+    bool all = true;
+    for (int r = 0; r < sc->nregions; ++r) all = all && sc->regions[r].n == sc->ambient_n;
+    return all;
+}
 
 // Variant of a plan launch whose shape nobody chose.
 inline int default_variant(int precision, uint64_t npackets, const DevScene &S)
 {
     if (precision == SMCRT_FP64) return npackets < kFewFp64Packets ? kFewFp64Variant : 1;
     if (S.general) return 2;
-    return npackets < kManyMixedPackets || S.cull_region >= 0 ? 1 : 0;
+    return npackets < (S.matched ? kManyMatchedPackets : kManyMixedPackets) || S.cull_region >= 0 ? 1 : 0;
 }
 
 // Kernel family of a scene: its register variants start at kNumVariants

@@ -225,6 +225,7 @@ int build_image(const smcrt_scene *sc, const smcrt_source *src, const smcrt_grid
     H.delta = sc->delta;
     H.ambient_n = sc->ambient_n;
     H.ambient_n32 = (float)sc->ambient_n;
+    H.matched = matched_regions(sc);
     H.cull_region = -1;   // no culling grid in the fixed scratch
     H.stepping = sc->stepping;
     H.nseg = nseg;

@@ -35,6 +35,7 @@ def test_spread_over_warps(precision, n):
 
 @pytest.mark.parametrize("make,precision,n", [
     (W.three_layer_slab, "mixed", (3 << 18) - 1), (W.three_layer_slab, "mixed", 3 << 18),
+    (lambda: W.iso_sphere(10.0), "mixed", (5 << 14) - 1), (lambda: W.iso_sphere(10.0), "mixed", 5 << 14),
     (W.vessel_network, "mixed", 20_000), (W.sdf_gallery, "mixed", 5_000),
     (W.glass_sphere_beam, "fp64", (1 << 19) - 1), (W.glass_sphere_beam, "fp64", 1 << 19)])
 def test_default_shape_same_results(make, precision, n):
