@@ -540,6 +540,7 @@ __global__ void __launch_bounds__(128, kMinBlocks) packets_fp64(JobWork *jobs, i
         const long long *s8 = reinterpret_cast<const long long *>(src);
         long long *d8 = reinterpret_cast<long long *>(&ws->S);
         for (int i = lane; i < (int)(sizeof(DevScene) / 8); i += 32) d8[i] = s8[i];
+        __syncwarp();                        // every lane reads what others copied, and all decide alike
         if (!scene_runs64<K>(ws->S)) {       // a scene of another family than this instantiation's
             if (lane == 0) {
                 atomicOr(status, kStatusBadJob);
