@@ -301,6 +301,8 @@ inline void fill_screen(DevScene &H, const smcrt_scene *sc, const smcrt_source *
     }
     R = R + 4.0 * sc->delta;
     H.screen_mask = H.fold_mask = H.soft_mask = 0;
+    for (int r = 0; r < sc->nregions; ++r)       // bounds the moves, screened or not
+        if (region_is_soft(sc, r)) H.soft_mask |= 1ull << r;
     H.feps = 0.f;
     H.tfix = 0;
     for (int a = 0; a < 3; ++a) H.gm32[a] = H.gr32[a] = INFINITY;
@@ -317,7 +319,6 @@ inline void fill_screen(DevScene &H, const smcrt_scene *sc, const smcrt_source *
         }
         if (fold) H.fold_mask |= bit;
         if (fold || smooth <= 8) H.screen_mask |= bit;
-        if (region_is_soft(sc, r)) H.soft_mask |= bit;
     }
     int k;
     std::frexp(R, &k);                           // R < 2^k: a move is shorter than 4 R <= 2^(k + 2)

@@ -1,0 +1,78 @@
+"""Segment stepping in FP64 moves a packet as far as the oracle does, bit for
+bit, in the scenes in which a bound of the move is easily lost: soft regions
+(folds of more than eight smooth unions, which bound a move by their distance
+alone) where the FP32 screening is off."""
+from dataclasses import replace
+
+import numpy as np
+import pytest
+
+import oracle as O
+import paper_2112_08035_gb300 as smc
+import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+KEYS = ("R", "T", "A", "killed", "gain", "packets", "scatters", "steps", "max_steps_hit")
+
+
+def _check(wl, fluence=True):
+    """Totals, records and (unless its units overflow) fluence of a plan launch and
+    of the launch without allocation against the oracle's."""
+    import torch
+    fo, to, ro = O.run(wl, fluence=fluence, records=True)
+    ctx = smc.Context(0)
+    plan = ctx.plan(wl, "fp64")
+    flu = torch.zeros(wl.grid.n[::-1], dtype=torch.int64, device="cuda") if fluence else None
+    tot = smc.totals_tensor()
+    rec = torch.zeros(wl.npackets * 8, dtype=torch.int64, device="cuda")
+    plan.launch(0, wl.npackets, wl.seed, flu, tot, rec)
+    f2, t2 = torch.zeros_like(flu) if fluence else None, smc.totals_tensor()
+    smc.run_noalloc(wl, 0, wl.npackets, wl.seed, f2, t2)
+    torch.cuda.synchronize()
+    assert plan.status() == 0
+    tg = smc.totals_from_tensor(tot)
+    for k in KEYS + (("pieces",) if fluence else ()):
+        assert tg[k] == to[k], (k, tg[k], to[k])
+    r = rec.cpu().numpy().view(smc.RECORD_DTYPE)
+    for f in ("R", "T", "A", "killed", "gain", "scatters", "steps"):
+        assert np.array_equal(r[f], ro[f]), f
+    assert torch.equal(t2[:14], tot[:14])
+    if fluence:
+        assert np.array_equal(flu.cpu().numpy().reshape(-1), np.asarray(fo).reshape(-1))
+        assert torch.equal(f2, flu)
+    plan.close()
+    ctx.close()
+
+
+def _scaled(wl, s):
+    """The same scene in other units: lengths times s, coefficients over s."""
+    prims = tuple(replace(p, params=tuple(v * s for v in p.params)) for p in wl.scene.prims)
+    regions = tuple(replace(r, mu_a=r.mu_a / s, mu_s=r.mu_s / s,
+                            program=tuple(replace(n, k=n.k * s) for n in r.program)) for r in wl.scene.regions)
+    by = lambda v: tuple(x * s for x in v)
+    scene = replace(wl.scene, prims=prims, regions=regions, delta=wl.scene.delta * s,
+                    bbox_lo=by(wl.scene.bbox_lo), bbox_hi=by(wl.scene.bbox_hi))
+    return replace(wl, scene=scene, source=replace(wl.source, pos=by(wl.source.pos), radius=wl.source.radius * s),
+                   grid=replace(wl.grid, lo=by(wl.grid.lo), hi=by(wl.grid.hi)))
+
+
+def _vessel(n=300):
+    return W.vessel_network(n, precision="fp64", grid_n=20).with_stepping(W.SEGMENT)
+
+
+def _wide(wl, half):
+    """The tissue box (primitive 0) widened beyond the volume of interest."""
+    p = wl.scene.prims[0].params
+    box = W.Prim(W.BOX, p[:3] + (half, half, p[5]))
+    return replace(wl, scene=replace(wl.scene, prims=(box,) + wl.scene.prims[1:]))
+
+
+@pytest.mark.parametrize("scale", [1e-7, 1e-6, 1e13])
+def test_soft_region_bounds_the_move_at_any_scale(scale):
+    """(At 1e13 cm a track length overflows the fluence's units.)"""
+    _check(_scaled(_vessel(), scale), fluence=scale < 1.0)
+
+
+def test_soft_region_bounds_the_move_beside_a_wide_box():
+    _check(_wide(_vessel(), 1e13))
