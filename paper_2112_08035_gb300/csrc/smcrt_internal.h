@@ -286,9 +286,10 @@ inline void fill_screen(DevScene &H, const smcrt_scene *sc, const smcrt_source *
                         const Instr *ins, const int2 *rr)
 {
     double R = 0.0;
+    const double spread = src->kind == SMCRT_SRC_DISC || src->kind == SMCRT_SRC_SQUARE ? src->radius : 0.0;
     for (int a = 0; a < 3; ++a) {
         R = std::fmax(R, std::fmax(std::fabs(sc->bbox_lo[a]), std::fabs(sc->bbox_hi[a])));
-        R = std::fmax(R, std::fabs(src->pos[a]) + std::fabs(src->radius));
+        R = std::fmax(R, std::fabs(src->pos[a]) + spread);
     }
     for (int i = 0; i < sc->nprims; ++i) {
         const smcrt_prim &P = sc->prims[i];

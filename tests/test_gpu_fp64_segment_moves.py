@@ -76,3 +76,9 @@ def test_soft_region_bounds_the_move_at_any_scale(scale):
 
 def test_soft_region_bounds_the_move_beside_a_wide_box():
     _check(_wide(_vessel(), 1e13))
+
+
+@pytest.mark.parametrize("radius", [1e13, float("inf")])
+def test_the_radius_of_a_pencil_changes_nothing(radius):
+    wl = _vessel()
+    _check(replace(wl, source=replace(wl.source, kind=W.PENCIL, radius=radius)))
