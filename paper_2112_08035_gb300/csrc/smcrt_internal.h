@@ -308,7 +308,11 @@ inline void fill_screen(DevScene &H, const smcrt_scene *sc, const smcrt_source *
     H.tfix = 0;
     for (int a = 0; a < 3; ++a) H.gm32[a] = H.gr32[a] = INFINITY;
     if (H.general || !(R > 1e-6 && R < 1e12)) return;   // FP32 squares stay in range
-    H.feps = (float)(R / 65536.0);
+    // the FP32 error; in scenes of simple regions also what the corners of all
+    // boxes grown by delta / 2 could take from a bound (segment_bound64_screened)
+    int nbox = 0;
+    for (int i = 0; i < sc->nprims; ++i) nbox += sc->prims[i].kind == SMCRT_BOX;
+    H.feps = (float)(R / 65536.0 + (H.singles ? 0.75 * (nbox + 1) * (0.5 * sc->delta) : 0.0));
     for (int r = 0; r < sc->nregions; ++r) {
         const uint64_t bit = 1ull << r;
         bool fold = rr[r].y - rr[r].x <= 60000;   // list entries are 16 bits

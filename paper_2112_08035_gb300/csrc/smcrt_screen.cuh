@@ -18,7 +18,8 @@
 // square root), of a capsule below 80 u R (the foot point along the axis),
 // and each of up to 8 smooth unions adds 14 u R (min, max and the
 // polynomial smooth minimum are 1-Lipschitz in their operands, so operand
-// errors do not grow).  DevScene.feps = 2^-16 R = 256 u R exceeds the sum.
+// errors do not grow).  DevScene.feps exceeds the sum: 2^-16 R = 256 u R, and in
+// scenes of simple regions a few delta more (segment_bound64_screened).
 #pragma once
 
 #include <cstddef>
@@ -478,6 +479,16 @@ __device__ __forceinline__ float scr_sphere(float4 A, float d, float e, const fl
     return scr_sqrt(disc - err) * kScrDown - b - eps;
 }
 
+// A lower bound of the distance along any ray to a primitive grown (d > 0) or
+// shrunk by e, |d| known within eps: |d| - e, but a box grows by e with sharp
+// corners, whose points lie up to sqrt(3) e from it.  Where every box's e is
+// delta / 2 (scenes of simple regions), feps has room for that (fill_screen).
+template <int K>
+__device__ __forceinline__ float scr_isotropic(int kind, float d, float e, float eps)
+{
+    return fabsf(d) - eps - (K == kPlainScene && kind == 1 && d > 0.f ? 1.7321f * e : e);
+}
+
 // A lower bound of the move bound (segment_bound64), or a value <= 0 when
 // FP32 cannot tell.
 template <int K>
@@ -490,8 +501,8 @@ static __device__ __noinline__ float segment_screen(const DevScene &S, float sof
         const int i = __ldg(S.seg_prims + j), kind = K == kBoxScene ? 1 : __ldg(S.pkind + i);
         const float e = __ldg(S.seg_m32 + j) * kScrUp + dh;
         const float d = scr_prim(S, kind, i, p[0], p[1], p[2]);
-        float b = fabsf(d) - eps - e;
-        if (!(b > 0.f)) return 0.f;
+        if (!(fabsf(d) - eps - e > 0.f)) return 0.f;
+        float b = scr_isotropic<K>(kind, d, e, eps);
         if (b >= t) continue;
         const float4 A = __ldg(S.p32 + 2 * i), B = __ldg(S.p32 + 2 * i + 1);
         const float c[3] = {A.x, A.y, A.z}, h[3] = {B.x, B.y, B.z};
@@ -573,6 +584,17 @@ __device__ __forceinline__ float scr_exit_most(const Ray32 &r, const float *c, c
 // conversions of FP64 tables that FP32 copies exist of (64 cycles each, as any
 // FP64 operation), and for the tree's fold a second time: vessel tree 1e4
 // packets 33.9 -> 26.2 ms, 4e4 51.4 -> 39.0, layered slab 1e5 44.7 -> 42.5.
+//
+// The reference passes a surface over when |d| - e is not below its bound so
+// far.  For all but a box seen from outside, whose ray bound may be smaller
+// than |d| - e (scr_isotropic), that changes nothing.  Surfaces left out here
+// lie beyond the bound so far, or beyond cap: then the reference's bound so
+// far may be another one above cap, and a box with |d| - e between cap and
+// ours may be one that it passes over.  Plain scenes start again without cap
+// there.  In scenes of simple regions (e = delta / 2 for every box) the result
+// cannot depend on it: cap exceeds the result by feps at least, and each such
+// box can only bring the bounds in question down by 0.74 delta / 2, all of
+// them together by less than feps has room for.
 template <int K>
 static __device__ __noinline__ double segment_bound64_screened(const DevScene &S, const Eval64 &E, const Screen64 &C,
                                                                double px, double py, double pz, double ux, double uy,
@@ -600,59 +622,68 @@ static __device__ __noinline__ double segment_bound64_screened(const DevScene &S
         }
         cap *= kScrUp;
     }
-    double t = __longlong_as_double(0x7ff0000000000000LL);
-    if (!(eps > 0.f && scr_box_exit(S.bbc32, S.bbh32, dhf * kScrUp, p, u, eps) > cap))
-        t = seg_face64(box, r, S.bbc32, S.bbh32, true, px, py, pz, ux, uy, uz, dh, dhf, eps);
-    if (!one_each<K>() && S.soft_mask != 0ull && !(C.soft - dhf * kScrUp > fminf(cap, (float)t * kScrUp))) {
-        double ds = __longlong_as_double(0x7ff0000000000000LL);
-        for (unsigned long long m = S.soft_mask; m != 0ull; m &= m - 1ull) {
-            const int k = __ffsll((long long)m) - 1;
-            double d = E.dmin;                   // the nearest surface's is known
-            if (k != E.istar) {
-                unsigned long long list = C.list;
-                int cnt = C.cnt;
-                if (k != C.flr) fold_list<K>(S, k, px, py, pz, 0.f, list, cnt);
-                d = fabs(region_exact<K>(S, k, px, py, pz, list, cnt));
+    for (;;) {
+        bool again = false;
+        double t = __longlong_as_double(0x7ff0000000000000LL);
+        if (!(eps > 0.f && scr_box_exit(S.bbc32, S.bbh32, dhf * kScrUp, p, u, eps) > cap))
+            t = seg_face64(box, r, S.bbc32, S.bbh32, true, px, py, pz, ux, uy, uz, dh, dhf, eps);
+        if (!one_each<K>() && S.soft_mask != 0ull && !(C.soft - dhf * kScrUp > fminf(cap, (float)t * kScrUp))) {
+            double ds = __longlong_as_double(0x7ff0000000000000LL);
+            for (unsigned long long m = S.soft_mask; m != 0ull; m &= m - 1ull) {
+                const int k = __ffsll((long long)m) - 1;
+                double d = E.dmin;                   // the nearest surface's is known
+                if (k != E.istar) {
+                    unsigned long long list = C.list;
+                    int cnt = C.cnt;
+                    if (k != C.flr) fold_list<K>(S, k, px, py, pz, 0.f, list, cnt);
+                    d = fabs(region_exact<K>(S, k, px, py, pz, list, cnt));
+                }
+                ds = min64(ds, d);
             }
-            ds = min64(ds, d);
+            t = min64(t, ds - dh);
         }
-        t = min64(t, ds - dh);
+        for (int j = 0; j < S.nseg; ++j) {
+            const int i = __ldg(S.seg_prims + j);
+            const int kind = K == kBoxScene ? 1 : __ldg(S.pkind + i);
+            const double e = __ldg(S.seg_m64 + j) + dh;
+            const float e32 = __ldg(S.seg_m32 + j) + dhf, ef = e32 * kScrUp, tu = fminf((float)t * kScrUp, cap);
+            const float df = scr_prim(S, kind, i, p[0], p[1], p[2]);
+            const float iso = fabsf(df) - eps - ef;
+            const float4 A = __ldg(S.p32 + 2 * i), B = __ldg(S.p32 + 2 * i + 1);
+            const float c[3] = {A.x, A.y, A.z}, h[3] = {B.x, B.y, B.z};
+            if (eps > 0.f && iso > 0.f) {        // certainly outside the margin
+                if (scr_isotropic<K>(kind, df, ef, eps) > tu) continue;
+                if (kind == 1 &&
+                    (df > 0.f ? scr_box_entry(c, h, ef, p, u, eps) : scr_box_exit(c, h, ef, p, u, eps)) > tu)
+                    continue;
+                if (kind == 0 && scr_sphere(A, df, ef, p, u, eps) > tu) continue;
+            }
+            // FP64 where FP32 leaves it open whether the primitive is passed over
+            // (|d| within its margin, or |d| - e not below the bound so far)
+            double d = (double)df;
+            if (!(eps > 0.f && iso > 0.f && fabsf(df) + eps - ef * kScrDown * kScrDown < tu * kScrDown * kScrDown)) {
+                d = prim64<false>(S, kind, i, px, py, pz);
+                if (!(fabs(d) > e)) return 0.0;
+                const double away = fabs(d) - e;
+                if (away >= t) continue;
+                if (K == kPlainScene && SMCRT_RARE(tu == cap && away >= (double)cap && t > (double)cap)) {
+                    again = true;            // the reference's bound so far is not known
+                    break;
+                }
+            }
+            const double *P = S.p64 + 8 * i;
+            double b;
+            if (kind == 0)
+                b = seg_sphere64(P, d, px, py, pz, ux, uy, uz, e);
+            else if (kind == 1)
+                b = seg_face64(P, r, c, h, !(d > 0.0), px, py, pz, ux, uy, uz, e, e32, eps);
+            else
+                b = seg_capsule64(P, d, px, py, pz, ux, uy, uz, e);
+            t = min64(t, b);
+        }
+        if (K != kPlainScene || !again) return t;
+        cap = __int_as_float(0x7f800000);
     }
-    for (int j = 0; j < S.nseg; ++j) {
-        const int i = __ldg(S.seg_prims + j);
-        const int kind = K == kBoxScene ? 1 : __ldg(S.pkind + i);
-        const double e = __ldg(S.seg_m64 + j) + dh;
-        const float e32 = __ldg(S.seg_m32 + j) + dhf, ef = e32 * kScrUp, tu = fminf((float)t * kScrUp, cap);
-        const float df = scr_prim(S, kind, i, p[0], p[1], p[2]);
-        const float iso = fabsf(df) - eps - ef;
-        const float4 A = __ldg(S.p32 + 2 * i), B = __ldg(S.p32 + 2 * i + 1);
-        const float c[3] = {A.x, A.y, A.z}, h[3] = {B.x, B.y, B.z};
-        if (eps > 0.f && iso > 0.f) {        // certainly outside the margin
-            if (iso > tu) continue;
-            if (kind == 1 &&
-                (df > 0.f ? scr_box_entry(c, h, ef, p, u, eps) : scr_box_exit(c, h, ef, p, u, eps)) > tu)
-                continue;
-            if (kind == 0 && scr_sphere(A, df, ef, p, u, eps) > tu) continue;
-        }
-        // FP64 where FP32 leaves it open whether the primitive is passed over
-        // (|d| within its margin, or |d| - e not below the bound so far)
-        double d = (double)df;
-        if (!(eps > 0.f && iso > 0.f && fabsf(df) + eps - ef * kScrDown * kScrDown < tu * kScrDown * kScrDown)) {
-            d = prim64<false>(S, kind, i, px, py, pz);
-            if (!(fabs(d) > e)) return 0.0;
-            if (fabs(d) - e >= t) continue;
-        }
-        const double *P = S.p64 + 8 * i;
-        double b;
-        if (kind == 0)
-            b = seg_sphere64(P, d, px, py, pz, ux, uy, uz, e);
-        else if (kind == 1)
-            b = seg_face64(P, r, c, h, !(d > 0.0), px, py, pz, ux, uy, uz, e, e32, eps);
-        else
-            b = seg_capsule64(P, d, px, py, pz, ux, uy, uz, e);
-        t = min64(t, b);
-    }
-    return t;
 }
 
 // ---------------------------------------------------------------------------
