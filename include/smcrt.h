@@ -276,7 +276,9 @@ int smcrt_plan_destroy(smcrt_plan *plan);
 
 /* Launch configuration of the persistent packet kernel: blocks (0 = SM
  * count x resident blocks per SM) and threads per block (a multiple of 32,
- * 32 .. 128; 0 = tuned default).  Other values return BAD_ARG. */
+ * 32 .. 128; 0 = tuned default).  Other values return BAD_ARG.  Where neither
+ * they nor a variant was chosen, FP64 launches of fewer than 2^19 packets run
+ * one block per SM. */
 int smcrt_plan_set_launch(smcrt_plan *plan, int32_t blocks, int32_t threads);
 
 /* Asynchronously propagate packets [id_begin, id_begin + npackets) with

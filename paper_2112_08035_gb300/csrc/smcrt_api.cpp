@@ -682,8 +682,10 @@ int build_plan(smcrt_ctx *ctx, const smcrt_scene *sc, const smcrt_source *src, c
 
 void default_launch(const smcrt_plan *pl, uint64_t npackets, int &blocks, int &threads, int &variant)
 {
-    const bool few = pl->precision == SMCRT_FP64 && !pl->chosen && npackets < kFewFp64Packets;
-    variant = pl->chosen ? pl->variant : default_variant(pl->precision, npackets, pl->host);
+    // blocks 0 beside a chosen number of threads: all that are resident
+    const bool shaped = pl->blocks > 0 || pl->threads > 0, fp64 = pl->precision == SMCRT_FP64;
+    const bool few = fp64 && !pl->chosen && !shaped && npackets < kFewFp64Packets;
+    variant = pl->chosen ? pl->variant : default_variant(pl->precision, fp64 && !few ? kFewFp64Packets : npackets, pl->host);
     threads = pl->threads > 0 ? pl->threads : 128;
     blocks = pl->blocks;
     if (blocks <= 0) {
