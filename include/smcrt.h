@@ -328,7 +328,9 @@ int smcrt_set_time_limit(smcrt_ctx *ctx, double seconds);
  * plans, scene tables in global or shared memory x threads per block x
  * resident blocks) on a short trial run of this plan and keep the
  * fastest; the choice is cached per scene shape in the context and applied
- * to later plans of the same shape.  Trial tallies go to scratch buffers.
+ * to later plans of the same shape.  FP64 trials of fewer than 2^19 packets
+ * also try one block per SM; if that is fastest, it is used for launches
+ * below that size only.  Trial tallies go to scratch buffers.
  * *blocks / *threads / *variant (may be NULL) receive the choice. */
 int smcrt_plan_autotune(smcrt_plan *plan, uint64_t trial_packets, int32_t *blocks,
                         int32_t *threads, int32_t *variant);

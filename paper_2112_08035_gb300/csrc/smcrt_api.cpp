@@ -230,8 +230,11 @@ struct smcrt_ctx {
     size_t budget = 0;
     double time_limit_s = 0.0;   // device time limit of smcrt_run and the default of new plans
     std::mutex tune_mu;
-    struct Tuned { int blocks, threads, variant; };
-    std::map<uint64_t, Tuned> tuned;  // scene shape -> launch shape
+    // scene shape -> launch shape; few: of FP64 launches below kFewFp64Packets,
+    // where one block per SM was faster (blocks 0: the same)
+    struct Shape { int blocks, threads, variant; };
+    struct Tuned { Shape all, few; };
+    std::map<uint64_t, Tuned> tuned;
 
     // serving
     std::mutex mu;
@@ -260,6 +263,7 @@ struct smcrt_plan {
     int *dstatus = nullptr;
     int blocks = 0, threads = 0, variant = 0;
     bool chosen = false;       // the caller or the autotuner chose the variant
+    smcrt_ctx::Shape few{0, 0, 0};   // tuned: FP64 launches below kFewFp64Packets (blocks 0: none)
     int stage = 0;             // mixed: stage the scene tables in shared memory
     double time_limit_s = 0.0; // device time limit of a launch (0 = none)
     size_t cells = 0;
@@ -438,6 +442,16 @@ void build_cull(const smcrt_scene *sc, CullGrid &cg)
         cg.lo[a] = (float)glo[a];
         cg.inv_s[a] = (float)(1.0 / s[a]);
     }
+}
+
+void use_tuned(smcrt_plan *pl, const smcrt_ctx::Tuned &t)
+{
+    pl->blocks = t.all.blocks;
+    pl->threads = t.all.threads;
+    pl->variant = t.all.variant % kNumVariants;
+    pl->stage = t.all.variant / kNumVariants;
+    pl->chosen = true;
+    pl->few = t.few;
 }
 
 // Validate, compile and upload a plan.  With a stream (the serving
@@ -669,11 +683,7 @@ int build_plan(smcrt_ctx *ctx, const smcrt_scene *sc, const smcrt_source *src, c
         std::lock_guard<std::mutex> lk(ctx->tune_mu);
         auto it = ctx->tuned.find(pl->shape_key);
         if (it != ctx->tuned.end()) {
-            pl->blocks = it->second.blocks;
-            pl->threads = it->second.threads;
-            pl->variant = it->second.variant % kNumVariants;
-            pl->chosen = true;
-            pl->stage = it->second.variant / kNumVariants;
+            use_tuned(pl.get(), it->second);
         }
     }
     *out = pl.release();
@@ -682,6 +692,12 @@ int build_plan(smcrt_ctx *ctx, const smcrt_scene *sc, const smcrt_source *src, c
 
 void default_launch(const smcrt_plan *pl, uint64_t npackets, int &blocks, int &threads, int &variant)
 {
+    if (pl->few.blocks > 0 && npackets < kFewFp64Packets) {
+        blocks = pl->few.blocks;
+        threads = pl->few.threads;
+        variant = pl->few.variant;
+        return;
+    }
     // blocks 0 beside a chosen number of threads: all that are resident
     const bool shaped = pl->blocks > 0 || pl->threads > 0, fp64 = pl->precision == SMCRT_FP64;
     const bool few = fp64 && !pl->chosen && !shaped && npackets < kFewFp64Packets;
@@ -1404,6 +1420,7 @@ int smcrt_plan_set_launch(smcrt_plan *pl, int32_t blocks, int32_t threads)
     if (!pl || blocks < 0 || threads < 0 || threads > kMaxThreads || (threads % 32) != 0) return SMCRT_ERR_BAD_ARG;
     pl->blocks = blocks;
     pl->threads = threads;
+    pl->few.blocks = 0;
     return SMCRT_OK;
 }
 
@@ -1426,6 +1443,7 @@ int smcrt_plan_set_variant(smcrt_plan *pl, int32_t variant)
     pl->variant = variant % kNumVariants;
     pl->chosen = true;
     pl->stage = variant / kNumVariants;
+    pl->few.blocks = 0;
     return SMCRT_OK;
 }
 
@@ -1468,8 +1486,11 @@ int smcrt_plan_autotune(smcrt_plan *pl, uint64_t trial, int32_t *blocks_out, int
     cudaEvent_t e0, e1;
     cudaEventCreate(&e0);
     cudaEventCreate(&e1);
-    float best = 1e30f;
-    int bb = 0, bt = 0, bv = 0;
+    // FP64 trials below kFewFp64Packets also try one block per SM, whose time
+    // says nothing about larger launches: that choice is kept apart
+    float best = 1e30f, best_few = 1e30f;
+    smcrt_ctx::Tuned tuned{{0, 0, 0}, {0, 0, 0}};
+    const bool try_few = pl->precision == SMCRT_FP64 && trial < kFewFp64Packets;
     const int thread_opts[] = {64, 128};
     const int saved_variant = pl->variant, saved_stage = pl->stage;
     int rc = SMCRT_OK;
@@ -1484,8 +1505,8 @@ int smcrt_plan_autotune(smcrt_plan *pl, uint64_t trial, int32_t *blocks_out, int
             const int occ = occupancy(pl->precision, t, v);
             if (occ < 1) continue;
             for (int mult : {0, 1, 2}) {
-                if (mult == 0 && pl->precision != SMCRT_FP64) continue;
-                const int b = pl->ctx->sm_count * (mult == 0 ? 1 : occ * mult);   // FP64: one block per SM too
+                if (mult == 0 && !try_few) continue;
+                const int b = pl->ctx->sm_count * (mult == 0 ? 1 : occ * mult);
                 float ms_best = 1e30f;
                 for (int rep = 0; rep < 2; ++rep) {
                     cudaMemsetAsync(flu, 0, pl->cells * 8, 0);
@@ -1502,11 +1523,10 @@ int smcrt_plan_autotune(smcrt_plan *pl, uint64_t trial, int32_t *blocks_out, int
                     ms_best = std::min(ms_best, ms);
                 }
                 if (rc != SMCRT_OK) break;
-                if (ms_best < best) {
-                    best = ms_best;
-                    bb = b;
-                    bt = t;
-                    bv = pv;
+                float &least = mult == 0 ? best_few : best;
+                if (ms_best < least) {
+                    least = ms_best;
+                    (mult == 0 ? tuned.few : tuned.all) = {b, t, pv};
                 }
             }
         }
@@ -1520,18 +1540,16 @@ int smcrt_plan_autotune(smcrt_plan *pl, uint64_t trial, int32_t *blocks_out, int
         pl->stage = saved_stage;
         return rc;
     }
-    pl->blocks = bb;
-    pl->threads = bt;
-    pl->variant = bv % kNumVariants;
-    pl->chosen = true;
-    pl->stage = bv / kNumVariants;
+    if (!(best_few < best)) tuned.few.blocks = 0;
+    use_tuned(pl, tuned);
     {
         std::lock_guard<std::mutex> lk(pl->ctx->tune_mu);
-        pl->ctx->tuned[pl->shape_key] = {bb, bt, bv};
+        pl->ctx->tuned[pl->shape_key] = tuned;
     }
-    if (blocks_out) *blocks_out = bb;
-    if (threads_out) *threads_out = bt;
-    if (variant_out) *variant_out = bv;
+    const smcrt_ctx::Shape &fastest = tuned.few.blocks > 0 ? tuned.few : tuned.all;
+    if (blocks_out) *blocks_out = fastest.blocks;
+    if (threads_out) *threads_out = fastest.threads;
+    if (variant_out) *variant_out = fastest.variant;
     return SMCRT_OK;
 }
 

@@ -42,3 +42,25 @@ def test_blocks_zero_means_all_resident_blocks(threads):
     assert _warps(plan, wl) > 1.5 * one
     plan.close()
     ctx.close()
+
+
+def test_a_small_trial_leaves_large_launches_their_shape():
+    """FP64, 5000 packets: one block per SM is fastest (13.3 against 17.6 ms
+    at 1e4), and the tuner reports it; a launch of 2^19 packets, of this plan
+    or of a later one of the same shape, runs at least twice the warps."""
+    import torch
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    ctx = smc.Context(0)
+    small = W.three_layer_slab(5_000, precision="fp64").with_stepping(W.SEGMENT)
+    large = small.with_packets(1 << 19)
+    plan = ctx.plan(small, "fp64")
+    blocks, threads, variant = plan.autotune(small.npackets)
+    assert blocks == sms and threads in (64, 128) and variant in range(3)
+    one = ctx.plan(large, "fp64")
+    one.set_launch(sms, 128)
+    few = _warps(one, large)
+    for p in (plan, ctx.plan(large, "fp64")):
+        assert _warps(p, large) > 1.5 * few
+        p.close()
+    one.close()
+    ctx.close()
