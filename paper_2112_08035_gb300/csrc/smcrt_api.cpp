@@ -1502,7 +1502,7 @@ int smcrt_plan_autotune(smcrt_plan *pl, uint64_t trial, int32_t *blocks_out, int
         pl->variant = v;
         pl->stage = pv / kNumVariants;
         for (int t : thread_opts) {
-            const int occ = occupancy(pl->precision, t, v);
+            const int occ = occupancy(pl->precision, t, kvariant(pl, v));
             if (occ < 1) continue;
             for (int mult : {0, 1, 2}) {
                 if (mult == 0 && !try_few) continue;
