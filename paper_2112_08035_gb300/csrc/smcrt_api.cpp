@@ -520,7 +520,8 @@ int build_plan(smcrt_ctx *ctx, const smcrt_scene *sc, const smcrt_source *src, c
     const size_t o_segm32 = take(sizeof(float) * nseg);
     const size_t o_xf64 = take(sizeof(double) * xf64.size());
     const size_t o_xf32 = take(sizeof(float4) * xf32.size());
-    const size_t o_planes = take(precision == SMCRT_FP64 ? sizeof(double) * plane_count(g) : 0);
+    const bool with_planes = precision == SMCRT_FP64 && walk_bits(screen_range(sc, src)) > 0;
+    const size_t o_planes = take(with_planes ? sizeof(double) * plane_count(g) : 0);
     const size_t total = off;
 
     std::unique_ptr<smcrt_plan> pl(new smcrt_plan());
@@ -627,7 +628,7 @@ int build_plan(smcrt_ctx *ctx, const smcrt_scene *sc, const smcrt_source *src, c
     H.src_radius32 = (float)src->radius;
     if (precision == SMCRT_FP64) {
         fill_screen(H, sc, src, g, ins.data(), rr.data());
-        H.planes = (const double *)(base + o_planes);
+        if (with_planes) H.planes = (const double *)(base + o_planes);
     }
 
     std::vector<char> hb(total, 0);
@@ -639,7 +640,7 @@ int build_plan(smcrt_ctx *ctx, const smcrt_scene *sc, const smcrt_source *src, c
     std::memcpy(hb.data() + o_p32, p32.data(), sizeof(float4) * 2 * np);
     std::memcpy(hb.data() + o_rr, rr.data(), sizeof(int2) * nr);
     std::memcpy(hb.data() + o_r64, reg64.data(), sizeof(double) * kReg64 * nr);
-    if (precision == SMCRT_FP64) fill_planes(g, (double *)(hb.data() + o_planes));
+    if (with_planes) fill_planes(g, (double *)(hb.data() + o_planes));
     std::memcpy(hb.data() + o_r32, reg32.data(), sizeof(float4) * 2 * nr);
     if (!cg.off.empty()) std::memcpy(hb.data() + o_coff, cg.off.data(), sizeof(int32_t) * cg.off.size());
     if (!cg.list.empty()) std::memcpy(hb.data() + o_clist, cg.list.data(), sizeof(int32_t) * cg.list.size());

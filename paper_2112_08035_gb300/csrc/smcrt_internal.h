@@ -277,13 +277,13 @@ struct DevScene {
     float tq[3];              // fixed-point walk: error of a plane's distance times |u|, in units, per axis
     int32_t tfix;             // ... its unit is 2^-tfix (0: no fixed-point walk)
     int32_t matched;          // every region has the ambient index (default_variant)
-    const double *planes;     // fill_planes; null: computed
+    const double *planes;     // fill_planes (where tfix > 0)
 };
 
-// The screening fields of a compiled scene without general shapes: the error
-// bounds and region classes that smcrt_screen.cuh states.
-inline void fill_screen(DevScene &H, const smcrt_scene *sc, const smcrt_source *src, const smcrt_grid *g,
-                        const Instr *ins, const int2 *rr)
+// The range of the FP64 screening: every coordinate, half extent and radius
+// of the scene and its source, plus four surface thresholds; 0 where there is
+// no screening (general shapes, FP32 squares out of range).
+inline double screen_range(const smcrt_scene *sc, const smcrt_source *src)
 {
     double R = 0.0;
     const double spread = src->kind == SMCRT_SRC_DISC || src->kind == SMCRT_SRC_SQUARE ? src->radius : 0.0;
@@ -293,6 +293,7 @@ inline void fill_screen(DevScene &H, const smcrt_scene *sc, const smcrt_source *
     }
     for (int i = 0; i < sc->nprims; ++i) {
         const smcrt_prim &P = sc->prims[i];
+        if (!plain_prim(P)) return 0.0;
         for (int a = 0; a < 3; ++a) {
             if (P.kind == SMCRT_SPHERE) R = std::fmax(R, std::fabs(P.p[a]) + P.p[3]);
             else if (P.kind == SMCRT_BOX) R = std::fmax(R, std::fabs(P.p[a]) + P.p[3 + a]);
@@ -301,13 +302,30 @@ inline void fill_screen(DevScene &H, const smcrt_scene *sc, const smcrt_source *
         }
     }
     R = R + 4.0 * sc->delta;
+    return R > 1e-6 && R < 1e12 ? R : 0.0;
+}
+
+// The fixed-point walk's unit is 2^-walk_bits of a centimetre; 0: no such walk.
+inline int walk_bits(double R)
+{
+    int k;
+    std::frexp(R, &k);                           // R < 2^k: a move is shorter than 4 R <= 2^(k + 2)
+    return R > 0.0 && 58 - k >= 40 ? 58 - k : 0;
+}
+
+// The screening fields of a compiled scene: the error bounds and region
+// classes that smcrt_screen.cuh states.
+inline void fill_screen(DevScene &H, const smcrt_scene *sc, const smcrt_source *src, const smcrt_grid *g,
+                        const Instr *ins, const int2 *rr)
+{
+    const double R = screen_range(sc, src);
     H.screen_mask = H.fold_mask = H.soft_mask = 0;
     for (int r = 0; r < sc->nregions; ++r)       // bounds the moves, screened or not
         if (region_is_soft(sc, r)) H.soft_mask |= 1ull << r;
     H.feps = 0.f;
     H.tfix = 0;
     for (int a = 0; a < 3; ++a) H.gm32[a] = H.gr32[a] = INFINITY;
-    if (H.general || !(R > 1e-6 && R < 1e12)) return;   // FP32 squares stay in range
+    if (R == 0.0) return;
     // the FP32 error; in scenes of simple regions also what the corners of all
     // boxes grown by delta / 2 could take from a bound (segment_bound64_screened)
     int nbox = 0;
@@ -325,9 +343,7 @@ inline void fill_screen(DevScene &H, const smcrt_scene *sc, const smcrt_source *
         if (fold) H.fold_mask |= bit;
         if (fold || smooth <= 8) H.screen_mask |= bit;
     }
-    int k;
-    std::frexp(R, &k);                           // R < 2^k: a move is shorter than 4 R <= 2^(k + 2)
-    H.tfix = 58 - k >= 40 ? 58 - k : 0;
+    H.tfix = walk_bits(R);
     for (int a = 0; a < 3; ++a) {
         const double Rg = std::fmax(R, std::fmax(std::fabs(g->lo[a]), std::fabs(g->hi[a])));
         const double dl = (g->hi[a] - g->lo[a]) / (double)g->n[a];

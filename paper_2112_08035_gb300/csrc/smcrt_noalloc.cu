@@ -159,14 +159,20 @@ int build_image(const smcrt_scene *sc, const smcrt_source *src, const smcrt_grid
     const size_t o_seg = take(sizeof(int32_t) * nseg);
     const size_t o_segm64 = take(sizeof(double) * nseg);
     const size_t o_segm32 = take(sizeof(float) * nseg);
-    const bool has_xf = sc->nxforms > 0;
+    bool has_xf = false;                         // some primitive has a frame
+    for (int i = 0; i < np; ++i) has_xf = has_xf || sc->prims[i].xform > 0;
     const size_t o_xf64 = take(has_xf ? sizeof(double) * kXf64 * np : 0);
     const size_t o_xf32 = take(has_xf ? sizeof(float4) * kXf32 * np : 0);
+    // the grid's planes, in scenes without frames: at the limits they fit too
+    static_assert(kImageOff + sizeof(DevScene) + kNoAllocMaxNodes * (sizeof(Instr) + sizeof(double)) +
+                          kNoAllocMaxPrims * (2 * sizeof(int32_t) + 9 * sizeof(double) + 2 * sizeof(float4) + sizeof(float)) +
+                          kNoAllocMaxRegions * (sizeof(int2) + kReg64 * sizeof(double) + 2 * sizeof(float4)) +
+                          3 * (kMaxGridSide + 1) * sizeof(double) + 16 * 16 <=
+                      kNoAllocScratchBytes,
+                  "image of the largest scene without frames");
+    const bool with_planes = precision == SMCRT_FP64 && walk_bits(screen_range(sc, src)) > 0;
+    const size_t o_planes = take(with_planes ? sizeof(double) * plane_count(g) : 0);
     if (kImageOff + off > kNoAllocScratchBytes) return SMCRT_ERR_NO_MEMORY;
-    // the grid's planes where they fit (else the kernel computes them)
-    const size_t plane_bytes = sizeof(double) * plane_count(g);
-    const bool with_planes = precision == SMCRT_FP64 && kImageOff + a16(off + plane_bytes) <= kNoAllocScratchBytes;
-    const size_t o_planes = take(with_planes ? plane_bytes : 0);
     std::memset(img, 0, off);
 
     int32_t *pkind = (int32_t *)(img + o_kind);

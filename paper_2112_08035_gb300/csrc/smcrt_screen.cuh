@@ -738,9 +738,7 @@ __device__ __forceinline__ unsigned long long fixed64(double x, int e)
 // The plane i of one axis.
 __device__ __forceinline__ double grid_plane(const DevScene &S, int a, int i)
 {
-    if (S.planes != nullptr)
-        return __ldg(S.planes + (a == 0 ? 0 : a == 1 ? S.g_n[0] + 1 : S.g_n[0] + S.g_n[1] + 2) + i);
-    return S.g_lo[a] + (double)i * S.g_dl[a];
+    return __ldg(S.planes + (a == 0 ? 0 : a == 1 ? S.g_n[0] + 1 : S.g_n[0] + S.g_n[1] + 2) + i);
 }
 
 // One axis of a fixed-point walk: the distance of the plane ahead along the

@@ -17,10 +17,11 @@ PROGRAM = r"""
 #include "smcrt_internal.h"
 int main(int argc, char **argv)
 {
-    if (argc != 3) return 2;
+    if (argc != 4) return 2;
     smcrt_prim prim{};
-    prim.kind = SMCRT_SPHERE;
+    prim.kind = std::atoi(argv[3]);
     prim.p[3] = 1.0;
+    prim.p[4] = 0.5;
     smcrt_csg_node node{};
     node.op = SMCRT_OP_PRIM;
     smcrt_region region{};
@@ -41,7 +42,7 @@ int main(int argc, char **argv)
     const int2 rr = make_int2(0, 1);
     smcrt::DevScene H{};
     smcrt::fill_screen(H, &sc, &src, &g, &ins, &rr);
-    std::printf("%.9g %d\n", H.feps, H.tfix);
+    std::printf("%.9g %d %d\n", H.feps, H.tfix, smcrt::walk_bits(smcrt::screen_range(&sc, &src)));
 }
 """
 
@@ -54,14 +55,16 @@ def bound(tmp_path_factory):
         f.write(PROGRAM)
     subprocess.check_call(["g++", "-std=c++17", f"-I{CSRC}", f"-I{CUDA}/include", src, "-o", exe])
 
-    def run(kind, radius):
-        feps, tfix = subprocess.check_output([exe, str(kind), repr(radius)], text=True).split()
+    def run(kind, radius, prim=SPHERE):
+        feps, tfix, walk = subprocess.check_output([exe, str(kind), repr(radius), str(prim)], text=True).split()
+        assert tfix == walk                      # the image has the planes where the kernel walks with them
         return float(feps), int(tfix)
 
     return run
 
 
 PENCIL, DISC, SQUARE, ISO_POINT = range(4)
+SPHERE, TORUS = 0, 3
 
 
 @pytest.mark.parametrize("kind", [PENCIL, ISO_POINT])
@@ -76,3 +79,13 @@ def test_a_source_with_a_radius_counts(bound, kind):
     assert narrow == bound(kind, 1.0)            # inside the volume of interest
     assert 15.9 < wide[0] / narrow[0] < 16.1     # 32 against the box's 2
     assert off == (0.0, 0)                       # beyond the screening's range
+
+
+def test_general_shapes_have_no_screening_and_no_planes(bound):
+    assert bound(PENCIL, 0.0, TORUS) == (0.0, 0)
+
+
+def test_the_fixed_point_walk_ends_before_the_screening(bound):
+    """The walk's unit is 2^-58 of the range and no coarser than 2^-40."""
+    assert bound(SQUARE, 2.0 ** 18 - 1.0)[1] == 40
+    assert bound(SQUARE, 2.0 ** 19)[1] == 0 and bound(SQUARE, 2.0 ** 19)[0] > 0.0
