@@ -1082,10 +1082,8 @@ __global__ void __launch_bounds__(128, kMinBlocks) packets_mixed_multi(JobWork *
 
 // Register budgets of the instantiations: variant v keeps kMinBlocks
 // blocks of 128 threads resident per SM (more blocks = fewer registers per
-// thread, possibly spilled); the autotuner picks per scene.  Variants
+// thread, possibly spilled): 5, 4 and 3; the autotuner picks per scene.  Variants
 // kNumVariants * k .. are the same budgets for scene family k (scene_family).
-constexpr int kVariantBlocks[kNumVariants] = {5, 4, 3};
-
 cudaError_t launch_mixed(JobWork *jobs, int njobs, int *status, int blocks, int threads, cudaStream_t stream,
                         int variant)
 {

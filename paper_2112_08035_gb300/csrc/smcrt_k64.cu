@@ -322,7 +322,7 @@ __device__ bool run_job_fp64(const DevScene &S, WarpAcc *wa, const volatile JobC
             if (alive && phase == kExact && !interact) {
                 Eval64 E;
                 if (K == kGeneralScene) {
-                    E = scene_eval64<true>(S, px, py, pz, -2);
+                    E = scene_eval64(S, px, py, pz);
                 } else {
                     C.neg = kneg; C.mask = kmask; C.list = klist; C.flr = kfold >> 8; C.cnt = (int)(int8_t)(kfold & 0xff);
                     C.soft = ksoft; C.db = kdb;
@@ -342,7 +342,7 @@ __device__ bool run_job_fp64(const DevScene &S, WarpAcc *wa, const volatile JobC
                         move = true;
                         interact = mu_t > 0.0 && tau < mu_t * L;
                         if (!interact && S.stepping == SMCRT_STEP_SEGMENT) {   // a longer move along u
-                            if (K == kGeneralScene) L = fmax(L, segment_bound64<true>(S, E.dsoft, E.dbox, px, py, pz, ux, uy, uz));
+                            if (K == kGeneralScene) L = fmax(L, segment_bound64(S, E.dsoft, E.dbox, px, py, pz, ux, uy, uz));
                             else L = max64(L, segment_bound64_screened<K>(S, E, C, px, py, pz, ux, uy, uz));
                             interact = mu_t > 0.0 && tau < mu_t * L;
                         }
@@ -569,9 +569,7 @@ __global__ void __launch_bounds__(128, kMinBlocks) packets_fp64(JobWork *jobs, i
 
 // Register budgets of the instantiations: variant v keeps kMinBlocks
 // blocks of 128 threads resident per SM (more blocks = fewer registers per
-// thread, possibly spilled); the autotuner picks per scene.
-constexpr int kVariantBlocks[kNumVariants] = {4, 3, 2};
-
+// thread, possibly spilled): 4, 3 and 2; the autotuner picks per scene.
 cudaError_t launch_fp64(JobWork *jobs, int njobs, int *status, int blocks, int threads, cudaStream_t stream,
                         int variant)
 {

@@ -193,7 +193,7 @@ __device__ __forceinline__ long long fx32(float x) { return __float2ll_rn(x * 42
 // loads measured 3.5 % faster than read-only-cache loads on the layered slab.
 // ---------------------------------------------------------------------------
 // dsoft: min |d| over soft regions (segment stepping), +inf if none.
-struct Eval64 { double dmin, dstar, dsel, dbox, dsoft; int istar, region; };
+struct Eval64 { double dmin, dstar, dbox, dsoft; int istar, region; };
 struct Eval32 { float dmin, dstar, dbox, dsoft; int istar, region; };
 
 // The larger / smaller of two numbers (not NaN), compared as integers: an
@@ -426,10 +426,9 @@ __device__ __forceinline__ float csg32(int op, float a, float b, float kinv)
 }
 
 // Evaluate instructions [i0, i1) as a register-stack program; when `full`,
-// record every region end (region, d_min, istar, and d of surface `sel`).
+// record every region end (region, d_min and istar).
 template <bool kFull, bool G>
-__device__ __forceinline__ double run_prog64(const DevScene &S, int i0, int i1, double x, double y, double z,
-                                             int sel, Eval64 *E)
+__device__ __forceinline__ double run_prog64(const DevScene &S, int i0, int i1, double x, double y, double z, Eval64 *E)
 {
     double s0 = 0.0, s1 = 0.0, s2 = 0.0, s3 = 0.0;
     for (int i = i0; i < i1; ++i) {
@@ -454,7 +453,6 @@ __device__ __forceinline__ double run_prog64(const DevScene &S, int i0, int i1, 
             const double ad = fabs(d);
             if (ad < E->dmin) { E->dmin = ad; E->istar = ins.z; E->dstar = d; }
             if ((ins.x & kSoftRegionEnd) && ad < E->dsoft) E->dsoft = ad;
-            if (ins.z == sel) E->dsel = d;
         }
     }
     return s0;
@@ -511,18 +509,16 @@ __device__ __forceinline__ bool scene_runs64(const DevScene &S)
 }
 
 // Full scene evaluation (Sec. 2.3): every region, then the bounding box.
-template <bool G>
-__device__ __forceinline__ Eval64 scene_eval64(const DevScene &S, double x, double y, double z, int sel)
+__device__ __forceinline__ Eval64 scene_eval64(const DevScene &S, double x, double y, double z)
 {
     Eval64 E;
     E.dmin = __longlong_as_double(0x7ff0000000000000LL);
     E.dsoft = E.dmin;
-    E.dstar = 0.0; E.dsel = 0.0; E.istar = -1; E.region = -1;
-    run_prog64<true, G>(S, 0, S.ninstr, x, y, z, sel, &E);
+    E.dstar = 0.0; E.istar = -1; E.region = -1;
+    run_prog64<true, true>(S, 0, S.ninstr, x, y, z, &E);
     const double db = box64(x, y, z, S.bbc[0], S.bbc[1], S.bbc[2], S.bbh[0], S.bbh[1], S.bbh[2]);
     E.dbox = db;
     if (fabs(db) < E.dmin) { E.dmin = fabs(db); E.istar = -1; E.dstar = db; }
-    if (sel == -1) E.dsel = db;
     return E;
 }
 
@@ -554,7 +550,6 @@ __device__ __forceinline__ float culled_region32(const DevScene &S, float x, flo
         }
         return fminf(acc, S.cull_rmax);
     }
-    if (K == kTreeScene) return S.cull_rmax;     // not reached
     int i = __ldg(S.cull_list + o0);
     float acc = prim32<false>(S, (*(S.pkind + i)), i, x, y, z);   // culled regions are plain
     for (int j = o0 + 1; j < o1; ++j) {
@@ -790,7 +785,7 @@ __device__ __forceinline__ double surface64(const DevScene &S, int r, double x, 
 {
     if (r < 0) return box64(x, y, z, S.bbc[0], S.bbc[1], S.bbc[2], S.bbh[0], S.bbh[1], S.bbh[2]);
     const int2 rr = (*(S.rrange + r));
-    return run_prog64<false, G>(S, rr.x, rr.y, x, y, z, -2, nullptr);
+    return run_prog64<false, G>(S, rr.x, rr.y, x, y, z, nullptr);
 }
 
 // ---------------------------------------------------------------------------
@@ -1044,7 +1039,6 @@ static __device__ __noinline__ double seg_xprim64(const DevScene &S, int kind, i
 // bound, then each listed primitive with margin e = m + delta/2 (its
 // regions' sum of k/4): 0 when |d| <= e, passed over when |d| - e cannot
 // lower the bound so far, else its ray bound.
-template <bool G>
 static __device__ __noinline__ double segment_bound64(const DevScene &S, double dsoft, double dbox, double px,
                                                       double py, double pz, double ux, double uy, double uz)
 {
@@ -1056,7 +1050,7 @@ static __device__ __noinline__ double segment_bound64(const DevScene &S, double 
         const int i = __ldg(S.seg_prims + j);
         const int kind = (*(S.pkind + i));
         const double e = __ldg(S.seg_m64 + j) + dh;
-        const double d = prim64<G>(S, kind, i, px, py, pz);
+        const double d = prim64<true>(S, kind, i, px, py, pz);
         if (!(fabs(d) > e)) return 0.0;
         if (fabs(d) - e >= t) continue;
         double b;
@@ -1066,7 +1060,7 @@ static __device__ __noinline__ double segment_bound64(const DevScene &S, double 
             const double *P = S.p64 + 8 * i;
             b = seg_box64(__ldg(P), __ldg(P + 1), __ldg(P + 2), __ldg(P + 3), __ldg(P + 4), __ldg(P + 5), d, px,
                           py, pz, ux, uy, uz, e);
-        } else if (!G || kind == 2) {
+        } else if (kind == 2) {
             b = seg_capsule64(S.p64 + 8 * i, d, px, py, pz, ux, uy, uz, e);
         } else if (kind & kXformFlag) {
             b = seg_xprim64(S, kind & 0xf, i, d, px, py, pz, ux, uy, uz, e);

@@ -290,7 +290,7 @@ static __device__ __noinline__ Eval64 scene_exact(const DevScene &S, double x, d
 {
     Eval64 E;
     E.dmin = __longlong_as_double(0x7ff0000000000000LL);
-    E.dstar = 0.0; E.dsel = 0.0; E.istar = -1; E.region = -1;
+    E.dstar = 0.0; E.istar = -1; E.region = -1;
     E.dsoft = (double)C.soft;
     E.dbox = (double)C.db;
     unsigned long long neg = C.neg, mask = C.mask;
@@ -346,7 +346,7 @@ static __device__ __noinline__ double surface_at64(const DevScene &S, int r, dou
 template <int K>
 static __device__ __noinline__ int region_at64(const DevScene &S, double x, double y, double z, int r, FoldNear f)
 {
-    if (K == kGeneralScene) return scene_eval64<K == kGeneralScene>(S, x, y, z, -2).region;
+    if (K == kGeneralScene) return scene_eval64(S, x, y, z).region;
     const Screen64 C = scene_screen<K>(S, (float)x, (float)y, (float)z, kForRegion, f.cnt >= 0 ? r : -1, f.list, f.cnt);
     return scene_exact<K>(S, x, y, z, C, kForRegion).region;
 }
