@@ -424,11 +424,15 @@ int occupancy_mixed_multi(int threads, int variant = 0);
 // autotuner chose a shape, one block of 128 threads per SM with the largest
 // register budget (variant 2): one warp per scheduler nearly fills the FP64
 // pipe, and four warps disturb one another's instruction fetch less than
-// twelve.  Measured, 1 x 128 against 3 x 128: layered slab 1e4 packets 13.3
-// / 17.6 ms, 1e5 42.6 / 45.1; vessel tree 1e4 25.7 / 34.0; glass container
-// 3e4 48.6 / 58.3; thick slab 3e3 109.9 / 117.0; sphere 1e5, sphere tracing,
-// 65.4 / 62.2 ms.  From the limit on the wider launch won (before the scene
-// families: glass container 5e5 237 / 232 ms, sphere 1e6 324 / 285).
+// twelve.  Measured, 1 x 128 against the 3 x 128 that larger launches run:
+// layered slab 1e4 packets 13.5 / 17.4 ms, 1e5 41.5 / 44.3; vessel tree 1e4
+// 26.8 / 35.5, 4e4 38.8 / 55.5; glass container 1e4 36.8 / 43.0, 1e5 74.5 /
+// 79.5; shape gallery (general) 1e3 86.9 / 91.5, 1e4 191 / 221, 1e5 559 / 629,
+// with sphere tracing 849 / 891.  Packets of short, even lives are better off
+// with the wider launch well below the limit: sphere 1e4 3.5 / 4.6 ms, 1e5 10.9
+// / 10.5, 5e5 47 / 40, with sphere tracing 163 / 146; layered slab 4e5 137 /
+// 131, with sphere tracing 206 / 168; glass sphere in a beam 3e5 6.0 / 4.2;
+// homogeneous sphere 1e5 19.2 / 16.1.
 constexpr uint64_t kFewFp64Packets = 1u << 19;
 constexpr int kFewFp64Variant = 2;
 

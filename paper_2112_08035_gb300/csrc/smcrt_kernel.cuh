@@ -91,9 +91,9 @@ __device__ __forceinline__ float u01_32(uint32_t w) { return ((float)(w >> 9) + 
 // Taylor series of sin to a^17, cos to a^16 on |a| <= pi/4.
 // ---------------------------------------------------------------------------
 // FP64 quotient and square root, one copy each: a call costs far less than
-// the ten or so FP64 instructions (16 cycles each) it leads to, while inline
-// copies made the FP64 kernel 194 KB of code, more than the instruction cache
-// holds (15 cycles of fetch stall per instruction).
+// the ten or so FP64 instructions it leads to (64 cycles of a scheduler each),
+// while inline copies made the FP64 kernel 194 KB of code, more than the
+// instruction cache holds (15 cycles of fetch stall per instruction).
 static __device__ __noinline__ double div64(double a, double b) { return a / b; }
 static __device__ __noinline__ double sqrt64(double a) { return sqrt(a); }
 

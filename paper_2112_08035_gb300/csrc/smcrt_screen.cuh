@@ -1,8 +1,8 @@
 // smcrt_screen.cuh -- FP32 screening for the FP64 packet kernel.
 //
-// GB300 has one FP64 pipe per SM, which takes 16 cycles for a warp
-// instruction: one FP64 operation costs as much issue time as 64 FP32 or
-// integer ones.  The kernel's results must be the reference's IEEE
+// An FP64 warp instruction takes a scheduler of GB300 64 cycles (measured; an
+// SM's four schedulers start one every 16 cycles between them, 19 with all at
+// it): as much issue time as 64 FP32 or integer ones.  The kernel's results must be the reference's IEEE
 // operations on the values that count, but most values do not: the distance
 // of a region that is not the nearest, the plane of an axis that the ray
 // does not reach, a move's bound when the packet interacts before it.  Here
