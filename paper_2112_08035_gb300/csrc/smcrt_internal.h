@@ -440,15 +440,15 @@ constexpr int kFewFp64Variant = 2;
 // (variant 1) unless the caller or the autotuner chose a shape, and 5 blocks
 // with 96 registers (variant 0) from this many packets on in scenes without
 // a cell list.  General scenes run 3 blocks (variant 2): their code exceeds the
-// instruction cache (9.6 cycles of fetch stall per instruction), and fewer
-// warps disturb one another's fetch less.  Measured, variant 0 / 1: layered slab 1e5
-// packets 3.22 / 3.03 ms, 5e5 7.36 / 7.83, 1e6 12.9 / 14.0, 1e7 111 / 124;
+// instruction cache (9.6 cycles of fetch stall per instruction with four
+// blocks, 6.6 with three), and fewer warps disturb one another's fetch less.
+// Measured, variant 0 / 1: layered slab 1e5 packets 3.22 / 3.03 ms, 5e5 7.36 / 7.83, 1e6 12.9 / 14.0, 1e7 111 / 124;
 // with sphere tracing 4e5 15.0 / 14.7, 1e6 25.3 / 25.6; glass container 5e5
 // 15.4 / 15.0, 1e6 21.4 / 21.6; thick slab 1e5 27.3 / 24.2, 4e5 37.6 / 35.3,
 // 1e6 65.7 / 66.5; vessel tree 1e5 21.1 / 19.7, 4e6 98 / 96 ms; shape gallery,
-// variants 0 / 1 / 2, 3e4 26.8 / 25.4 / 23.9, 5e5 126 / 127 / 122, 1e6 172 /
-// 178 / 171, with sphere tracing 5e5 316 / 312 / 300.  (Layered slabs alone would cross over at
-// 2e5; thick ones and sphere tracing near 1e6.)
+// variants 0 / 1 / 2, 3e4 18.2 / 18.3 / 17.2, 1e5 53.2 / 53.7 / 49.1, 5e5 84.7 /
+// 87.3 / 81.5, with sphere tracing 316 / 312 / 300.  (Layered slabs alone would
+// cross over at 2e5; thick ones and sphere tracing near 1e6.)
 //
 // Scenes without an index step, whose packets meet no Fresnel surface, cross
 // over earlier: homogeneous sphere (isotropic, optical radius 10) 6e4 packets
