@@ -291,11 +291,12 @@ cudaError_t launch_kernel(int precision, JobWork *jobs, int njobs, int *status, 
                                    : launch_mixed(jobs, njobs, status, blocks, threads, s, variant);
 }
 
-uint64_t shape_key(const smcrt_scene *sc, int precision, const smcrt_grid *g)
+uint64_t shape_key(const smcrt_scene *sc, int precision, const smcrt_grid *g, int family)
 {
     uint64_t h = 1469598103934665603ull;
     auto mix = [&](uint64_t v) { h = (h ^ v) * 1099511628211ull; };
     mix((uint64_t)precision);
+    mix((uint64_t)family);
     mix((uint64_t)sc->stepping);
     mix((uint64_t)sc->nxforms);
     mix((uint64_t)sc->nprims);
@@ -678,7 +679,7 @@ int build_plan(smcrt_ctx *ctx, const smcrt_scene *sc, const smcrt_source *src, c
         return SMCRT_ERR_NO_MEMORY;
     }
     pl->cells = (size_t)g->n[0] * g->n[1] * g->n[2];
-    pl->shape_key = shape_key(sc, precision, g);
+    pl->shape_key = shape_key(sc, precision, g, scene_family(precision, pl->host));
     pl->time_limit_s = ctx->time_limit_s;
     {
         std::lock_guard<std::mutex> lk(ctx->tune_mu);
