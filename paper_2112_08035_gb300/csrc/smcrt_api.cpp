@@ -701,9 +701,8 @@ void default_launch(const smcrt_plan *pl, uint64_t npackets, int &blocks, int &t
         return;
     }
     // blocks 0 beside a chosen number of threads: all that are resident
-    const bool shaped = pl->blocks > 0 || pl->threads > 0, fp64 = pl->precision == SMCRT_FP64;
-    const bool few = fp64 && !pl->chosen && !shaped && npackets < kFewFp64Packets;
-    variant = pl->chosen ? pl->variant : default_variant(pl->precision, fp64 && !few ? kFewFp64Packets : npackets, pl->host);
+    const bool few = pl->precision == SMCRT_FP64 && !pl->chosen && pl->threads == 0 && npackets < kFewFp64Packets;
+    variant = pl->chosen ? pl->variant : default_variant(pl->precision, npackets, pl->host);
     threads = pl->threads > 0 ? pl->threads : 128;
     blocks = pl->blocks;
     if (blocks <= 0) {

@@ -27,10 +27,9 @@ def _warps(plan, wl):
 
 @pytest.mark.parametrize("threads", [32, 64, 128])
 def test_blocks_zero_means_all_resident_blocks(threads):
-    """One block per SM against blocks = 0 with the same threads: at least
-    two blocks of up to 128 threads fit on an SM (a third of the registers
-    each), so the second runs about that many times the warps; midway is the
-    limit."""
+    """One block per SM against blocks = 0 with the same threads: at least two
+    blocks of up to 128 threads are resident on an SM, so the second runs about
+    that many times the warps; midway is the limit."""
     import torch
     sms = torch.cuda.get_device_properties(0).multi_processor_count
     ctx = smc.Context(0)
