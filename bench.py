@@ -682,7 +682,7 @@ def main():
                                     "achieved_per_s": tipp * args.packets / kernel_s, "peak_per_s": issue_peak,
                                     "frac": tipp * args.packets / kernel_s / issue_peak,
                                     "note": "thread instructions per packet from the ncu summary in profiles/ "
-                                            "(2e5-packet capture of this kernel source)"}
+                                            "(2e6-packet capture of this kernel source)"}
     out["counters_per_packet"] = {k: totals_mixed[k] / args.packets for k in
                                   ("steps", "scene_evals", "scatters", "interfaces", "fresnel", "pieces")}
     out["counters_per_packet"]["refined_fraction_of_fresnel"] = (
